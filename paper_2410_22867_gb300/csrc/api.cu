@@ -465,6 +465,8 @@ dp_status upload_weights(Model* m) {
   if (m->prec == DP_MIX_BF16 || m->prec == DP_MIX_FP16) {
     DP_TRY(launch_tc_setup(m));
     DP_TRY(launch_emb_images(m));
+  } else {
+    DP_TRY(dig_upload(m));
   }
   return DP_OK;
 }
@@ -579,6 +581,10 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
     A_(vir_rep, 72 * R + 64);
     A_(tc_weights, mix_fit_weight_bytes(nt));
     A_(emb_img, mix_emb_image_bytes(nt));
+  } else {
+    A_(dig_emb, dig_emb_bytes(nt, prec == DP_FP64));
+    A_(dig_dT, es * N * (4 * kN3 + 4));
+    if (prec == DP_FP64) A_(dig_tanh, dig_tanh_bytes());
   }
   m->pg_cap = std::min(max_atoms, kPgAtoms);
   m->pg_roff_cap = 2 * (size_t)nt * N + 64;
@@ -598,6 +604,10 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
   m->geom_host = m->geom_stage[0];
   if (halloc(m, &m->err_host, 64) != DP_OK) return fail(DP_ERR_OOM, m->last_error);
 
+  if (prec == DP_FP64) {
+    dp_status s0 = dig_upload_tanh(m);
+    if (s0 != DP_OK) return fail(s0, m->last_error);
+  }
   {
     dp_status s1 = upload_weights(m);
     if (s1 != DP_OK) return fail(s1, m->last_error);

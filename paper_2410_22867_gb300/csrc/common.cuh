@@ -176,6 +176,11 @@ struct Model {
   int* err = nullptr;         // sticky error word
   int* err_host = nullptr;    // pinned
   int* small_i = nullptr;     // [64] device: small integer tables (sel, offsets)
+  // FP64 / FP32: embedding weights as digit fragments (emb_digits.cu), the table of its tanh, dE/dT
+  void* dig_emb = nullptr;
+  void* dig_tanh = nullptr;
+  void* dig_dT = nullptr;     // [N][100][4], then [N][4] maxima
+  bool dig_ok = false;        // the weights are within the range of the fixed-point layers
   // mixed-precision path
   int* rowoff = nullptr;      // [nt][N + 1] row offsets of each atom in the per-type neighbour streams
   int* scan_blk = nullptr;    // [nt][N / 1024 + 1]
@@ -238,8 +243,9 @@ struct Model {
 inline int cdiv(long a, long b) { return (int)((a + b - 1) / b); }
 
 // Raise a kernel's dynamic shared-memory limit once (not from inside stream capture
-// after the first call: the attribute call is skipped when already large enough).
-inline cudaError_t ensure_smem(const void* fn, size_t smem) {
+// after the first call: the attribute call is skipped when already large enough).  one_cta: a kernel that
+// runs one CTA per SM and reads weights through L1 gets no larger carveout than it needs.
+inline cudaError_t ensure_smem(const void* fn, size_t smem, bool one_cta = false) {
   static std::mutex mu;  // models may be driven from several host threads
   static std::vector<std::pair<const void*, size_t>> done;
   std::lock_guard<std::mutex> lock(mu);
@@ -247,7 +253,9 @@ inline cudaError_t ensure_smem(const void* fn, size_t smem) {
     if (e.first == fn && e.second >= smem) return cudaSuccess;
   cudaError_t err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err == cudaSuccess)  // prefer the largest shared-memory carveout so several CTAs fit per SM
-    err = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    err = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                               one_cta ? (int)std::min<size_t>(100, (smem + 2048) * 100 / (228 * 1024) + 1)
+                                       : (int)cudaSharedmemCarveoutMaxShared);
   if (err == cudaSuccess) done.push_back({fn, smem});
   return err;
 }
@@ -318,6 +326,13 @@ dp_status launch_pad_rows(Model* m);  // pad64 / pad32 from the current weights 
 dp_status launch_descriptor(Model* m, int N);
 dp_status launch_fitting(Model* m, int N);
 dp_status launch_embed_backward(Model* m, int N);
+// emb_digits.cu (FP64 / FP32 embedding net as digit products on the tensor cores)
+size_t dig_emb_bytes(int ntypes, bool fp64);
+size_t dig_tanh_bytes();
+dp_status dig_upload_tanh(Model* m);
+dp_status dig_upload(Model* m);
+dp_status launch_dig_descriptor(Model* m, int N);
+dp_status launch_dig_embed_backward(Model* m, int N);
 // mix_embed.cu (tensor-core embedding net)
 dp_status launch_mix_descriptor(Model* m, int N);
 dp_status launch_mix_embed_backward(Model* m, int N);

@@ -679,6 +679,7 @@ dp_status launch_pad_rows(Model* m) {
 
 dp_status launch_descriptor(Model* m, int N) {
   if (is_mixed(m)) return launch_mix_descriptor(m, N);
+  if (m->dig_ok && m->tab_n == 0) return launch_dig_descriptor(m, N);
   return m->prec == DP_FP64 ? run_descriptor<double>(m, N) : run_descriptor<float>(m, N);
 }
 dp_status launch_fitting(Model* m, int N) {
@@ -687,6 +688,7 @@ dp_status launch_fitting(Model* m, int N) {
 }
 dp_status launch_embed_backward(Model* m, int N) {
   if (is_mixed(m)) return launch_mix_embed_backward(m, N);
+  if (m->dig_ok && m->tab_n == 0) return launch_dig_embed_backward(m, N);
   return m->prec == DP_FP64 ? run_embed_backward<double>(m, N) : run_embed_backward<float>(m, N);
 }
 
