@@ -429,36 +429,17 @@ extern "C" {
 const char* dp_version(void) { return "dpgb300 0.1"; }
 
 // Device copies of the parameters from m->theta_host (and davg / dstd): theta in FP64 and
-// FP32, transposed fitting weights, normalisation statistics, and for the mixed precisions
-// the 16-bit tensor-core operand copies.  Synchronous.
+// FP32, normalisation statistics, and the tensor-core operand copies: 16-bit ones for the mixed
+// precisions, digit fragments for FP64 / FP32.  Synchronous.
 dp_status upload_weights(Model* m) {
   const int nt = m->ntypes;
   const std::vector<double>& theta = m->theta_host;
-  const size_t tsz = (size_t)kF * kKD + 2 * (size_t)kF * kF;
   std::vector<float> t32(theta.begin(), theta.end());
-  std::vector<double> wT(tsz * nt);
-  const size_t emb_total = (size_t)nt * nt * kEmbParams;
-  for (int t = 0; t < nt; ++t) {
-    const double* Pf = theta.data() + emb_total + (size_t)t * kFitParams;
-    double* dst = wT.data() + t * tsz;
-    for (int k = 0; k < kKD; ++k)
-      for (int o = 0; o < kF; ++o) dst[(size_t)o * kKD + k] = Pf[kFW1 + (size_t)k * kF + o];
-    double* d2 = dst + (size_t)kF * kKD;
-    double* d3 = d2 + (size_t)kF * kF;
-    for (int k = 0; k < kF; ++k)
-      for (int o = 0; o < kF; ++o) {
-        d2[(size_t)o * kF + k] = Pf[kFW2 + (size_t)k * kF + o];
-        d3[(size_t)o * kF + k] = Pf[kFW3 + (size_t)k * kF + o];
-      }
-  }
-  std::vector<float> wT32(wT.begin(), wT.end());
   std::vector<double> stat(8 * nt);
   for (int q = 0; q < 4 * nt; ++q) { stat[q] = m->davg_host[q]; stat[4 * nt + q] = 1.0 / m->dstd_host[q]; }
   std::vector<float> stat32(stat.begin(), stat.end());
   DP_CUDA_TRY(m, cudaMemcpy(m->w64, theta.data(), 8 * theta.size(), cudaMemcpyHostToDevice));
   DP_CUDA_TRY(m, cudaMemcpy(m->w32, t32.data(), 4 * t32.size(), cudaMemcpyHostToDevice));
-  DP_CUDA_TRY(m, cudaMemcpy(m->fitT64, wT.data(), 8 * wT.size(), cudaMemcpyHostToDevice));
-  DP_CUDA_TRY(m, cudaMemcpy(m->fitT32, wT32.data(), 4 * wT32.size(), cudaMemcpyHostToDevice));
   DP_CUDA_TRY(m, cudaMemcpy(m->stat64, stat.data(), 8 * stat.size(), cudaMemcpyHostToDevice));
   DP_CUDA_TRY(m, cudaMemcpy(m->stat32, stat32.data(), 4 * stat32.size(), cudaMemcpyHostToDevice));
   DP_TRY(launch_pad_rows(m));
@@ -467,6 +448,7 @@ dp_status upload_weights(Model* m) {
     DP_TRY(launch_emb_images(m));
   } else {
     DP_TRY(dig_upload(m));
+    DP_TRY(dig_fit_upload(m));
   }
   return DP_OK;
 }
@@ -544,9 +526,6 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
 #define A_(p, bytes) do { dp_status s_ = dalloc(m, &m->p, (bytes)); if (s_ != DP_OK) return fail(s_, m->last_error); } while (0)
   A_(w64, 8 * P.theta.size());
   A_(w32, 4 * P.theta.size());
-  const size_t tsz = (size_t)kF * kKD + 2 * (size_t)kF * kF;
-  A_(fitT64, 8 * tsz * nt);
-  A_(fitT32, 4 * tsz * nt);
   A_(stat64, 8 * 8 * nt);
   A_(stat32, 4 * 8 * nt);
   A_(pad64, 8 * (size_t)nt * nt * 4 * kN3);
@@ -584,6 +563,8 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
   } else {
     A_(dig_emb, dig_emb_bytes(nt, prec == DP_FP64));
     A_(dig_dT, es * N * (4 * kN3 + 4));
+    A_(dig_fit, dig_fit_bytes(nt, prec == DP_FP64));
+    A_(dig_max, 4 * 4 * N);
     if (prec == DP_FP64) A_(dig_tanh, dig_tanh_bytes());
   }
   m->pg_cap = std::min(max_atoms, kPgAtoms);

@@ -88,8 +88,6 @@ struct Model {
   // weights (device)
   double* w64 = nullptr;      // theta FP64 (blob order)
   float* w32 = nullptr;       // theta FP32
-  double* fitT64 = nullptr;   // per type: W1^T [kF][kKD], W2^T [kF][kF], W3^T [kF][kF]
-  float* fitT32 = nullptr;
   double* stat64 = nullptr;   // davg [nt][4], 1/dstd [nt][4]
   float* stat32 = nullptr;
   // One padded neighbour slot's contribution to S*T per (ti, tj): R_pad^T G(R_pad_0), c-major
@@ -180,6 +178,8 @@ struct Model {
   void* dig_emb = nullptr;
   void* dig_tanh = nullptr;
   void* dig_dT = nullptr;     // [N][100][4], then [N][4] maxima
+  void* dig_fit = nullptr;    // fitting weights as digit fragments (fit_digits.cu)
+  void* dig_max = nullptr;    // [4][N] top bits of the largest element of a row: D, dz3, dz2, dz1
   bool dig_ok = false;        // the weights are within the range of the fixed-point layers
   // mixed-precision path
   int* rowoff = nullptr;      // [nt][N + 1] row offsets of each atom in the per-type neighbour streams
@@ -333,6 +333,10 @@ dp_status dig_upload_tanh(Model* m);
 dp_status dig_upload(Model* m);
 dp_status launch_dig_descriptor(Model* m, int N);
 dp_status launch_dig_embed_backward(Model* m, int N);
+// fit_digits.cu (FP64 / FP32 fitting net as digit products)
+size_t dig_fit_bytes(int ntypes, bool fp64);
+dp_status dig_fit_upload(Model* m);
+dp_status launch_dig_fitting(Model* m, int N);
 // mix_embed.cu (tensor-core embedding net)
 dp_status launch_mix_descriptor(Model* m, int N);
 dp_status launch_mix_embed_backward(Model* m, int N);

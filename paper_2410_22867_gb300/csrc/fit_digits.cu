@@ -1,0 +1,503 @@
+// FP64 / FP32 fitting net (1600 -> 240 -> 240 -> 240 -> 1, forward and data gradient) with digit
+// products on the tensor cores (digits.cuh): seven launches for all centre types.
+//
+// A GEMM C = A B works on the atoms of one type (rows) and one weight matrix, whose digits are stored as
+// m16n8k16 B fragments (built once per weight upload, 15.7 MB a type in FP64, resident in L2).  A is read
+// in FP64 / FP32 and cut into digits on the way: lane (g, t) of a warp loads four consecutive k of rows
+// g and g + 8, which are its A fragment when k = 16 s + 4 t + {0, 1, 2, 3} stands at the fragment's columns
+// 2t, 2t + 1, 2t + 8, 2t + 9.  Rows carry a power of two of their own (largest element of the row, or
+// the bound of an activation), matrices one.
+//
+// Eight warps a CTA share a tile of 16 (8 / WK) rows: WK warps split K (their sums meet in shared
+// memory), so that a box of a few hundred atoms, where 16-row tiles times column blocks do not fill
+// 152 SMs, is not one long serial chain of K; with many atoms WK = 1 and the warps read the same
+// fragments through L1.
+#include <cmath>
+
+#include "digits.cuh"
+#include "tc_common.cuh"
+
+namespace dpg {
+namespace {
+
+using dig::Fmt;
+
+constexpr int kMats = 6;  // W1, W2, W3 (forward), W3^T, W2^T, W1^T (backward)
+struct Mat {
+  int K, N;
+};
+__host__ __device__ __forceinline__ Mat mat_of(int q) {
+  return q == 0 ? Mat{kKD, kF} : q == 5 ? Mat{kF, kKD} : Mat{kF, kF};
+}
+// fragment sets (n-tile, k step) before matrix q of a type
+__host__ __device__ __forceinline__ int mat_off(int q) {
+  constexpr int big = (kKD / 16) * (kF / 8), small = (kF / 16) * (kF / 8);
+  return q == 0 ? 0 : big + (q - 1) * small;
+}
+constexpr int kTypeFrags = 2 * (kKD / 16) * (kF / 8) + 4 * (kF / 16) * (kF / 8);
+
+template <class T> struct NTiles { static constexpr int v = sizeof(T) == 8 ? 3 : 6; };  // n-tiles of a warp
+// k steps whose digit products stay below 2^24 in the accumulators: 7 x 128 x 2^14, 3 x 80 x 2^16
+template <class T> struct Flush { static constexpr int v = sizeof(T) == 8 ? 8 : 5; };
+constexpr int kWarps = 8;
+
+enum EpiMode { EPI_TANH = 0, EPI_RES_TANH = 1, EPI_BWD = 2, EPI_NONE = 3 };
+
+template <class T>
+struct GemmArgs {
+  int ntypes, mat, mode;
+  const int* type_off;
+  const int* type_count;
+  const uint4* frag;       // [type][kTypeFrags][Q][32]
+  const int* wscale;       // [type][kMats]: |W| 2^sw within the digits' range
+  const T* A;              // [rows][K]
+  const unsigned* rowmax;  // [rows] top bits of each row's largest |a|, or null: |a| < 2^a_exp
+  int a_exp;
+  const T* w4;             // B3: the bound of dz3 is max |w4| of the type (in w4max), residual w4
+  T* C;                    // [rows][N]
+  const T* bias;           // theta: bias of type 0 (types bias_stride apart)
+  long stride;             // parameters of a fitting block
+  const T* res;            // [rows][N] or, with res_vec, [N] of type 0
+  int res_vec;
+  const T* aux_in;
+  T* aux_out;
+  unsigned* outmax;        // row maxima of C, or null
+};
+
+// Top bits of |v|: the high word of a double, a float's bits; ordered as unsigned integers.
+__device__ __forceinline__ unsigned top_bits(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned top_bits(float v) { return (unsigned)__float_as_int(v) & 0x7fffffffu; }
+// Exponent e with |v| < 2^e for all v with these top bits; not finite: a large one.
+__device__ __forceinline__ int exp_of(unsigned b, double) { return max((int)(b >> 20) - 1022, -800); }
+__device__ __forceinline__ int exp_of(unsigned b, float) {  // with the margin the full digit range needs
+  return max((int)((b + 0x10000u) >> 23) - 126, -80);
+}
+template <class T> struct RowBits { static constexpr int v = sizeof(T) == 8 ? 54 : 26; };
+
+// v 2^(54 - e) rounded, as integers do it (|v| < 2^e): the conversion instruction would take the FP64 pipe.
+__device__ __forceinline__ unsigned long long fix_digits(double v, int e) {
+  const int hi = __double2hiint(v);
+  const int ex = (hi >> 20) & 0x7ff;
+  const unsigned long long m = ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 33) |
+                               ((unsigned long long)(unsigned)__double2loint(v) << 1);  // mantissa x 2
+  const int r = min(max(1022 + e - ex, 0), 62);  // (m >> r): v 2^(54 - e) = m 2^(ex - 1076 + 54 - e)
+  const long long q = (long long)((m + ((1ull << r) >> 1)) >> r);
+  return dig::biased(hi < 0 ? -q : q);
+}
+__device__ __forceinline__ uint32_t fix_digits(float v, int e) {
+  return dig::biased(__float2int_rn(v * __int_as_float((127 + min(26 - e, 127)) << 23)));
+}
+
+__device__ __forceinline__ void load4(const double* p, double* v) {
+  const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
+  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+__device__ __forceinline__ void load4(const float* p, float* v) {
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+
+__device__ __forceinline__ double gtanh(double x) { return tanh(x); }
+__device__ __forceinline__ float gtanh(float x) { return tanhf(x); }
+
+// Running sums of a warp's outputs over flushes: joined integers (FP64, exact) or floats.
+template <class T> struct Sum;
+template <> struct Sum<double> {
+  long long hi = 0, lo = 0;
+  __device__ __forceinline__ void add(const float (*acc)[4], int e) {
+    const dig::Pair64 p = dig::join(acc, e);
+    hi += p.hi;
+    lo += p.lo;
+  }
+  __device__ __forceinline__ double value() const { return fma((double)hi, 4294967296.0, (double)lo); }
+};
+template <> struct Sum<float> {
+  float s = 0.f;
+  __device__ __forceinline__ void add(const float (*acc)[4], int e) { s += dig::join_f(acc, e); }
+  __device__ __forceinline__ float value() const { return s; }
+};
+__device__ __forceinline__ double out_scale(int e, int sw, double) {  // 2^(40 - (54 - e) - sw)
+  return e > 1024 ? __longlong_as_double(0x7ff8000000000000ll) : dig::pow2d(40 - 54 + e - sw);
+}
+__device__ __forceinline__ float out_scale(int e, int sw, float) {    // 2^(36 - (26 - e) - sw)
+  return e > 128 ? __int_as_float(0x7fc00000) : __int_as_float((127 + min(max(36 - 26 + e - sw, -126), 127)) << 23);
+}
+
+// The fragments run through shared memory in stages of KS k steps by cp.async, ST stages deep: with WK = 1 one
+// pipeline for the CTA (every warp multiplies the same fragments), else one for each warp.  Loads straight
+// into registers left each k step waiting for L2 (32,000 FP32 rows: 3.04 ms for the six GEMMs).
+template <class T, int WK> struct Pipe {
+  static constexpr int KS = (WK == 1 && sizeof(T) == 4) ? 2 : 1;
+  static constexpr int ST = WK == 1 ? 4 : 3;
+  static constexpr int kWords = KS * NTiles<T>::v * dig::Frag<T>::Q * 32;  // uint4 of a stage
+  static constexpr int kPipes = WK == 1 ? 1 : kWarps;
+  static constexpr size_t kBytes = (size_t)kPipes * ST * kWords * 16;
+};
+
+template <class T, int WK>
+__global__ void __launch_bounds__(32 * kWarps, 1) k_dig_gemm(GemmArgs<T> g) {
+  constexpr int ND = Fmt<T>::ND, NO = Fmt<T>::NO, Q = dig::Frag<T>::Q, NT = NTiles<T>::v, MW = kWarps / WK;
+  using P = Pipe<T, WK>;
+  static_assert(WK == 1 || P::kBytes >= sizeof(T) * kWarps * NT * 4 * 32, "the partial sums reuse the pipeline's memory");
+  extern __shared__ __align__(16) uint4 sm[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, kw = w % WK, mw = w / WK;
+  const int tq = lane & 3, gr = lane >> 2;
+  // the CTA's type and rows
+  int ty = 0, blk = blockIdx.x;
+  for (; ty < g.ntypes; ++ty) {
+    const int b = (g.type_count[ty] + 16 * MW - 1) / (16 * MW);
+    if (blk < b) break;
+    blk -= b;
+  }
+  if (ty == g.ntypes) return;
+  const int rows = g.type_count[ty], r0 = (blk * MW + mw) * 16;
+  const size_t base = (size_t)g.type_off[ty];
+  const Mat mt = mat_of(g.mat);
+  const int ntile0 = blockIdx.y * NT, ntiles = mt.N / 8, ksteps = mt.K / 16;
+  const uint4* fr = g.frag + ((size_t)ty * kTypeFrags + mat_off(g.mat)) * Q * 32;
+  const int sw = g.wscale[ty * kMats + g.mat];
+  int ea[2];
+  const T* ap[2];
+  bool ok[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int row = r0 + gr + 8 * r;
+    ok[r] = row < rows;
+    const size_t gi = base + (ok[r] ? row : 0);
+    ap[r] = g.A + gi * mt.K + 4 * tq;
+    ea[r] = g.rowmax ? exp_of(g.rowmax[gi], T(0)) : g.a_exp;
+  }
+  Sum<T> sum[NT][4];
+  {
+    float acc[NT][NO][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n) dig::zero_acc<T>(acc[n]);
+    const int k0 = ksteps * kw / WK, k1 = ksteps * (kw + 1) / WK;
+    const int nst = (k1 - k0 + P::KS - 1) / P::KS;
+    uint4* pipe = sm + (WK == 1 ? 0 : w) * P::ST * P::kWords;
+    auto issue = [&](int st) {
+      if (st < nst) {
+        uint4* dst = pipe + (st % P::ST) * P::kWords;
+        for (int q = WK == 1 ? (int)threadIdx.x : lane; q < P::kWords; q += WK == 1 ? 32 * kWarps : 32) {
+          const int ln = q % (Q * 32), f = q / (Q * 32), n = f % NT, s = k0 + st * P::KS + f / NT;
+          if (s < k1 && ntile0 + n < ntiles) tc::cp_async16(dst + q, fr + ((size_t)(ntile0 + n) * ksteps + s) * Q * 32 + ln);
+        }
+      }
+      tc::cp_async_commit();
+    };
+    T v[P::KS][2][4];
+    auto load_a = [&](int st) {
+#pragma unroll
+      for (int k = 0; k < P::KS; ++k) {
+        const int s = k0 + st * P::KS + k;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+          if (ok[r] && s < k1) load4(ap[r] + 16 * s, v[k][r]);
+      }
+    };
+#pragma unroll
+    for (int k = 0; k < P::KS; ++k)
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[k][r][q] = T(0);
+    for (int st = 0; st < P::ST - 1; ++st) issue(st);
+    load_a(0);
+    int left = Flush<T>::v;
+    for (int st = 0; st < nst; ++st) {
+      tc::cp_async_wait_group<P::ST - 2>();
+      if (WK == 1) __syncthreads();  // the stage has landed, and everyone is done with the one refilled next
+      else __syncwarp();
+      issue(st + P::ST - 1);
+      uint4 a[P::KS][ND];
+#pragma unroll
+      for (int k = 0; k < P::KS; ++k) {
+        uint32_t x[ND], y[ND], z[ND], u[ND];
+        dig::split2(fix_digits(v[k][0][0], ea[0]), fix_digits(v[k][0][1], ea[0]), x);
+        dig::split2(fix_digits(v[k][1][0], ea[1]), fix_digits(v[k][1][1], ea[1]), y);
+        dig::split2(fix_digits(v[k][0][2], ea[0]), fix_digits(v[k][0][3], ea[0]), z);
+        dig::split2(fix_digits(v[k][1][2], ea[1]), fix_digits(v[k][1][3], ea[1]), u);
+#pragma unroll
+        for (int i = 0; i < ND; ++i) a[k][i] = make_uint4(x[i], y[i], z[i], u[i]);
+      }
+      if (st + 1 < nst) load_a(st + 1);
+      const uint4* buf = pipe + (st % P::ST) * P::kWords + lane;
+#pragma unroll
+      for (int k = 0; k < P::KS; ++k) {
+        const int s = k0 + st * P::KS + k;
+        if (s >= k1) break;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          if (ntile0 + n < ntiles) {
+            uint4 b[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) b[q] = buf[((k * NT + n) * Q + q) * 32];
+            dig::block16<T>(acc[n], a[k], b);
+          }
+        }
+        if (--left == 0 || s + 1 == k1) {
+#pragma unroll
+          for (int n = 0; n < NT; ++n) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sum[n][e].add(acc[n], e);
+            dig::zero_acc<T>(acc[n]);
+          }
+          left = Flush<T>::v;
+        }
+      }
+    }
+    tc::cp_async_wait_group<0>();
+  }
+  T(*part)[NT * 4][32] = reinterpret_cast<T(*)[NT * 4][32]>(sm);  // [warp]
+  if (WK > 1) {
+    __syncthreads();  // every pipeline is drained
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) part[w][4 * n + e][lane] = sum[n][e].value();
+    __syncthreads();
+  }
+  if (r0 >= rows) return;
+  const T* bias = g.bias + (long)ty * g.stride;
+  const T* resv = g.res + (g.res_vec ? (long)ty * g.stride : 0);
+#pragma unroll
+  for (int q = 0; q < NT * 4; ++q) {
+    if (WK > 1 && q % WK != kw) continue;
+    const int n = q >> 2, e = q & 3, r = e >> 1;
+    T v;
+    if (WK > 1) {
+      v = T(0);
+#pragma unroll
+      for (int k = 0; k < WK; ++k) v += part[mw * WK + k][q][lane];
+    } else {
+      v = sum[n][e].value();
+    }
+    v *= out_scale(ea[r], sw, T(0));
+    const int col = 8 * (ntile0 + n) + 2 * tq + (e & 1);
+    const bool in = ok[r] && ntile0 + n < ntiles;
+    T out = T(0);
+    if (in) {
+      const size_t o = (base + r0 + gr + 8 * r) * mt.N + col;
+      if (g.mode == EPI_TANH) {
+        out = gtanh(v + bias[col]);
+      } else if (g.mode == EPI_RES_TANH) {
+        const T t = gtanh(v + bias[col]);
+        g.aux_out[o] = t;
+        out = g.res[o] + t;
+      } else if (g.mode == EPI_BWD) {
+        const T h = v + (g.res_vec ? resv[col] : g.res[o]);
+        const T f = g.aux_in[o];
+        if (g.aux_out) g.aux_out[o] = h;
+        out = h * (T(1) - f * f);
+      } else {
+        out = v;
+      }
+      g.C[o] = out;
+    }
+    if (g.outmax) {
+      unsigned m = in ? top_bits(out) : 0u;
+      m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+      m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+      if (in && tq == 0) atomicMax(g.outmax + base + r0 + gr + 8 * r, m);
+    }
+  }
+}
+
+// Row maxima of D (the descriptor), one warp a row.
+template <class T>
+__global__ void k_dig_rowmax(int N, const T* __restrict__ D, unsigned* out) {
+  const int lane = threadIdx.x & 31;
+  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (row >= N) return;
+  unsigned m = 0;
+  for (int q = 4 * lane; q < kKD; q += 128) {
+    T v[4];
+    load4(D + (size_t)row * kKD + q, v);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m = max(m, top_bits(v[k]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) out[row] = m;
+}
+
+template <class T>
+__device__ __forceinline__ T warp_sum(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// E_i = H3 . w4 + b4 + e_bias[t];  dZ3 = w4 * (1 - T3^2) written over H3, with its row maximum.
+template <class T>
+__global__ void k_dig_head(int N, const int* __restrict__ itype, T* H3, const T* __restrict__ T3,
+                           const T* __restrict__ fit, const T* __restrict__ ebias, double* e_atom, unsigned* outmax) {
+  const int lane = threadIdx.x & 31;
+  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (row >= N) return;
+  const int ty = itype[row];
+  const T* P = fit + (size_t)ty * kFitParams;
+  const size_t r = (size_t)row;
+  T e = T(0);
+  unsigned m = 0;
+  for (int n = lane; n < kF; n += 32) {
+    const T h = H3[r * kF + n], t = T3[r * kF + n], w = P[kFw4 + n];
+    e += h * w;
+    const T dz = w * (T(1) - t * t);
+    H3[r * kF + n] = dz;
+    m = max(m, top_bits(dz));
+  }
+  e = warp_sum<T>(e);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) {
+    e_atom[r] = (double)e + (double)P[kFb4] + (double)ebias[ty];
+    outmax[r] = m;
+  }
+}
+
+// ------------------------------------------------------------------ weights
+// Scale exponent of every matrix (one block each): the largest |w|.
+template <class T>
+__global__ void __launch_bounds__(1024) k_dig_fit_scale(const T* __restrict__ fit, int* wscale) {
+  __shared__ unsigned s[32];
+  const int ty = blockIdx.x / 3, q = blockIdx.x % 3;  // W1, W2, W3; the transposes share their scale
+  const T* W = fit + (size_t)ty * kFitParams + (q == 0 ? kFW1 : q == 1 ? kFW2 : kFW3);
+  const int n = (q == 0 ? kKD : kF) * kF;
+  unsigned m = 0;
+  for (int k = threadIdx.x; k < n; k += 1024) m = max(m, top_bits(W[k]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 32; ++k) m = max(m, s[k]);
+    const int e = max(exp_of(m, T(0)), sizeof(T) == 8 ? -60 : -30);
+    const int sw = RowBits<T>::v - e;
+    wscale[ty * kMats + q] = sw;
+    wscale[ty * kMats + 5 - q] = sw;
+  }
+}
+
+// B fragments: one warp per fragment set (n-tile, k step) of a type; rows k = 16 s + 4 t + {0..3}.
+template <class T>
+__global__ void __launch_bounds__(256) k_dig_fit_weights(const T* __restrict__ fit, const int* __restrict__ wscale,
+                                                        uint4* frag) {
+  constexpr int Q = dig::Frag<T>::Q;
+  const int f = blockIdx.x * 8 + (threadIdx.x >> 5), ty = blockIdx.y, lane = threadIdx.x & 31;
+  if (f >= kTypeFrags) return;
+  int q = 0;
+  while (q + 1 < kMats && f >= mat_off(q + 1)) ++q;
+  const Mat mt = mat_of(q);
+  const int ks = mt.K / 16, idx = f - mat_off(q), nt = idx / ks, s = idx % ks;
+  const int col = 8 * nt + (lane >> 2), k0 = 16 * s + 4 * (lane & 3);
+  const T* W = fit + (size_t)ty * kFitParams +
+               (q == 0 || q == 5 ? kFW1 : q == 1 || q == 4 ? kFW2 : kFW3);
+  const int e = RowBits<T>::v - wscale[ty * kMats + q];
+  decltype(fix_digits(T(0), 0)) u[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)  // q < 3: W[k][n]; transposes: W[n][k] of a matrix with K columns
+    u[k] = fix_digits(q < 3 ? W[(size_t)(k0 + k) * mt.N + col] : W[(size_t)col * mt.K + k0 + k], e);
+  uint32_t lo[2 * Q], hi[2 * Q];
+  lo[2 * Q - 1] = hi[2 * Q - 1] = 0u;
+  dig::split2(u[0], u[1], lo);
+  dig::split2(u[2], u[3], hi);
+  uint4* dst = frag + ((size_t)ty * kTypeFrags + f) * Q * 32 + lane;
+#pragma unroll
+  for (int p = 0; p < Q; ++p) dst[p * 32] = make_uint4(lo[2 * p], hi[2 * p], lo[2 * p + 1], hi[2 * p + 1]);
+}
+
+template <class T>
+const T* theta_of(const Model* m) {
+  return sizeof(T) == 8 ? reinterpret_cast<const T*>(m->w64) : reinterpret_cast<const T*>(m->w32);
+}
+
+template <class T>
+dp_status upload(Model* m) {
+  const T* fit = theta_of<T>(m) + (size_t)m->ntypes * m->ntypes * kEmbParams;
+  int* ws = static_cast<int*>(m->dig_fit);
+  uint4* fr = reinterpret_cast<uint4*>(static_cast<unsigned char*>(m->dig_fit) + 1024);
+  k_dig_fit_scale<T><<<3 * m->ntypes, 1024>>>(fit, ws);
+  k_dig_fit_weights<T><<<dim3(cdiv(kTypeFrags, 8), m->ntypes), 256>>>(fit, ws, fr);
+  m->launches += 2;
+  DP_LAUNCH_CHECK(m);
+  return DP_OK;
+}
+
+template <class T, int WK>
+dp_status gemm(Model* m, int N, const GemmArgs<T>& g) {
+  const int mt = 16 * (kWarps / WK);
+  DP_CUDA_TRY(m, ensure_smem(reinterpret_cast<const void*>(k_dig_gemm<T, WK>), Pipe<T, WK>::kBytes));
+  const dim3 grid(cdiv(N, mt) + m->ntypes, cdiv(mat_of(g.mat).N / 8, NTiles<T>::v));
+  k_dig_gemm<T, WK><<<grid, 32 * kWarps, Pipe<T, WK>::kBytes, m->stream>>>(g);
+  m->launches += 1;
+  DP_LAUNCH_CHECK(m);
+  return DP_OK;
+}
+
+template <class T>
+dp_status run(Model* m, int N) {
+  const T* theta = theta_of<T>(m);
+  const size_t emb = (size_t)m->ntypes * m->ntypes * kEmbParams;
+  const T* fit = theta + emb;
+  const T* ebias = fit + (size_t)m->ntypes * kFitParams;
+  T* act[5];
+  for (int q = 0; q < 5; ++q) act[q] = static_cast<T*>(m->act[q]);
+  unsigned* mx = static_cast<unsigned*>(m->dig_max);
+  const size_t R = (size_t)m->max_atoms;
+  DP_CUDA_TRY(m, cudaMemsetAsync(mx + 2 * R, 0, 4 * 2 * R, m->stream));
+  k_dig_rowmax<T><<<cdiv(N, 8), 256, 0, m->stream>>>(N, static_cast<const T*>(m->Dm), mx);
+  m->launches += 1;
+  GemmArgs<T> g{};
+  g.ntypes = m->ntypes; g.type_off = m->type_off; g.type_count = m->type_count;
+  g.wscale = static_cast<const int*>(m->dig_fit);
+  g.frag = reinterpret_cast<const uint4*>(static_cast<unsigned char*>(m->dig_fit) + 1024);
+  g.stride = kFitParams;
+  // rows in 16-row tiles times column blocks against the SMs decides how far K is split inside a CTA:
+  // below about two CTAs an SM with 128-row CTAs, all eight warps share 16 rows
+  auto go = [&](const GemmArgs<T>& a) {
+    const long ctas = (long)cdiv(N, 128) * cdiv(mat_of(a.mat).N / 8, NTiles<T>::v);
+    return ctas >= 4l * num_sms() ? gemm<T, 1>(m, N, a) : gemm<T, 8>(m, N, a);
+  };
+#define DP_GO(a)                      \
+  do {                                \
+    const dp_status s_ = go(a);       \
+    if (s_ != DP_OK) return s_;       \
+  } while (0)
+  // F1: H1 = tanh(D W1 + b1)
+  g.mat = 0; g.A = static_cast<const T*>(m->Dm); g.rowmax = mx; g.C = act[0]; g.bias = fit + kFb1; g.mode = EPI_TANH;
+  DP_GO(g);
+  // F2: T2 = tanh(H1 W2 + b2), H2 = H1 + T2   (|H1| <= 1 < 2^1, |H2| <= 2 < 2^2)
+  g.mat = 1; g.A = act[0]; g.rowmax = nullptr; g.a_exp = 1; g.C = act[2]; g.bias = fit + kFb2; g.res = act[0];
+  g.aux_out = act[1]; g.mode = EPI_RES_TANH;
+  DP_GO(g);
+  // F3: T3 = tanh(H2 W3 + b3), H3 = H2 + T3
+  g.mat = 2; g.A = act[2]; g.a_exp = 2; g.C = act[4]; g.bias = fit + kFb3; g.res = act[2]; g.aux_out = act[3];
+  DP_GO(g);
+  k_dig_head<T><<<cdiv(N, 8), 256, 0, m->stream>>>(N, m->itype, act[4], act[3], fit, ebias, m->e_atom, mx + R);
+  m->launches += 1;
+  // B3: dH2 = w4 + dZ3 W3^T ; dZ2 = dH2 (1 - T2^2)  (dH2 -> act[3], dZ2 -> act[2])
+  g.mat = 3; g.A = act[4]; g.rowmax = mx + R; g.C = act[2]; g.res = fit + kFw4; g.res_vec = 1; g.aux_in = act[1];
+  g.aux_out = act[3]; g.mode = EPI_BWD; g.outmax = mx + 2 * R;
+  DP_GO(g);
+  // B2: dH1 = dH2 + dZ2 W2^T ; dZ1 = dH1 (1 - H1^2)  (dZ1 -> act[1])
+  g.mat = 4; g.A = act[2]; g.rowmax = mx + 2 * R; g.C = act[1]; g.res = act[3]; g.res_vec = 0; g.aux_in = act[0];
+  g.aux_out = nullptr; g.outmax = mx + 3 * R;
+  DP_GO(g);
+  // B1: dD = dZ1 W1^T
+  g.mat = 5; g.A = act[1]; g.rowmax = mx + 3 * R; g.C = static_cast<T*>(m->dD); g.mode = EPI_NONE; g.outmax = nullptr;
+  DP_GO(g);
+#undef DP_GO
+  DP_LAUNCH_CHECK(m);
+  return DP_OK;
+}
+
+}  // namespace
+
+size_t dig_fit_bytes(int ntypes, bool fp64) {
+  return 1024 + (size_t)ntypes * kTypeFrags * 512 * (fp64 ? dig::Frag<double>::Q : dig::Frag<float>::Q);
+}
+dp_status dig_fit_upload(Model* m) { return m->prec == DP_FP64 ? upload<double>(m) : upload<float>(m); }
+dp_status launch_dig_fitting(Model* m, int N) { return m->prec == DP_FP64 ? run<double>(m, N) : run<float>(m, N); }
+
+}  // namespace dpg
