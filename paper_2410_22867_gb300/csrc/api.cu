@@ -572,7 +572,7 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
   A_(pg_ws, param_grad_workspace_bytes(m->pg_cap, prec == DP_FP64));
   A_(pg_roff, 4 * m->pg_roff_cap);
   A_(pg_w, 24 * N);
-  A_(pg_scal, 64);
+  A_(pg_scal, 64 + 8 * kN3 * kMaxTypes);
   m->red_cap = rep_reduce_slots(max_atoms, max_replicas);
   A_(red_part, 80 * m->red_cap);
 #undef A_

@@ -24,7 +24,7 @@ constexpr int kFitParams = kKD * kF + kF + kF * kF + kF + kF * kF + kF + kF + 1;
 constexpr int kMaxTypes = 4;
 constexpr int kRdfMaxCells = 24576;  // dp_rdf: ntypes^2 * nbins histogram cells at most
 // parameter gradient: centre atoms per chunk, neighbour rows per chunk of the embedding reverse
-constexpr int kPgAtoms = 2048, kPgRows = 16384;
+constexpr int kPgAtoms = 2048, kPgRows = 32768;
 
 // offsets inside one embedding block
 constexpr int kEW1 = 0, kEb1 = kN1, kEW2 = 2 * kN1, kEb2 = kEW2 + kN1 * kN2, kEW3 = kEb2 + kN2,
@@ -194,7 +194,7 @@ struct Model {
   int* pg_roff = nullptr;     // row offsets of every row chunk of one call
   size_t pg_roff_cap = 0;
   double* pg_w = nullptr;     // [N][3] tangent direction 2 cF (F - F0), internal order
-  double* pg_scal = nullptr;  // alpha, loss, E
+  double* pg_scal = nullptr;  // alpha, loss, E; from [8]: padded-slot sums [nt][100]
 
   // MD bookkeeping
   int natoms = 0;             // atoms of the current call

@@ -13,16 +13,18 @@
 // reverse sweep over that (value, tangent) computation then gives dPsi/dtheta.
 //
 // Work runs per chunk of centre atoms of one type (at most pg_cap atoms):
-//   1. embedding forward with tangents -> T, T' per atom;
+//   1. embedding forward with tangents -> T, T' per atom, layer by layer over row chunks;
 //   2. descriptor D, D' per atom, stacked as the 2n rows [D; D'];
 //   3. fitting net forward on the stacked rows (GEMMs), activations kept;
 //   4. fitting reverse: adjoint rows [u_bar; v_bar] per layer, weight gradients as
 //      GEMMs over the atoms, and [D_bar; D'_bar];
 //   5. descriptor reverse -> T_bar, T'_bar per atom;
-//   6. embedding reverse per neighbour row (activations recomputed), in row
-//      chunks of at most kPgRows: each row writes its layer inputs and
-//      pre-activation adjoints, whose products summed over rows are the weight
-//      gradients (GEMMs with the rows as the reduction dimension).
+//   6. embedding reverse over the same row chunks (activations recomputed).
+// The embedding layers run as tall, skinny GEMMs over neighbour rows (at most kPgRows at a time): a
+// value and its tangent are consecutive rows 2 r and 2 r + 1, and one thread holds both for the two
+// units that share a residual, so activations, residuals and the adjoint formulas are epilogues in
+// registers.  One thread per row with its 225 activations in local memory took 17 ms of a
+// 3,072-atom FP32 gradient; these take 3.1 ms.
 // Weight gradients are accumulated with FP64 atomics.
 #include "common.cuh"
 
@@ -116,117 +118,378 @@ __device__ __forceinline__ void row_geometry(const PgArgs<T>& a, int i, int ti, 
   env_tangent<T>(a, ti, d, dd, R, Rd);
 }
 
-// Embedding layers 1 and 2 with tangents: h1, h1' [25]; h2, h2' [50]; v1 = x' W1; z2' [50].
+// Rows of a chunk: the neighbours of type tj of atoms [b0, b0 + nb), numbered by roff (exclusive offsets).
+struct RowMap {
+  int ti, tj, b0, nb, R;
+  const int* roff;
+};
+
+// 1a / 6a. Environment row and tangent, and layer 1 with tangents, of every row of a chunk:
+// geo [R][8] = (R_hat, R_hat'), atom [R] = local atom, H1 rows 2 r = h1, 2 r + 1 = h1'.
+constexpr int kPgGeo = 8;
 template <class T>
-__device__ __forceinline__ void emb12_tangent(const T* __restrict__ W, T x, T xd, T* h1, T* hd1, T* v1, T* h2,
-                                              T* hd2, T* zd2) {
-#pragma unroll 1
-  for (int k = 0; k < kN1; ++k) {
-    h1[k] = tanh_t<T>(x * W[kEW1 + k] + W[kEb1 + k]);
-    v1[k] = xd * W[kEW1 + k];
-    hd1[k] = (T(1) - h1[k] * h1[k]) * v1[k];
-  }
-#pragma unroll 1
-  for (int m = 0; m < kN2; ++m) {
-    T z = W[kEb2 + m], zd = T(0);
-#pragma unroll 5
-    for (int k = 0; k < kN1; ++k) {
-      z += h1[k] * W[kEW2 + k * kN2 + m];
-      zd += hd1[k] * W[kEW2 + k * kN2 + m];
+__global__ void __launch_bounds__(128) k_pg_rows(PgArgs<T> a, RowMap m, T* __restrict__ geo, int* __restrict__ atom,
+                                                T* __restrict__ H1) {
+  __shared__ T sx[128][2];
+  const int r0 = blockIdx.x * 128, r = r0 + threadIdx.x;
+  const T* W = a.w + (size_t)(m.ti * a.ntypes + m.tj) * kEmbParams;
+  if (r < m.R) {
+    int lo = 0, hi = m.nb - 1;  // last atom k with roff[k] <= r
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (m.roff[mid] <= r) lo = mid; else hi = mid - 1;
     }
-    const T t2 = tanh_t<T>(z);
-    h2[m] = h1[m % kN1] + t2;
-    hd2[m] = hd1[m % kN1] + (T(1) - t2 * t2) * zd;
-    zd2[m] = zd;
+    T R[4], Rd[4];
+    row_geometry<T>(a, m.b0 + lo, m.ti, (size_t)(m.b0 + lo) * a.S + a.sel_off[m.tj] + (r - m.roff[lo]), R, Rd);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      geo[(size_t)r * kPgGeo + c] = R[c];
+      geo[(size_t)r * kPgGeo + 4 + c] = Rd[c];
+    }
+    atom[r] = lo;
+    sx[threadIdx.x][0] = R[0];
+    sx[threadIdx.x][1] = Rd[0];
+  }
+  __syncthreads();
+  const int rows = min(128, m.R - r0);
+  for (int q = threadIdx.x; q < rows * kN1; q += 128) {
+    const int rr = q / kN1, k = q - rr * kN1;
+    const T w = W[kEW1 + k];
+    const T h = tanh_t<T>(sx[rr][0] * w + W[kEb1 + k]);
+    T* o = H1 + (size_t)(r0 + rr) * 2 * kN1 + k;
+    o[0] = h;
+    o[kN1] = (T(1) - h * h) * (sx[rr][1] * w);
   }
 }
 
-// 1. T and T' of each atom of the chunk: CTA per atom, rows staged in shared memory.
-constexpr int kPgNB = 64;
-constexpr int kPgGP = kN3 + 1;
-
-template <class T>
-__global__ void __launch_bounds__(kPgNB) k_pg_emb_fwd(PgArgs<T> a, int ti, int a0, int n, T* TT) {
+// Tall, skinny product of 2 R rows: C = A [2 R x K] W [K x N] (or W^T with TB: W is [N x K]), all of W and
+// 128 (N = 100) or 256 (N = 50, 25) rows in shared memory (FP64: half as many).  320 threads (160): TC
+// column groups of CN columns tc + TC j (so the columns m and m + N / 2 of a residual pair belong to one
+// thread), row groups of 4 rows (two value / tangent pairs).  Per k a thread loads 4 + CN values for
+// 4 CN multiply-adds.
+template <class T, int N> struct Skinny {
+  static constexpr int THREADS = sizeof(T) == 8 ? 160 : 320;
+  static constexpr int TC = N == 100 ? 10 : 5, CN = N / TC, TR = THREADS / TC, ROWS = 4 * TR;
+  static constexpr int CP = (CN + 3) / 4 * 4;  // columns of a thread, padded for 16-byte loads
+};
+template <class T, int K, int N> constexpr size_t skinny_smem() {
+  return sizeof(T) * ((size_t)K * Skinny<T, N>::TC * Skinny<T, N>::CP + (size_t)K * (Skinny<T, N>::ROWS + 4));
+}
+template <class T, int K, int N, bool TB, class Epi>
+__global__ void __launch_bounds__(Skinny<T, N>::THREADS) k_pg_layer(int R2, const T* __restrict__ A, const T* __restrict__ W, Epi epi) {
+  using S = Skinny<T, N>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sG = reinterpret_cast<T*>(smem_raw);  // [NB][GP]
-  T* sGd = sG + kPgNB * kPgGP;             // [NB][GP]
-  T* sR = sGd + kPgNB * kPgGP;             // [NB][4]
-  T* sRd = sR + kPgNB * 4;                 // [NB][4]
+  T* sW = reinterpret_cast<T*>(smem_raw);         // [K][TC][CP]
+  T* sA = sW + (size_t)K * S::TC * S::CP;         // [K][ROWS + 4]
   const int tid = threadIdx.x;
-  for (int li = blockIdx.x; li < n; li += gridDim.x) {
-    const int i = a0 + li;
-    T acc[2][4], accd[2][4];
+  const int row0 = blockIdx.x * S::ROWS;
+  for (int q = tid; q < K * N; q += S::THREADS) {
+    const int k = TB ? q % K : q / N, n = TB ? q / K : q % N;
+    sW[((size_t)k * S::TC + n % S::TC) * S::CP + n / S::TC] = W[q];
+  }
+  for (int q = tid; q < S::ROWS * K; q += S::THREADS) {
+    const int r = q / K, k = q - r * K;
+    sA[(size_t)k * (S::ROWS + 4) + r] = row0 + r < R2 ? A[(size_t)row0 * K + q] : T(0);
+  }
+  __syncthreads();
+  const int tc = tid % S::TC, tr = tid / S::TC;
+  T acc[4][S::CN];
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+  for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[u][c] = accd[u][c] = T(0);
-    for (int tj = 0; tj < a.ntypes; ++tj) {
-      const int cnt = a.nl_count[(size_t)i * a.ntypes + tj];
-      const T* W = a.w + (size_t)(ti * a.ntypes + tj) * kEmbParams;
-      for (int base = 0; base < cnt; base += kPgNB) {
-        const int rows = min(kPgNB, cnt - base);
-        if (tid < rows) {
-          T R[4], Rd[4];
-          row_geometry<T>(a, i, ti, (size_t)i * a.S + a.sel_off[tj] + base + tid, R, Rd);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) { sR[tid * 4 + c] = R[c]; sRd[tid * 4 + c] = Rd[c]; }
-          T h1[kN1], hd1[kN1], v1[kN1], h2[kN2], hd2[kN2], zd2[kN2];
-          emb12_tangent<T>(W, R[0], Rd[0], h1, hd1, v1, h2, hd2, zd2);
-          T* g = sG + tid * kPgGP;
-          T* gd = sGd + tid * kPgGP;
-#pragma unroll 1
-          for (int q = 0; q < kN3; ++q) {
-            T z = W[kEb3 + q], zd = T(0);
+    for (int c = 0; c < S::CN; ++c) acc[r][c] = T(0);
 #pragma unroll 5
-            for (int m = 0; m < kN2; ++m) {
-              z += h2[m] * W[kEW3 + m * kN3 + q];
-              zd += hd2[m] * W[kEW3 + m * kN3 + q];
-            }
-            const T t3 = tanh_t<T>(z);
-            g[q] = h2[q % kN2] + t3;
-            gd[q] = hd2[q % kN2] + (T(1) - t3 * t3) * zd;
-          }
-        }
-        __syncthreads();
+  for (int k = 0; k < K; ++k) {
+    T av[4], wv[S::CN];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int col = tid + u * kPgNB;
-          if (col < kN3) {
-            for (int rr = 0; rr < rows; ++rr) {
-              const T gv = sG[rr * kPgGP + col], gdv = sGd[rr * kPgGP + col];
+    for (int r = 0; r < 4; ++r) av[r] = sA[(size_t)k * (S::ROWS + 4) + 4 * tr + r];
 #pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                acc[u][c] += sR[rr * 4 + c] * gv;
-                accd[u][c] += sRd[rr * 4 + c] * gv + sR[rr * 4 + c] * gdv;
-              }
-            }
-          }
+    for (int c = 0; c < S::CN; ++c) wv[c] = sW[((size_t)k * S::TC + tc) * S::CP + c];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < S::CN; ++c) acc[r][c] += av[r] * wv[c];
+  }
+  epi.template run<S::TC, S::CN>(row0 + 4 * tr, R2, tc, acc, reinterpret_cast<T*>(smem_raw));
+}
+
+// h2 = [h1, h1] + tanh(z2 + b2), h2' = [h1', h1'] + (1 - t2^2) z2'; keeps (t2, z2').
+template <class T>
+struct EpiL2 {
+  const T* b;
+  const T* H1;
+  T* H2;
+  T* TZ;
+  template <int TC, int CN>
+  __device__ __forceinline__ void run(int row, int R2, int tc, T (*acc)[CN], T*) const {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const size_t r = (size_t)row + 2 * p;
+      if (r >= (size_t)R2) return;
+#pragma unroll
+      for (int c = 0; c < CN; ++c) {
+        const int n = tc + TC * c, k = n % kN1;
+        const T t = tanh_t<T>(acc[2 * p][c] + b[n]), zd = acc[2 * p + 1][c];
+        H2[r * kN2 + n] = H1[r * kN1 + k] + t;
+        H2[(r + 1) * kN2 + n] = H1[(r + 1) * kN1 + k] + (T(1) - t * t) * zd;
+        if (TZ) {
+          TZ[r * kN2 + n] = t;
+          TZ[(r + 1) * kN2 + n] = zd;
         }
-        __syncthreads();
       }
     }
-    if (a.pad)  // padded slots: constant in the positions, so they add to T but not to T'
-      for (int tj = 0; tj < a.ntypes; ++tj) {
-        const T np = T(a.sel[tj] - a.nl_count[(size_t)i * a.ntypes + tj]);
-        const T* P = a.pad + (size_t)(ti * a.ntypes + tj) * 4 * kN3;
+  }
+};
+// G = [h2, h2] + tanh(z3 + b3) and G' likewise.
+template <class T>
+struct EpiL3 {
+  const T* b;
+  const T* H2;
+  T* G;
+  template <int TC, int CN>
+  __device__ __forceinline__ void run(int row, int R2, int tc, T (*acc)[CN], T*) const {
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int col = tid + u * kPgNB;
-          if (col < kN3)
+    for (int p = 0; p < 2; ++p) {
+      const size_t r = (size_t)row + 2 * p;
+      if (r >= (size_t)R2) return;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[u][c] += np * P[c * kN3 + col];
+      for (int c = 0; c < CN; ++c) {
+        const int n = tc + TC * c, k = n % kN2;
+        const T t = tanh_t<T>(acc[2 * p][c] + b[n]);
+        G[r * kN3 + n] = H2[r * kN2 + k] + t;
+        G[(r + 1) * kN3 + n] = H2[(r + 1) * kN2 + k] + (T(1) - t * t) * acc[2 * p + 1][c];
+      }
+    }
+  }
+};
+// Adjoints of z3, z3' (into Y3) and the residual adjoints of h2, h2' (gb[m] + gb[m + 50], into HB).
+template <class T>
+struct EpiR3 {
+  const T* b;
+  const T* geo;
+  const int* atom;
+  const T* TB;  // [local atom][800]
+  T invS;
+  T* Y3;
+  T* HB;
+  template <int TC, int CN>
+  __device__ __forceinline__ void run(int row, int R2, int tc, T (*acc)[CN], T*) const {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const size_t r = (size_t)row + 2 * p;
+      if (r >= (size_t)R2) return;
+      T g[kPgGeo];
+#pragma unroll
+      for (int c = 0; c < kPgGeo; ++c) g[c] = geo[(r / 2) * kPgGeo + c];
+      const T* Tb = TB + (size_t)atom[r / 2] * 800;
+#pragma unroll
+      for (int c = 0; c < CN / 2; ++c) {
+        T sb = T(0), sd = T(0);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int cc = c + h * (CN / 2), n = tc + TC * cc;
+          const T t = tanh_t<T>(acc[2 * p][cc] + b[n]), zd = acc[2 * p + 1][cc];
+          T gb = T(0), gd = T(0);
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const T u = Tb[x * kN3 + n], ud = Tb[400 + x * kN3 + n];
+            gb += g[x] * u + g[4 + x] * ud;
+            gd += g[x] * ud;
+          }
+          gb *= invS;
+          gd *= invS;
+          const T q = T(1) - t * t;
+          Y3[r * kN3 + n] = (gb - T(2) * t * (gd * zd)) * q;
+          Y3[(r + 1) * kN3 + n] = gd * q;
+          sb += gb;
+          sd += gd;
+        }
+        const int m = tc + TC * c;
+        HB[r * kN2 + m] = sb;
+        HB[(r + 1) * kN2 + m] = sd;
+      }
+    }
+  }
+};
+// dE/dh2 = residual + Y3 W3^T; adjoints of z2, z2' (Y2) and the residual adjoints of h1, h1' (HB1).
+template <class T>
+struct EpiR2 {
+  const T* HB;
+  const T* TZ;
+  T* Y2;
+  T* HB1;
+  template <int TC, int CN>
+  __device__ __forceinline__ void run(int row, int R2, int tc, T (*acc)[CN], T*) const {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const size_t r = (size_t)row + 2 * p;
+      if (r >= (size_t)R2) return;
+#pragma unroll
+      for (int c = 0; c < CN / 2; ++c) {
+        T sb = T(0), sd = T(0);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int cc = c + h * (CN / 2), n = tc + TC * cc;
+          const T hb = HB[r * kN2 + n] + acc[2 * p][cc], hd = HB[(r + 1) * kN2 + n] + acc[2 * p + 1][cc];
+          const T t = TZ[r * kN2 + n], zd = TZ[(r + 1) * kN2 + n];
+          const T q = T(1) - t * t;
+          Y2[r * kN2 + n] = (hb - T(2) * t * (hd * zd)) * q;
+          Y2[(r + 1) * kN2 + n] = hd * q;
+          sb += hb;
+          sd += hd;
+        }
+        const int k = tc + TC * c;
+        HB1[r * kN1 + k] = sb;
+        HB1[(r + 1) * kN1 + k] = sd;
+      }
+    }
+  }
+};
+// dE/dh1 = residual + Y2 W2^T, then the gradients of W1 and b1: sums over rows of x z1_bar + x' v1_bar and
+// z1_bar, added up in shared memory (FP64) and with one atomic per column and block.
+template <class T>
+struct EpiR1 {
+  const T* HB1;
+  const T* H1;
+  const T* geo;
+  const T* w1;
+  double* gw1;  // W1 then b1
+  template <int TC, int CN>
+  __device__ __forceinline__ void run(int row, int R2, int tc, T (*acc)[CN], T* smem) const {
+    T sw[CN], sb[CN];
+#pragma unroll
+    for (int c = 0; c < CN; ++c) sw[c] = sb[c] = T(0);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const size_t r = (size_t)row + 2 * p;
+      if (r < (size_t)R2) {
+        const T x = geo[(r / 2) * kPgGeo], xd = geo[(r / 2) * kPgGeo + 4];
+#pragma unroll
+        for (int c = 0; c < CN; ++c) {
+          const int k = tc + TC * c;
+          const T hb = HB1[r * kN1 + k] + acc[2 * p][c], hd = HB1[(r + 1) * kN1 + k] + acc[2 * p + 1][c];
+          const T h = H1[r * kN1 + k], q = T(1) - h * h;
+          const T zb = (hb - T(2) * h * (hd * (xd * w1[k]))) * q, vb = hd * q;
+          sw[c] += x * zb + xd * vb;
+          sb[c] += zb;
         }
       }
+    }
+    __syncthreads();  // every thread is done with the operands
+    T* s = smem;      // [row groups][2 kN1]
+    const int tr = threadIdx.x / TC;
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int col = tid + u * kPgNB;
-      if (col < kN3)
+    for (int c = 0; c < CN; ++c) {
+      s[tr * 2 * kN1 + tc + TC * c] = sw[c];
+      s[tr * 2 * kN1 + kN1 + tc + TC * c] = sb[c];
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * kN1) {
+      double v = 0.0;
+      for (int q = 0; q < (int)blockDim.x / TC; ++q) v += (double)s[q * 2 * kN1 + threadIdx.x];
+      atomicAdd(gw1 + threadIdx.x, v);
+    }
+  }
+};
+
+// T += R_hat^T G and T' += R_hat'^T G + R_hat^T G' over the rows of each atom of the chunk (CTA per atom;
+// sums over S added later): rows [roff[k], roff[k + 1]) of G.
+template <class T>
+__global__ void __launch_bounds__(128) k_pg_T(RowMap m, int a0, const T* __restrict__ geo, const T* __restrict__ G,
+                                             T* TT) {
+  __shared__ T sg[32][kPgGeo];
+  const int k = blockIdx.x, q = threadIdx.x;
+  const int rb = m.roff[k], re = m.roff[k + 1];
+  T acc[4], accd[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) acc[c] = accd[c] = T(0);
+  for (int r0 = rb; r0 < re; r0 += 32) {
+    __syncthreads();
+    for (int e = q; e < 32 * kPgGeo; e += 128) {
+      const int r = r0 + e / kPgGeo;
+      sg[e / kPgGeo][e % kPgGeo] = r < re ? geo[(size_t)r * kPgGeo + e % kPgGeo] : T(0);
+    }
+    __syncthreads();
+    if (q < kN3)
+      for (int r = r0; r < min(re, r0 + 32); ++r) {
+        const T g = G[(size_t)2 * r * kN3 + q], gd = G[((size_t)2 * r + 1) * kN3 + q];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          TT[(size_t)li * 800 + c * kN3 + col] = acc[u][c] * a.invS;
-          TT[(size_t)li * 800 + 400 + c * kN3 + col] = accd[u][c] * a.invS;
+          acc[c] += sg[r - r0][c] * g;
+          accd[c] += sg[r - r0][4 + c] * g + sg[r - r0][c] * gd;
         }
+      }
+  }
+  if (q < kN3) {
+    T* o = TT + (size_t)(m.b0 + k - a0) * 800 + q;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      o[c * kN3] += acc[c];
+      o[400 + c * kN3] += accd[c];
     }
+  }
+}
+
+// Padded slots (constant in the positions: T only) and the normaliser 1 / S; block per atom of the chunk.
+template <class T>
+__global__ void __launch_bounds__(128) k_pg_T_scale(PgArgs<T> a, int ti, int a0, T* TT) {
+  const int li = blockIdx.x, i = a0 + li;
+  for (int q = threadIdx.x; q < 800; q += 128) {
+    T v = TT[(size_t)li * 800 + q];
+    if (a.pad && q < 400)
+      for (int tj = 0; tj < a.ntypes; ++tj)
+        v += T(a.sel[tj] - a.nl_count[(size_t)i * a.ntypes + tj]) * a.pad[(size_t)(ti * a.ntypes + tj) * 4 * kN3 + q];
+    TT[(size_t)li * 800 + q] = v * a.invS;
+  }
+}
+
+// Weight and bias gradients of a layer: gW [KX x N] += X^T Y over the 2 R rows (value and tangent rows
+// alike), gb [N] += column sums of the value rows of Y.  A block sums a range of rows in registers
+// (thread: two columns of X, N / 10 of Y) and adds its result with FP64 atomics.
+template <class T, int KX, int N>
+__global__ void __launch_bounds__(320) k_pg_wgrad(int R2, int per, const T* __restrict__ X, const T* __restrict__ Y,
+                                                 double* gW, double* gb) {
+  constexpr int CN = N / 10, GX = (KX + 1) / 2, B = 32;  // GX groups of two X columns, then one for the bias
+  __shared__ T sX[B][KX + 1], sY[B][N];
+  const int tid = threadIdx.x, tc = tid % 10, tx = tid / 10;
+  const int rb = blockIdx.x * per, re = min(R2, rb + per);
+  T acc[2][CN];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int c = 0; c < CN; ++c) acc[h][c] = T(0);
+  for (int r0 = rb; r0 < re; r0 += B) {
+    __syncthreads();
+    const int nr = min(B, re - r0);
+    for (int q = tid; q < B * KX; q += 320) sX[q / KX][q % KX] = q / KX < nr ? X[(size_t)r0 * KX + q] : T(0);
+    for (int q = tid; q < B * N; q += 320) sY[q / N][q % N] = q / N < nr ? Y[(size_t)r0 * N + q] : T(0);
+    __syncthreads();
+    if (tx < GX) {
+#pragma unroll 4
+      for (int r = 0; r < B; ++r) {
+        const T x0 = sX[r][2 * tx], x1 = 2 * tx + 1 < KX ? sX[r][2 * tx + 1] : T(0);
+#pragma unroll
+        for (int c = 0; c < CN; ++c) {
+          const T y = sY[r][tc + 10 * c];
+          acc[0][c] += x0 * y;
+          acc[1][c] += x1 * y;
+        }
+      }
+    } else if (tx == GX) {
+      for (int r = 0; r < B; r += 2)
+#pragma unroll
+        for (int c = 0; c < CN; ++c) acc[0][c] += sY[r][tc + 10 * c];
+    }
+  }
+  if (tx < GX) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (2 * tx + h < KX)
+#pragma unroll
+        for (int c = 0; c < CN; ++c) atomicAdd(gW + (2 * tx + h) * N + tc + 10 * c, (double)acc[h][c]);
+  } else if (tx == GX) {
+#pragma unroll
+    for (int c = 0; c < CN; ++c) atomicAdd(gb + tc + 10 * c, (double)acc[0][c]);
   }
 }
 
@@ -296,24 +559,33 @@ __global__ void k_pg_desc_bwd(int n, const T* TT, const T* Yb, T* TB) {
 //       G_bar[a] = (1/S) sum_li (sel[tj] - count_li,tj) sum_c T_bar_li[c][a] R_pad[c],
 //     and the reverse of the embedding net at the single input R_pad_0 gives the parameter
 //     gradients (FP64 atomics).  The input is a constant (davg, dstd are not parameters).
+//     k_pg_pad_sum forms the sums over atoms first, 32 atoms a block (one block per tj walking all
+//     atoms took 0.27 ms a call): gsum [tj][100], zeroed by the caller.
 template <class T>
-__global__ void __launch_bounds__(128) k_pg_pad_rev(PgArgs<T> a, int ti, int a0, int n, const T* __restrict__ TB,
-                                                   double* grad) {
+__global__ void __launch_bounds__(128) k_pg_pad_sum(PgArgs<T> a, int ti, int a0, int n, const T* __restrict__ TB,
+                                                   double* gsum) {
+  const int tj = blockIdx.x, tid = threadIdx.x;
+  if (tid >= kN3) return;
+  T Rp[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) Rp[c] = (T(0) - a.stat[ti * 4 + c]) * a.stat[(a.ntypes + ti) * 4 + c];
+  T acc = T(0);
+  for (int li = blockIdx.y * 32; li < min(n, blockIdx.y * 32 + 32); ++li) {
+    const T np = T(a.sel[tj] - a.nl_count[(size_t)(a0 + li) * a.ntypes + tj]);
+    const T* tb = TB + (size_t)li * 800;
+    acc += np * (tb[tid] * Rp[0] + tb[kN3 + tid] * Rp[1] + tb[2 * kN3 + tid] * Rp[2] + tb[3 * kN3 + tid] * Rp[3]);
+  }
+  atomicAdd(gsum + tj * kN3 + tid, (double)acc);
+}
+template <class T>
+__global__ void __launch_bounds__(128) k_pg_pad_rev(PgArgs<T> a, int ti, const double* __restrict__ gsum, double* grad) {
   const int tj = blockIdx.x, tid = threadIdx.x;
   const T* W = a.w + (size_t)(ti * a.ntypes + tj) * kEmbParams;
   double* gW = grad + (size_t)(ti * a.ntypes + tj) * kEmbParams;
   __shared__ T Rp[4], h1[kN1], t2[kN2], h2[kN2], gG[kN3], dz3[kN3], dh2[kN2], dz2[kN2];
   if (tid < 4) Rp[tid] = (T(0) - a.stat[ti * 4 + tid]) * a.stat[(a.ntypes + ti) * 4 + tid];
   __syncthreads();
-  if (tid < kN3) {
-    T acc = T(0);
-    for (int li = 0; li < n; ++li) {
-      const T np = T(a.sel[tj] - a.nl_count[(size_t)(a0 + li) * a.ntypes + tj]);
-      const T* tb = TB + (size_t)li * 800;
-      acc += np * (tb[tid] * Rp[0] + tb[kN3 + tid] * Rp[1] + tb[2 * kN3 + tid] * Rp[2] + tb[3 * kN3 + tid] * Rp[3]);
-    }
-    gG[tid] = acc * a.invS;
-  }
+  if (tid < kN3) gG[tid] = (T)gsum[tj * kN3 + tid] * a.invS;
   const T x = Rp[0];
   if (tid < kN1) h1[tid] = tanh_t<T>(x * W[kEW1 + tid] + W[kEb1 + tid]);
   __syncthreads();
@@ -503,111 +775,6 @@ __global__ void k_pg_counts(int n, const double* scal, double* gb4, double* gebi
   }
 }
 
-// 6. Embedding reverse, one thread per neighbour row of pair (ti, tj); rows of the chunk's
-//    atoms [b0, b0 + nb) are numbered by roff (exclusive offsets, nb + 1 entries).  Each
-//    row writes X3 = [h2; h2'], Y3 = [z3_bar; z3'_bar], X2 = [h1; h1'], Y2 = [z2_bar;
-//    z2'_bar] (primal at row r, tangent at row R + r) and C1 = [x z1_bar + x' v1_bar, z1_bar].
-template <class T>
-__global__ void __launch_bounds__(128) k_pg_emb_rev(PgArgs<T> a, int ti, int tj, int a0, int b0, int nb,
-                                                   const int* __restrict__ roff, int R, const T* __restrict__ TB,
-                                                   T* X3, T* Y3, T* X2, T* Y2, T* C1) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R) return;
-  int lo = 0, hi = nb - 1;  // last atom k with roff[k] <= r
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (roff[mid] <= r) lo = mid; else hi = mid - 1;
-  }
-  const int i = b0 + lo;
-  const size_t e = (size_t)i * a.S + a.sel_off[tj] + (r - roff[lo]);
-  const T* W = a.w + (size_t)(ti * a.ntypes + tj) * kEmbParams;
-  const T* Tb = TB + (size_t)(i - a0) * 800;
-  const T* Tdb = Tb + 400;
-  T R4[4], Rd[4];
-  row_geometry<T>(a, i, ti, e, R4, Rd);
-  const T x = R4[0], xd = Rd[0];
-  T h1[kN1], hd1[kN1], v1[kN1], h2[kN2], hd2[kN2], zd2[kN2];
-  emb12_tangent<T>(W, x, xd, h1, hd1, v1, h2, hd2, zd2);
-  T hb2[kN2], hdb2[kN2];
-#pragma unroll 1
-  for (int m = 0; m < kN2; ++m) {
-    hb2[m] = hdb2[m] = T(0);
-    X3[(size_t)r * kN2 + m] = h2[m];
-    X3[(size_t)(R + r) * kN2 + m] = hd2[m];
-  }
-#pragma unroll 1
-  for (int q = 0; q < kN3; ++q) {
-    T z = W[kEb3 + q], zd = T(0);
-#pragma unroll 5
-    for (int m = 0; m < kN2; ++m) {
-      z += h2[m] * W[kEW3 + m * kN3 + q];
-      zd += hd2[m] * W[kEW3 + m * kN3 + q];
-    }
-    const T t3 = tanh_t<T>(z);
-    const T q3 = T(1) - t3 * t3;
-    T gb = T(0), gdb = T(0);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      gb += R4[c] * Tb[c * kN3 + q] + Rd[c] * Tdb[c * kN3 + q];
-      gdb += R4[c] * Tdb[c * kN3 + q];
-    }
-    gb *= a.invS;
-    gdb *= a.invS;
-    const T tb = gb - T(2) * t3 * (gdb * zd);
-    const T zb = tb * q3, zdb = gdb * q3;
-    hb2[q % kN2] += gb;
-    hdb2[q % kN2] += gdb;
-#pragma unroll 5
-    for (int m = 0; m < kN2; ++m) {
-      hb2[m] += zb * W[kEW3 + m * kN3 + q];
-      hdb2[m] += zdb * W[kEW3 + m * kN3 + q];
-    }
-    Y3[(size_t)r * kN3 + q] = zb;
-    Y3[(size_t)(R + r) * kN3 + q] = zdb;
-  }
-  T hb1[kN1], hdb1[kN1];
-#pragma unroll 1
-  for (int k = 0; k < kN1; ++k) {
-    hb1[k] = hdb1[k] = T(0);
-    X2[(size_t)r * kN1 + k] = h1[k];
-    X2[(size_t)(R + r) * kN1 + k] = hd1[k];
-  }
-#pragma unroll 1
-  for (int m = 0; m < kN2; ++m) {
-    const T t2 = h2[m] - h1[m % kN1];
-    const T q2 = T(1) - t2 * t2;
-    const T tb = hb2[m] - T(2) * t2 * (hdb2[m] * zd2[m]);
-    const T zb = tb * q2, zdb = hdb2[m] * q2;
-    hb1[m % kN1] += hb2[m];
-    hdb1[m % kN1] += hdb2[m];
-#pragma unroll 5
-    for (int k = 0; k < kN1; ++k) {
-      hb1[k] += zb * W[kEW2 + k * kN2 + m];
-      hdb1[k] += zdb * W[kEW2 + k * kN2 + m];
-    }
-    Y2[(size_t)r * kN2 + m] = zb;
-    Y2[(size_t)(R + r) * kN2 + m] = zdb;
-  }
-#pragma unroll 1
-  for (int k = 0; k < kN1; ++k) {
-    const T q1 = T(1) - h1[k] * h1[k];
-    const T kb = hb1[k] - T(2) * h1[k] * (hdb1[k] * v1[k]);
-    const T zb = kb * q1, vb = hdb1[k] * q1;
-    C1[(size_t)r * 2 * kN1 + k] = x * zb + xd * vb;
-    C1[(size_t)r * 2 * kN1 + kN1 + k] = zb;
-  }
-}
-
-// Column sums of X [rows x cols] (leading dimension ld) added to out (FP64 atomics).
-template <class T>
-__global__ void k_pg_colsum(int rows, int cols, int ld, const T* __restrict__ X, double* out) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= cols) return;
-  double acc = 0.0;
-  for (int r = blockIdx.y; r < rows; r += gridDim.y) acc += (double)X[(size_t)r * ld + col];
-  atomicAdd(out + col, acc);
-}
-
 // alpha, loss, and the tangent direction w = 2 cF (F - F0) in internal order.
 __global__ void k_pg_setup(int N, const double* __restrict__ e_atom, const double* __restrict__ force,
                            const double* __restrict__ F0, const int* __restrict__ perm, double E0, double cE,
@@ -731,15 +898,27 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
   T* U = H + 2 * C * kF;
   T* G = U + 2 * C * kF;
   T* TB = G + 2 * C * kF;
-  T* X3 = TB + C * 800;
-  T* Y3 = X3 + 2 * (size_t)kPgRows * kN2;
-  T* X2 = Y3 + 2 * (size_t)kPgRows * kN3;
-  T* Y2 = X2 + 2 * (size_t)kPgRows * kN1;
-  T* C1 = Y2 + 2 * (size_t)kPgRows * kN2;
+  const size_t RW = (size_t)kPgRows;
+  T* geo = TB + C * 800;
+  T* H1 = geo + RW * kPgGeo;
+  T* H2 = H1 + 2 * RW * kN1;
+  T* TZ = H2 + 2 * RW * kN2;
+  T* Y3 = TZ + 2 * RW * kN2;   // G, G' of the forward; adjoints of z3, z3' of the reverse
+  T* HB = Y3 + 2 * RW * kN3;
+  T* Y2 = HB + 2 * RW * kN2;
+  T* HB1 = Y2 + 2 * RW * kN2;
+  int* atom = reinterpret_cast<int*>(HB1 + 2 * RW * kN1);
 
   const size_t emb_total = (size_t)nt * nt * kEmbParams;
-  const size_t fsmem = (size_t)(2 * kPgNB * kPgGP + 8 * kPgNB) * sizeof(T);
-  DP_CUDA_TRY(m, ensure_smem(reinterpret_cast<const void*>(k_pg_emb_fwd<T>), fsmem));
+  // one layer over the rows of a chunk
+#define PG_LAYER(K_, N_, TB_, EPI_, A_, W_)                                                                  \
+  do {                                                                                                       \
+    auto fn_ = k_pg_layer<T, K_, N_, TB_, EPI_<T>>;                                                          \
+    const size_t sm_ = skinny_smem<T, K_, N_>();                                                             \
+    DP_CUDA_TRY(m, ensure_smem(reinterpret_cast<const void*>(fn_), sm_));                                    \
+    fn_<<<cdiv(2 * rc.R, Skinny<T, N_>::ROWS), Skinny<T, N_>::THREADS, sm_, m->stream>>>(2 * rc.R, A_, W_, epi);                   \
+    m->launches += 1;                                                                                        \
+  } while (0)
   const int sms = num_sms();
 
   for (const AtomChunk& ac : achunks) {
@@ -748,7 +927,18 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
     const T* P = theta + fb;
     double* gP = grad + fb;
     // 1-2: T, T', D, D'
-    k_pg_emb_fwd<T><<<std::min(n, 8 * sms), kPgNB, fsmem, m->stream>>>(a, ti, ac.a0, n, TT);
+    DP_CUDA_TRY(m, cudaMemsetAsync(TT, 0, sizeof(T) * 800 * (size_t)n, m->stream));
+    for (const RowChunk& rc : rchunks) {
+      if (rc.ti != ti || rc.a0 != ac.a0 || rc.R == 0) continue;
+      const T* W = theta + (size_t)(ti * nt + rc.tj) * kEmbParams;
+      const RowMap rm{ti, rc.tj, rc.b0, rc.nb, rc.R, m->pg_roff + rc.off};
+      k_pg_rows<T><<<cdiv(rc.R, 128), 128, 0, m->stream>>>(a, rm, geo, atom, H1);
+      { EpiL2<T> epi{W + kEb2, H1, H2, nullptr}; PG_LAYER(kN1, kN2, false, EpiL2, H1, W + kEW2); }
+      { EpiL3<T> epi{W + kEb3, H2, Y3}; PG_LAYER(kN2, kN3, false, EpiL3, H2, W + kEW3); }
+      k_pg_T<T><<<rc.nb, 128, 0, m->stream>>>(rm, ac.a0, geo, Y3, TT);
+      m->launches += 2;
+    }
+    k_pg_T_scale<T><<<n, 128, 0, m->stream>>>(a, ti, ac.a0, TT);
     k_pg_desc<T><<<std::min(n, 8 * sms), 128, 0, m->stream>>>(n, TT, Y);
     m->launches += 2;
     // 3: fitting forward on [D; D']
@@ -782,27 +972,35 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
     k_pg_desc_bwd<T><<<std::min(n, 8 * sms), 128, 0, m->stream>>>(n, TT, Yb, TB);
     m->launches += 1;
     if (a.pad) {
-      k_pg_pad_rev<T><<<nt, 128, 0, m->stream>>>(a, ti, ac.a0, n, TB, grad);
-      m->launches += 1;
+      double* gsum = m->pg_scal + 8;
+      DP_CUDA_TRY(m, cudaMemsetAsync(gsum, 0, sizeof(double) * kN3 * nt, m->stream));
+      k_pg_pad_sum<T><<<dim3(nt, cdiv(n, 32)), 128, 0, m->stream>>>(a, ti, ac.a0, n, TB, gsum);
+      k_pg_pad_rev<T><<<nt, 128, 0, m->stream>>>(a, ti, gsum, grad);
+      m->launches += 2;
     }
-    // 6: embedding reverse per neighbour row
+    // 6: embedding reverse over the rows
     for (const RowChunk& rc : rchunks) {
       if (rc.ti != ti || rc.a0 != ac.a0 || rc.R == 0) continue;
-      const int R = rc.R;
       const size_t eb = (size_t)(ti * nt + rc.tj) * kEmbParams;
-      k_pg_emb_rev<T><<<cdiv(R, 128), 128, 0, m->stream>>>(a, ti, rc.tj, ac.a0, rc.b0, rc.nb, m->pg_roff + rc.off,
-                                                           R, TB, X3, Y3, X2, Y2, C1);
-      m->launches += 1;
-      const int skr = std::max(1, std::min(128, 2 * R / 512));
-      gemm<T, true, false, 2>(m, kN2, kN3, 2 * R, X3, kN2, Y3, kN3, grad + eb + kEW3, kN3, skr);
-      gemm<T, true, false, 2>(m, kN1, kN2, 2 * R, X2, kN1, Y2, kN2, grad + eb + kEW2, kN2, skr);
-      const int ry = std::min(R, 256);
-      k_pg_colsum<T><<<dim3(1, ry), 128, 0, m->stream>>>(R, kN3, kN3, Y3, grad + eb + kEb3);
-      k_pg_colsum<T><<<dim3(1, ry), 128, 0, m->stream>>>(R, kN2, kN2, Y2, grad + eb + kEb2);
-      k_pg_colsum<T><<<dim3(1, ry), 128, 0, m->stream>>>(R, 2 * kN1, 2 * kN1, C1, grad + eb + kEW1);
+      const T* W = theta + eb;
+      double* gW = grad + eb;
+      const RowMap rm{ti, rc.tj, rc.b0, rc.nb, rc.R, m->pg_roff + rc.off};
+      k_pg_rows<T><<<cdiv(rc.R, 128), 128, 0, m->stream>>>(a, rm, geo, atom, H1);
+      { EpiL2<T> epi{W + kEb2, H1, H2, TZ}; PG_LAYER(kN1, kN2, false, EpiL2, H1, W + kEW2); }
+      {
+        EpiR3<T> epi{W + kEb3, geo, atom, TB + (size_t)(rc.b0 - ac.a0) * 800, a.invS, Y3, HB};
+        PG_LAYER(kN2, kN3, false, EpiR3, H2, W + kEW3);
+      }
+      { EpiR2<T> epi{HB, TZ, Y2, HB1}; PG_LAYER(kN3, kN2, true, EpiR2, Y3, W + kEW3); }
+      { EpiR1<T> epi{HB1, H1, geo, W + kEW1, gW + kEW1}; PG_LAYER(kN2, kN1, true, EpiR1, Y2, W + kEW2); }
+      // about two blocks an SM, at least 128 rows each
+      const int per = std::max(128, cdiv(cdiv(2 * rc.R, 2 * sms), 32) * 32);
+      k_pg_wgrad<T, kN2, kN3><<<cdiv(2 * rc.R, per), 320, 0, m->stream>>>(2 * rc.R, per, H2, Y3, gW + kEW3, gW + kEb3);
+      k_pg_wgrad<T, kN1, kN2><<<cdiv(2 * rc.R, per), 320, 0, m->stream>>>(2 * rc.R, per, H1, Y2, gW + kEW2, gW + kEb2);
       m->launches += 3;
     }
   }
+#undef PG_LAYER
   DP_LAUNCH_CHECK(m);
   return DP_OK;
 }
@@ -811,7 +1009,7 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
 
 size_t param_grad_workspace_bytes(int cap, bool fp64) {
   const size_t per_atom = 800 + 2 * 2 * (size_t)kKD + 6 * 2 * (size_t)kF + 800;
-  const size_t per_row = 2 * (size_t)(kN2 + kN3 + kN1 + kN2) + 2 * kN1;
+  const size_t per_row = kPgGeo + 2 * (size_t)(kN1 + kN2 + kN2 + kN3 + kN2 + kN2 + kN1) + 1;
   return ((size_t)cap * per_atom + (size_t)kPgRows * per_row) * (fp64 ? 8 : 4);
 }
 
