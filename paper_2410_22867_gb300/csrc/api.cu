@@ -196,12 +196,12 @@ dp_status setup_replicas(Model* m, int nrep, const int* offs, const double* boxe
 
 // One force evaluation on the current internal positions (lists already valid):
 // format -> descriptor -> fitting -> embedding backward (forces, virials).
-dp_status force_eval(Model* m, int N) {
+dp_status force_eval(Model* m, int N, bool fold = true) {
   DP_TRY(launch_format(m, N));
   DP_TRY(launch_zero_forces(m, N));
   DP_TRY(launch_descriptor(m, N));
   DP_TRY(launch_fitting(m, N));
-  DP_TRY(launch_embed_backward(m, N));
+  DP_TRY(launch_embed_backward(m, N, fold));
   return DP_OK;
 }
 
@@ -229,8 +229,8 @@ dp_status md_step(Model* m, int N, double dt, bool rebuild) {
   } else {
     DP_TRY(launch_delta(m, N));
   }
-  DP_TRY(force_eval(m, N));
-  DP_TRY(launch_kick(m, N, dt));
+  DP_TRY(force_eval(m, N, false));
+  DP_TRY(launch_kick(m, N, dt, is_mixed(m)));  // adds the mixed backward's forces on the way
   return DP_OK;
 }
 
@@ -377,9 +377,8 @@ dp_status run_md(Model* m, dp_md_state* st, double dt, int nsteps, int capture, 
     DP_CUDA_TRY(m, cudaMemcpyAsync(mass_t_dev, st->mass_by_type, sizeof(double) * m->ntypes,
                                    cudaMemcpyHostToDevice, m->stream));
     DP_TRY(launch_type_sort(m, st->types, N));
-    DP_TRY(launch_load_positions(m, st->x, N));
     DP_TRY(launch_load_state(m, N, st->v, mass_t_dev));
-    DP_TRY(launch_rebuild(m, N, true));
+    DP_TRY(launch_rebuild(m, N, true, st->x));
     DP_TRY(force_eval(m, N));
   }
   Model::GraphCache& gc = m->graphs;
@@ -538,9 +537,9 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
   A_(force, 24 * N); A_(mass, 8 * N);
   A_(geom, sizeof(RepGeom) * R);
   A_(cell_of, 4 * N);
-  A_(cell_count, 4 * (size_t)m->max_cells); A_(cell_start, 4 * ((size_t)m->max_cells + 1));
-  A_(cell_fill, 4 * (size_t)m->max_cells); A_(cell_atoms, 4 * N); A_(cell_xf, 16 * N);
-  A_(vl_e, 16 * N * m->VS); A_(vl_img, 4 * N * m->VS); A_(vl_work, 4 * (N + 1)); A_(vcount, 4 * N * nt);
+  A_(cell_count, 4 * (2 * (size_t)m->max_cells + 1)); A_(cell_start, 4 * ((size_t)m->max_cells + 1));
+  A_(cell_atoms, 4 * N); A_(cell_xf, 16 * N);
+  A_(vl_e, 16 * N * m->VS); A_(vl_img, 4 * N * m->VS); A_(vl_work, 4 * N); A_(vcount, 4 * N * nt);
   A_(nl_j, 4 * N * m->S); A_(nl_img, 4 * N * m->S);
   A_(nl_d, (prec == DP_FP64 ? 32 : 16) * N * m->S);
   A_(nl_count, 4 * N * nt);
@@ -615,8 +614,7 @@ dp_status dp_compute_batch(dp_model* h, int nrep, const int* atom_offsets, const
   DP_TRY(setup_replicas(m, nrep, atom_offsets, boxes, N, false));
   m->natoms = N;
   DP_TRY(launch_type_sort(m, types, N));
-  DP_TRY(launch_load_positions(m, coords, N));
-  DP_TRY(launch_rebuild(m, N, false));
+  DP_TRY(launch_rebuild(m, N, false, coords));
   DP_TRY(force_eval(m, N));
   DP_TRY(launch_outputs(m, N, energies, atom_energy, forces, virials));
   return DP_OK;
@@ -842,8 +840,7 @@ extern "C" dp_status dp_param_grad(dp_model* h, int natoms, const double* coords
   DP_TRY(setup_replicas(m, 1, offs, box, natoms, false));
   m->natoms = natoms;
   DP_TRY(launch_type_sort(m, types, natoms));
-  DP_TRY(launch_load_positions(m, coords, natoms));
-  DP_TRY(launch_rebuild(m, natoms, false));
+  DP_TRY(launch_rebuild(m, natoms, false, coords));
   DP_TRY(force_eval(m, natoms));
   return launch_param_grad(m, natoms, F0, E0, cE, cF, grad, loss);
 }

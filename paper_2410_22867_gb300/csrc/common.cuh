@@ -141,16 +141,15 @@ struct Model {
 
   // cell list
   int* cell_of = nullptr;
-  int* cell_count = nullptr;
+  int* cell_count = nullptr;  // [ncells], then [ncells] fill counters and the Verlet work count (zeroed together)
   int* cell_start = nullptr;
-  int* cell_fill = nullptr;
   int* cell_atoms = nullptr;
   float4* cell_xf = nullptr;  // [N] FP32 positions in cell order (beside cell_atoms)
 
   // Verlet list (r_c + skin)
   float4* vl_e = nullptr;     // [N*VS] pair vector at rebuild (fp32), w = neighbour index
   int* vl_img = nullptr;      // [N*VS] image code
-  int* vl_work = nullptr;     // [N + 1] atoms the per-atom Verlet kernel builds, their count last
+  int* vl_work = nullptr;     // [N] atoms the per-atom Verlet kernel builds
   int* vcount = nullptr;      // [N*nt]
 
   // formatted list (r_c), compacted per type segment
@@ -306,11 +305,11 @@ __host__ __device__ __forceinline__ int cdiv_dev(int a, int b) { return (a + b -
 // host-side launchers (each returns DP_OK or DP_ERR_CUDA)
 // nlist.cu
 dp_status launch_type_sort(Model* m, const int* types_user, int N);
-dp_status launch_load_positions(Model* m, const double* coords_user, int N);
 // Cell binning and the Verlet list of every atom.  with_skin: pairs within r_c + skin (MD: the
 // list serves the next steps); otherwise within r_c (a single evaluation: the list is rebuilt on
 // every call, so the skin would only add entries).
-dp_status launch_rebuild(Model* m, int N, bool with_skin);
+// coords: positions in the caller's order to start from (null: the internal ones).
+dp_status launch_rebuild(Model* m, int N, bool with_skin, const double* coords = nullptr);
 dp_status launch_delta(Model* m, int N);
 dp_status launch_format(Model* m, int N, bool images = false);  // images: also the image codes
 dp_status launch_get_nlist(Model* m, int N, int* nlist, int* images);
@@ -325,7 +324,7 @@ dp_status launch_mix_atom_virial(Model* m, int N);  // synchronous; n = 0 drops 
 dp_status launch_pad_rows(Model* m);  // pad64 / pad32 from the current weights (synchronous caller)
 dp_status launch_descriptor(Model* m, int N);
 dp_status launch_fitting(Model* m, int N);
-dp_status launch_embed_backward(Model* m, int N);
+dp_status launch_embed_backward(Model* m, int N, bool fold = true);  // fold: mixed forces into m->force
 // emb_digits.cu (FP64 / FP32 embedding net as digit products on the tensor cores)
 size_t dig_emb_bytes(int ntypes, bool fp64);
 size_t dig_tanh_bytes();
@@ -339,7 +338,7 @@ dp_status dig_fit_upload(Model* m);
 dp_status launch_dig_fitting(Model* m, int N);
 // mix_embed.cu (tensor-core embedding net)
 dp_status launch_mix_descriptor(Model* m, int N);
-dp_status launch_mix_embed_backward(Model* m, int N);
+dp_status launch_mix_embed_backward(Model* m, int N, bool fold);
 // mix_fit.cu (tensor-core fitting net)
 dp_status mix_fit_setup(Model* m);
 size_t mix_fit_weight_bytes(int ntypes);
@@ -359,7 +358,8 @@ dp_status launch_outputs(Model* m, int N, double* energy_rep, double* atom_energ
                          double* virial_rep);
 dp_status launch_zero_forces(Model* m, int N);
 dp_status launch_kick_drift(Model* m, int N, double dt);
-dp_status launch_kick(Model* m, int N, double dt);
+// fold: first add the mixed backward's FP32 forces (launch_embed_backward was told to leave them)
+dp_status launch_kick(Model* m, int N, double dt, bool fold);
 dp_status launch_load_state(Model* m, int N, const double* v_user, const double* mass_by_type);
 dp_status launch_store_state(Model* m, int N, double* x_user, double* v_user);
 dp_status launch_kinetic(Model* m, int N, double* ke_rep);

@@ -26,72 +26,87 @@ __global__ void k_unpermute(int N, const int* __restrict__ perm, const double* _
 
 // Per-replica energy and virial: sums of the per-atom values (caller order), or for the
 // virial the per-replica accumulator vir_rep when the backward produced one.  Deterministic:
-// block (c, r) sums chunk c (kRedChunk atoms) of replica r over a fixed strided partition (four
-// independent loads per pass) and a fixed tree; with one chunk per replica it writes the result,
-// otherwise its partial, which k_rep_final adds in chunk order.
+// block (c, r) sums chunk c (kRedChunk atoms) of replica r over a fixed strided partition and a fixed
+// tree of warp shuffles; with one chunk per replica it writes the result, otherwise its partial,
+// which k_rep_final adds in a fixed order.  NQ = 1 (no per-atom virial) or 10 quantities: FP64 adds are
+// slow here, and the mixed precisions paid for ten columns of zeros (9.8 us a call, now 2.9).
 constexpr int kRedThreads = 256;
-constexpr int kRedChunk = 8192;
+constexpr int kRedChunk = 2048;
+template <int NQ>
 __global__ void __launch_bounds__(kRedThreads) k_rep_reduce(int nrep, int nchunk, const int* __restrict__ rep_off,
                                                            const double* __restrict__ e_user,
                                                            const double* __restrict__ vir_user,
                                                            const double* __restrict__ vir_rep, double* energy,
                                                            double* virial, double* part_out,
                                                            const int* __restrict__ err) {
-  __shared__ double part[10][kRedThreads];
-  const int r = blockIdx.y, c = blockIdx.x;
+  __shared__ double part[kRedThreads / 32][NQ];
+  const int r = blockIdx.y, c = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (r >= nrep) return;
   const int rb = rep_off[r], re = rep_off[r + 1];
   const int beg = min(re, rb + c * kRedChunk), end = min(re, beg + kRedChunk);
-  double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (int u0 = beg + threadIdx.x; u0 < end; u0 += 4 * kRedThreads) {
-    double e[4];
+  double acc[NQ];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+  for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
+  constexpr int kU = NQ == 1 ? 8 : 2;  // atoms a pass, their loads in flight together
+  for (int u0 = beg + threadIdx.x; u0 < end; u0 += kU * kRedThreads) {
+    double v[kU][NQ];
+#pragma unroll
+    for (int k = 0; k < kU; ++k) {
       const int u = u0 + k * kRedThreads;
-      e[k] = u < end ? e_user[u] : 0.0;
+      v[k][0] = u < end ? e_user[u] : 0.0;
+#pragma unroll
+      for (int q = 1; q < NQ; ++q) v[k][q] = u < end ? vir_user[(size_t)u * 9 + q - 1] : 0.0;
     }
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc[0] += e[k];
-    if (vir_user) {
+    for (int k = 0; k < kU; ++k)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int u = u0 + k * kRedThreads;
-        if (u < end)
-          for (int q = 0; q < 9; ++q) acc[1 + q] += vir_user[(size_t)u * 9 + q];
-      }
-    }
+      for (int q = 0; q < NQ; ++q) acc[q] += v[k][q];
   }
-  for (int q = 0; q < 10; ++q) part[q][threadIdx.x] = acc[q];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_down_sync(0xffffffffu, acc[q], o);
+    if (lane == 0) part[w][q] = acc[q];
+  }
   __syncthreads();
-  for (int st = kRedThreads / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st)
-      for (int q = 0; q < 10; ++q) part[q][threadIdx.x] += part[q][threadIdx.x + st];
-    __syncthreads();
-  }
+  if (threadIdx.x >= 10) return;
+  const int q = threadIdx.x;
+  double s = 0.0;
+  if (q < NQ)
+#pragma unroll
+    for (int k = 0; k < kRedThreads / 32; ++k) s += part[k][q];
   if (nchunk > 1) {
-    if (threadIdx.x < 10) part_out[((size_t)r * nchunk + c) * 10 + threadIdx.x] = part[threadIdx.x][0];
+    part_out[((size_t)r * nchunk + c) * 10 + q] = s;
     return;
   }
-  if (threadIdx.x == 0) {
-    bool bad = err && *err != 0;
-    if (energy) energy[r] = bad ? __longlong_as_double(0x7ff8000000000000ll) : part[0][0];
-    if (virial)
-      for (int q = 0; q < 9; ++q) virial[r * 9 + q] = vir_rep ? vir_rep[r * 9 + q] : part[1 + q][0];
-  }
-}
-
-// The chunk partials of each replica added in chunk order (lane q: quantity q).
-__global__ void k_rep_final(int nrep, int nchunk, const double* __restrict__ part, const double* __restrict__ vir_rep,
-                            double* energy, double* virial, const int* __restrict__ err) {
-  const int r = blockIdx.x, q = threadIdx.x;
-  if (r >= nrep || q >= 10) return;
-  double s = 0.0;
-  for (int c = 0; c < nchunk; ++c) s += part[((size_t)r * nchunk + c) * 10 + q];
   if (q == 0) {
-    bool bad = err && *err != 0;
+    const bool bad = err && *err != 0;
     if (energy) energy[r] = bad ? __longlong_as_double(0x7ff8000000000000ll) : s;
   } else if (virial) {
     virial[r * 9 + q - 1] = vir_rep ? vir_rep[r * 9 + q - 1] : s;
+  }
+}
+
+// The chunk partials of each replica (warp q: quantity q; lane l adds chunks l, l + 32, ..., then a tree).
+__global__ void __launch_bounds__(320) k_rep_final(int nrep, int nchunk, const double* __restrict__ part,
+                                                  const double* __restrict__ vir_rep, double* energy, double* virial,
+                                                  const int* __restrict__ err) {
+  const int r = blockIdx.x, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (r >= nrep) return;
+  if (q > 0 && (!virial || vir_rep)) {
+    if (virial && lane == 0) virial[r * 9 + q - 1] = vir_rep[r * 9 + q - 1];
+    return;
+  }
+  double s = 0.0;
+  for (int c = lane; c < nchunk; c += 32) s += part[((size_t)r * nchunk + c) * 10 + q];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane != 0) return;
+  if (q == 0) {
+    const bool bad = err && *err != 0;
+    if (energy) energy[r] = bad ? __longlong_as_double(0x7ff8000000000000ll) : s;
+  } else {
+    virial[r * 9 + q - 1] = s;
   }
 }
 
@@ -107,12 +122,20 @@ __global__ void k_kick_drift(int N, dvec4* x, dvec4* v, const double* __restrict
   x[k] = xx;
 }
 
-__global__ void k_kick(int N, dvec4* v, const double* __restrict__ F, const double* __restrict__ mass, double dt) {
+// f32: the mixed backward's FP32 forces, still to be added to F (null: F is complete).
+__global__ void k_kick(int N, dvec4* v, double* __restrict__ F, const float4* __restrict__ f32,
+                       const double* __restrict__ mass, double dt) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= N) return;
   double a = 0.5 * dt * kKappa / mass[k];
+  double f[3] = {F[3 * k], F[3 * k + 1], F[3 * k + 2]};
+  if (f32) {
+    const float4 g = f32[k];
+    f[0] += (double)g.x; f[1] += (double)g.y; f[2] += (double)g.z;
+    F[3 * k] = f[0]; F[3 * k + 1] = f[1]; F[3 * k + 2] = f[2];
+  }
   dvec4 vv = v[k];
-  vv.x += a * F[3 * k]; vv.y += a * F[3 * k + 1]; vv.z += a * F[3 * k + 2];
+  vv.x += a * f[0]; vv.y += a * f[1]; vv.z += a * f[2];
   v[k] = vv;
 }
 
@@ -166,11 +189,12 @@ dp_status launch_rep_reduce(Model* m, const double* e_user, const double* vir_us
     m->last_error = "reduction workspace too small";
     return DP_ERR_CAPACITY;
   }
-  k_rep_reduce<<<dim3(nchunk, m->nrep), kRedThreads, 0, m->stream>>>(m->nrep, nchunk, m->rep_off_dev, e_user, vir_user,
-                                                                     vir_rep, energy, virial, m->red_part, err);
+  const auto fn = vir_user ? k_rep_reduce<10> : k_rep_reduce<1>;
+  fn<<<dim3(nchunk, m->nrep), kRedThreads, 0, m->stream>>>(m->nrep, nchunk, m->rep_off_dev, e_user, vir_user, vir_rep,
+                                                           energy, virial, m->red_part, err);
   m->launches += 1;
   if (nchunk > 1) {
-    k_rep_final<<<m->nrep, 32, 0, m->stream>>>(m->nrep, nchunk, m->red_part, vir_rep, energy, virial, err);
+    k_rep_final<<<m->nrep, 320, 0, m->stream>>>(m->nrep, nchunk, m->red_part, vir_rep, energy, virial, err);
     m->launches += 1;
   }
   return DP_OK;
@@ -194,7 +218,9 @@ dp_status launch_outputs(Model* m, int N, double* energy_rep, double* atom_energ
   return DP_OK;
 }
 
+// (The mixed precisions zero their forces with the other accumulators, in launch_mix_descriptor.)
 dp_status launch_zero_forces(Model* m, int N) {
+  if (is_mixed(m)) return DP_OK;
   DP_CUDA_TRY(m, cudaMemsetAsync(m->force, 0, sizeof(double) * 3 * N, m->stream));
   return DP_OK;
 }
@@ -206,8 +232,9 @@ dp_status launch_kick_drift(Model* m, int N, double dt) {
   return DP_OK;
 }
 
-dp_status launch_kick(Model* m, int N, double dt) {
-  k_kick<<<cdiv(N, 256), 256, 0, m->stream>>>(N, m->v, m->force, m->mass, dt);
+dp_status launch_kick(Model* m, int N, double dt, bool fold) {
+  k_kick<<<cdiv(N, 256), 256, 0, m->stream>>>(N, m->v, m->force, fold ? reinterpret_cast<const float4*>(m->force32) : nullptr,
+                                              m->mass, dt);
   m->launches += 1;
   DP_LAUNCH_CHECK(m);
   return DP_OK;

@@ -234,7 +234,9 @@ constexpr int kSmall = 64;
 // Forward operand image of one embedding pair (built once per weight upload, copied into shared
 // memory by three bulk copies per pair change): B2 | B3 (head, remainder) | small.
 constexpr uint32_t kImgFwdB3 = 8192, kImgFwdSmall = kImgFwdB3 + 2 * 14336, kImgFwd = kImgFwdSmall + kSmall * 4;
-constexpr uint32_t kImgBytes = kImgFwd;
+// Backward image behind it: B2 | B3 | small, used where a CTA walks few tiles (k_mix_embed_bwd<.., IMG>).
+constexpr uint32_t kImgBwdB3 = 8192, kImgBwdSmall = kImgBwdB3 + 16384, kImgBwd = kImgBwdSmall + kSmall * 4;
+constexpr uint32_t kImgBytes = kImgFwd + kImgBwd;
 
 // The three bulk copies of one operand image (B2 | B3 | small, `b3` and `sm_off` bytes in) into
 // shared memory on mbarrier `bar`; issued by one thread.  Out of line: the kernels' register
@@ -751,7 +753,9 @@ __device__ void load_bwd_ops(const float* __restrict__ W, unsigned char* sB2, un
 // dh2' product.  dR_hat and dG use dE/dT and G in FP32 on the CUDA cores.
 // ATOMVIR: a second pass over the stored state that accumulates only the per-atom (centre)
 // virial -sum g (x) d into a.vir_atom (FP64) and leaves forces and per-replica virials alone.
-template <bool F16, bool TAB, bool ATOMVIR = false>
+// IMG: the operand blocks come from the pair's image (three bulk copies) instead of being converted from
+// the weights by every CTA; see launch_mix_embed_backward for where that pays.
+template <bool F16, bool TAB, bool ATOMVIR = false, bool IMG = false>
 __global__ void __launch_bounds__(kRows, 3) k_mix_embed_bwd(MixArgs a) {
   extern __shared__ unsigned char sraw[];
   unsigned char* sm = align1024(sraw);
@@ -822,9 +826,15 @@ __global__ void __launch_bounds__(kRows, 3) k_mix_embed_bwd(MixArgs a) {
     if (w == kLocWarp && cur + ti.nrows < c1) locate_window(a, cur + ti.nrows, wk, s_tot, sWin);
     const int np = ti.ti * a.ntypes + ti.tj;
     if (np != pair) {
-      // the backward builds its operand blocks itself: fetching them from the image (bulk or
-      // cooperative copy) changed the register allocation of its main loop and cost 4-8%
-      if (!TAB) load_bwd_ops<F16>(a.w + (size_t)np * kEmbParams, sB2, sB3, small);
+      // over many tiles the backward builds its operand blocks itself: fetching them from the image
+      // changes the register allocation of its main loop and costs 4-8%
+      if (!TAB && !IMG) load_bwd_ops<F16>(a.w + (size_t)np * kEmbParams, sB2, sB3, small);
+      if (!TAB && IMG) {  // on the product barrier, idle here
+        if (t == 0)
+          fetch_image(a.img + (size_t)np * kImgBytes + kImgFwd, kImgBwdB3, kImgBwdSmall, kImgBwd, sB2, sB3, small, &bar);
+        ok = tc::mbar_wait(&bar, phase, a.err) && ok;
+        phase ^= 1u;
+      }
       pair = np;
       __syncthreads();
     }
@@ -1184,25 +1194,53 @@ __global__ void k_scan_local(int N, int ntypes, const int* __restrict__ cnt, int
   __syncthreads();
   const int excl = x - v + (w > 0 ? ws[w - 1] : 0);
   if (i < N) rowoff[(size_t)tj * (N + 1) + i] = excl;
-  if (threadIdx.x == 1023) blk[tj * gridDim.x + blockIdx.x] = ws[31];
+  if (threadIdx.x == 1023) {
+    if (gridDim.x == 1) rowoff[(size_t)tj * (N + 1) + N] = ws[31];  // no second pass
+    else blk[tj * gridDim.x + blockIdx.x] = ws[31];
+  }
 }
 
 __global__ void k_scan_fix(int N, int nblk, int* rowoff, const int* blk) {
   const int tj = blockIdx.y;
   __shared__ int off;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
     int s = 0;
-    for (int b = 0; b < blockIdx.x; ++b) s += blk[tj * nblk + b];
-    off = s;
-    if (blockIdx.x == nblk - 1) {
-      int tot = s;
-      tot += blk[tj * nblk + blockIdx.x];
-      rowoff[(size_t)tj * (N + 1) + N] = tot;
+    for (int b = threadIdx.x; b < blockIdx.x; b += 32) s += blk[tj * nblk + b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) {
+      off = s;
+      if (blockIdx.x == nblk - 1) rowoff[(size_t)tj * (N + 1) + N] = s + blk[tj * nblk + blockIdx.x];
     }
   }
   __syncthreads();
   const int i = blockIdx.x * 1024 + threadIdx.x;
   if (i < N) rowoff[(size_t)tj * (N + 1) + i] += off;
+}
+
+// Zeroes what an evaluation accumulates: forces (both arrays), per-replica virials, and the partial T
+// of the (atom, type) segments that the forward does not store whole: those without rows and those
+// split between two CTAs (chunks of `per` rows as in k_mix_embed_fwd with `grid` CTAs).  Clearing all
+// of Tseg wrote 1.6 KB an atom and type (38 us a step at 131,072 atoms).  One warp per atom.
+__global__ void __launch_bounds__(256) k_mix_zero(int N, int ntypes, int grid, int nrep, const int* __restrict__ rowoff,
+                                                  float4* Tseg, double* force, float4* force32, double* vir_rep) {
+  const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  for (int q = blockIdx.x * 256 + threadIdx.x; q < 9 * nrep; q += gridDim.x * 256) vir_rep[q] = 0.0;
+  if (i >= N) return;
+  if (lane < 3) force[(size_t)i * 3 + lane] = 0.0;
+  if (lane == 3) force32[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  int total = 0;
+  for (int tj = 0; tj < ntypes; ++tj) total += rowoff[(size_t)tj * (N + 1) + N];
+  const int per = max(kRows, (total + grid - 1) / grid);
+  int base = 0;
+  for (int tj = 0; tj < ntypes; ++tj) {
+    const int* ro = rowoff + (size_t)tj * (N + 1);
+    const int b = base + ro[i], e = base + ro[i + 1];
+    base += ro[N];
+    if (b < e && b / per == (e - 1) / per) continue;
+    float4* t = Tseg + ((size_t)tj * N + i) * 100;
+    for (int q = lane; q < 100; q += 32) t[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
 }
 
 // T = sum over neighbour types of the partial sums, scaled by 1/S (kept in FP32, feature-major,
@@ -1423,8 +1461,10 @@ __global__ void __launch_bounds__(kRows) k_emb_images(const float* __restrict__ 
   const float* W = w + (size_t)blockIdx.x * kEmbParams;
   unsigned char* r = img + (size_t)blockIdx.x * kImgBytes;
   load_fwd_weights<F16>(W, r, r + kImgFwdB3, reinterpret_cast<float*>(r + kImgFwdSmall));
+  unsigned char* b = r + kImgFwd;
+  load_bwd_ops<F16>(W, b, b + kImgBwdB3, reinterpret_cast<float*>(b + kImgBwdSmall));
 }
-static_assert(kImgFwd % 16 == 0 && kImgFwdB3 % 16 == 0 && kImgFwdSmall % 16 == 0,
+static_assert(kImgBwd % 16 == 0 && kImgBwdSmall % 16 == 0 && kImgFwd % 16 == 0 && kImgFwdB3 % 16 == 0 && kImgFwdSmall % 16 == 0,
               "bulk copies need 16-byte sizes and offsets");
 
 constexpr size_t kFwdSmem = 32768 + 4096 + 8192 + 2 * 14336 + kSmall * 4 + 160 + 1024;
@@ -1449,8 +1489,7 @@ dp_status launch_emb_images(Model* m) {
 dp_status launch_mix_descriptor(Model* m, int N) {
   const int nblk = cdiv(N, 1024);
   k_scan_local<<<dim3(nblk, m->ntypes), 1024, 0, m->stream>>>(N, m->ntypes, m->nl_count, m->rowoff, m->scan_blk);
-  k_scan_fix<<<dim3(nblk, m->ntypes), 1024, 0, m->stream>>>(N, nblk, m->rowoff, m->scan_blk);
-  DP_CUDA_TRY(m, cudaMemsetAsync(m->Tseg, 0, sizeof(float) * 400 * (size_t)N * m->ntypes, m->stream));
+  if (nblk > 1) k_scan_fix<<<dim3(nblk, m->ntypes), 1024, 0, m->stream>>>(N, nblk, m->rowoff, m->scan_blk);
   MixArgs a = make_mix_args(m, N);
   const bool f16 = m->prec == DP_MIX_FP16;
   const bool tab = m->tab_n > 0;
@@ -1459,6 +1498,8 @@ dp_status launch_mix_descriptor(Model* m, int N) {
   const void* fn = reinterpret_cast<const void*>(fk);
   DP_CUDA_TRY(m, ensure_smem(fn, kFwdSmem));
   const int grid = tuned_grid(m, 0, num_sms() * blocks_per_sm(fn, kRows, kFwdSmem, kTmemCols));
+  k_mix_zero<<<cdiv(N, 8), 256, 0, m->stream>>>(N, m->ntypes, grid, m->nrep, m->rowoff, reinterpret_cast<float4*>(m->Tseg),
+                                                m->force, reinterpret_cast<float4*>(m->force32), m->vir_rep);
   fk<<<grid, kRows, kFwdSmem, m->stream>>>(a);
   if (m->sub_ev[0]) DP_CUDA_TRY(m, cudaEventRecord(m->sub_ev[0], m->stream));
   const int dgrid = std::max(1, std::min((N + kDescWarps - 1) / kDescWarps, tuned_grid(m, 3, 8 * num_sms())));
@@ -1479,30 +1520,36 @@ dp_status launch_mix_descriptor(Model* m, int N) {
     k_mix_descriptor<false><<<dgrid, 32 * kDescWarps, dsm, m->stream>>>(
         N, m->ntypes, 1.f / (float)m->S, m->Tseg, static_cast<float4*>(m->Tm), static_cast<unsigned short*>(m->Dm),
         pa);
-  m->launches += 4;
+  m->launches += nblk > 1 ? 5 : 4;
   DP_LAUNCH_CHECK(m);
   return DP_OK;
 }
 
-dp_status launch_mix_embed_backward(Model* m, int N) {
+// Up to this many neighbour slots (atoms x S) a CTA of the backward walks few tiles and converting the
+// weights is a good part of its time: the image variant runs instead.  Measured, converting -> image: 192
+// water atoms (26 k slots) 42 -> 32 us, 4,500 (0.6 M) 118 -> 112, 8,100 (1.1 M) 161 -> 157; 6,912 Cu atoms
+// (3.5 M) 195 -> 198.
+constexpr long kImgSlots = 1200000;
+
+dp_status launch_mix_embed_backward(Model* m, int N, bool fold) {
   const int dt_grid = std::max(1, std::min((N + kDtWarps - 1) / kDtWarps, tuned_grid(m, 2, 5 * num_sms())));
   k_mix_dT<<<dt_grid, 32 * kDtWarps, 0, m->stream>>>(N, 1.f / (float)m->S, static_cast<const float4*>(m->Tm),
                                                               static_cast<const unsigned short*>(m->dD),
                                                               static_cast<float4*>(m->dTm));
-  DP_CUDA_TRY(m, cudaMemsetAsync(m->vir_rep, 0, sizeof(double) * 9 * (size_t)m->nrep, m->stream));
-  DP_CUDA_TRY(m, cudaMemsetAsync(m->force32, 0, sizeof(float) * 4 * (size_t)N, m->stream));
   if (m->sub_ev[1]) DP_CUDA_TRY(m, cudaEventRecord(m->sub_ev[1], m->stream));
   MixArgs a = make_mix_args(m, N);
   const bool f16 = m->prec == DP_MIX_FP16;
   const bool tab = m->tab_n > 0;
+  const bool img = !tab && (long)N * m->S <= kImgSlots;
   auto bk = f16 ? (tab ? k_mix_embed_bwd<true, true> : k_mix_embed_bwd<true, false>)
                 : (tab ? k_mix_embed_bwd<false, true> : k_mix_embed_bwd<false, false>);
+  if (img) bk = f16 ? k_mix_embed_bwd<true, false, false, true> : k_mix_embed_bwd<false, false, false, true>;
   const void* fn = reinterpret_cast<const void*>(bk);
   DP_CUDA_TRY(m, ensure_smem(fn, kBwdSmem));
   const int grid = tuned_grid(m, 1, num_sms() * blocks_per_sm(fn, kRows, kBwdSmem, kTmemCols));
   bk<<<grid, kRows, kBwdSmem, m->stream>>>(a);
-  k_fold_force32<<<cdiv(3L * N, 256), 256, 0, m->stream>>>(3 * N, m->force32, m->force);
-  m->launches += 3;
+  if (fold) k_fold_force32<<<cdiv(3L * N, 256), 256, 0, m->stream>>>(3 * N, m->force32, m->force);
+  m->launches += fold ? 3 : 2;
   DP_LAUNCH_CHECK(m);
   return DP_OK;
 }

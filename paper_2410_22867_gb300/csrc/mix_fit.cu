@@ -74,13 +74,14 @@ struct FitMaps {
 
 struct FitArgs {
   int N, ntypes;
+  int parts;               // CTAs a tile: each computes dz1 and its share of the B1 chunks (1, 2 or 5)
   const int* type_off;
   const int* type_count;
   const float* w;          // theta fp32
   long fit_base;           // offset of the first fitting block in theta
   long ebias_off;
-  unsigned short* f1;      // [N][240] 16-bit: 1 - h1^2
-  unsigned short* f2;      // [N][240] 16-bit: 1 - t2^2
+  unsigned short* f1[5];   // per part [N][240] 16-bit: 1 - h1^2
+  unsigned short* f2[5];   // per part [N][240] 16-bit: 1 - t2^2
   unsigned short* dD;      // [N][1600] fp16
   double* e_atom;
   int* err;
@@ -225,6 +226,10 @@ __device__ __forceinline__ TileOf tile_of(int tile, const int* s_tiles, const Fi
 //   warp 8 (lane 0)      the MMAs of each GEMM once its operands landed and the epilogue that
 //                        writes its A operand finished (events epi, alternating barriers);
 //   warps 0..7           the epilogues after each GEMM's accumulator is complete (accb).
+// With fewer tiles than SMs, `parts` CTAs take the same tile: the GEMMs up to dz1 run in each (their
+// latency is what a lone tile costs), and each does its share of the B1 chunks, the longest part of a
+// tile (14 of 64 us alone).  All parts of a tile walk the weights in the same order, so they hold
+// the same dz1; part 0 writes E_i.
 // Each waits only with bounded polls; a role that gives up sets the shared abort flag and the
 // others leave their loops at their next wait.
 template <bool F16>
@@ -256,6 +261,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
   tc::tc_fence_after();
   const uint32_t tmem = tslot;
   const int ntiles = s_tiles[a.ntypes];
+  const int part = blockIdx.x % a.parts, tile0 = blockIdx.x / a.parts, tstep = gridDim.x / a.parts;
+  const int nb1 = kB1Chunks / a.parts;                                   // B1 chunks of this CTA
+  const int b1_first = (tile0 % kB1Chunks + part * nb1) % kB1Chunks;     // the first of them
   volatile int* abort_flag = &s_abort;
 
   if (w >= kLoadWarp) {
@@ -267,23 +275,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
       for (int q = 0; q < 10; ++q) L.uses[q] = L.issued[q] = 0;
       L.keep = tc::make_policy_evict_last();
       L.stream = tc::make_policy_evict_first();
-      L.rot_l1 = blockIdx.x % kL1Jobs;
-      L.rot_s = blockIdx.x & 3;
-      L.rot_b1 = blockIdx.x % kB1Chunks;
+      L.rot_l1 = tile0 % kL1Jobs;
+      L.rot_s = tile0 & 3;
+      L.rot_b1 = b1_first;
       uint32_t rph[3] = {0, 0, 0};
       auto wait_rf = [&](int r) {
         L.ok = L.ok && tc::mbar_wait(&rf[r], rph[r] & 1u, a.err);
         rph[r] += 1;
       };
-      for (int tile = blockIdx.x; tile < ntiles && L.ok && !*abort_flag; tile += gridDim.x) {
+      for (int tile = tile0; tile < ntiles && L.ok && !*abort_flag; tile += tstep) {
         const TileOf T = tile_of(tile, s_tiles, a);
-        if (tile != (int)blockIdx.x) wait_rf(2);  // the B1 MMAs of the previous tile read X and the B1 slots
+        if (tile != tile0) wait_rf(2);  // the B1 MMAs of the previous tile read X and the B1 slots
         for (int j = 0; j < kL1Jobs; ++j) L.l1(T.ty, T.row0, j);
         wait_rf(0);  // the split slots overlay L1 slot 2
         for (int g = 0; g < 4; ++g)
           for (int i = 0; i < kSplitJobs; ++i) L.split(T.ty, g, i);
         wait_rf(1);  // the B1 slots overlay X_lo (read by the B2 MMAs) and the split slots
-        for (int j = 0; j < kB1Jobs; ++j) L.b1(T.ty, j);
+        for (int j = 0; j < 2 * nb1; ++j) L.b1(T.ty, j);
       }
       if (!L.ok) *abort_flag = 1;
       // copies still in flight land before the CTA can finish
@@ -295,7 +303,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
     // ------------------------------------------------------------------ MMA issue
     if (lane == 0) {
       const uint32_t id240 = tc::idesc_f16(128, 240, F16), id160 = tc::idesc_f16(128, kBChunk, F16);
-      const int rot_s = blockIdx.x & 3;
+      const int rot_s = tile0 & 3;
       uint32_t uses[10];
       for (int q = 0; q < 10; ++q) uses[q] = 0;
       bool ok = true;
@@ -348,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
         }
         tc::mma_commit(&accb[n & 1]);
       };
-      for (int tile = blockIdx.x; tile < ntiles && ok && !*abort_flag; tile += gridDim.x) {
+      for (int tile = tile0; tile < ntiles && ok && !*abort_flag; tile += tstep) {
         // L1: z1 = D W1 into columns 0..239 (free: the previous tile's B1 drains are done)
         for (int j = 0; j < kL1Jobs && ok; ++j) {
           const int k = j % kL1Slots;
@@ -366,14 +374,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
           tc::mma_commit(&accb[0]);
           if (g == 3) tc::mma_commit(&rf[1]);
         }
-        // B1 in ten chunks over two TMEM regions: chunk n + 2 once chunk n has been drained
+        // B1 in nb1 >= 2 chunks over two TMEM regions: chunk n + 2 once chunk n has been drained
         if (ok && wait_epi()) {
           issue_b1(0);
           issue_b1(1);
-          for (int n = 0; n < kB1Chunks && ok; ++n) {
+          if (nb1 == 2) tc::mma_commit(&rf[2]);
+          for (int n = 0; n < nb1 && ok; ++n) {
             if (!wait_epi()) break;
-            if (n + 2 < kB1Chunks) issue_b1(n + 2);
-            if (n + 2 == kB1Chunks - 1) tc::mma_commit(&rf[2]);
+            if (n + 2 < nb1) issue_b1(n + 2);
+            if (n + 2 == nb1 - 1) tc::mma_commit(&rf[2]);
           }
         }
       }
@@ -413,7 +422,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
       ev += 1;
     };
 
-    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    for (int tile = tile0; tile < ntiles && ok; tile += tstep) {
       const TileOf T = tile_of(tile, s_tiles, a);
       const int ty = T.ty, row0 = T.row0, nrow = T.nrow;
       const bool valid = row < nrow;
@@ -447,7 +456,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
         }
         store_x16<F16>(sm, row, 16 * c, h, true);
         tc::tmem_st16(resid + 16 * c, h);
-        if (valid) store_g16<F16>(a.f1 + grow * kF + 16 * c, f);
+        if (valid) store_g16<F16>(a.f1[part] + grow * kF + 16 * c, f);
       }
       if (half == 1) {  // K columns 240..255 stay zero (hi and lo)
         tc::st_chunk(sm + kXHi + 3 * kBlk, row, 48, make_uint4(0, 0, 0, 0));
@@ -475,7 +484,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
         }
         store_x16<F16>(sm, row, 16 * c, r, true);
         tc::tmem_st16(resid + 16 * c, r);
-        if (valid) store_g16<F16>(a.f2 + grow * kF + 16 * c, f);
+        if (valid) store_g16<F16>(a.f2[part] + grow * kF + 16 * c, f);
       }
       tc::tmem_wait_st();
       if (!sync_epi()) break;
@@ -502,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
       if (half == 1) sE[row] = e;
       if (!sync_epi()) break;
       signal();
-      if (half == 0 && valid)
+      if (half == 0 && valid && part == 0)
         a.e_atom[grow] = (double)e + (double)sE[row] + (double)P[kFb4] + (double)a.w[a.ebias_off + ty];
 
       // ---- B3 epilogue: dh2 = w4 + dz3 W3^T ; dz2 = dh2 (1 - t2^2)
@@ -512,7 +521,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
         for (int c = 0; c < 8; ++c) {
           const int cc = c_beg + c;
           if (valid && cc < c_end) {
-            const uint4* src = reinterpret_cast<const uint4*>(a.f2 + grow * kF + 16 * cc);
+            const uint4* src = reinterpret_cast<const uint4*>(a.f2[part] + grow * kF + 16 * cc);
             fq[2 * c] = src[0];
             fq[2 * c + 1] = src[1];
           } else {
@@ -550,7 +559,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
         for (int c = 0; c < 8; ++c) {
           const int cc = c_beg + c;
           if (valid && cc < c_end) {
-            const uint4* src = reinterpret_cast<const uint4*>(a.f1 + grow * kF + 16 * cc);
+            const uint4* src = reinterpret_cast<const uint4*>(a.f1[part] + grow * kF + 16 * cc);
             fq[2 * c] = src[0];
             fq[2 * c + 1] = src[1];
           } else {
@@ -577,7 +586,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
       signal();
 
       // ---- B1 drains: dE/dD = dz1 W1^T, chunk n from TMEM region n & 1 through the staging tile
-      for (int n = 0; n < kB1Chunks; ++n) {
+      for (int n = 0; n < nb1; ++n) {
         const int rg = n & 1;
         wait_acc(rg);
         const uint32_t src = rg ? acc1 : acc0;
@@ -599,10 +608,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
         }
         if (!sync_epi()) break;
         // TMEM region n & 1 is free: chunk n + 2 may start under the write-out
-        if (n + 1 < kB1Chunks) signal();
+        if (n + 1 < nb1) signal();
         // whole row segments (320 B) to dE/dD: warp w writes rows w, w + 8, ...; lanes 0..19
         {
-          const int col0 = kBChunk * (((blockIdx.x % kB1Chunks) + n) % kB1Chunks);
+          const int col0 = kBChunk * ((b1_first + n) % kB1Chunks);
           for (int r = w; r < nrow; r += kEpi / 32)
             if (lane < kBChunk / 8) {
               const uint4 v = *reinterpret_cast<const uint4*>(sm + kStage + r * kStageRow + 16 * lane);
@@ -612,7 +621,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mix_fit(const __grid_constant__
         if (!sync_epi()) break;
         // the last chunk's signal also frees the staging tile, which the next tile's split
         // slots overlay
-        if (n + 1 == kB1Chunks) signal();
+        if (n + 1 == nb1) signal();
       }
     }
   }
@@ -754,8 +763,10 @@ dp_status launch_mix_fitting(Model* m, int N) {
   a.N = N; a.ntypes = m->ntypes; a.type_off = m->type_off; a.type_count = m->type_count; a.w = m->w32;
   a.fit_base = (long)m->ntypes * m->ntypes * kEmbParams;
   a.ebias_off = a.fit_base + (long)m->ntypes * kFitParams;
-  a.f1 = static_cast<unsigned short*>(m->act[0]);
-  a.f2 = static_cast<unsigned short*>(m->act[1]);
+  for (int p = 0; p < 5; ++p) {  // each activation buffer holds two 16-bit arrays
+    a.f1[p] = static_cast<unsigned short*>(m->act[p]);
+    a.f2[p] = a.f1[p] + (size_t)m->max_atoms * kF;
+  }
   a.dD = static_cast<unsigned short*>(m->dD);
   a.e_atom = m->e_atom;
   a.err = m->err;
@@ -763,7 +774,9 @@ dp_status launch_mix_fitting(Model* m, int N) {
   const void* fn = f16 ? reinterpret_cast<const void*>(k_mix_fit<true>) : reinterpret_cast<const void*>(k_mix_fit<false>);
   DP_CUDA_TRY(m, ensure_smem(fn, kFitSmem));
   const int tiles_upper = cdiv(N, kFR) + m->ntypes;
-  const int grid = std::max(1, std::min(num_sms(), tiles_upper));
+  // a tile for 2 or 5 CTAs while all of them run at once
+  a.parts = 5 * tiles_upper <= num_sms() ? 5 : 2 * tiles_upper <= num_sms() ? 2 : 1;
+  const int grid = a.parts * std::max(1, std::min(num_sms() / a.parts, tiles_upper));
   if (f16) k_mix_fit<true><<<grid, kThreads, kFitSmem, m->stream>>>(*maps_of(m), a);
   else k_mix_fit<false><<<grid, kThreads, kFitSmem, m->stream>>>(*maps_of(m), a);
   m->launches += 1;

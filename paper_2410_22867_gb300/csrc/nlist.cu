@@ -88,22 +88,31 @@ __global__ void k_type_count(const int* __restrict__ types, int N, int ntypes, i
 }
 
 __global__ void k_type_scan(int nblk, int ntypes, int* blk_count, int* type_count, int* type_off) {
-  // single thread: nblk <= a few hundred
-  if (threadIdx.x != 0) return;
+  // one warp: 32 blocks' counts at a time
+  const int lane = threadIdx.x;
   int off = 0;
   for (int t = 0; t < ntypes; ++t) {
-    type_off[t] = off;
+    if (lane == 0) type_off[t] = off;
     int run = off;
-    for (int b = 0; b < nblk; ++b) {
-      int c = blk_count[b * kMaxTypes + t];
-      blk_count[b * kMaxTypes + t] = run;
-      run += c;
+    for (int b0 = 0; b0 < nblk; b0 += 32) {
+      const int b = b0 + lane;
+      const int c = b < nblk ? blk_count[b * kMaxTypes + t] : 0;
+      int x = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (b < nblk) blk_count[b * kMaxTypes + t] = run + x - c;
+      run += __shfl_sync(0xffffffffu, x, 31);
     }
-    type_count[t] = run - off;
+    if (lane == 0) type_count[t] = run - off;
     off = run;
   }
-  type_off[ntypes] = off;
-  type_count[kMaxTypes] = off;
+  if (lane == 0) {
+    type_off[ntypes] = off;
+    type_count[kMaxTypes] = off;
+  }
 }
 
 __global__ void k_type_scatter(const int* __restrict__ types, int N, int ntypes, const int* blk_off,
@@ -133,24 +142,24 @@ __global__ void k_type_scatter(const int* __restrict__ types, int N, int ntypes,
   }
 }
 
-__global__ void k_load_positions(const double* __restrict__ coords, const int* __restrict__ perm, int N,
-                                 dvec4* x) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= N) return;
-  int u = perm[k];
-  x[k] = make_dvec4(coords[3 * u], coords[3 * u + 1], coords[3 * u + 2], 0.0);
-}
-
 // ------------------------------------------------------------------ cells
 // xf.w carries the atom's type (bit pattern), read by the Verlet-list gather; xq holds the
-// wrapped position in fixed point for exact pair vectors.
-__global__ void k_wrap_bin(int N, const int* __restrict__ irep, const int* __restrict__ itype,
+// wrapped position in fixed point for exact pair vectors.  Starts from the caller's positions (coords,
+// permuted) or, in an MD rebuild (coords null), from the internal ones.
+__global__ void k_wrap_bin(int N, const double* __restrict__ coords, const int* __restrict__ perm,
+                           const int* __restrict__ irep, const int* __restrict__ itype,
                            const RepGeom* __restrict__ geom, dvec4* x, dvec4* xref, float4* xf, qvec4* xq,
                            float4* delta, int* cell_of, int* cell_count) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= N) return;
   const RepGeom& g = geom[irep[k]];
-  dvec4 p = x[k];
+  dvec4 p;
+  if (coords) {
+    const size_t u = (size_t)perm[k];
+    p = make_dvec4(coords[3 * u], coords[3 * u + 1], coords[3 * u + 2], 0.0);
+  } else {
+    p = x[k];
+  }
   double w[3], sf[3] = {0.0, 0.0, 0.0};
   if (!g.tri) {
     w[0] = wrap1(p.x, g.L[0]);
@@ -438,23 +447,26 @@ __global__ void __launch_bounds__(32 * kVerletWarps) k_verlet(VerletArgs a) {
 // instead of once per atom.  Accepted candidates go to a per-warp queue with their list slots;
 // the exact pair vectors (an L2 gather of the fixed-point position and integer arithmetic) are
 // formed 32 at a time from the queue, with every lane busy, instead of in the test loop where a
-// quarter of the lanes or fewer accept.  Cells whose stencil has more than kMaxStencil cells or
-// more than kCellCap candidates (small, sparse or triclinic boxes) hand their atoms to k_verlet.
+// quarter of the lanes or fewer accept.  Cells whose stencil has more than MAXS cells or
+// more than kCellCap candidates (dense or very flat cells) hand their atoms to k_verlet.  A triclinic
+// stencil has one more layer (7 x 7 x 7 cells): handing those over made k_verlet 87 of the 90 us of
+// a 4,500-atom box's list.
 constexpr int kCellWarps = 8;
 constexpr int kCellCap = 2048;
-constexpr int kMaxStencil = 125;
+constexpr int kStencilOrtho = 125, kStencilTri = 343;  // template variants: the larger costs a CTA an SM
 constexpr int kQueue = 64;
 constexpr size_t kCellSmem = (size_t)kCellCap * (sizeof(float4) + sizeof(int));
 
+template <int MAXS>
 __global__ void __launch_bounds__(32 * kCellWarps) k_verlet_cell(VerletArgs a) {
   extern __shared__ float4 s_cx[];                      // [kCellCap] position + shift, w = type | stencil slot << 8
   int* s_cj = reinterpret_cast<int*>(s_cx + kCellCap);  // [kCellCap] atom
-  __shared__ int s_beg[kMaxStencil], s_off[kMaxStencil + 1], s_code[kMaxStencil];
-  __shared__ float s_sh[kMaxStencil][3];
-  __shared__ long long s_shq[kMaxStencil][3];
+  __shared__ int s_beg[MAXS], s_off[MAXS + 1], s_code[MAXS];
+  __shared__ float s_sh[MAXS][3];
+  __shared__ long long s_shq[MAXS][3];
   __shared__ int s_wsum[kCellWarps], s_total, s_wbase;
   __shared__ int s_qj[kCellWarps][kQueue], s_qe[kCellWarps][kQueue];  // queue: atom, slot in the row
-  __shared__ unsigned char s_qk[kCellWarps][kQueue];                  // queue: stencil slot
+  __shared__ unsigned short s_qk[kCellWarps][kQueue];                 // queue: stencil slot
   const int cid = blockIdx.x;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int cb = a.cell_start[cid], ce = a.cell_start[cid + 1];
@@ -468,7 +480,7 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_verlet_cell(VerletArgs a) {
   const RepGeom& g = a.geom[a.irep[a.cell_atoms[cb]]];
   const int sy = 2 * g.m[1] + 1, sz = 2 * g.m[2] + 1;
   const int ncell = (2 * g.m[0] + 1) * sy * sz;
-  if (ncell > kMaxStencil) {
+  if (ncell > MAXS) {
     hand_over();
     return;
   }
@@ -477,29 +489,34 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_verlet_cell(VerletArgs a) {
   const int kc = (g.m[0] * sy + g.m[1]) * sz + g.m[2];
   const int rel = cid - g.cell_off;
   const int ci[3] = {rel / (g.nc[1] * g.nc[2]), (rel / g.nc[2]) % g.nc[1], rel % g.nc[2]};
-  int num = 0;
-  if (t < ncell) {
-    const int o[3] = {t / (sy * sz) - g.m[0], (t / sz) % sy - g.m[1], t % sz - g.m[2]};
-    int n[3], cc[3];
+  // thread t holds the stencil slots 2 t and 2 t + 1 (ncell <= 343 < 64 * kCellWarps)
+  int num[2] = {0, 0};
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const int v = ci[q] + o[q];
-      n[q] = floor_div(v, g.nc[q]);
-      cc[q] = v - n[q] * g.nc[q];
-    }
+  for (int h = 0; h < 2; ++h) {
+    const int sl = 2 * t + h;
+    if (sl < ncell) {
+      const int o[3] = {sl / (sy * sz) - g.m[0], (sl / sz) % sy - g.m[1], sl % sz - g.m[2]};
+      int n[3], cc[3];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      s_sh[t][q] = ((float)n[0] * g.Hf[q] + (float)n[1] * g.Hf[3 + q]) + (float)n[2] * g.Hf[6 + q];
-      s_shq[t][q] = g.tri ? (long long)n[0] * g.Hq[q] + (long long)n[1] * g.Hq[3 + q] + (long long)n[2] * g.Hq[6 + q]
-                          : (long long)n[q] * g.Hq[4 * q];
+      for (int q = 0; q < 3; ++q) {
+        const int v = ci[q] + o[q];
+        n[q] = floor_div(v, g.nc[q]);
+        cc[q] = v - n[q] * g.nc[q];
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        s_sh[sl][q] = ((float)n[0] * g.Hf[q] + (float)n[1] * g.Hf[3 + q]) + (float)n[2] * g.Hf[6 + q];
+        s_shq[sl][q] = g.tri ? (long long)n[0] * g.Hq[q] + (long long)n[1] * g.Hq[3 + q] + (long long)n[2] * g.Hq[6 + q]
+                             : (long long)n[q] * g.Hq[4 * q];
+      }
+      const int c = g.cell_off + (cc[0] * g.nc[1] + cc[1]) * g.nc[2] + cc[2];
+      s_beg[sl] = a.cell_start[c];
+      num[h] = a.cell_start[c + 1] - s_beg[sl];
+      s_code[sl] = pack_img(n[0], n[1], n[2]);
     }
-    const int c = g.cell_off + (cc[0] * g.nc[1] + cc[1]) * g.nc[2] + cc[2];
-    s_beg[t] = a.cell_start[c];
-    num = a.cell_start[c + 1] - s_beg[t];
-    s_code[t] = pack_img(n[0], n[1], n[2]);
   }
-  // exclusive prefix of the stencil cells' sizes (ncell <= 125 < 32 * kCellWarps)
-  int incl = num;
+  // exclusive prefix of the stencil cells' sizes
+  int incl = num[0] + num[1];
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -509,7 +526,9 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_verlet_cell(VerletArgs a) {
   __syncthreads();
   int base = 0;
   for (int u = 0; u < w; ++u) base += s_wsum[u];
-  if (t < ncell) s_off[t] = base + incl - num;
+  const int off0 = base + incl - num[0] - num[1];
+  if (2 * t < ncell) s_off[2 * t] = off0;
+  if (2 * t + 1 < ncell) s_off[2 * t + 1] = off0 + num[0];
   if (t == 32 * kCellWarps - 1) s_total = base + incl;
   __syncthreads();
   const int T = s_total;
@@ -615,7 +634,7 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_verlet_cell(VerletArgs a) {
       if (off >= 0) {
         const int qs = qn + __popc(qm & lt);
         s_qj[w][qs] = j;
-        s_qk[w][qs] = (unsigned char)k;
+        s_qk[w][qs] = (unsigned short)k;
         s_qe[w][qs] = off;
       }
       qn += __popc(qm);
@@ -625,7 +644,7 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_verlet_cell(VerletArgs a) {
         int rj = 0, re = 0, rk = 0;
         if (lane < qn - 32) { rj = s_qj[w][32 + lane]; re = s_qe[w][32 + lane]; rk = s_qk[w][32 + lane]; }
         __syncwarp();
-        if (lane < qn - 32) { s_qj[w][lane] = rj; s_qe[w][lane] = re; s_qk[w][lane] = (unsigned char)rk; }
+        if (lane < qn - 32) { s_qj[w][lane] = rj; s_qe[w][lane] = re; s_qk[w][lane] = (unsigned short)rk; }
         qn -= 32;
       }
     }
@@ -885,13 +904,6 @@ dp_status launch_type_sort(Model* m, const int* types_user, int N) {
   return DP_OK;
 }
 
-dp_status launch_load_positions(Model* m, const double* coords_user, int N) {
-  k_load_positions<<<cdiv(N, 256), 256, 0, m->stream>>>(coords_user, m->perm, N, m->x);
-  m->launches += 1;
-  DP_LAUNCH_CHECK(m);
-  return DP_OK;
-}
-
 // Largest |x| a wrapped coordinate or a single-cell shift can have: max over rows of sum |H_ac|.
 static double max_box_length(const Model* m) {
   double Lmax = 0;
@@ -904,14 +916,16 @@ static double max_box_length(const Model* m) {
   return Lmax;
 }
 
-dp_status launch_rebuild(Model* m, int N, bool with_skin) {
+dp_status launch_rebuild(Model* m, int N, bool with_skin, const double* coords) {
   cudaStream_t s = m->stream;
-  DP_CUDA_TRY(m, cudaMemsetAsync(m->cell_count, 0, sizeof(int) * m->ncells, s));
-  DP_CUDA_TRY(m, cudaMemsetAsync(m->cell_fill, 0, sizeof(int) * m->ncells, s));
-  k_wrap_bin<<<cdiv(N, 256), 256, 0, s>>>(N, m->irep, m->itype, m->geom, m->x, m->xref, m->xf, m->xq,
+  // cell counters, fill counters and the work count of the Verlet build: one memset
+  int* cell_fill = m->cell_count + m->ncells;
+  int* work_n = cell_fill + m->ncells;
+  DP_CUDA_TRY(m, cudaMemsetAsync(m->cell_count, 0, sizeof(int) * (2 * (size_t)m->ncells + 1), s));
+  k_wrap_bin<<<cdiv(N, 128), 128, 0, s>>>(N, coords, m->perm, m->irep, m->itype, m->geom, m->x, m->xref, m->xf, m->xq,
                                           m->delta, m->cell_of, m->cell_count);
   k_scan_cells<<<1, 1024, 0, s>>>(m->ncells, m->cell_count, m->cell_start);
-  k_fill_cells<<<cdiv(N, 256), 256, 0, s>>>(N, m->cell_of, m->cell_start, m->xf, m->cell_fill, m->cell_atoms,
+  k_fill_cells<<<cdiv(N, 256), 256, 0, s>>>(N, m->cell_of, m->cell_start, m->xf, cell_fill, m->cell_atoms,
                                             m->cell_xf);
   VerletArgs a;
   a.N = N; a.ntypes = m->ntypes; a.VS = m->VS;
@@ -931,10 +945,15 @@ dp_status launch_rebuild(Model* m, int N, bool with_skin) {
   // cells by k_verlet_cell; the atoms of the cells it hands over by k_verlet, whose grid-stride
   // loop over the work list costs little when the list is empty
   a.work = m->vl_work;
-  a.work_n = m->vl_work + m->max_atoms;
-  DP_CUDA_TRY(m, cudaMemsetAsync(a.work_n, 0, sizeof(int), s));
-  DP_CUDA_TRY(m, ensure_smem(reinterpret_cast<const void*>(k_verlet_cell), kCellSmem));
-  k_verlet_cell<<<m->ncells, 32 * kCellWarps, kCellSmem, s>>>(a);
+  a.work_n = work_n;
+  int stencil = 0;  // the largest stencil of any replica
+  for (int r = 0; r < m->nrep; ++r) {
+    const int* h = m->geom_host[r].m;
+    stencil = std::max(stencil, (2 * h[0] + 1) * (2 * h[1] + 1) * (2 * h[2] + 1));
+  }
+  const auto fn = stencil > kStencilOrtho ? k_verlet_cell<kStencilTri> : k_verlet_cell<kStencilOrtho>;
+  DP_CUDA_TRY(m, ensure_smem(reinterpret_cast<const void*>(fn), kCellSmem));
+  fn<<<m->ncells, 32 * kCellWarps, kCellSmem, s>>>(a);
   k_verlet<<<std::min(cdiv(N, kVerletWarps), 8 * num_sms()), 32 * kVerletWarps, 0, s>>>(a);
   m->launches += 5;
   DP_LAUNCH_CHECK(m);

@@ -530,8 +530,8 @@ dp_status launch_fitting(Model* m, int N) {
   if (is_mixed(m)) return launch_mix_fitting(m, N);
   return launch_dig_fitting(m, N);
 }
-dp_status launch_embed_backward(Model* m, int N) {
-  if (is_mixed(m)) return launch_mix_embed_backward(m, N);
+dp_status launch_embed_backward(Model* m, int N, bool fold) {
+  if (is_mixed(m)) return launch_mix_embed_backward(m, N, fold);
   if (m->dig_ok && m->tab_n == 0) return launch_dig_embed_backward(m, N);
   return m->prec == DP_FP64 ? run_embed_backward<double>(m, N) : run_embed_backward<float>(m, N);
 }
