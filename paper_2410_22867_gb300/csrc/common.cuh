@@ -103,6 +103,7 @@ struct Model {
   unsigned long long* rdf_hist = nullptr;  // [kRdfMaxCells] pair-distance histogram (dp_rdf)
   double* tab64 = nullptr;
   float* tab32 = nullptr;
+  float* tab_nodes32 = nullptr;  // FP32 node data for the shared-memory table kernels (tab_mix.cu)
   void* tab_mem = nullptr;
   // 16-bit operand copies for the tensor-core kernels (per type), laid out by those kernels
   void* tc_weights = nullptr;
@@ -315,6 +316,14 @@ dp_status launch_format(Model* m, int N, bool images = false);  // images: also 
 dp_status launch_get_nlist(Model* m, int N, int* nlist, int* images);
 // tab.cu
 dp_status launch_tabulate(Model* m, double x0, double x1, int n);
+// tab_mix.cu (mixed precisions, table in shared memory)
+// Neighbour slots (atoms x S) from which the shared-memory kernels pay for loading the table: evaluations of 26 k
+// slots 331 us without, 385 with them; 212 k 485 / 407; 442 k 455 / 386; 2 M 1005 / 642.
+constexpr long kTabSlots = 100000;
+bool tab_smem_path(const Model* m, int N);
+dp_status launch_tab_nodes32(Model* m, int n, double h, const double* v, float* out);
+dp_status launch_tab_forward(Model* m, int N);
+dp_status launch_tab_backward(Model* m, int N);
 // diag.cu
 dp_status launch_rdf(Model* m, int nbins, double r_max, unsigned long long* hist_dev);
 dp_status launch_atom_virial_out(Model* m, int N, double* out);

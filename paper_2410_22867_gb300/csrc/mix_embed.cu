@@ -1500,7 +1500,12 @@ dp_status launch_mix_descriptor(Model* m, int N) {
   const int grid = tuned_grid(m, 0, num_sms() * blocks_per_sm(fn, kRows, kFwdSmem, kTmemCols));
   k_mix_zero<<<cdiv(N, 8), 256, 0, m->stream>>>(N, m->ntypes, grid, m->nrep, m->rowoff, reinterpret_cast<float4*>(m->Tseg),
                                                 m->force, reinterpret_cast<float4*>(m->force32), m->vir_rep);
-  fk<<<grid, kRows, kFwdSmem, m->stream>>>(a);
+  if (tab_smem_path(m, N)) {
+    const dp_status st = launch_tab_forward(m, N);
+    if (st != DP_OK) return st;
+  } else {
+    fk<<<grid, kRows, kFwdSmem, m->stream>>>(a);
+  }
   if (m->sub_ev[0]) DP_CUDA_TRY(m, cudaEventRecord(m->sub_ev[0], m->stream));
   const int dgrid = std::max(1, std::min((N + kDescWarps - 1) / kDescWarps, tuned_grid(m, 3, 8 * num_sms())));
   const size_t dsm = (size_t)kDescWarps * 2 * m->ntypes * kN3 * sizeof(float4);
@@ -1547,7 +1552,12 @@ dp_status launch_mix_embed_backward(Model* m, int N, bool fold) {
   const void* fn = reinterpret_cast<const void*>(bk);
   DP_CUDA_TRY(m, ensure_smem(fn, kBwdSmem));
   const int grid = tuned_grid(m, 1, num_sms() * blocks_per_sm(fn, kRows, kBwdSmem, kTmemCols));
-  bk<<<grid, kRows, kBwdSmem, m->stream>>>(a);
+  if (tab_smem_path(m, N)) {
+    const dp_status st = launch_tab_backward(m, N);
+    if (st != DP_OK) return st;
+  } else {
+    bk<<<grid, kRows, kBwdSmem, m->stream>>>(a);
+  }
   if (fold) k_fold_force32<<<cdiv(3L * N, 256), 256, 0, m->stream>>>(3 * N, m->force32, m->force);
   m->launches += fold ? 3 : 2;
   DP_LAUNCH_CHECK(m);

@@ -100,13 +100,14 @@ dp_status launch_tabulate(Model* m, double x0, double x1, int n) {
     m->tab_mem = nullptr;
     m->tab64 = nullptr;
     m->tab32 = nullptr;
+    m->tab_nodes32 = nullptr;
   }
   m->tab_n = 0;
   if (n == 0) return DP_OK;
   const int npairs = m->ntypes * m->ntypes;
   const size_t nodes = (size_t)npairs * (n + 1) * kN3 * 3;        // doubles
   const size_t coef = (size_t)npairs * n * kN3 * 8;               // entries
-  const size_t bytes = nodes * 8 + coef * 8 + coef * 4;
+  const size_t bytes = nodes * 8 + coef * 8 + coef * 4 + nodes * 4;
   void* mem = nullptr;
   cudaError_t e = cudaMalloc(&mem, bytes);
   if (e != cudaSuccess) {
@@ -117,12 +118,15 @@ dp_status launch_tabulate(Model* m, double x0, double x1, int n) {
   double* v = static_cast<double*>(mem);
   m->tab64 = v + nodes;
   m->tab32 = reinterpret_cast<float*>(m->tab64 + coef);
+  m->tab_nodes32 = m->tab32 + coef;
   const double h = (x1 - x0) / n;
   k_tab_nodes<<<dim3(n + 1, npairs), 128, 0, m->stream>>>(n, x0, h, m->w64, v);
   const size_t total = (size_t)npairs * n * kN3;
   k_tab_coef<<<(unsigned)((total + 255) / 256), 256, 0, m->stream>>>(npairs, n, h, v, m->tab64, m->tab32);
   m->launches += 2;
   DP_LAUNCH_CHECK(m);
+  const dp_status st = launch_tab_nodes32(m, n, h, v, m->tab_nodes32);
+  if (st != DP_OK) return st;
   DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));
   m->tab_n = n;
   m->tab_x0 = x0;
