@@ -6,7 +6,8 @@
 // accumulators of mma.sync hold them exactly.  Digit products of one order i + j share an
 // accumulator; orders above NO - 1 are dropped.
 //   FP64: 7 digits of 8 bits, orders 0..7:  34 digit products, 7 x K x 2^14 < 2^24 for K <= 146
-//   FP32: 3 digits of 9 bits, orders 0..2:   6 digit products, 3 x K x 2^16 < 2^24 for K <= 85
+//   FP32: 3 digits (9, 9 and up to 11 bits), orders 0..2: 6 digit products; orders 0 and 1 are exact sums,
+//         2 x K x 2^16 < 2^24 for K <= 127
 //
 // Why on this GPU: the FP64 pipe gives 2 multiply-adds a clock and SM (DFMA measured at 588 G/s; one
 // warp instruction occupies a sub-partition's pipe for 64 clocks), mma.sync with fp16 operands 1,032.
@@ -49,6 +50,13 @@ __device__ __forceinline__ void hmma8(float* c, uint32_t a0, uint32_t a1, uint32
       : "r"(a0), "r"(a1), "r"(b0));
 }
 
+// The same with a zero accumulator (no registers to clear first).
+__device__ __forceinline__ void hmma16z(float* c, const uint4& a, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1), "f"(0.f));
+}
+
 // Two bytes u0 (digit + 128 of the even column) and u1 (odd column) as a half2 of the digits:
 // 0x6400 | u is 1024 + u in fp16, and 1024 + 128 is taken off exactly.
 __device__ __forceinline__ uint32_t bytes_to_half2(uint32_t both) {
@@ -61,8 +69,6 @@ __device__ __forceinline__ uint32_t bytes_to_half2(uint32_t both) {
 __device__ __forceinline__ unsigned long long biased(long long v) {
   return (unsigned long long)v + 0x0080808080808080ull;
 }
-__device__ __forceinline__ uint32_t biased(int v) { return (uint32_t)v + (256u + (256u << 9) + (256u << 18)); }
-
 // out[i] = half2 of digit i of (u0, u1).
 __device__ __forceinline__ void split2(unsigned long long u0, unsigned long long u1, uint32_t* out) {
   const uint32_t l0 = (uint32_t)u0, h0 = (uint32_t)(u0 >> 32), l1 = (uint32_t)u1, h1 = (uint32_t)(u1 >> 32);
@@ -75,21 +81,26 @@ __device__ __forceinline__ void split2(unsigned long long u0, unsigned long long
   out[5] = bytes_to_half2(__byte_perm(l0, l1, 0x0501));
   out[6] = bytes_to_half2(__byte_perm(l0, l1, 0x0400));
 }
-// (two 9-bit fields as 1024 + field in fp16, 1024 + 256 taken off)
-__device__ __forceinline__ uint32_t fields_to_half2(uint32_t lo, uint32_t hi16) {
-  const uint32_t h = (((lo & 0xffffu) | (hi16 & 0xffff0000u)) & 0x01ff01ffu) | 0x64006400u;
-  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&h), __halves2half2(__ushort_as_half(0x6500), __ushort_as_half(0x6500)));
-  return *reinterpret_cast<const uint32_t*>(&d);
-}
-__device__ __forceinline__ void split2(uint32_t u0, uint32_t u1, uint32_t* out) {
-  out[0] = fields_to_half2(u0 >> 18, u1 >> 2);
-  out[1] = fields_to_half2(u0 >> 9, u1 << 7);
-  out[2] = fields_to_half2(u0, u1 << 16);
+// FP32: x as three fp16 numbers that carry their own weights: the nearest multiples of 2^-G and of 2^-(G+9) of what
+// is left (nine bits each, by adding and subtracting 1.5 x 2^23 times the step), and the rest.  Subnormal
+// fp16 is exact in the products.  Five additions a value, where integer digits took ten instructions.
+template <int G>
+__device__ __forceinline__ void split2f(float x0, float x1, uint32_t* out) {
+  constexpr float m0 = 12582912.f / (float)(1 << G), m1 = m0 / 512.f;
+  const float a0 = __fsub_rn(__fadd_rn(x0, m0), m0), a1 = __fsub_rn(__fadd_rn(x1, m0), m0);
+  const float r0 = __fsub_rn(x0, a0), r1 = __fsub_rn(x1, a1);
+  const float b0 = __fsub_rn(__fadd_rn(r0, m1), m1), b1 = __fsub_rn(__fadd_rn(r1, m1), m1);
+  const __half2 h0 = __floats2half2_rn(a0, a1), h1 = __floats2half2_rn(b0, b1),
+                h2 = __floats2half2_rn(__fsub_rn(r0, b0), __fsub_rn(r1, b1));
+  out[0] = *reinterpret_cast<const uint32_t*>(&h0);
+  out[1] = *reinterpret_cast<const uint32_t*>(&h1);
+  out[2] = *reinterpret_cast<const uint32_t*>(&h2);
 }
 
 // All kept digit products of one (16 x 16) x (16 x 8) block: consecutive instructions go to different
 // accumulators.
-template <class T>
+// FIRST: the block's first product of each order overwrites the accumulator.
+template <class T, bool FIRST = false>
 __device__ __forceinline__ void block16(float (*acc)[4], const uint4* a, const uint4* b) {
   constexpr int ND = Fmt<T>::ND, NO = Fmt<T>::NO;
 #pragma unroll
@@ -97,7 +108,10 @@ __device__ __forceinline__ void block16(float (*acc)[4], const uint4* a, const u
     const uint32_t b0 = (j & 1) ? b[j >> 1].z : b[j >> 1].x, b1 = (j & 1) ? b[j >> 1].w : b[j >> 1].y;
 #pragma unroll
     for (int i = 0; i < ND; ++i)
-      if (i + j < NO) hmma16(acc[i + j], a[i], b0, b1);
+      if (i + j < NO) {
+        if (FIRST && (j == 0 || i == ND - 1)) hmma16z(acc[i + j], a[i], b0, b1);
+        else hmma16(acc[i + j], a[i], b0, b1);
+      }
   }
 }
 template <class T>
@@ -136,10 +150,8 @@ __device__ __forceinline__ Pair64 join(const float (*acc)[4], int e) {
   p.lo = join4(acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
   return p;
 }
-// FP32: sum of the orders in units of 2^(BD 2 (ND - 1)).
-__device__ __forceinline__ float join_f(const float (*acc)[4], int e) {
-  return fmaf(fmaf(acc[2][e], 0.001953125f, acc[1][e]), 0.001953125f, acc[0][e]);
-}
+// FP32: sum of the orders (the digits carry their weights).
+__device__ __forceinline__ float join_f(const float (*acc)[4], int e) { return acc[0][e] + (acc[1][e] + acc[2][e]); }
 
 // 2^e as FP64 / FP32 (normal range).
 __host__ __device__ __forceinline__ double pow2d(int e) {

@@ -34,6 +34,10 @@ constexpr int kT2T = 4, kK2T = 4;           // dz2 W2^T (likewise)
 constexpr int kF2 = 0, kF3 = kF2 + kT2 * kK2, kF3T = kF3 + kT3 * kK3, kF2T = kF3T + kT3T * kK3T,
               kFrags = kF2T + kT2T * kK2T;  // fragment sets of a pair
 
+// uint4 words of a fragment set: FP64 four 16-byte loads a lane (digits 2q, 2q + 1; the eighth is zero); FP32
+// a 16-byte load (digits 0, 1) and an 8-byte one (digit 2).
+template <class T> struct SetWords { static constexpr int v = sizeof(T) == 8 ? 128 : 48; };
+
 __host__ __device__ __forceinline__ int unit2(int p, int t, int e) { return 4 * p + t < kN1 ? 4 * p + t + kN1 * e : -1; }
 __host__ __device__ __forceinline__ int unit3m(int j, int t) {
   if (j < 12) return 4 * (j >> 1) + t + kN1 * (j & 1);
@@ -60,7 +64,7 @@ struct DigArgs {
   T rc, rs, winv;
   int switch_kind;
   const T* stat;
-  const uint4* frag;           // [pair][kFrags][Q][32]
+  const uint4* frag;           // [pair][kFrags][SetWords]
   const PairScale* scale;      // [pair]
   const PairSmall<T>* small;   // [pair]
   const dig::TanhTab* tab;     // FP64
@@ -135,9 +139,9 @@ struct LayerF {
 __device__ __forceinline__ LayerD layer(const PairScale& p, int which, double) {
   return which == 2 ? LayerD{p.zs2, p.s2} : LayerD{p.zs3, p.s3};
 }
-// FP32: z = 2^(36 - sh - sw) (sum of orders) + b, the activations' scale sh being 25 (h1) or 24 (h2)
+// FP32: z = 2^(18 - sw) (sum of orders) + b
 __device__ __forceinline__ LayerF layer(const PairScale& p, int which, float) {
-  const int e = which == 2 ? 36 - 25 - p.sw2 : 36 - 24 - p.sw3;
+  const int e = 18 - (which == 2 ? p.sw2 : p.sw3);
   return LayerF{__int_as_float((127 + e) << 23)};
 }
 __device__ __forceinline__ long long act(const float (*acc)[4], int e, const LayerD& L, long long b,
@@ -154,79 +158,128 @@ __device__ __forceinline__ float act(const float (*acc)[4], int e, const LayerF&
 // The biased digits of activations: h1 (|h1| <= 1) and h2 (|h2| <= 2).
 __device__ __forceinline__ unsigned long long dig_h1(long long h) { return dig::biased(h); }
 __device__ __forceinline__ unsigned long long dig_h2(long long h) { return dig::biased((h + 1) >> 1); }
-__device__ __forceinline__ uint32_t dig_h1(float h) { return dig::biased(__float2int_rn(h * 33554432.f)); }
-__device__ __forceinline__ uint32_t dig_h2(float h) { return dig::biased(__float2int_rn(h * 16777216.f)); }
+__device__ __forceinline__ float dig_h1(float h) { return h; }  // FP32 splits the value itself
+__device__ __forceinline__ float dig_h2(float h) { return h; }
 __device__ __forceinline__ unsigned long long dig_of(double v) { return dig::biased(__double2ll_rn(v)); }
-__device__ __forceinline__ uint32_t dig_of(float v) { return dig::biased(__float2int_rn(v)); }
+__device__ __forceinline__ float dig_of(float v) { return v; }
 
 template <class T> struct DigWord;
 template <> struct DigWord<double> { using U = unsigned long long; };
-template <> struct DigWord<float> { using U = uint32_t; };
+template <> struct DigWord<float> { using U = float; };
+// G: fraction bits of the leading FP32 digit, 7 for activations (|h| <= 2), 0 for gradients scaled below 256
+template <int G>
+__device__ __forceinline__ void split2(unsigned long long u0, unsigned long long u1, uint32_t* out) { dig::split2(u0, u1, out); }
+template <int G>
+__device__ __forceinline__ void split2(float u0, float u1, uint32_t* out) { dig::split2f<G>(u0, u1, out); }
 
 // A fragment of one k step (all digits) from the lane's four slots of rows g (u[0]) and g + 8 (u[1]); only the
 // first two slots unless `full`.
-template <class T>
+template <class T, int G>
 __device__ __forceinline__ void get_a(uint4* a, const typename DigWord<T>::U (*u)[4], bool full) {
   constexpr int ND = Fmt<T>::ND;
   uint32_t x[ND], y[ND], z[ND], w[ND];
-  dig::split2(u[0][0], u[0][1], x);
-  dig::split2(u[1][0], u[1][1], y);
+  split2<G>(u[0][0], u[0][1], x);
+  split2<G>(u[1][0], u[1][1], y);
   if (full) {
-    dig::split2(u[0][2], u[0][3], z);
-    dig::split2(u[1][2], u[1][3], w);
+    split2<G>(u[0][2], u[0][3], z);
+    split2<G>(u[1][2], u[1][3], w);
   }
 #pragma unroll
   for (int i = 0; i < ND; ++i) a[i] = make_uint4(x[i], y[i], full ? z[i] : 0u, full ? w[i] : 0u);
 }
 // The same into the warp's shared memory.
-template <class T>
+template <class T, int G>
 __device__ __forceinline__ void put_a16(uint4* sA, int lane, const typename DigWord<T>::U (*u)[4]) {
   constexpr int ND = Fmt<T>::ND;
   uint4 a[ND];
-  get_a<T>(a, u, true);
+  get_a<T, G>(a, u, true);
 #pragma unroll
   for (int i = 0; i < ND; ++i) sA[i * 32 + lane] = a[i];
 }
-template <class T>
+template <class T, int G>
 __device__ __forceinline__ void put_a8(uint4* sA, int lane, const typename DigWord<T>::U (*u)[4]) {
   constexpr int ND = Fmt<T>::ND;
   uint32_t x[ND], y[ND];
-  dig::split2(u[0][0], u[0][1], x);
-  dig::split2(u[1][0], u[1][1], y);
+  split2<G>(u[0][0], u[0][1], x);
+  split2<G>(u[1][0], u[1][1], y);
 #pragma unroll
   for (int i = 0; i < ND; ++i) reinterpret_cast<uint2*>(sA)[i * 32 + lane] = make_uint2(x[i], y[i]);
 }
 
-// acc += A (k steps 0..KS-1 of sA) times the fragments of one n-tile; with TAIL the last step has 8 columns.
+// The lane's B fragments of one set.
+template <class T>
+__device__ __forceinline__ void load_b(uint4* b, const uint4* __restrict__ set, int lane) {
+  if constexpr (sizeof(T) == 8) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = __ldg(set + q * 32 + lane);
+  } else {
+    b[0] = __ldg(set + lane);
+    const uint2 c = __ldg(reinterpret_cast<const uint2*>(set + 32) + lane);
+    b[1] = make_uint4(c.x, c.y, 0u, 0u);
+  }
+}
+
+// acc = A (KS k steps) times the fragments of one n-tile; with TAIL the last step has 8 columns.
+// FP64: A from the warp's shared memory (its digits are 100 registers); FP32: from registers, since reading
+// A again for every n-tile made the kernels bound by shared-memory bandwidth.
 template <class T, int KS, bool TAIL>
-__device__ __forceinline__ void product(float (*acc)[4], const uint4* sA, const uint4* __restrict__ fr, int lane) {
+__device__ __forceinline__ void product(float (*acc)[4], const uint4* A, const uint4* __restrict__ fr, int lane) {
   constexpr int ND = Fmt<T>::ND, Q = dig::Frag<T>::Q;
-  dig::zero_acc<T>(acc);
+  constexpr bool D = sizeof(T) == 8;
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
     uint4 b[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) b[q] = __ldg(fr + (s * Q + q) * 32 + lane);
+    load_b<T>(b, fr + s * SetWords<T>::v, lane);
     if (TAIL && s == KS - 1) {
       uint2 a[ND];
 #pragma unroll
-      for (int i = 0; i < ND; ++i) a[i] = reinterpret_cast<const uint2*>(sA + s * ND * 32)[i * 32 + lane];
+      for (int i = 0; i < ND; ++i) {
+        if constexpr (D) a[i] = reinterpret_cast<const uint2*>(A + s * ND * 32)[i * 32 + lane];
+        else a[i] = make_uint2(A[s * ND + i].x, A[s * ND + i].y);
+      }
       dig::block8<T>(acc, a, b);
     } else {
       uint4 a[ND];
 #pragma unroll
-      for (int i = 0; i < ND; ++i) a[i] = sA[(s * ND + i) * 32 + lane];
-      dig::block16<T>(acc, a, b);
+      for (int i = 0; i < ND; ++i) a[i] = D ? A[(s * ND + i) * 32 + lane] : A[s * ND + i];
+      if (s == 0) dig::block16<T, true>(acc, a, b);
+      else dig::block16<T>(acc, a, b);
     }
   }
 }
+// A fragments of k step s: into shared memory (FP64) or the register array (FP32).
+template <class T, int G>
+__device__ __forceinline__ void put_a(uint4* A, int s, bool full, int lane, const typename DigWord<T>::U (*u)[4]) {
+  constexpr int ND = Fmt<T>::ND;
+  if constexpr (sizeof(T) == 8) {
+    if (full) put_a16<T, G>(A + s * ND * 32, lane, u);
+    else put_a8<T, G>(A + s * ND * 32, lane, u);
+  } else {
+    get_a<T, G>(A + s * ND, u, full);
+  }
+}
+// FP32: the activation of h2 slot (p, e), row r, back from the digits in registers (24 bits and more).
+__device__ __forceinline__ float from_digits(const uint4* A, int p, int e, int r) {
+  constexpr int ND = Fmt<float>::ND;
+  float v = 0.f;
+#pragma unroll
+  for (int i = ND - 1; i >= 0; --i) {
+    const uint4& w = A[(p >> 1) * ND + i];
+    const uint32_t h = (p & 1) ? (r ? w.w : w.z) : (r ? w.y : w.x);
+    const __half2 x = *reinterpret_cast<const __half2*>(&h);
+    v += e ? __high2float(x) : __low2float(x);
+  }
+  return v;
+}
 
-// Layers 1 and 2 of a tile: h1 [slot][row], h2 [n-tile][e][row] (rows g, g + 8), and the digits of h2 in sA.
+// Layers 1 and 2 of a tile: h1 [slot][row], h2 [n-tile][e][row] (rows g, g + 8; FP64), and the digits of h2
+// in A (shared memory, FP64) or A (registers, FP32, which takes h2 back from them).
 template <class T>
 __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale& ps, const uint4* __restrict__ fr,
-                                         T x0, T x1, const dig::TanhTab* tab, uint4* sA, int lane,
+                                         T x0, T x1, const dig::TanhTab* tab, uint4* A, int lane,
                                          typename Fmt<T>::V (*h1)[2], typename Fmt<T>::V (*h2)[2][2]) {
-  constexpr int ND = Fmt<T>::ND, Q = dig::Frag<T>::Q;
+  constexpr int ND = Fmt<T>::ND;
+  constexpr bool D = sizeof(T) == 8;
   using V = typename Fmt<T>::V;
   using U = typename DigWord<T>::U;
   const int t = lane & 3;
@@ -236,6 +289,8 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale
     h1[p][0] = act1(x0, w, b, tab);
     h1[p][1] = act1(x1, w, b, tab);
   }
+  uint4 A1r[D ? 1 : kK2 * ND];
+  uint4* A1 = D ? A : A1r;
 #pragma unroll
   for (int s = 0; s < kK2; ++s) {
     U u[2][4];
@@ -243,36 +298,48 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale
     for (int q = 0; q < 4; ++q)
 #pragma unroll
       for (int r = 0; r < 2; ++r) u[r][q] = 4 * s + q < kS1 ? dig_h1(h1[4 * s + q < kS1 ? 4 * s + q : 0][r]) : dig_h1(V(0));
-    put_a16<T>(sA + s * ND * 32, lane, u);
+    put_a<T, 7>(A1, s, true, lane, u);
   }
-  __syncwarp();
+  if (D) __syncwarp();
   const auto L = layer(ps, 2, T(0));
+  U u[2][4];
 #pragma unroll
   for (int p = 0; p < kT2; ++p) {
     float acc[Fmt<T>::NO][4];
-    product<T, kK2, false>(acc, sA, fr + (size_t)(kF2 + p * kK2) * Q * 32, lane);
+    product<T, kK2, false>(acc, A1, fr + (size_t)(kF2 + p * kK2) * SetWords<T>::v, lane);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const V b = sm.b2[8 * p + 2 * t + e];
 #pragma unroll
-      for (int r = 0; r < 2; ++r) h2[p][e][r] = h1[p][r] + act(acc, 2 * r + e, L, b, tab);
-    }
-  }
-  __syncwarp();
-#pragma unroll
-  for (int s = 0; s < kK3; ++s) {
-    U u[2][4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const int p = 2 * s + (q >> 1);
-        u[r][q] = p < kT2 ? dig_h2(h2[p < kT2 ? p : 0][q & 1][r]) : dig_h2(V(0));
+        const V h = h1[p][r] + act(acc, 2 * r + e, L, b, tab);
+        if constexpr (D) h2[p][e][r] = h;
+        else u[r][2 * (p & 1) + e] = dig_h2(h);
       }
-    if (s + 1 < kK3) put_a16<T>(sA + s * ND * 32, lane, u);
-    else put_a8<T>(sA + s * ND * 32, lane, u);
+    }
+    if constexpr (!D)
+      if ((p & 1) || p == kT2 - 1) put_a<T, 7>(A, p >> 1, p & 1, lane, u);
   }
-  __syncwarp();
+  if constexpr (D) {
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < kK3; ++s) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int p = 2 * s + (q >> 1);
+          u[r][q] = p < kT2 ? dig_h2(h2[p < kT2 ? p : 0][q & 1][r]) : dig_h2(V(0));
+        }
+      put_a<T, 7>(A, s, s + 1 < kK3, lane, u);
+    }
+    __syncwarp();
+  }
+}
+template <class T>
+__device__ __forceinline__ typename Fmt<T>::V h2_of(const uint4* A, const typename Fmt<T>::V (*h2)[2][2], int p, int e, int r) {
+  if constexpr (sizeof(T) == 8) return h2[p][e][r];
+  else return from_digits(A, p, e, r);
 }
 
 __device__ __forceinline__ double to_t(long long v) { return (double)v; }  // times 2^-54 later
@@ -288,7 +355,7 @@ template <class T> struct FwdWarps { static constexpr int v = sizeof(T) == 8 ? 8
 template <class T> struct AWords { static constexpr int v = (kK3 - 1) * Fmt<T>::ND * 32 + Fmt<T>::ND * 16; };
 template <class T>
 struct FwdWarp {  // shared memory of one warp
-  uint4 A[AWords<T>::v];
+  uint4 A[sizeof(T) == 8 ? AWords<T>::v : 1];
   T G[16][34];
   T R[16][4];
 };
@@ -325,7 +392,7 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
       const int pair = ti * a.ntypes + tj;
       const PairScale ps = a.scale[pair];
       const PairSmall<T>& sm = a.small[pair];
-      const uint4* fr = a.frag + (size_t)pair * kFrags * Q * 32;
+      const uint4* fr = a.frag + (size_t)pair * kFrags * SetWords<T>::v;
       int first = (sub - q0) % a.sp;
       if (first < 0) first += a.sp;
       q0 += nt;
@@ -344,8 +411,10 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
           for (int c = 0; c < 4; ++c) sw.R[lane][c] = v.R[c];
         }
         __syncwarp();
-        V h1[kS1][2], h2[kT2][2][2];
-        layers12<T>(sm, ps, fr, sw.R[g][0], sw.R[g + 8][0], tab, sw.A, lane, h1, h2);
+        V h1[kS1][2], h2[D ? kT2 : 1][2][2];
+        uint4 Ar[D ? 1 : kK3 * Fmt<T>::ND];
+        uint4* A = D ? sw.A : Ar;
+        layers12<T>(sm, ps, fr, sw.R[g][0], sw.R[g + 8][0], tab, A, lane, h1, h2);
         const auto L = layer(ps, 3, T(0));
 #pragma unroll
         for (int grp = 0; grp < 4; ++grp) {
@@ -354,15 +423,15 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
             const int j = 4 * grp + jj;
             if (j >= kT3) break;
             float acc[Fmt<T>::NO][4];
-            product<T, kK3, true>(acc, sw.A, fr + (size_t)(kF3 + j * kK3) * Q * 32, lane);
+            product<T, kK3, true>(acc, A, fr + (size_t)(kF3 + j * kK3) * SetWords<T>::v, lane);
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
               V res;
               if (j < 12) {
-                res = h2[j < 12 ? j >> 1 : 0][j & 1][r];
+                res = h2_of<T>(A, h2, j < 12 ? j >> 1 : 0, j & 1, r);
               } else {  // unit 24 (lane 0 of the quad, its own) and unit 49 (held by lane 0, used by lane 1)
-                const V o = __shfl_sync(0xffffffffu, h2[6][1][r], lane & ~3);
-                res = t == 0 ? h2[6][0][r] : o;
+                const V o = __shfl_sync(0xffffffffu, h2_of<T>(A, h2, 6, 1, r), lane & ~3);
+                res = t == 0 ? h2_of<T>(A, h2, 6, 0, r) : o;
               }
 #pragma unroll
               for (int e = 0; e < 2; ++e)
@@ -483,13 +552,13 @@ __global__ void __launch_bounds__(128) k_dig_dT(int N, T invS, const T* __restri
 }
 
 // ------------------------------------------------------------------ backward
-// FP64 keeps the digits of dz3 (Z) and the residual part of dE/dh2 (r) in shared memory: 44 KB a
-// warp, four warps an SM.  FP32 multiplies each k step of dz3 as soon as its digits exist and sums
-// dE/dh2 in registers, so that twelve warps fit.
+// FP64 keeps digits and the residual part of dE/dh2 (r) in shared memory: 44 KB a warp, four warps an SM.
+// FP32 holds the digits in registers, multiplies each k step of dz3 as soon as it exists and sums dE/dh2 in
+// registers; shared memory is left to L1, which keeps the weights (100 KB a pair).
 template <class T>
 struct BwdWarp {
   static constexpr bool D = sizeof(T) == 8;
-  uint4 A[AWords<T>::v];                                        // digits of h1, h2, then dz2
+  uint4 A[D ? AWords<T>::v : 1];                                // digits of h1, h2, then dz2
   uint4 Z[D ? 6 * Fmt<T>::ND * 32 + Fmt<T>::ND * 16 : 1];       // digits of dz3
   T r[D ? 2 * 2 * kT2 : 1][32];                                 // dG[m] + dG[m + 50], then dz2, lane-private
   union {
@@ -500,10 +569,13 @@ struct BwdWarp {
     T out[16][5];                                               // dR_hat, d s_hat (after the last read of R)
   };
   T env[6][16];                                                 // d, 1/r, switch and derivative of each row
-  double g3[3][16];                                             // dE/dd of each row
+  T g3[3][16];                                                  // dE/dd of each row
   int sd[16];
 };
-template <class T> struct BwdWarps { static constexpr int v = sizeof(T) == 8 ? 4 : 12; };
+// Warps a CTA.  FP32: 12 (168 registers) with one atom type; 16 (128 registers, some spills) with more, whose
+// weights (100 KB a pair) overflow L1 and leave more latency to hide: 32,000 Cu atoms 4.79 (12) and 5.10 ms (16),
+// 2,331 water atoms 325 and 282 us.
+constexpr int kBwdWarps64 = 4, kBwdWarps32 = 12, kBwdWarps32Types = 16;
 
 // Exponent e with |v| <= 2^e (v finite), from the bits; zero and tiny values give the lower limit.
 __device__ __forceinline__ int exp_above(double v) {
@@ -517,15 +589,15 @@ __device__ __forceinline__ int exp_above(float v) {
 __device__ __forceinline__ double pow2t(int e, double) { return dig::pow2d(e); }
 __device__ __forceinline__ float pow2t(int e, float) { return __int_as_float((127 + min(max(e, -126), 127)) << 23); }
 
-// Product value of element e times 2^sh (FP64: orders joined in units of 2^40; FP32: of 2^36).
+// Product value of element e times 2^sh (FP64: orders joined in units of 2^40; FP32: weights are 2^(18 - sw) times their digits).
 __device__ __forceinline__ double value(const float (*acc)[4], int e, double scale) {
   const dig::Pair64 p = dig::join(acc, e);
   return fma((double)p.hi, 4294967296.0, (double)p.lo) * scale;
 }
 __device__ __forceinline__ float value(const float (*acc)[4], int e, float scale) { return dig::join_f(acc, e) * scale; }
-// Gradients are scaled to |v| <= 2^GradBits (1 - 1/128): the digits' whole range is 2^(BD ND - 1).
-template <class T> struct GradBits { static constexpr int v = Fmt<T>::BD * Fmt<T>::ND - 1; };
-template <class T> struct ProdUnit { static constexpr int v = sizeof(T) == 8 ? 40 : 36; };
+// Gradients are scaled to |v| <= 2^GradBits (1 - 1/128), the digits' whole range.
+template <class T> struct GradBits { static constexpr int v = sizeof(T) == 8 ? 55 : 8; };
+template <class T> struct ProdUnit { static constexpr int v = sizeof(T) == 8 ? 40 : 18; };
 
 // g (1 - t^2) with t = tau 2^-54 (FP64) or tau (FP32)
 __device__ __forceinline__ double times_sech2(double g, long long tau) {
@@ -534,14 +606,41 @@ __device__ __forceinline__ double times_sech2(double g, long long tau) {
 }
 __device__ __forceinline__ float times_sech2(float g, float tau) { return g * fmaf(-tau, tau, 1.f); }
 
+// The value as FP64.  The conversion instruction takes the FP64 pipe for 64 clocks; a float's bits move by
+// integer instructions (subnormals become zero).
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = (uint32_t)__float_as_int(v), e = (b >> 23) & 0xffu, m = b & 0x7fffffu;
+  const uint32_t x = e == 255u ? 0x7ffu : e + 896u;
+  return __hiloint2double((int)((b & 0x80000000u) | (e == 0u ? 0u : (x << 20) | (m >> 3))), (int)(e == 0u ? 0u : m << 29));
+}
+// Sum over a tile's rows of g (plain) or -g d, in FP64; FP32 rows with exact products and a compensated sum
+// (two floats, 48 bits), widened once a tile: the FP64 form was 18% of the FP64 pipe and a chain of 16 DFMAs.
+__device__ __forceinline__ double tile_sum(const double* g, const double* d, bool plain, int rows) {
+  double s = 0.0;
+  for (int k = 0; k < rows; ++k) s = fma(g[k], plain ? 1.0 : -d[k], s);
+  return s;
+}
+__device__ __forceinline__ double tile_sum(const float* g, const float* d, bool plain, int rows) {
+  float s = 0.f, c = 0.f;
+  for (int k = 0; k < rows; ++k) {
+    const float x = g[k], y = plain ? 1.f : -d[k];
+    const float p = __fmul_rn(x, y), e = __fmaf_rn(x, y, -p);
+    const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b)), e));
+    s = t;
+  }
+  return (double)s + (double)c;
+}
+
 // Embedding backward with recompute, prod_force and the per-atom virial.  Everything downstream of
 // dG = R_hat . dT carries the row's power of two 2^sd (a bound of |dG| from max |dT|), so dz3 is ready
 // to be cut into digits and the products come out in one scale for the whole warp.
-template <class T>
-__global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a) {
+template <class T, int W>
+__global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
   extern __shared__ __align__(16) unsigned char raw[];
   constexpr bool D = sizeof(T) == 8;
-  constexpr int ND = Fmt<T>::ND, Q = dig::Frag<T>::Q, W = BwdWarps<T>::v;
+  constexpr int ND = Fmt<T>::ND, Q = dig::Frag<T>::Q;
   using V = typename Fmt<T>::V;
   using U = typename DigWord<T>::U;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = lane & 3, g = lane >> 2;
@@ -569,7 +668,7 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
       const int pair = ti * a.ntypes + tj;
       const PairScale ps = a.scale[pair];
       const PairSmall<T>& sm = a.small[pair];
-      const uint4* fr = a.frag + (size_t)pair * kFrags * Q * 32;
+      const uint4* fr = a.frag + (size_t)pair * kFrags * SetWords<T>::v;
       int first = (sub - q0) % a.sp;
       if (first < 0) first += a.sp;
       q0 += nt;
@@ -605,8 +704,10 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
           for (int c = 0; c < 4; ++c) sw.R[lane][c] = v.R[c] * f;
         }
         __syncwarp();
-        V h1[kS1][2], h2[kT2][2][2];
-        layers12<T>(sm, ps, fr, sw.x[g], sw.x[g + 8], tab, sw.A, lane, h1, h2);
+        V h1[kS1][2], h2[D ? kT2 : 1][2][2];
+        uint4 Ar[D ? 1 : kK3 * ND];
+        uint4* A = D ? sw.A : Ar;
+        layers12<T>(sm, ps, fr, sw.x[g], sw.x[g + 8], tab, A, lane, h1, h2);
         T R[2][4], dR[2][4];
 #pragma unroll
         for (int r = 0; r < 2; ++r)
@@ -631,7 +732,7 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
 #pragma unroll
         for (int j = 0; j < kT3; ++j) {
           float acc[Fmt<T>::NO][4];
-          product<T, kK3, true>(acc, sw.A, fr + (size_t)(kF3 + j * kK3) * Q * 32, lane);
+          product<T, kK3, true>(acc, A, fr + (size_t)(kF3 + j * kK3) * SetWords<T>::v, lane);
           const int m = unit3m(j, t);
           T dt[2][4];
 #pragma unroll
@@ -642,10 +743,10 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
           for (int r = 0; r < 2; ++r) {
             V res;
             if (j < 12) {
-              res = h2[j < 12 ? j >> 1 : 0][j & 1][r];
+              res = h2_of<T>(A, h2, j < 12 ? j >> 1 : 0, j & 1, r);
             } else {
-              const V o = __shfl_sync(0xffffffffu, h2[6][1][r], lane & ~3);
-              res = t == 0 ? h2[6][0][r] : o;
+              const V o = __shfl_sync(0xffffffffu, h2_of<T>(A, h2, 6, 1, r), lane & ~3);
+              res = t == 0 ? h2_of<T>(A, h2, 6, 0, r) : o;
             }
             T sum = T(0);
 #pragma unroll
@@ -676,25 +777,20 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
             }
           }
           if constexpr (D) {
-            if (j & 1) put_a16<T>(sw.Z + (j >> 1) * ND * 32, lane, u);
-            else if (j == kT3 - 1) put_a8<T>(sw.Z + (j >> 1) * ND * 32, lane, u);
+            if ((j & 1) || j == kT3 - 1) put_a<T, 0>(sw.Z, j >> 1, j & 1, lane, u);
           } else if ((j & 1) || j == kT3 - 1) {  // this k step against every n-tile of W3^T
             uint4 za[ND];
-            get_a<T>(za, u, j & 1);
+            get_a<T, 0>(za, u, j & 1);
 #pragma unroll
             for (int p = 0; p < kT3T; ++p) {
-              const uint4* bf = fr + (size_t)(kF3T + p * kK3T + (j >> 1)) * Q * 32 + lane;
-              uint4 b[Q];
-#pragma unroll
-              for (int q = 0; q < Q; ++q) b[q] = __ldg(bf + q * 32);
-              dig::zero_acc<T>(acc);
+              const uint4* set = fr + (size_t)(kF3T + p * kK3T + (j >> 1)) * SetWords<T>::v;
               if (j & 1) {
-                dig::block16<T>(acc, za, b);
+                uint4 b[Q];
+                load_b<T>(b, set, lane);
+                dig::block16<T, true>(acc, za, b);
               } else {
-                uint2 z8[ND];
-#pragma unroll
-                for (int i = 0; i < ND; ++i) z8[i] = make_uint2(za[i].x, za[i].y);
-                dig::block8<T>(acc, z8, b);
+                dig::zero_acc<T>(acc);
+                product<T, 1, true>(acc, za, set, lane);
               }
 #pragma unroll
               for (int e = 0; e < 2; ++e)
@@ -708,7 +804,7 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
 #pragma unroll
         for (int p = 0; p < kT3T; ++p) {
           float acc[Fmt<T>::NO][4];
-          if constexpr (D) product<T, kK3T, true>(acc, sw.Z, fr + (size_t)(kF3T + p * kK3T) * Q * 32, lane);
+          if constexpr (D) product<T, kK3T, true>(acc, sw.Z, fr + (size_t)(kF3T + p * kK3T) * SetWords<T>::v, lane);
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
             dh1[p][r] = T(0);
@@ -717,7 +813,7 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
               T g2;
               if constexpr (D) g2 = sw.r[4 * p + 2 * e + r][lane] + value(acc, 2 * r + e, sc3);
               else g2 = dh2[p][e][r];
-              const T dz = times_sech2(g2, h2[p][e][r] - h1[p][r]);
+              const T dz = times_sech2(g2, h2_of<T>(A, h2, p, e, r) - h1[p][r]);
               if constexpr (D) sw.r[4 * p + 2 * e + r][lane] = dz;
               else dh2[p][e][r] = dz;
               top[r] = fmax(top[r], fabs(dz));
@@ -749,8 +845,7 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
                 }
                 z[r][q] = dig_of(v * f[r]);
               }
-            if (s + 1 < kK2T) put_a16<T>(sw.A + s * ND * 32, lane, z);
-            else put_a8<T>(sw.A + s * ND * 32, lane, z);
+            put_a<T, 0>(A, s, s + 1 < kK2T, lane, z);  // the digits of h2 are no longer needed
           }
         }
         __syncwarp();
@@ -763,7 +858,7 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
 #pragma unroll
           for (int n = 0; n < kT2T; ++n) {
             float acc[Fmt<T>::NO][4];
-            product<T, kK2T, true>(acc, sw.A, fr + (size_t)(kF2T + n * kK2T) * Q * 32, lane);
+            product<T, kK2T, true>(acc, A, fr + (size_t)(kF2T + n * kK2T) * SetWords<T>::v, lane);
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               const int p = 2 * n + e;
@@ -810,16 +905,16 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
           const int jn = a.nl_j[e0];
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            const double g3 = (double)(common * d[c] + qv * o[1 + c]);
+            const T g3 = common * d[c] + qv * o[1 + c];
             sw.g3[c][lane] = g3;
-            atomicAdd(&a.force[3 * (size_t)jn + c], -g3);
+            atomicAdd(&a.force[3 * (size_t)jn + c], -widen(g3));
           }
         }
         __syncwarp();
         if (lane < 12) {  // lane c: sum of g_c; lane 3 + 3 p + q: -sum of g_p d_q
           const int rows = min(16, cnt - base);
           const int c = lane < 3 ? lane : (lane - 3) / 3, q = lane < 3 ? 0 : (lane - 3) % 3;
-          for (int k = 0; k < rows; ++k) mine = fma(sw.g3[c][k], lane < 3 ? 1.0 : -(double)sw.env[q][k], mine);
+          mine += tile_sum(sw.g3[c], sw.env[q], lane < 3, rows);
         }
       }
     }
@@ -835,14 +930,14 @@ __global__ void __launch_bounds__(32 * BwdWarps<T>::v, 1) k_dig_bwd(DigArgs<T> a
 __device__ __forceinline__ unsigned long long weight_digits(double v, int sw, double) {
   return dig::biased(__double2ll_rn(v * dig::pow2d(sw)));
 }
-__device__ __forceinline__ uint32_t weight_digits(float v, int sw, float) {
-  return dig::biased(__float2int_rn(v * __int_as_float((127 + sw) << 23)));
+__device__ __forceinline__ float weight_digits(float v, int sw, float) {
+  return v * __int_as_float((127 + sw - 18) << 23);  // |.| < 256
 }
 
 // B fragments of every pair: block (fragment set, pair), one warp.
 template <class T>
 __global__ void __launch_bounds__(32) k_dig_weights(const T* __restrict__ theta, const PairScale* scale, uint4* frag) {
-  constexpr int ND = Fmt<T>::ND, Q = dig::Frag<T>::Q;
+  constexpr int Q = dig::Frag<T>::Q;
   const int lane = threadIdx.x, t = lane & 3, n = lane >> 2;  // B fragment: k rows 2t.., column n
   const int f = blockIdx.x, pair = blockIdx.y;
   const T* W = theta + (size_t)pair * kEmbParams;
@@ -878,12 +973,16 @@ __global__ void __launch_bounds__(32) k_dig_weights(const T* __restrict__ theta,
   }
   uint32_t lo[2 * Q], hi[2 * Q];
   lo[2 * Q - 1] = hi[2 * Q - 1] = 0u;  // an odd number of digits
-  dig::split2(u[0], u[1], lo);
-  dig::split2(u[2], u[3], hi);
-  uint4* dst = frag + ((size_t)pair * kFrags + f) * Q * 32 + lane;
+  split2<0>(u[0], u[1], lo);
+  split2<0>(u[2], u[3], hi);
+  uint4* dst = frag + ((size_t)pair * kFrags + f) * SetWords<T>::v;
+  if constexpr (sizeof(T) == 8) {
 #pragma unroll
-  for (int q = 0; q < Q; ++q) dst[q * 32] = make_uint4(lo[2 * q], hi[2 * q], lo[2 * q + 1], hi[2 * q + 1]);
-  (void)ND;
+    for (int q = 0; q < Q; ++q) dst[q * 32 + lane] = make_uint4(lo[2 * q], hi[2 * q], lo[2 * q + 1], hi[2 * q + 1]);
+  } else {
+    dst[lane] = make_uint4(lo[0], hi[0], lo[1], hi[1]);
+    reinterpret_cast<uint2*>(dst + 32)[lane] = make_uint2(lo[2], hi[2]);
+  }
 }
 
 __device__ __forceinline__ long long bias_v(double b, int zs) { return __double2ll_rn(b * dig::pow2d(zs)); }
@@ -998,8 +1097,8 @@ size_t fwd_smem() {
   return (sizeof(T) == 8 ? (sizeof(dig::TanhTab) + 15) / 16 * 16 : 0) + FwdWarps<T>::v * sizeof(FwdWarp<T>);
 }
 template <class T>
-size_t bwd_smem() {
-  return (sizeof(T) == 8 ? (sizeof(dig::TanhTab) + 15) / 16 * 16 : 0) + BwdWarps<T>::v * sizeof(BwdWarp<T>);
+size_t bwd_smem(int warps) {
+  return (sizeof(T) == 8 ? (sizeof(dig::TanhTab) + 15) / 16 * 16 : 0) + warps * sizeof(BwdWarp<T>);
 }
 
 // Tasks per atom: enough warp tasks (about 16 a resident warp) that the last wave is short; at most one per two
@@ -1037,15 +1136,21 @@ dp_status backward(Model* m, int N) {
   DigArgs<T> a = make_args<T>(m, N);
   k_dig_dT<T><<<N, 128, 0, m->stream>>>(N, T(1) / (T)m->S, a.Tm, static_cast<const T*>(m->dD), const_cast<T*>(a.dT),
                                         const_cast<T*>(a.dTmax));
-  const size_t smem = bwd_smem<T>();
-  const void* fn = reinterpret_cast<const void*>(k_dig_bwd<T>);
+  auto kern = k_dig_bwd<T, sizeof(T) == 8 ? kBwdWarps64 : kBwdWarps32>;
+  int W = sizeof(T) == 8 ? kBwdWarps64 : kBwdWarps32;
+  if constexpr (sizeof(T) == 4)
+    if (m->ntypes > 1) {
+      kern = k_dig_bwd<T, kBwdWarps32Types>;
+      W = kBwdWarps32Types;
+    }
+  const size_t smem = bwd_smem<T>(W);
+  const void* fn = reinterpret_cast<const void*>(kern);
   DP_CUDA_TRY(m, ensure_smem(fn, smem, true));
-  constexpr int W = BwdWarps<T>::v;
   const int per = blocks_per_sm(fn, 32 * W, smem);
   a.sp = split_of(m, N, W * per);
   DP_CUDA_TRY(m, cudaMemsetAsync(m->vir_atom, 0, sizeof(double) * 9 * (size_t)N, m->stream));
   const int grid = (int)std::min((long)num_sms() * per, ((long)N * a.sp + W - 1) / W);
-  k_dig_bwd<T><<<grid, 32 * W, smem, m->stream>>>(a);
+  kern<<<grid, 32 * W, smem, m->stream>>>(a);
   m->launches += 2;
   DP_LAUNCH_CHECK(m);
   return DP_OK;
@@ -1055,8 +1160,8 @@ dp_status backward(Model* m, int N) {
 
 size_t dig_emb_bytes(int ntypes, bool fp64) {
   const size_t np = (size_t)ntypes * ntypes;
-  return fp64 ? 1024 + np * (sizeof(PairSmall<double>) + (size_t)kFrags * dig::Frag<double>::Q * 512)
-              : 1024 + np * (sizeof(PairSmall<float>) + (size_t)kFrags * dig::Frag<float>::Q * 512);
+  return fp64 ? 1024 + np * (sizeof(PairSmall<double>) + (size_t)kFrags * SetWords<double>::v * 16)
+              : 1024 + np * (sizeof(PairSmall<float>) + (size_t)kFrags * SetWords<float>::v * 16);
 }
 size_t dig_tanh_bytes() { return sizeof(dig::TanhTab); }
 

@@ -37,7 +37,7 @@ __host__ __device__ __forceinline__ int mat_off(int q) {
 constexpr int kTypeFrags = 2 * (kKD / 16) * (kF / 8) + 4 * (kF / 16) * (kF / 8);
 
 template <class T> struct NTiles { static constexpr int v = sizeof(T) == 8 ? 3 : 6; };  // n-tiles of a warp
-// k steps whose digit products stay below 2^24 in the accumulators: 7 x 128 x 2^14, 3 x 80 x 2^16
+// k steps whose digit products stay below 2^24 in the accumulators: 7 x 128 x 2^14, 2 x 80 x 2^16
 template <class T> struct Flush { static constexpr int v = sizeof(T) == 8 ? 8 : 5; };
 constexpr int kWarps = 8;
 
@@ -84,9 +84,11 @@ __device__ __forceinline__ unsigned long long fix_digits(double v, int e) {
   const long long q = (long long)((m + ((1ull << r) >> 1)) >> r);
   return dig::biased(hi < 0 ? -q : q);
 }
-__device__ __forceinline__ uint32_t fix_digits(float v, int e) {
-  return dig::biased(__float2int_rn(v * __int_as_float((127 + min(26 - e, 127)) << 23)));
+__device__ __forceinline__ float fix_digits(float v, int e) {  // below 256
+  return v * __int_as_float((127 + min(8 - e, 127)) << 23);
 }
+__device__ __forceinline__ void split2(unsigned long long u0, unsigned long long u1, uint32_t* out) { dig::split2(u0, u1, out); }
+__device__ __forceinline__ void split2(float u0, float u1, uint32_t* out) { dig::split2f<0>(u0, u1, out); }
 
 __device__ __forceinline__ void load4(const double* p, double* v) {
   const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
@@ -213,10 +215,10 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_dig_gemm(GemmArgs<T> g) {
 #pragma unroll
       for (int k = 0; k < P::KS; ++k) {
         uint32_t x[ND], y[ND], z[ND], u[ND];
-        dig::split2(fix_digits(v[k][0][0], ea[0]), fix_digits(v[k][0][1], ea[0]), x);
-        dig::split2(fix_digits(v[k][1][0], ea[1]), fix_digits(v[k][1][1], ea[1]), y);
-        dig::split2(fix_digits(v[k][0][2], ea[0]), fix_digits(v[k][0][3], ea[0]), z);
-        dig::split2(fix_digits(v[k][1][2], ea[1]), fix_digits(v[k][1][3], ea[1]), u);
+        split2(fix_digits(v[k][0][0], ea[0]), fix_digits(v[k][0][1], ea[0]), x);
+        split2(fix_digits(v[k][1][0], ea[1]), fix_digits(v[k][1][1], ea[1]), y);
+        split2(fix_digits(v[k][0][2], ea[0]), fix_digits(v[k][0][3], ea[0]), z);
+        split2(fix_digits(v[k][1][2], ea[1]), fix_digits(v[k][1][3], ea[1]), u);
 #pragma unroll
         for (int i = 0; i < ND; ++i) a[k][i] = make_uint4(x[i], y[i], z[i], u[i]);
       }
@@ -400,8 +402,8 @@ __global__ void __launch_bounds__(256) k_dig_fit_weights(const T* __restrict__ f
     u[k] = fix_digits(q < 3 ? W[(size_t)(k0 + k) * mt.N + col] : W[(size_t)col * mt.K + k0 + k], e);
   uint32_t lo[2 * Q], hi[2 * Q];
   lo[2 * Q - 1] = hi[2 * Q - 1] = 0u;
-  dig::split2(u[0], u[1], lo);
-  dig::split2(u[2], u[3], hi);
+  split2(u[0], u[1], lo);
+  split2(u[2], u[3], hi);
   uint4* dst = frag + ((size_t)ty * kTypeFrags + f) * Q * 32 + lane;
 #pragma unroll
   for (int p = 0; p < Q; ++p) dst[p * 32] = make_uint4(lo[2 * p], hi[2 * p], lo[2 * p + 1], hi[2 * p + 1]);
