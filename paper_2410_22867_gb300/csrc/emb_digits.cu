@@ -187,24 +187,6 @@ __device__ __forceinline__ void get_a(uint4* a, const typename DigWord<T>::U (*u
 #pragma unroll
   for (int i = 0; i < ND; ++i) a[i] = make_uint4(x[i], y[i], full ? z[i] : 0u, full ? w[i] : 0u);
 }
-// The same into the warp's shared memory.
-template <class T, int G>
-__device__ __forceinline__ void put_a16(uint4* sA, int lane, const typename DigWord<T>::U (*u)[4]) {
-  constexpr int ND = Fmt<T>::ND;
-  uint4 a[ND];
-  get_a<T, G>(a, u, true);
-#pragma unroll
-  for (int i = 0; i < ND; ++i) sA[i * 32 + lane] = a[i];
-}
-template <class T, int G>
-__device__ __forceinline__ void put_a8(uint4* sA, int lane, const typename DigWord<T>::U (*u)[4]) {
-  constexpr int ND = Fmt<T>::ND;
-  uint32_t x[ND], y[ND];
-  split2<G>(u[0][0], u[0][1], x);
-  split2<G>(u[1][0], u[1][1], y);
-#pragma unroll
-  for (int i = 0; i < ND; ++i) reinterpret_cast<uint2*>(sA)[i * 32 + lane] = make_uint2(x[i], y[i]);
-}
 
 // The lane's B fragments of one set.
 template <class T>
@@ -219,41 +201,76 @@ __device__ __forceinline__ void load_b(uint4* b, const uint4* __restrict__ set, 
   }
 }
 
+// Where a tile's A operand lives.  FP32 (kRegs): digits in registers, since reading A again for every n-tile
+// made those kernels bound by shared-memory bandwidth.  FP64 forward (kDigits): digits in the warp's
+// shared memory, 112 bytes a lane and k step.  FP64 backward (kWords): the slots' 56-bit digit words, 64
+// bytes, cut into digits on every use, so that six warps fit an SM instead of four (8.66 -> 7.30 ms for 4,000 Cu
+// atoms; the forward, which has its eight warps anyway, would lose: 2.73 -> 3.10 ms).
+enum Store { kRegs, kDigits, kWords };
+
 // acc = A (KS k steps) times the fragments of one n-tile; with TAIL the last step has 8 columns.
-// FP64: A from the warp's shared memory (its digits are 100 registers); FP32: from registers, since reading
-// A again for every n-tile made the kernels bound by shared-memory bandwidth.
-template <class T, int KS, bool TAIL>
+template <class T, int KS, bool TAIL, Store ST>
 __device__ __forceinline__ void product(float (*acc)[4], const uint4* A, const uint4* __restrict__ fr, int lane) {
   constexpr int ND = Fmt<T>::ND, Q = dig::Frag<T>::Q;
-  constexpr bool D = sizeof(T) == 8;
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
-    uint4 b[Q];
+    const bool tail = TAIL && s == KS - 1;
+    uint4 b[Q], a[ND];
     load_b<T>(b, fr + s * SetWords<T>::v, lane);
-    if (TAIL && s == KS - 1) {
-      uint2 a[ND];
+    if constexpr (ST == kWords) {
+      typename DigWord<T>::U u[2][4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (tail && q >= 2) break;
+        const uint4 w = A[(4 * s + q) * 32 + lane];
+        u[0][q] = ((unsigned long long)w.y << 32) | w.x;
+        u[1][q] = ((unsigned long long)w.w << 32) | w.z;
+      }
+      get_a<T, 0>(a, u, !tail);
+    } else if constexpr (ST == kDigits) {
 #pragma unroll
       for (int i = 0; i < ND; ++i) {
-        if constexpr (D) a[i] = reinterpret_cast<const uint2*>(A + s * ND * 32)[i * 32 + lane];
-        else a[i] = make_uint2(A[s * ND + i].x, A[s * ND + i].y);
+        if (tail) {
+          const uint2 w = reinterpret_cast<const uint2*>(A + s * ND * 32)[i * 32 + lane];
+          a[i] = make_uint4(w.x, w.y, 0u, 0u);
+        } else {
+          a[i] = A[(s * ND + i) * 32 + lane];
+        }
       }
-      dig::block8<T>(acc, a, b);
     } else {
-      uint4 a[ND];
 #pragma unroll
-      for (int i = 0; i < ND; ++i) a[i] = D ? A[(s * ND + i) * 32 + lane] : A[s * ND + i];
-      if (s == 0) dig::block16<T, true>(acc, a, b);
-      else dig::block16<T>(acc, a, b);
+      for (int i = 0; i < ND; ++i) a[i] = A[s * ND + i];
+    }
+    if (tail) {
+      uint2 a8[ND];
+#pragma unroll
+      for (int i = 0; i < ND; ++i) a8[i] = make_uint2(a[i].x, a[i].y);
+      dig::block8<T>(acc, a8, b);
+    } else if (s == 0) {
+      dig::block16<T, true>(acc, a, b);
+    } else {
+      dig::block16<T>(acc, a, b);
     }
   }
 }
-// A fragments of k step s: into shared memory (FP64) or the register array (FP32).
-template <class T, int G>
+// A of k step s into its store.
+template <class T, int G, Store ST>
 __device__ __forceinline__ void put_a(uint4* A, int s, bool full, int lane, const typename DigWord<T>::U (*u)[4]) {
   constexpr int ND = Fmt<T>::ND;
-  if constexpr (sizeof(T) == 8) {
-    if (full) put_a16<T, G>(A + s * ND * 32, lane, u);
-    else put_a8<T, G>(A + s * ND * 32, lane, u);
+  if constexpr (ST == kWords) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (full || q < 2)
+        A[(4 * s + q) * 32 + lane] = make_uint4((uint32_t)u[0][q], (uint32_t)(u[0][q] >> 32), (uint32_t)u[1][q],
+                                                (uint32_t)(u[1][q] >> 32));
+  } else if constexpr (ST == kDigits) {
+    uint4 a[ND];
+    get_a<T, G>(a, u, full);
+#pragma unroll
+    for (int i = 0; i < ND; ++i) {
+      if (full) A[(s * ND + i) * 32 + lane] = a[i];
+      else reinterpret_cast<uint2*>(A + s * ND * 32)[i * 32 + lane] = make_uint2(a[i].x, a[i].y);
+    }
   } else {
     get_a<T, G>(A + s * ND, u, full);
   }
@@ -274,7 +291,7 @@ __device__ __forceinline__ float from_digits(const uint4* A, int p, int e, int r
 
 // Layers 1 and 2 of a tile: h1 [slot][row], h2 [n-tile][e][row] (rows g, g + 8; FP64), and the digits of h2
 // in A (shared memory, FP64) or A (registers, FP32, which takes h2 back from them).
-template <class T>
+template <class T, Store ST>
 __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale& ps, const uint4* __restrict__ fr,
                                          T x0, T x1, const dig::TanhTab* tab, uint4* A, int lane,
                                          typename Fmt<T>::V (*h1)[2], typename Fmt<T>::V (*h2)[2][2]) {
@@ -298,7 +315,7 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale
     for (int q = 0; q < 4; ++q)
 #pragma unroll
       for (int r = 0; r < 2; ++r) u[r][q] = 4 * s + q < kS1 ? dig_h1(h1[4 * s + q < kS1 ? 4 * s + q : 0][r]) : dig_h1(V(0));
-    put_a<T, 7>(A1, s, true, lane, u);
+    put_a<T, 7, ST>(A1, s, true, lane, u);
   }
   if (D) __syncwarp();
   const auto L = layer(ps, 2, T(0));
@@ -306,7 +323,7 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale
 #pragma unroll
   for (int p = 0; p < kT2; ++p) {
     float acc[Fmt<T>::NO][4];
-    product<T, kK2, false>(acc, A1, fr + (size_t)(kF2 + p * kK2) * SetWords<T>::v, lane);
+    product<T, kK2, false, ST>(acc, A1, fr + (size_t)(kF2 + p * kK2) * SetWords<T>::v, lane);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const V b = sm.b2[8 * p + 2 * t + e];
@@ -318,7 +335,7 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale
       }
     }
     if constexpr (!D)
-      if ((p & 1) || p == kT2 - 1) put_a<T, 7>(A, p >> 1, p & 1, lane, u);
+      if ((p & 1) || p == kT2 - 1) put_a<T, 7, ST>(A, p >> 1, p & 1, lane, u);
   }
   if constexpr (D) {
     __syncwarp();
@@ -331,7 +348,7 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale
           const int p = 2 * s + (q >> 1);
           u[r][q] = p < kT2 ? dig_h2(h2[p < kT2 ? p : 0][q & 1][r]) : dig_h2(V(0));
         }
-      put_a<T, 7>(A, s, s + 1 < kK3, lane, u);
+      put_a<T, 7, ST>(A, s, s + 1 < kK3, lane, u);
     }
     __syncwarp();
   }
@@ -352,10 +369,11 @@ template <> struct Unit<float> { static constexpr float v = 1.f; };
 // atom are numbered in one sequence; tile q belongs to the task with sub = q % sp.
 // warps a CTA (one CTA an SM): FP64 needs 255 registers a thread, FP32 runs in 128
 template <class T> struct FwdWarps { static constexpr int v = sizeof(T) == 8 ? 8 : 16; };
-template <class T> struct AWords { static constexpr int v = (kK3 - 1) * Fmt<T>::ND * 32 + Fmt<T>::ND * 16; };
+constexpr int kADigits = (kK3 - 1) * Fmt<double>::ND * 32 + Fmt<double>::ND * 16;  // FP64 digits of a tile, in uint4
+constexpr int kAWords = (4 * (kK3 - 1) + 2) * 32, kZWords = (4 * (kK3T - 1) + 2) * 32;  // FP64 digit words
 template <class T>
 struct FwdWarp {  // shared memory of one warp
-  uint4 A[sizeof(T) == 8 ? AWords<T>::v : 1];
+  uint4 A[sizeof(T) == 8 ? kADigits : 1];
   T G[16][34];
   T R[16][4];
 };
@@ -365,7 +383,8 @@ template <class T>
 __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a) {
   extern __shared__ __align__(16) unsigned char raw[];
   constexpr bool D = sizeof(T) == 8;
-  constexpr int Q = dig::Frag<T>::Q, W = FwdWarps<T>::v;
+  constexpr int W = FwdWarps<T>::v;
+  constexpr Store ST = D ? kDigits : kRegs;
   using V = typename Fmt<T>::V;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = lane & 3, g = lane >> 2;
   dig::TanhTab* tab = reinterpret_cast<dig::TanhTab*>(raw);
@@ -414,7 +433,7 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
         V h1[kS1][2], h2[D ? kT2 : 1][2][2];
         uint4 Ar[D ? 1 : kK3 * Fmt<T>::ND];
         uint4* A = D ? sw.A : Ar;
-        layers12<T>(sm, ps, fr, sw.R[g][0], sw.R[g + 8][0], tab, A, lane, h1, h2);
+        layers12<T, ST>(sm, ps, fr, sw.R[g][0], sw.R[g + 8][0], tab, A, lane, h1, h2);
         const auto L = layer(ps, 3, T(0));
 #pragma unroll
         for (int grp = 0; grp < 4; ++grp) {
@@ -423,7 +442,7 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
             const int j = 4 * grp + jj;
             if (j >= kT3) break;
             float acc[Fmt<T>::NO][4];
-            product<T, kK3, true>(acc, A, fr + (size_t)(kF3 + j * kK3) * SetWords<T>::v, lane);
+            product<T, kK3, true, ST>(acc, A, fr + (size_t)(kF3 + j * kK3) * SetWords<T>::v, lane);
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
               V res;
@@ -552,14 +571,14 @@ __global__ void __launch_bounds__(128) k_dig_dT(int N, T invS, const T* __restri
 }
 
 // ------------------------------------------------------------------ backward
-// FP64 keeps digits and the residual part of dE/dh2 (r) in shared memory: 44 KB a warp, four warps an SM.
+// FP64 keeps digit words and the residual part of dE/dh2 (r) in shared memory: 29.5 KB a warp, six warps an SM.
 // FP32 holds the digits in registers, multiplies each k step of dz3 as soon as it exists and sums dE/dh2 in
 // registers; shared memory is left to L1, which keeps the weights (100 KB a pair).
 template <class T>
 struct BwdWarp {
   static constexpr bool D = sizeof(T) == 8;
-  uint4 A[D ? AWords<T>::v : 1];                                // digits of h1, h2, then dz2
-  uint4 Z[D ? 6 * Fmt<T>::ND * 32 + Fmt<T>::ND * 16 : 1];       // digits of dz3
+  uint4 A[D ? kAWords : 1];                                // digits of h1, h2, then dz2
+  uint4 Z[D ? kZWords : 1];                                     // digits of dz3
   T r[D ? 2 * 2 * kT2 : 1][32];                                 // dG[m] + dG[m + 50], then dz2, lane-private
   union {
     struct {
@@ -575,7 +594,7 @@ struct BwdWarp {
 // Warps a CTA.  FP32: 12 (168 registers) with one atom type; 16 (128 registers, some spills) with more, whose
 // weights (100 KB a pair) overflow L1 and leave more latency to hide: 32,000 Cu atoms 4.79 (12) and 5.10 ms (16),
 // 2,331 water atoms 325 and 282 us.
-constexpr int kBwdWarps64 = 4, kBwdWarps32 = 12, kBwdWarps32Types = 16;
+constexpr int kBwdWarps64 = 6, kBwdWarps32 = 12, kBwdWarps32Types = 16;
 
 // Exponent e with |v| <= 2^e (v finite), from the bits; zero and tiny values give the lower limit.
 __device__ __forceinline__ int exp_above(double v) {
@@ -641,6 +660,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
   extern __shared__ __align__(16) unsigned char raw[];
   constexpr bool D = sizeof(T) == 8;
   constexpr int ND = Fmt<T>::ND, Q = dig::Frag<T>::Q;
+  constexpr Store ST = D ? kWords : kRegs;
   using V = typename Fmt<T>::V;
   using U = typename DigWord<T>::U;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, t = lane & 3, g = lane >> 2;
@@ -707,7 +727,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
         V h1[kS1][2], h2[D ? kT2 : 1][2][2];
         uint4 Ar[D ? 1 : kK3 * ND];
         uint4* A = D ? sw.A : Ar;
-        layers12<T>(sm, ps, fr, sw.x[g], sw.x[g + 8], tab, A, lane, h1, h2);
+        layers12<T, ST>(sm, ps, fr, sw.x[g], sw.x[g + 8], tab, A, lane, h1, h2);
         T R[2][4], dR[2][4];
 #pragma unroll
         for (int r = 0; r < 2; ++r)
@@ -732,7 +752,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
 #pragma unroll
         for (int j = 0; j < kT3; ++j) {
           float acc[Fmt<T>::NO][4];
-          product<T, kK3, true>(acc, A, fr + (size_t)(kF3 + j * kK3) * SetWords<T>::v, lane);
+          product<T, kK3, true, ST>(acc, A, fr + (size_t)(kF3 + j * kK3) * SetWords<T>::v, lane);
           const int m = unit3m(j, t);
           T dt[2][4];
 #pragma unroll
@@ -777,7 +797,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
             }
           }
           if constexpr (D) {
-            if ((j & 1) || j == kT3 - 1) put_a<T, 0>(sw.Z, j >> 1, j & 1, lane, u);
+            if ((j & 1) || j == kT3 - 1) put_a<T, 0, ST>(sw.Z, j >> 1, j & 1, lane, u);
           } else if ((j & 1) || j == kT3 - 1) {  // this k step against every n-tile of W3^T
             uint4 za[ND];
             get_a<T, 0>(za, u, j & 1);
@@ -790,7 +810,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
                 dig::block16<T, true>(acc, za, b);
               } else {
                 dig::zero_acc<T>(acc);
-                product<T, 1, true>(acc, za, set, lane);
+                product<T, 1, true, ST>(acc, za, set, lane);
               }
 #pragma unroll
               for (int e = 0; e < 2; ++e)
@@ -804,7 +824,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
 #pragma unroll
         for (int p = 0; p < kT3T; ++p) {
           float acc[Fmt<T>::NO][4];
-          if constexpr (D) product<T, kK3T, true>(acc, sw.Z, fr + (size_t)(kF3T + p * kK3T) * SetWords<T>::v, lane);
+          if constexpr (D) product<T, kK3T, true, ST>(acc, sw.Z, fr + (size_t)(kF3T + p * kK3T) * SetWords<T>::v, lane);
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
             dh1[p][r] = T(0);
@@ -845,7 +865,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
                 }
                 z[r][q] = dig_of(v * f[r]);
               }
-            put_a<T, 0>(A, s, s + 1 < kK2T, lane, z);  // the digits of h2 are no longer needed
+            put_a<T, 0, ST>(A, s, s + 1 < kK2T, lane, z);  // the digits of h2 are no longer needed
           }
         }
         __syncwarp();
@@ -858,7 +878,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
 #pragma unroll
           for (int n = 0; n < kT2T; ++n) {
             float acc[Fmt<T>::NO][4];
-            product<T, kK2T, true>(acc, A, fr + (size_t)(kF2T + n * kK2T) * SetWords<T>::v, lane);
+            product<T, kK2T, true, ST>(acc, A, fr + (size_t)(kF2T + n * kK2T) * SetWords<T>::v, lane);
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               const int p = 2 * n + e;
