@@ -260,6 +260,14 @@ long long dp_ntheta(const dp_model* m);
 dp_status dp_set_params(dp_model* m, const double* theta, long long ntheta);
 
 /*
+ * dp_set_params_device -- dp_set_params with theta in device memory, FP32 (is_fp32 != 0) or FP64, as a
+ * training loop on the GPU holds it: checked and converted there; only what host code reads (the embedding
+ * parameters; all of them for the mixed precisions' 16-bit copies) comes to the host.  theta must be ready
+ * on the device (work that writes it has completed).  Synchronous.  Errors as dp_set_params.
+ */
+dp_status dp_set_params_device(dp_model* m, const void* theta, int is_fp32, long long ntheta);
+
+/*
  * dp_get_nlist -- copy the formatted neighbour list of the last dp_compute /
  * MD step: nlist [natoms*S] and images [natoms*S] device int32 in caller order,
  * S = sum(sel).  Row i holds, per neighbour type t in order, the neighbours of

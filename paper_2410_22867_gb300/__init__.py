@@ -33,7 +33,7 @@ EXPORTS = ("dp_create", "dp_compute", "dp_compute_batch", "dp_verlet_step", "dp_
            "dp_ntheta", "dp_get_nlist", "dp_phase_times", "dp_kernel_launches", "dp_sync", "dp_last_error",
            "dp_destroy", "dp_version", "dp_selftest", "dp_selftest_noalloc", "dp_set_params", "dp_autotune",
            "dp_wait_selftest", "dp_measure_peak", "dp_tabulate", "dp_rdf", "dp_atom_virial",
-           "dp_set_truncation")
+           "dp_set_truncation", "dp_set_params_device")
 
 _P = ctypes.c_void_p
 _I = ctypes.c_int
@@ -88,6 +88,7 @@ def lib():
             L.dp_selftest.argtypes = [_I, _P]
             L.dp_selftest_noalloc.argtypes = [_P, _I, _P]
             L.dp_set_params.argtypes = [_P, _P, ctypes.c_longlong]
+            L.dp_set_params_device.argtypes = [_P, _P, _I, ctypes.c_longlong]
             L.dp_autotune.argtypes = [_P, _I, _P]
             L.dp_wait_selftest.argtypes = [ctypes.c_uint]
             L.dp_measure_peak.argtypes = [_I, _P]
@@ -98,7 +99,8 @@ def lib():
             for name in ("dp_create", "dp_compute", "dp_compute_batch", "dp_verlet_step", "dp_md_run_batch",
                          "dp_param_grad", "dp_get_nlist", "dp_phase_times", "dp_sync", "dp_selftest",
                          "dp_selftest_noalloc", "dp_set_params", "dp_autotune", "dp_wait_selftest",
-                         "dp_measure_peak", "dp_tabulate", "dp_rdf", "dp_atom_virial", "dp_set_truncation"):
+                         "dp_measure_peak", "dp_tabulate", "dp_rdf", "dp_atom_virial", "dp_set_truncation",
+                         "dp_set_params_device"):
                 getattr(L, name).restype = _I
             _lib = L
     return _lib
@@ -348,7 +350,14 @@ class DPModel:
         """Replace the network parameters (dp_set_params): theta [ntheta] float64 in the weight
         blob's parameter order (numpy array or torch tensor on any device)."""
         if hasattr(theta, "detach"):
-            theta = theta.detach().to("cpu").numpy()
+            import torch
+            theta = theta.detach()
+            if theta.device == self.device and theta.dtype in (torch.float32, torch.float64) and theta.is_contiguous():
+                torch.cuda.current_stream(self.device).synchronize()  # theta's values are there
+                self._check(lib().dp_set_params_device(self.h, _ptr(theta), int(theta.dtype == torch.float32),
+                                                       int(theta.numel())))
+                return
+            theta = theta.to("cpu").numpy()
         th = np.ascontiguousarray(theta, dtype=np.float64).ravel()
         self._check(lib().dp_set_params(self.h, th.ctypes.data_as(_P), int(th.size)))
 

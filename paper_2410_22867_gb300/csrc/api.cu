@@ -430,17 +430,17 @@ const char* dp_version(void) { return "dpgb300 0.1"; }
 // Device copies of the parameters from m->theta_host (and davg / dstd): theta in FP64 and
 // FP32, normalisation statistics, and the tensor-core operand copies: 16-bit ones for the mixed
 // precisions, digit fragments for FP64 / FP32.  Synchronous.
+dp_status derive_weights(Model* m);
 dp_status upload_weights(Model* m) {
-  const int nt = m->ntypes;
   const std::vector<double>& theta = m->theta_host;
   std::vector<float> t32(theta.begin(), theta.end());
-  std::vector<double> stat(8 * nt);
-  for (int q = 0; q < 4 * nt; ++q) { stat[q] = m->davg_host[q]; stat[4 * nt + q] = 1.0 / m->dstd_host[q]; }
-  std::vector<float> stat32(stat.begin(), stat.end());
   DP_CUDA_TRY(m, cudaMemcpy(m->w64, theta.data(), 8 * theta.size(), cudaMemcpyHostToDevice));
   DP_CUDA_TRY(m, cudaMemcpy(m->w32, t32.data(), 4 * t32.size(), cudaMemcpyHostToDevice));
-  DP_CUDA_TRY(m, cudaMemcpy(m->stat64, stat.data(), 8 * stat.size(), cudaMemcpyHostToDevice));
-  DP_CUDA_TRY(m, cudaMemcpy(m->stat32, stat32.data(), 4 * stat32.size(), cudaMemcpyHostToDevice));
+  return derive_weights(m);
+}
+
+// Everything made from w64 / w32: padded-slot terms and the operand copies.
+dp_status derive_weights(Model* m) {
   DP_TRY(launch_pad_rows(m));
   if (m->prec == DP_MIX_BF16 || m->prec == DP_MIX_FP16) {
     DP_TRY(launch_tc_setup(m));
@@ -449,6 +449,17 @@ dp_status upload_weights(Model* m) {
     DP_TRY(dig_upload(m));
     DP_TRY(dig_fit_upload(m));
   }
+  return DP_OK;
+}
+
+// Normalisation statistics (fixed for the life of the model).
+dp_status upload_stats(Model* m) {
+  const int nt = m->ntypes;
+  std::vector<double> stat(8 * nt);
+  for (int q = 0; q < 4 * nt; ++q) { stat[q] = m->davg_host[q]; stat[4 * nt + q] = 1.0 / m->dstd_host[q]; }
+  std::vector<float> stat32(stat.begin(), stat.end());
+  DP_CUDA_TRY(m, cudaMemcpy(m->stat64, stat.data(), 8 * stat.size(), cudaMemcpyHostToDevice));
+  DP_CUDA_TRY(m, cudaMemcpy(m->stat32, stat32.data(), 4 * stat32.size(), cudaMemcpyHostToDevice));
   return DP_OK;
 }
 
@@ -589,7 +600,8 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
     if (s0 != DP_OK) return fail(s0, m->last_error);
   }
   {
-    dp_status s1 = upload_weights(m);
+    dp_status s1 = upload_stats(m);
+    if (s1 == DP_OK) s1 = upload_weights(m);
     if (s1 != DP_OK) return fail(s1, m->last_error);
   }
   if (cudaMemset(m->err, 0, 16) != cudaSuccess) return fail(DP_ERR_CUDA, "memset failed");
@@ -676,6 +688,34 @@ dp_status dp_set_params(dp_model* h, const double* theta, long long ntheta) {
   return DP_OK;
 }
 
+dp_status dp_set_params_device(dp_model* h, const void* theta, int is_fp32, long long ntheta) {
+  if (!h) return DP_ERR_ARG;
+  Model* m = &h->m;
+  if (!theta) { m->last_error = "null theta"; return DP_ERR_ARG; }
+  if (ntheta != m->ntheta) { m->last_error = "ntheta does not match the model"; return DP_ERR_ARG; }
+  DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));
+  // The host keeps the parameters that host code reads: all of them for the mixed precisions' 16-bit copies,
+  // the embedding nets' (for the scales of their digits) otherwise.
+  const size_t keep = is_mixed(m) ? (size_t)ntheta : (size_t)m->ntypes * m->ntypes * kEmbParams;
+  std::vector<double> host(keep);
+  std::vector<float> host32(is_fp32 ? keep : 0);
+  DP_TRY(launch_check_finite(m, theta, is_fp32 != 0, ntheta, m->err + 1));
+  int bad = 0;
+  void* dst = is_fp32 ? static_cast<void*>(host32.data()) : static_cast<void*>(host.data());
+  DP_CUDA_TRY(m, cudaMemcpyAsync(dst, theta, (is_fp32 ? 4 : 8) * keep, cudaMemcpyDeviceToHost, m->stream));
+  DP_CUDA_TRY(m, cudaMemcpyAsync(&bad, m->err + 1, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
+  DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));
+  if (bad) { m->last_error = "non-finite parameter"; return DP_ERR_WEIGHTS; }
+  if (is_fp32) std::copy(host32.begin(), host32.end(), host.begin());
+  std::copy(host.begin(), host.end(), m->theta_host.begin());
+  DP_TRY(launch_copy_params(m, theta, is_fp32 != 0, ntheta));
+  DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));  // derive_weights also uses the legacy default stream
+  DP_TRY(derive_weights(m));
+  DP_CUDA_TRY(m, cudaDeviceSynchronize());
+  if (m->tab_n > 0) DP_TRY(launch_tabulate(m, m->tab_x0, m->tab_x0 + m->tab_n * m->tab_h, m->tab_n));
+  return DP_OK;
+}
+
 dp_status dp_rdf(dp_model* h, int nbins, double r_max, unsigned long long* counts) {
   if (!h || !counts) return DP_ERR_ARG;
   Model* m = &h->m;
@@ -744,8 +784,9 @@ dp_status dp_get_nlist(dp_model* h, int* nlist, int* images) {
 dp_status dp_sync(dp_model* h) {
   if (!h) return DP_ERR_ARG;
   Model* m = &h->m;
+  // the error word rides behind the work: one wait
+  DP_CUDA_TRY(m, cudaMemcpyAsync(m->err_host, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
   DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));
-  DP_CUDA_TRY(m, cudaMemcpy(m->err_host, m->err, sizeof(int), cudaMemcpyDeviceToHost));
   int bits = *m->err_host;
   if (bits) DP_CUDA_TRY(m, cudaMemset(m->err, 0, sizeof(int)));
   return map_err_bits(m, bits);

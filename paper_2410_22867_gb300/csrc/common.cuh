@@ -374,5 +374,8 @@ dp_status launch_store_state(Model* m, int N, double* x_user, double* v_user);
 dp_status launch_kinetic(Model* m, int N, double* ke_rep);
 size_t rep_reduce_slots(int max_atoms, int max_reps);  // chunk slots of red_part (10 doubles each)
 dp_status launch_nan_energy(Model* m, double* energy, int n);
+// parameters in device memory: *bad = 1 if any is not finite; w64 and w32 from them
+dp_status launch_check_finite(Model* m, const void* theta, bool fp32, long long n, int* bad);
+dp_status launch_copy_params(Model* m, const void* theta, bool fp32, long long n);
 
 }  // namespace dpg

@@ -172,7 +172,38 @@ __global__ void k_nan(double* p, int n) {
   if (k < n) p[k] = __longlong_as_double(0x7ff8000000000000ll);
 }
 
+template <class T>
+__global__ void k_check_finite(const T* __restrict__ p, long long n, int* bad) {
+  bool b = false;
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
+    b = b || !isfinite(p[k]);
+  if (b) *bad = 1;
+}
+template <class T>
+__global__ void k_copy_params(const T* __restrict__ p, long long n, double* w64, float* w32) {
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
+    w64[k] = (double)p[k];
+    w32[k] = (float)p[k];
+  }
+}
+
 }  // namespace
+
+dp_status launch_check_finite(Model* m, const void* theta, bool fp32, long long n, int* bad) {
+  DP_CUDA_TRY(m, cudaMemsetAsync(bad, 0, sizeof(int), m->stream));
+  if (fp32) k_check_finite<float><<<2 * num_sms(), 256, 0, m->stream>>>(static_cast<const float*>(theta), n, bad);
+  else k_check_finite<double><<<2 * num_sms(), 256, 0, m->stream>>>(static_cast<const double*>(theta), n, bad);
+  m->launches += 1;
+  DP_LAUNCH_CHECK(m);
+  return DP_OK;
+}
+dp_status launch_copy_params(Model* m, const void* theta, bool fp32, long long n) {
+  if (fp32) k_copy_params<float><<<2 * num_sms(), 256, 0, m->stream>>>(static_cast<const float*>(theta), n, m->w64, m->w32);
+  else k_copy_params<double><<<2 * num_sms(), 256, 0, m->stream>>>(static_cast<const double*>(theta), n, m->w64, m->w32);
+  m->launches += 1;
+  DP_LAUNCH_CHECK(m);
+  return DP_OK;
+}
 
 // Chunk slots of the reduction workspace: every replica may need ceil(max_atoms / kRedChunk).
 size_t rep_reduce_slots(int max_atoms, int max_reps) {
