@@ -125,22 +125,22 @@ __device__ __forceinline__ float out_scale(int e, int sw, float) {    // 2^(36 -
   return e > 128 ? __int_as_float(0x7fc00000) : __int_as_float((127 + min(max(36 - 26 + e - sw, -126), 127)) << 23);
 }
 
-// The fragments run through shared memory in stages of KS k steps by cp.async, ST stages deep: with WK = 1 one
-// pipeline for the CTA (every warp multiplies the same fragments), else one for each warp.  Loads straight
+// The fragments run through shared memory in stages of KS k steps by cp.async, ST stages deep: one pipeline for
+// the warps that share a part of K (they multiply the same fragments).  Loads straight
 // into registers left each k step waiting for L2 (32,000 FP32 rows: 3.04 ms for the six GEMMs).
 template <class T, int WK> struct Pipe {
   static constexpr int KS = (WK == 1 && sizeof(T) == 4) ? 2 : 1;
   static constexpr int ST = WK == 1 ? 4 : 3;
   static constexpr int kWords = KS * NTiles<T>::v * dig::Frag<T>::Q * 32;  // uint4 of a stage
-  static constexpr int kPipes = WK == 1 ? 1 : kWarps;
-  static constexpr size_t kBytes = (size_t)kPipes * ST * kWords * 16;
+  static constexpr size_t kPipe = (size_t)WK * ST * kWords * 16;
+  static constexpr size_t kPart = WK == 1 ? 0 : sizeof(T) * kWarps * NTiles<T>::v * 4 * 32;  // the partial sums reuse it
+  static constexpr size_t kBytes = kPipe > kPart ? kPipe : kPart;
 };
 
 template <class T, int WK>
 __global__ void __launch_bounds__(32 * kWarps, 1) k_dig_gemm(GemmArgs<T> g) {
   constexpr int ND = Fmt<T>::ND, NO = Fmt<T>::NO, Q = dig::Frag<T>::Q, NT = NTiles<T>::v, MW = kWarps / WK;
   using P = Pipe<T, WK>;
-  static_assert(WK == 1 || P::kBytes >= sizeof(T) * kWarps * NT * 4 * 32, "the partial sums reuse the pipeline's memory");
   extern __shared__ __align__(16) uint4 sm[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, kw = w % WK, mw = w / WK;
   const int tq = lane & 3, gr = lane >> 2;
@@ -176,11 +176,11 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_dig_gemm(GemmArgs<T> g) {
     for (int n = 0; n < NT; ++n) dig::zero_acc<T>(acc[n]);
     const int k0 = ksteps * kw / WK, k1 = ksteps * (kw + 1) / WK;
     const int nst = (k1 - k0 + P::KS - 1) / P::KS;
-    uint4* pipe = sm + (WK == 1 ? 0 : w) * P::ST * P::kWords;
+    uint4* pipe = sm + kw * P::ST * P::kWords;
     auto issue = [&](int st) {
       if (st < nst) {
         uint4* dst = pipe + (st % P::ST) * P::kWords;
-        for (int q = WK == 1 ? (int)threadIdx.x : lane; q < P::kWords; q += WK == 1 ? 32 * kWarps : 32) {
+        for (int q = 32 * mw + lane; q < P::kWords; q += 32 * MW) {
           const int ln = q % (Q * 32), f = q / (Q * 32), n = f % NT, s = k0 + st * P::KS + f / NT;
           if (s < k1 && ntile0 + n < ntiles) tc::cp_async16(dst + q, fr + ((size_t)(ntile0 + n) * ksteps + s) * Q * 32 + ln);
         }
@@ -208,8 +208,9 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_dig_gemm(GemmArgs<T> g) {
     int left = Flush<T>::v;
     for (int st = 0; st < nst; ++st) {
       tc::cp_async_wait_group<P::ST - 2>();
-      if (WK == 1) __syncthreads();  // the stage has landed, and everyone is done with the one refilled next
-      else __syncwarp();
+      // the stage has landed, and everyone is done with the one refilled next
+      if (MW == 1) __syncwarp();
+      else asm volatile("bar.sync %0, %1;" ::"r"(kw + 1), "n"(32 * MW) : "memory");
       issue(st + P::ST - 1);
       uint4 a[P::KS][ND];
 #pragma unroll
@@ -455,11 +456,14 @@ dp_status run(Model* m, int N) {
   g.wscale = static_cast<const int*>(m->dig_fit);
   g.frag = reinterpret_cast<const uint4*>(static_cast<unsigned char*>(m->dig_fit) + 1024);
   g.stride = kFitParams;
-  // rows in 16-row tiles times column blocks against the SMs decides how far K is split inside a CTA:
-  // below about two CTAs an SM with 128-row CTAs, all eight warps share 16 rows
+  // rows times column blocks against the SMs decide how far K is split inside a CTA: the least splitting
+  // (most reuse of the fragments) that still gives four CTAs an SM
   auto go = [&](const GemmArgs<T>& a) {
-    const long ctas = (long)cdiv(N, 128) * cdiv(mat_of(a.mat).N / 8, NTiles<T>::v);
-    return ctas >= 4l * num_sms() ? gemm<T, 1>(m, N, a) : gemm<T, 8>(m, N, a);
+    const long blocks = cdiv(mat_of(a.mat).N / 8, NTiles<T>::v), want = 4l * num_sms();
+    if (cdiv(N, 128) * blocks >= want) return gemm<T, 1>(m, N, a);
+    if (cdiv(N, 64) * blocks >= want) return gemm<T, 2>(m, N, a);
+    if (cdiv(N, 32) * blocks >= want) return gemm<T, 4>(m, N, a);
+    return gemm<T, 8>(m, N, a);
   };
 #define DP_GO(a)                      \
   do {                                \
