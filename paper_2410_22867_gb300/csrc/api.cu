@@ -441,6 +441,7 @@ dp_status upload_weights(Model* m) {
 
 // Everything made from w64 / w32: padded-slot terms and the operand copies.
 dp_status derive_weights(Model* m) {
+  const bool dig = m->dig_ok;
   DP_TRY(launch_pad_rows(m));
   if (m->prec == DP_MIX_BF16 || m->prec == DP_MIX_FP16) {
     DP_TRY(launch_tc_setup(m));
@@ -448,6 +449,7 @@ dp_status derive_weights(Model* m) {
   } else {
     DP_TRY(dig_upload(m));
     DP_TRY(dig_fit_upload(m));
+    if (m->dig_ok != dig) drop_graphs(m);  // captured steps hold the other embedding kernels
   }
   return DP_OK;
 }
@@ -578,8 +580,10 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
     if (prec == DP_FP64) A_(dig_tanh, dig_tanh_bytes());
   }
   m->pg_cap = std::min(max_atoms, kPgAtoms);
+  const long sel_max = *std::max_element(sel, sel + nt);
+  m->pg_rows = (int)std::max(sel_max, std::min<long>(kPgRows, (long)max_atoms * sel_max));
   m->pg_roff_cap = 2 * (size_t)nt * N + 64;
-  A_(pg_ws, param_grad_workspace_bytes(m->pg_cap, prec == DP_FP64));
+  A_(pg_ws, param_grad_workspace_bytes(m->pg_cap, m->pg_rows, prec == DP_FP64));
   A_(pg_roff, 4 * m->pg_roff_cap);
   A_(pg_w, 24 * N);
   A_(pg_scal, 64 + 8 * kN3 * kMaxTypes);

@@ -23,8 +23,8 @@ constexpr int kEmbParams = kN1 + kN1 + kN1 * kN2 + kN2 + kN2 * kN3 + kN3;       
 constexpr int kFitParams = kKD * kF + kF + kF * kF + kF + kF * kF + kF + kF + 1;  // 500161
 constexpr int kMaxTypes = 4;
 constexpr int kRdfMaxCells = 24576;  // dp_rdf: ntypes^2 * nbins histogram cells at most
-// parameter gradient: centre atoms per chunk, neighbour rows per chunk of the embedding reverse
-constexpr int kPgAtoms = 2048, kPgRows = 32768;
+// parameter gradient: centre atoms per chunk, neighbour rows per chunk at most, largest sel it takes
+constexpr int kPgAtoms = 2048, kPgRows = 32768, kPgSel = 16384;
 
 // offsets inside one embedding block
 constexpr int kEW1 = 0, kEb1 = kN1, kEW2 = 2 * kN1, kEb2 = kEW2 + kN1 * kN2, kEW3 = kEb2 + kN2,
@@ -191,6 +191,7 @@ struct Model {
   // parameter gradient
   void* pg_ws = nullptr;      // per-chunk activations and adjoints (FP64 or FP32)
   int pg_cap = 0;             // centre atoms per chunk
+  int pg_rows = 0;            // neighbour rows per chunk
   int* pg_roff = nullptr;     // row offsets of every row chunk of one call
   size_t pg_roff_cap = 0;
   double* pg_w = nullptr;     // [N][3] tangent direction 2 cF (F - F0), internal order
@@ -358,7 +359,7 @@ void mix_fit_release(Model* m);
 // grid of a tunable mixed kernel: the autotuned value if set, else the default
 inline int tuned_grid(const Model* m, int which, int dflt) { return m->tune_grid[which] > 0 ? m->tune_grid[which] : dflt; }
 // parameter gradient (pgrad.cu)
-size_t param_grad_workspace_bytes(int cap, bool fp64);
+size_t param_grad_workspace_bytes(int cap, int rows, bool fp64);
 dp_status launch_param_grad(Model* m, int N, const double* F0, double E0, double cE, double cF, double* grad,
                             double* loss);
 inline bool is_mixed(const Model* m) { return m->prec == DP_MIX_BF16 || m->prec == DP_MIX_FP16; }

@@ -1121,11 +1121,12 @@ size_t bwd_smem(int warps) {
   return (sizeof(T) == 8 ? (sizeof(dig::TanhTab) + 15) / 16 * 16 : 0) + warps * sizeof(BwdWarp<T>);
 }
 
-// Tasks per atom: enough warp tasks (about 16 a resident warp) that the last wave is short; at most one per two
-// tiles of a full list, since a task's sums cost a few hundred atomics.
+// Tasks per atom: enough warp tasks (about 16 a resident warp) that the last wave is short; at most about one a
+// tile (lists hold two thirds of S in water, a third in Cu), since a task's sums cost a few hundred atomics.
+// A 192-atom water box has six tiles an atom: with four tasks half the warps took two tiles (forward 146 us).
 int split_of(const Model* m, int N, int warps) {
   const long want = 16l * num_sms() * warps;
-  const int most = std::max(1, m->S / 32);
+  const int most = std::max(1, m->S / 23);
   return (int)std::max(1l, std::min((long)most, (want + N - 1) / N));
 }
 

@@ -118,11 +118,12 @@ template <> struct Sum<float> {
   __device__ __forceinline__ void add(const float (*acc)[4], int e) { s += dig::join_f(acc, e); }
   __device__ __forceinline__ float value() const { return s; }
 };
+constexpr int kBadScale = -100000;  // a matrix with an infinity or a NaN: every product is NaN
 __device__ __forceinline__ double out_scale(int e, int sw, double) {  // 2^(40 - (54 - e) - sw)
-  return e > 1024 ? __longlong_as_double(0x7ff8000000000000ll) : dig::pow2d(40 - 54 + e - sw);
+  return e > 1024 || sw == kBadScale ? __longlong_as_double(0x7ff8000000000000ll) : dig::pow2d(40 - 54 + e - sw);
 }
 __device__ __forceinline__ float out_scale(int e, int sw, float) {    // 2^(36 - (26 - e) - sw)
-  return e > 128 ? __int_as_float(0x7fc00000) : __int_as_float((127 + min(max(36 - 26 + e - sw, -126), 127)) << 23);
+  return e > 128 || sw == kBadScale ? __int_as_float(0x7fc00000) : __int_as_float((127 + min(max(36 - 26 + e - sw, -126), 127)) << 23);
 }
 
 // The fragments run through shared memory in stages of KS k steps by cp.async, ST stages deep: one pipeline for
@@ -376,7 +377,7 @@ __global__ void __launch_bounds__(1024) k_dig_fit_scale(const T* __restrict__ fi
   if (threadIdx.x == 0) {
     for (int k = 1; k < 32; ++k) m = max(m, s[k]);
     const int e = max(exp_of(m, T(0)), sizeof(T) == 8 ? -60 : -30);
-    const int sw = RowBits<T>::v - e;
+    const int sw = e > (sizeof(T) == 8 ? 1024 : 128) ? kBadScale : RowBits<T>::v - e;
     wscale[ty * kMats + q] = sw;
     wscale[ty * kMats + 5 - q] = sw;
   }

@@ -847,8 +847,8 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
   std::vector<int> roffs;
   const int cap = m->pg_cap;
   for (int t = 0; t < nt; ++t)
-    if (m->sel[t] > kPgRows) {
-      m->last_error = "param_grad: sel larger than the row chunk";
+    if (m->sel[t] > kPgSel) {
+      m->last_error = "param_grad: sel larger than 16384";
       return DP_ERR_UNSUPPORTED;
     }
   int start = 0;
@@ -864,7 +864,7 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
           RowChunk rc{ti, tj, ac.a0, b, 0, 0, roffs.size()};
           int rows = 0;
           roffs.push_back(0);
-          while (b < bend && rows + cnt[(size_t)b * nt + tj] <= kPgRows) {
+          while (b < bend && rows + cnt[(size_t)b * nt + tj] <= m->pg_rows) {
             rows += cnt[(size_t)b * nt + tj];
             roffs.push_back(rows);
             ++b;
@@ -898,7 +898,7 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
   T* U = H + 2 * C * kF;
   T* G = U + 2 * C * kF;
   T* TB = G + 2 * C * kF;
-  const size_t RW = (size_t)kPgRows;
+  const size_t RW = (size_t)m->pg_rows;
   T* geo = TB + C * 800;
   T* H1 = geo + RW * kPgGeo;
   T* H2 = H1 + 2 * RW * kN1;
@@ -1007,10 +1007,10 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
 
 }  // namespace
 
-size_t param_grad_workspace_bytes(int cap, bool fp64) {
+size_t param_grad_workspace_bytes(int cap, int rows, bool fp64) {
   const size_t per_atom = 800 + 2 * 2 * (size_t)kKD + 6 * 2 * (size_t)kF + 800;
   const size_t per_row = kPgGeo + 2 * (size_t)(kN1 + kN2 + kN2 + kN3 + kN2 + kN2 + kN1) + 1;
-  return ((size_t)cap * per_atom + (size_t)kPgRows * per_row) * (fp64 ? 8 : 4);
+  return ((size_t)cap * per_atom + (size_t)rows * per_row) * (fp64 ? 8 : 4);
 }
 
 dp_status launch_param_grad(Model* m, int N, const double* F0, double E0, double cE, double cF, double* grad,
