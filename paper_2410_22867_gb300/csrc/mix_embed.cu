@@ -36,7 +36,6 @@ struct MixArgs {
   int sel_off[kMaxTypes + 1];
   float rc, rs, invS;
   int switch_kind;
-  const float* w;        // theta (fp32)
   const float* stat;     // davg [nt][4], 1/dstd [nt][4]
   const int* itype;
   const int* type_off;   // device [nt + 1]
@@ -234,7 +233,7 @@ constexpr int kSmall = 64;
 // Forward operand image of one embedding pair (built once per weight upload, copied into shared
 // memory by three bulk copies per pair change): B2 | B3 (head, remainder) | small.
 constexpr uint32_t kImgFwdB3 = 8192, kImgFwdSmall = kImgFwdB3 + 2 * 14336, kImgFwd = kImgFwdSmall + kSmall * 4;
-// Backward image behind it: B2 | B3 | small, used where a CTA walks few tiles (k_mix_embed_bwd<.., IMG>).
+// Backward image behind it: B2 | B3 | small.
 constexpr uint32_t kImgBwdB3 = 8192, kImgBwdSmall = kImgBwdB3 + 16384, kImgBwd = kImgBwdSmall + kSmall * 4;
 constexpr uint32_t kImgBytes = kImgFwd + kImgBwd;
 
@@ -371,10 +370,8 @@ __device__ __forceinline__ void row_compute(const MixArgs& a, const TileInfo& ti
   for (int c = 0; c < 4; ++c) f.R[c] = (f.R[c] - a.stat[ti.ti * 4 + c]) * a.stat[(a.ntypes + ti.ti) * 4 + c];
 }
 
-// h1 = tanh(s_hat W1 + b1) and its 16-bit copy into the A block (K = 32: 25 units, then the
-// two bias ones; with SPLIT the copy again in K slots 32..63 for the remainder of W2).
-template <bool F16, bool SPLIT = false>
-__device__ __forceinline__ void layer1(const float* small, float x, float* h1, unsigned char* sA, int t) {
+// h1 = tanh(s_hat W1 + b1).
+__device__ __forceinline__ void layer1_h(const float* small, float x, float* h1) {
 #pragma unroll
   for (int k4 = 0; k4 < 7; ++k4) {
     const float4 wv = reinterpret_cast<const float4*>(small)[k4];
@@ -384,6 +381,13 @@ __device__ __forceinline__ void layer1(const float* small, float x, float* h1, u
     for (int u = 0; u < 4; ++u)
       if (4 * k4 + u < kN1) h1[4 * k4 + u] = tc::tanh_fast(fmaf(x, w4[u], b4[u]));
   }
+}
+
+// h1 and its 16-bit copy into the A block (K = 32: 25 units, then the
+// two bias ones; with SPLIT the copy again in K slots 32..63 for the remainder of W2).
+template <bool F16, bool SPLIT = false>
+__device__ __forceinline__ void layer1(const float* small, float x, float* h1, unsigned char* sA, int t) {
+  layer1_h(small, x, h1);
 #pragma unroll
   for (int k0 = 0; k0 < 32; k0 += 8) {
     uint32_t p[4];
@@ -753,9 +757,12 @@ __device__ void load_bwd_ops(const float* __restrict__ W, unsigned char* sB2, un
 // dh2' product.  dR_hat and dG use dE/dT and G in FP32 on the CUDA cores.
 // ATOMVIR: a second pass over the stored state that accumulates only the per-atom (centre)
 // virial -sum g (x) d into a.vir_atom (FP64) and leaves forces and per-replica virials alone.
-// IMG: the operand blocks come from the pair's image (three bulk copies) instead of being converted from
-// the weights by every CTA; see launch_mix_embed_backward for where that pays.
-template <bool F16, bool TAB, bool ATOMVIR = false, bool IMG = false>
+// The operand blocks come from the pair's image (three bulk copies); converting the weights in every CTA
+// took 10 us of a small box's 42.  h1 is computed twice, so that its 25 registers are free in the layer-3
+// epilogue for the packed dG (four instructions a unit pair less): 131,072 Cu atoms 2.99 -> 2.89 ms, 12,288 water
+// atoms 206 -> 191 us, 16,384 Cu atoms (bf16) 430 -> 391 us.  Either change without the other, or with 16
+// columns at a time in the layer-2 backward, spills and is slower (2.94 to 3.45 ms).
+template <bool F16, bool TAB, bool ATOMVIR = false>
 __global__ void __launch_bounds__(kRows, 3) k_mix_embed_bwd(MixArgs a) {
   extern __shared__ unsigned char sraw[];
   unsigned char* sm = align1024(sraw);
@@ -826,10 +833,7 @@ __global__ void __launch_bounds__(kRows, 3) k_mix_embed_bwd(MixArgs a) {
     if (w == kLocWarp && cur + ti.nrows < c1) locate_window(a, cur + ti.nrows, wk, s_tot, sWin);
     const int np = ti.ti * a.ntypes + ti.tj;
     if (np != pair) {
-      // over many tiles the backward builds its operand blocks itself: fetching them from the image
-      // changes the register allocation of its main loop and costs 4-8%
-      if (!TAB && !IMG) load_bwd_ops<F16>(a.w + (size_t)np * kEmbParams, sB2, sB3, small);
-      if (!TAB && IMG) {  // on the product barrier, idle here
+      if (!TAB) {  // on the product barrier, idle here: every earlier product has completed
         if (t == 0)
           fetch_image(a.img + (size_t)np * kImgBytes + kImgFwd, kImgBwdB3, kImgBwdSmall, kImgBwd, sB2, sB3, small, &bar);
         ok = tc::mbar_wait(&bar, phase, a.err) && ok;
@@ -925,6 +929,8 @@ __global__ void __launch_bounds__(kRows, 3) k_mix_embed_bwd(MixArgs a) {
     {
       const float4* dTa = sdT + f.la * kN3;
       const uint64_t m1 = tc::f2(-1.f, -1.f);
+      const uint64_t R2[4] = {tc::f2(f.R[0], f.R[0]), tc::f2(f.R[1], f.R[1]), tc::f2(f.R[2], f.R[2]),
+                              tc::f2(f.R[3], f.R[3])};
       uint64_t ax = tc::f2(0.f, 0.f), ay = ax, az = ax, aw = ax;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {  // columns 8 c .. 8 c + 7 of each member
@@ -949,9 +955,7 @@ __global__ void __launch_bounds__(kRows, 3) k_mix_embed_bwd(MixArgs a) {
             ay = tc::f2fma(Py, G2, ay);
             az = tc::f2fma(Pz, G2, az);
             aw = tc::f2fma(Pw, G2, aw);
-            const float ga = fmaf(f.R[3], phi.z, fmaf(f.R[2], phi.x, fmaf(f.R[1], plo.z, f.R[0] * plo.x)));
-            const float gb = fmaf(f.R[3], phi.w, fmaf(f.R[2], phi.y, fmaf(f.R[1], plo.w, f.R[0] * plo.y)));
-            const uint64_t g = tc::f2(ga, gb);
+            const uint64_t g = tc::f2fma(R2[3], Pw, tc::f2fma(R2[2], Pz, tc::f2fma(R2[1], Py, tc::f2mul(R2[0], Px))));
             const uint64_t dzn = tc::f2mul(g, tc::f2fma(T2, T2, m1));  // -dz3 of (m, m + 50)
             da[u] = tc::f2lo(dzn);
             db[u] = tc::f2hi(dzn);
@@ -990,6 +994,13 @@ __global__ void __launch_bounds__(kRows, 3) k_mix_embed_bwd(MixArgs a) {
       locate_tile(a, cur + ti.nrows, c0, c1, wk, s_tot, s_tiend, &sti, sRow, sWin, true, &sNat);
       if (lane == 0) fetch_dT(a, sti.a0, sNat, sdT, &dbar);  // values this lane has just written
     }
+    // h1 again, under the MMA: its 25 registers were free for the layer-3 epilogue (the compiler must not
+    // see that it is the same value)
+    {
+      float x = f.R[0];
+      asm volatile("" : "+f"(x));
+      layer1_h(small, x, h1);
+    }
     mma_sync_wait(&bar, phase, a.err, ok);
     if (cur + ti.nrows < c1) {
       dT_pending = true;
@@ -1001,30 +1012,31 @@ __global__ void __launch_bounds__(kRows, 3) k_mix_embed_bwd(MixArgs a) {
     float dh1[kN1];
 #pragma unroll
     for (int k = 0; k < kN1; ++k) dh1[k] = 0.f;
+// (eight columns at a time: this is the tile's peak of live registers)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float z[16], rr[16];
-      tc::tmem_ld16(tl + 16 * c, z);
-      tc::tmem_ld16(tl + 64 + 16 * c, rr);
-      tc::tmem_wait_ld();
-      float d2[16];
+    for (int c = 0; c < 8; ++c) {
+      float d2[8];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
-        const int m = 16 * c + u;
-        d2[u] = 0.f;
-        if (m < kN2) {
-          const float g2 = rr[u] - z[u];  // dh2' comes out negated (dz3 was stored negated)
-          const float t2 = h2[m] - h1[m % kN1];
-          d2[u] = g2 * (1.f - t2 * t2);
-          dh1[m % kN1] += g2;
+      for (int u = 0; u < 8; ++u) d2[u] = 0.f;
+      if (8 * c < kN2) {
+        float z[8], rr[8];
+        tc::tmem_ld8(tl + 8 * c, z);
+        tc::tmem_ld8(tl + 64 + 8 * c, rr);
+        tc::tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int m = 8 * c + u;
+          if (m < kN2) {
+            const float g2 = rr[u] - z[u];  // dh2' comes out negated (dz3 was stored negated)
+            const float t2 = h2[m] - h1[m % kN1];
+            d2[u] = g2 * (1.f - t2 * t2);
+            dh1[m % kN1] += g2;
+          }
         }
       }
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh)
-        tc::st_chunk(sA, t, 16 * c + 8 * hh,
-                     make_uint4(tc::pack2<F16>(d2[8 * hh], d2[8 * hh + 1]), tc::pack2<F16>(d2[8 * hh + 2], d2[8 * hh + 3]),
-                                tc::pack2<F16>(d2[8 * hh + 4], d2[8 * hh + 5]),
-                                tc::pack2<F16>(d2[8 * hh + 6], d2[8 * hh + 7])));
+      tc::st_chunk(sA, t, 8 * c,
+                   make_uint4(tc::pack2<F16>(d2[0], d2[1]), tc::pack2<F16>(d2[2], d2[3]), tc::pack2<F16>(d2[4], d2[5]),
+                              tc::pack2<F16>(d2[6], d2[7])));
     }
     operand_barrier();
     // dh1' = dz2 W2^T (B = the rows of B2 read MN-major: K = layer-2 unit, N = layer-1 unit)
@@ -1440,7 +1452,7 @@ MixArgs make_mix_args(Model* m, int N) {
   a.N = N; a.ntypes = m->ntypes; a.S = m->S;
   for (int t = 0; t <= m->ntypes; ++t) a.sel_off[t] = m->sel_off[t];
   a.rc = (float)m->rc; a.rs = (float)m->rs; a.invS = 1.f / (float)m->S; a.switch_kind = m->switch_kind;
-  a.w = m->w32; a.stat = m->stat32; a.itype = m->itype; a.type_off = m->type_off; a.rowoff = m->rowoff;
+  a.stat = m->stat32; a.itype = m->itype; a.type_off = m->type_off; a.rowoff = m->rowoff;
   a.tab = reinterpret_cast<const float4*>(m->tab32);
   a.img = static_cast<const unsigned char*>(m->emb_img);
   a.tab_n = m->tab_n;
@@ -1530,12 +1542,6 @@ dp_status launch_mix_descriptor(Model* m, int N) {
   return DP_OK;
 }
 
-// Up to this many neighbour slots (atoms x S) a CTA of the backward walks few tiles and converting the
-// weights is a good part of its time: the image variant runs instead.  Measured, converting -> image: 192
-// water atoms (26 k slots) 42 -> 32 us, 4,500 (0.6 M) 118 -> 112, 8,100 (1.1 M) 161 -> 157; 6,912 Cu atoms
-// (3.5 M) 195 -> 198.
-constexpr long kImgSlots = 1200000;
-
 dp_status launch_mix_embed_backward(Model* m, int N, bool fold) {
   const int dt_grid = std::max(1, std::min((N + kDtWarps - 1) / kDtWarps, tuned_grid(m, 2, 5 * num_sms())));
   k_mix_dT<<<dt_grid, 32 * kDtWarps, 0, m->stream>>>(N, 1.f / (float)m->S, static_cast<const float4*>(m->Tm),
@@ -1545,10 +1551,8 @@ dp_status launch_mix_embed_backward(Model* m, int N, bool fold) {
   MixArgs a = make_mix_args(m, N);
   const bool f16 = m->prec == DP_MIX_FP16;
   const bool tab = m->tab_n > 0;
-  const bool img = !tab && (long)N * m->S <= kImgSlots;
   auto bk = f16 ? (tab ? k_mix_embed_bwd<true, true> : k_mix_embed_bwd<true, false>)
                 : (tab ? k_mix_embed_bwd<false, true> : k_mix_embed_bwd<false, false>);
-  if (img) bk = f16 ? k_mix_embed_bwd<true, false, false, true> : k_mix_embed_bwd<false, false, false, true>;
   const void* fn = reinterpret_cast<const void*>(bk);
   DP_CUDA_TRY(m, ensure_smem(fn, kBwdSmem));
   const int grid = tuned_grid(m, 1, num_sms() * blocks_per_sm(fn, kRows, kBwdSmem, kTmemCols));
