@@ -6,7 +6,9 @@
 // (50 of 100) as node data (value and h-scaled first and second derivative at the n + 1 nodes, 154 KB
 // for 256 intervals) and a warp walks the neighbours of an atom with lane = two outputs: its
 // shared-memory reads are consecutive, the six Hermite basis values of a row are the same for all
-// outputs, and T (forward) or dR_hat, d s_hat (backward) are sums in registers.  Half the CTAs hold
+// outputs, and T (forward) or dR_hat, d s_hat (backward) are sums in registers.  A row outside the table
+// (an input below the first or above the last node) is evaluated from the edge interval's coefficients: u intervals
+// beyond the edge the Hermite basis values grow as u^5 and cancel, which costs all FP32 digits.  Half the CTAs hold
 // outputs 0..49, half 50..99; the backward's force terms are linear in those sums, so each half adds its own.
 // Bound by shared-memory wavefronts and issue (about 32 and 54 a row forward): 32,000 Cu atoms 2.48 -> 0.72 ms
 // forward, 2.50 -> 1.23 ms backward.
@@ -26,6 +28,7 @@ struct TabArgs {
   int switch_kind;
   const float* stat;
   const float* nodes;        // [pair][2][n + 1][3][50]
+  const float4* coef;        // [pair][n][100][2]: quintic coefficients (rows outside the table)
   const int* type_off;
   const int* type_count;
   const int* nl_j;
@@ -68,11 +71,19 @@ __device__ __forceinline__ void env_row(const TabArgs& a, int ti, float4 dv, Row
 }
 
 // The interval of x (edge intervals beyond the ends) and the quintic Hermite basis at u = (x - x_i) / h for
-// (f, h f', h^2 f'') at its left and right node; D: the derivatives of the basis.
-__device__ __forceinline__ int basis(const TabArgs& a, float x, float* H) {
+// (f, h f', h^2 f'') at its left and right node; D: the derivatives of the basis.  Outside the table the basis is
+// zero and `out` is set.
+__device__ __forceinline__ int basis(const TabArgs& a, float x, float& u, bool& out, float* H) {
   const float f = (x - a.x0) * a.ih;
   const int i = min(max((int)floorf(f), 0), a.n - 1);
-  const float u = f - (float)i, u2 = u * u, u3 = u2 * u;
+  u = f - (float)i;
+  out = !(u >= 0.f && u <= 1.f);
+  if (out) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) H[k] = 0.f;
+    return i;
+  }
+  const float u2 = u * u, u3 = u2 * u;
   const float s = u3 * fmaf(u, fmaf(6.f, u, -15.f), 10.f);
   H[0] = 1.f - s;
   H[1] = u + u3 * fmaf(u, fmaf(-3.f, u, 8.f), -6.f);
@@ -82,8 +93,8 @@ __device__ __forceinline__ int basis(const TabArgs& a, float x, float* H) {
   H[5] = 0.5f * u3 * fmaf(u, fmaf(1.f, u, -2.f), 1.f);
   return i;
 }
-__device__ __forceinline__ void basis_d(const TabArgs& a, float x, int i, float* D) {
-  const float u = (x - a.x0) * a.ih - (float)i, u2 = u * u;
+__device__ __forceinline__ void basis_d(float u, float* D) {
+  const float u2 = u * u;
   const float s = u2 * fmaf(u, fmaf(30.f, u, -60.f), 30.f);
   D[0] = -s;
   D[1] = 1.f + u2 * fmaf(u, fmaf(-15.f, u, 32.f), -18.f);
@@ -91,6 +102,17 @@ __device__ __forceinline__ void basis_d(const TabArgs& a, float x, int i, float*
   D[3] = s;
   D[4] = u2 * fmaf(u, fmaf(-15.f, u, 28.f), -12.f);
   D[5] = u2 * fmaf(u, fmaf(2.5f, u, -4.f), 1.5f);
+}
+
+// P(u) and P'(u) of outputs q and q + 1 from the coefficients of interval i.
+__device__ __forceinline__ void poly2(const TabArgs& a, int pair, int i, int q, float u, float* g, float* gu) {
+  const float4* p = a.coef + (((size_t)pair * a.n + i) * kN3 + q) * 2;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float4 lo = __ldg(p + 2 * k), hi = __ldg(p + 2 * k + 1);
+    g[k] = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, hi.y, hi.x), lo.w), lo.z), lo.y), lo.x);
+    gu[k] = fmaf(u, fmaf(u, fmaf(u, fmaf(u, 5.f * hi.y, 4.f * hi.x), 3.f * lo.w), 2.f * lo.z), lo.y);
+  }
 }
 
 __device__ __forceinline__ void load_nodes(const TabArgs& a, int pair, int half, float* tab) {
@@ -130,19 +152,33 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_tab_fwd(TabArgs a) {
         const float4 dv = nxt;
         if (b + 32 + lane < cnt) nxt = dp[b + 32 + lane];
         __syncwarp();
+        bool out = false;
         if (b + lane < cnt) {
           Row f;
-          float H[6];
+          float H[6], u;
           env_row(a, ti, dv, f);
-          const int k = basis(a, f.R[0], H);
+          const int k = basis(a, f.R[0], u, out, H);
 #pragma unroll
           for (int c = 0; c < 4; ++c) f.R[c] = __half2float(__float2half_rn(f.R[c]));
           mine[lane][0] = make_float4(H[0], H[1], H[2], H[3]);
           mine[lane][1] = make_float4(H[4], H[5], __int_as_float(k * kNode), f.R[0]);
-          mine[lane][2] = make_float4(f.R[1], f.R[2], f.R[3], 0.f);
+          mine[lane][2] = make_float4(f.R[1], f.R[2], f.R[3], u);
         }
+        unsigned far = __ballot_sync(0xffffffffu, out);
         __syncwarp();
         const int nr = min(32, cnt - b);
+        for (; far; far &= far - 1) {
+          const int r = __ffs(far) - 1;
+          const float4 q = mine[r][1], s = mine[r][2];
+          float g[2], gu[2];
+          poly2(a, pair, __float_as_int(q.z) / kNode, half * kHalf + fo, s.w, g, gu);
+          const float2 G = __half22float2(__floats2half2_rn(g[0], g[1]));
+          const uint64_t gg = tc::f2(G.x, G.y);
+          acc[0] = tc::f2fma(dup(q.w), gg, acc[0]);
+          acc[1] = tc::f2fma(dup(s.x), gg, acc[1]);
+          acc[2] = tc::f2fma(dup(s.y), gg, acc[2]);
+          acc[3] = tc::f2fma(dup(s.z), gg, acc[3]);
+        }
 #pragma unroll 2
         for (int r = 0; r < nr; ++r) {
           const float4 p = mine[r][0], q = mine[r][1], s = mine[r][2];
@@ -254,22 +290,25 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_tab_bwd(TabArgs a) {
       for (int b = 0; b < cnt; b += 32) {
         Row f;
         const bool in = b + lane < cnt;
+        bool out = false;
         __syncwarp();
         {
           float H[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, D[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+          float u = 0.f;
           int k = 0;
           f.R[0] = f.R[1] = f.R[2] = f.R[3] = 0.f;
           if (in) {
             env_row(a, ti, a.nl_d[e0 + b + lane], f);
-            k = basis(a, f.R[0], H);
-            basis_d(a, f.R[0], k, D);
+            k = basis(a, f.R[0], u, out, H);
+            if (!out) basis_d(u, D);
           }
           mine[lane][0] = make_float4(H[0], H[1], H[2], H[3]);
           mine[lane][1] = make_float4(H[4], H[5], __int_as_float(k * kNode), f.R[0]);
           mine[lane][2] = make_float4(f.R[1], f.R[2], f.R[3], D[0]);
           mine[lane][3] = make_float4(D[1], D[2], D[3], D[4]);
-          mine[lane][4] = make_float4(D[5], 0.f, 0.f, 0.f);
+          mine[lane][4] = make_float4(D[5], u, 0.f, 0.f);
         }
+        unsigned far = __ballot_sync(0xffffffffu, out);
         __syncwarp();
         const int nr = min(32, cnt - b);
         float own[5] = {0.f, 0.f, 0.f, 0.f, 0.f};  // this lane's row
@@ -313,6 +352,25 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_tab_bwd(TabArgs a) {
           for (int q = 0; q < 5; ++q) {
             const float y = __shfl_sync(0xffffffffu, o[q], src);
             if ((lane & ~7) == r0) own[q] = y;
+          }
+        }
+        for (; far; far &= far - 1) {
+          const int r = __ffs(far) - 1;
+          const float4 q = mine[r][1], s = mine[r][2];
+          float g[2], gu[2], v[5];
+          poly2(a, pair, __float_as_int(q.z) / kNode, half * kHalf + fo, mine[r][4].y, g, gu);
+          const uint64_t gg = tc::f2(g[0], g[1]);
+          uint64_t dg = tc::f2mul(dup(q.w), dt[0]);
+          dg = tc::f2fma(dup(s.x), dt[1], dg);
+          dg = tc::f2fma(dup(s.y), dt[2], dg);
+          dg = tc::f2fma(dup(s.z), dt[3], dg);
+#pragma unroll
+          for (int c = 0; c < 5; ++c) {
+            const uint64_t m = c < 4 ? tc::f2mul(dt[c], gg) : tc::f2mul(dg, tc::f2(gu[0], gu[1]));
+            v[c] = lane < kHalf / 2 ? tc::f2lo(m) + tc::f2hi(m) : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+            if (lane == r) own[c] = v[c];
           }
         }
         if (in) {
@@ -368,6 +426,7 @@ TabArgs make_args(Model* m, int N) {
   a.rc = (float)m->rc; a.rs = (float)m->rs; a.winv = 1.f / (a.rc - a.rs);
   a.x0 = (float)m->tab_x0; a.ih = (float)(1.0 / m->tab_h);
   a.switch_kind = m->switch_kind; a.stat = m->stat32; a.nodes = m->tab_nodes32;
+  a.coef = reinterpret_cast<const float4*>(m->tab32);
   a.type_off = m->type_off; a.type_count = m->type_count; a.nl_j = m->nl_j;
   a.nl_d = static_cast<const float4*>(m->nl_d); a.nl_count = m->nl_count;
   a.Tseg = m->Tseg; a.dT = static_cast<const float4*>(m->dTm); a.force32 = m->force32;

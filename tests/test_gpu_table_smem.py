@@ -49,3 +49,26 @@ def test_table_forms(prec, n, form):
         else:
             assert e["f_rel"] <= 5 * bar["f_rel"], e
     m.close()
+
+
+@pytest.mark.parametrize("prec", ["mix_bf16", "mix_fp16"])
+def test_rows_outside_the_table(prec):
+    """A table that ends below the bonded O-H pairs: their rows (about 700) lie up to 98 intervals beyond
+    the last node and take the edge interval's polynomial, which is within 0.015 of the net there (outputs of
+    up to 2.9), so the same bars hold."""
+    import paper_2410_22867_gb300 as dp
+    w = synth.normalised_weights("water", env_stats())
+    s = synth.water_box(250, 255)
+    m = dp.DPModel(w, prec, max_atoms=s.natoms)
+    x0, x1, _ = m.tabulate(256)
+    x1 = x0 + 0.48 * (x1 - x0)
+    m.tabulate(256, x0, x1)
+    orc = oracle.Model(w.to_blob())
+    orc.tabulate(x0, x1, 256)
+    out = m.compute(torch.tensor(s.coords, device="cuda"), torch.tensor(s.types, device="cuda"), s.box)
+    ref = orc.compute(s.coords, s.types, s.box)
+    e = errors({q: out[q] for q in ("forces", "atom_energy")}, ref, s.types)
+    bar = BARS["water"][prec]
+    assert e["f_rel"] <= bar["f_rel"], e
+    assert e["dev_rel"] <= bar["dev_rel"], e
+    m.close()
