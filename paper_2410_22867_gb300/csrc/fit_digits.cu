@@ -36,7 +36,11 @@ __host__ __device__ __forceinline__ int mat_off(int q) {
 }
 constexpr int kTypeFrags = 2 * (kKD / 16) * (kF / 8) + 4 * (kF / 16) * (kF / 8);
 
-template <class T> struct NTiles { static constexpr int v = sizeof(T) == 8 ? 3 : 6; };  // n-tiles of a warp
+// n-tiles of a warp.  FP32: three, so that two CTAs of 128 registers a thread fit an SM; six in one CTA reuse the
+// A digits twice as often but leave a warp's latency open (six GEMMs, 32,000 rows: 2.46 -> 1.97 ms, 6,912:
+// 0.71 -> 0.50, 2,331: 0.33 -> 0.23, 192: 0.089 -> 0.070; five spill: 2.04, 0.54, 0.35, 0.091).  FP64's three
+// take 228 to 244 registers.
+constexpr int kNTiles = 3;
 // k steps whose digit products stay below 2^24 in the accumulators: 7 x 128 x 2^14, 2 x 80 x 2^16
 template <class T> struct Flush { static constexpr int v = sizeof(T) == 8 ? 8 : 5; };
 constexpr int kWarps = 8;
@@ -132,15 +136,15 @@ __device__ __forceinline__ float out_scale(int e, int sw, float) {    // 2^(36 -
 template <class T, int WK> struct Pipe {
   static constexpr int KS = (WK == 1 && sizeof(T) == 4) ? 2 : 1;
   static constexpr int ST = WK == 1 ? 4 : 3;
-  static constexpr int kWords = KS * NTiles<T>::v * dig::Frag<T>::Q * 32;  // uint4 of a stage
+  static constexpr int kWords = KS * kNTiles * dig::Frag<T>::Q * 32;  // uint4 of a stage
   static constexpr size_t kPipe = (size_t)WK * ST * kWords * 16;
-  static constexpr size_t kPart = WK == 1 ? 0 : sizeof(T) * kWarps * NTiles<T>::v * 4 * 32;  // the partial sums reuse it
+  static constexpr size_t kPart = WK == 1 ? 0 : sizeof(T) * kWarps * kNTiles * 4 * 32;  // the partial sums reuse it
   static constexpr size_t kBytes = kPipe > kPart ? kPipe : kPart;
 };
 
 template <class T, int WK>
-__global__ void __launch_bounds__(32 * kWarps, 1) k_dig_gemm(GemmArgs<T> g) {
-  constexpr int ND = Fmt<T>::ND, NO = Fmt<T>::NO, Q = dig::Frag<T>::Q, NT = NTiles<T>::v, MW = kWarps / WK;
+__global__ void __launch_bounds__(32 * kWarps, sizeof(T) == 8 ? 1 : 2) k_dig_gemm(GemmArgs<T> g) {
+  constexpr int ND = Fmt<T>::ND, NO = Fmt<T>::NO, Q = dig::Frag<T>::Q, NT = kNTiles, MW = kWarps / WK;
   using P = Pipe<T, WK>;
   extern __shared__ __align__(16) uint4 sm[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, kw = w % WK, mw = w / WK;
@@ -432,7 +436,7 @@ template <class T, int WK>
 dp_status gemm(Model* m, int N, const GemmArgs<T>& g) {
   const int mt = 16 * (kWarps / WK);
   DP_CUDA_TRY(m, ensure_smem(reinterpret_cast<const void*>(k_dig_gemm<T, WK>), Pipe<T, WK>::kBytes));
-  const dim3 grid(cdiv(N, mt) + m->ntypes, cdiv(mat_of(g.mat).N / 8, NTiles<T>::v));
+  const dim3 grid(cdiv(N, mt) + m->ntypes, cdiv(mat_of(g.mat).N / 8, kNTiles));
   k_dig_gemm<T, WK><<<grid, 32 * kWarps, Pipe<T, WK>::kBytes, m->stream>>>(g);
   m->launches += 1;
   DP_LAUNCH_CHECK(m);
@@ -460,7 +464,7 @@ dp_status run(Model* m, int N) {
   // rows times column blocks against the SMs decide how far K is split inside a CTA: the least splitting
   // (most reuse of the fragments) that still gives four CTAs an SM
   auto go = [&](const GemmArgs<T>& a) {
-    const long blocks = cdiv(mat_of(a.mat).N / 8, NTiles<T>::v), want = 4l * num_sms();
+    const long blocks = cdiv(mat_of(a.mat).N / 8, kNTiles), want = 4l * num_sms();
     if (cdiv(N, 128) * blocks >= want) return gemm<T, 1>(m, N, a);
     if (cdiv(N, 64) * blocks >= want) return gemm<T, 2>(m, N, a);
     if (cdiv(N, 32) * blocks >= want) return gemm<T, 4>(m, N, a);
