@@ -44,17 +44,32 @@ __host__ __device__ __forceinline__ int unit3m(int j, int t) {
   return t == 0 ? 24 : t == 1 ? 49 : -1;
 }
 
-// Per-pair scales: |W2| 2^sw2 below half (FP64) or 255/256 (FP32) of the digits' range, and likewise W3; FP64: z of a layer is a fixed-point
-// number with zs fraction bits, the upper four orders shifted left by s, the lower four right by 32 - s.
+// Scales of a pair, one for every output of a product (a column of W, a row of W for the transposes): its weights
+// times 2^sw fill half (FP64) or 255/256 (FP32) of the digits' range.  The dropped digit products count against
+// the largest weight of a column, so a scale for the whole matrix let one large weight take the bits of every other
+// column (largest weight 30,000 beside 0.1: G 1.2e-3 off in FP32, 6e-14 in FP64; with these 6e-8 and 2e-16).
+// FP64: z of an output is a fixed-point number with zs fraction bits, the upper four orders shifted left by s, the
+// lower four right by 32 - s.
 struct PairScale {
-  int sw2, sw3, zs2, zs3, s2, s3;
+  int sw2[kN2], zs2[kN2], s2[kN2], sw3[kN3], zs3[kN3], s3[kN3];
+  int swt3[kN2], swt2[kN1];  // rows of W3, W2
 };
 
-// Bias and layer-1 constants of a pair.
+// Constants of one output: bias and scale.
+template <class T> struct Out;
+template <> struct __align__(16) Out<double> {
+  long long b;  // fixed point, zs bits
+  int zs, s;
+};
+template <> struct __align__(8) Out<float> {
+  float b, c;   // z = c (sum of orders) + b
+};
+// Bias and layer-1 constants of a pair, and the factors of the transposed products.
 template <class T>
-struct PairSmall {
-  T w1[4 * kS1], b1[4 * kS1];              // [slot][t]
-  typename Fmt<T>::V b2[8 * kT2], b3[8 * kT3];  // [n-tile][2 t + e] (FP64: fixed point, zs2 / zs3 bits)
+struct __align__(16) PairSmall {
+  T w1[4 * kS1], b1[4 * kS1];       // [slot][t]
+  Out<T> o2[8 * kT2], o3[8 * kT3];  // [n-tile][2 t + e]
+  T c3t[8 * kT3T], c2t[4 * kS1];    // [n-tile][2 t + e], [slot][t]: unit of dz3 W3^T, dz2 W2^T
 };
 
 template <class T>
@@ -65,7 +80,6 @@ struct DigArgs {
   int switch_kind;
   const T* stat;
   const uint4* frag;           // [pair][kFrags][SetWords]
-  const PairScale* scale;      // [pair]
   const PairSmall<T>* small;   // [pair]
   const dig::TanhTab* tab;     // FP64
   const int* itype;
@@ -130,29 +144,15 @@ __device__ __forceinline__ long long act1(double x, double w, double b, const di
 }
 __device__ __forceinline__ float act1(float x, float w, float b, const dig::TanhTab*) { return tanhf(fmaf(x, w, b)); }
 
-struct LayerD {  // a layer's constants
-  int zs, s;
-};
-struct LayerF {
-  float c;
-};
-__device__ __forceinline__ LayerD layer(const PairScale& p, int which, double) {
-  return which == 2 ? LayerD{p.zs2, p.s2} : LayerD{p.zs3, p.s3};
-}
-// FP32: z = 2^(18 - sw) (sum of orders) + b
-__device__ __forceinline__ LayerF layer(const PairScale& p, int which, float) {
-  const int e = 18 - (which == 2 ? p.sw2 : p.sw3);
-  return LayerF{__int_as_float((127 + e) << 23)};
-}
-__device__ __forceinline__ long long act(const float (*acc)[4], int e, const LayerD& L, long long b,
-                                         const dig::TanhTab* tab) {
+// tanh of element e's output.
+__device__ __forceinline__ long long act(const float (*acc)[4], int e, const Out<double>& o, const dig::TanhTab* tab) {
   const dig::Pair64 p = dig::join(acc, e);
-  const int r = 32 - L.s;
-  const long long z = (p.hi << L.s) + ((p.lo + ((1ll << r) >> 1)) >> r) + b;
-  return dig::tanh_fixed(z, L.zs, tab);
+  const int r = 32 - o.s;
+  const long long z = (p.hi << o.s) + ((p.lo + ((1ll << r) >> 1)) >> r) + o.b;
+  return dig::tanh_fixed(z, o.zs, tab);
 }
-__device__ __forceinline__ float act(const float (*acc)[4], int e, const LayerF& L, float b, const dig::TanhTab*) {
-  return tanhf(fmaf(dig::join_f(acc, e), L.c, b));
+__device__ __forceinline__ float act(const float (*acc)[4], int e, const Out<float>& o, const dig::TanhTab*) {
+  return tanhf(fmaf(dig::join_f(acc, e), o.c, o.b));
 }
 
 // The biased digits of activations: h1 (|h1| <= 1) and h2 (|h2| <= 2).
@@ -292,7 +292,7 @@ __device__ __forceinline__ float from_digits(const uint4* A, int p, int e, int r
 // Layers 1 and 2 of a tile: h1 [slot][row], h2 [n-tile][e][row] (rows g, g + 8; FP64), and the digits of h2
 // in A (shared memory, FP64) or A (registers, FP32, which takes h2 back from them).
 template <class T, Store ST>
-__device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale& ps, const uint4* __restrict__ fr,
+__device__ __forceinline__ void layers12(const PairSmall<T>& sm, const uint4* __restrict__ fr,
                                          T x0, T x1, const dig::TanhTab* tab, uint4* A, int lane,
                                          typename Fmt<T>::V (*h1)[2], typename Fmt<T>::V (*h2)[2][2]) {
   constexpr int ND = Fmt<T>::ND;
@@ -318,7 +318,6 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale
     put_a<T, 7, ST>(A1, s, true, lane, u);
   }
   if (D) __syncwarp();
-  const auto L = layer(ps, 2, T(0));
   U u[2][4];
 #pragma unroll
   for (int p = 0; p < kT2; ++p) {
@@ -326,10 +325,10 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const PairScale
     product<T, kK2, false, ST>(acc, A1, fr + (size_t)(kF2 + p * kK2) * SetWords<T>::v, lane);
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const V b = sm.b2[8 * p + 2 * t + e];
+      const Out<T> o = sm.o2[8 * p + 2 * t + e];
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const V h = h1[p][r] + act(acc, 2 * r + e, L, b, tab);
+        const V h = h1[p][r] + act(acc, 2 * r + e, o, tab);
         if constexpr (D) h2[p][e][r] = h;
         else u[r][2 * (p & 1) + e] = dig_h2(h);
       }
@@ -409,7 +408,6 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
       const int cnt = a.nl_count[(size_t)i * a.ntypes + tj];
       const int nt = (cnt + 15) >> 4;
       const int pair = ti * a.ntypes + tj;
-      const PairScale ps = a.scale[pair];
       const PairSmall<T>& sm = a.small[pair];
       const uint4* fr = a.frag + (size_t)pair * kFrags * SetWords<T>::v;
       int first = (sub - q0) % a.sp;
@@ -433,8 +431,7 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
         V h1[kS1][2], h2[D ? kT2 : 1][2][2];
         uint4 Ar[D ? 1 : kK3 * Fmt<T>::ND];
         uint4* A = D ? sw.A : Ar;
-        layers12<T, ST>(sm, ps, fr, sw.R[g][0], sw.R[g + 8][0], tab, A, lane, h1, h2);
-        const auto L = layer(ps, 3, T(0));
+        layers12<T, ST>(sm, fr, sw.R[g][0], sw.R[g + 8][0], tab, A, lane, h1, h2);
 #pragma unroll
         for (int grp = 0; grp < 4; ++grp) {
 #pragma unroll
@@ -454,7 +451,7 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
               }
 #pragma unroll
               for (int e = 0; e < 2; ++e)
-                sw.G[g + 8 * r][8 * jj + 2 * t + e] = to_t(res + act(acc, 2 * r + e, L, sm.b3[8 * j + 2 * t + e], tab));
+                sw.G[g + 8 * r][8 * jj + 2 * t + e] = to_t(res + act(acc, 2 * r + e, sm.o3[8 * j + 2 * t + e], tab));
             }
           }
           __syncwarp();
@@ -607,8 +604,10 @@ __device__ __forceinline__ int exp_above(float v) {
 }
 __device__ __forceinline__ double pow2t(int e, double) { return dig::pow2d(e); }
 __device__ __forceinline__ float pow2t(int e, float) { return __int_as_float((127 + min(max(e, -126), 127)) << 23); }
+// 1 / c of a power of two c
+__device__ __forceinline__ float unit_inv(float c) { return __int_as_float((254 << 23) - __float_as_int(c)); }
 
-// Product value of element e times 2^sh (FP64: orders joined in units of 2^40; FP32: weights are 2^(18 - sw) times their digits).
+// Product value of element e (FP64: orders joined in units of 2^40; FP32: weights are 2^(18 - sw) times their digits).
 __device__ __forceinline__ double value(const float (*acc)[4], int e, double scale) {
   const dig::Pair64 p = dig::join(acc, e);
   return fma((double)p.hi, 4294967296.0, (double)p.lo) * scale;
@@ -686,7 +685,6 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
       const int cnt = a.nl_count[(size_t)i * a.ntypes + tj];
       const int nt = (cnt + 15) >> 4;
       const int pair = ti * a.ntypes + tj;
-      const PairScale ps = a.scale[pair];
       const PairSmall<T>& sm = a.small[pair];
       const uint4* fr = a.frag + (size_t)pair * kFrags * SetWords<T>::v;
       int first = (sub - q0) % a.sp;
@@ -727,7 +725,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
         V h1[kS1][2], h2[D ? kT2 : 1][2][2];
         uint4 Ar[D ? 1 : kK3 * ND];
         uint4* A = D ? sw.A : Ar;
-        layers12<T, ST>(sm, ps, fr, sw.x[g], sw.x[g + 8], tab, A, lane, h1, h2);
+        layers12<T, ST>(sm, fr, sw.x[g], sw.x[g + 8], tab, A, lane, h1, h2);
         T R[2][4], dR[2][4];
 #pragma unroll
         for (int r = 0; r < 2; ++r)
@@ -738,10 +736,8 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
           }
         // layer 3: G, dR_hat, dG, dz3 (digits), residual dG[m] + dG[m + 50]; then
         // dE/dh2 = residual + dz3 W3^T, dz2 = dE/dh2 (1 - t2^2), the residual part of dE/dh1
-        const auto L = layer(ps, 3, T(0));
-        const T sc3 = pow2t(ProdUnit<T>::v - ps.sw3, T(0));
         T dh1[kS1][2];
-        T dh2[D ? 1 : kT2][2][2];  // FP32: dE/dh2, then dz2
+        T dh2[D ? 1 : kT2][2][2];  // FP32: dE/dh2 in the units of dz3 W3^T, then dz2
         if constexpr (!D) {
 #pragma unroll
           for (int p = 0; p < kT2; ++p)
@@ -771,7 +767,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
             T sum = T(0);
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-              const V t3 = act(acc, 2 * r + e, L, sm.b3[8 * j + 2 * t + e], tab);
+              const V t3 = act(acc, 2 * r + e, sm.o3[8 * j + 2 * t + e], tab);
               const T G = to_t(res + t3);
               T dg = T(0);
 #pragma unroll
@@ -784,15 +780,15 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
             }
             if (j < 12) {
               if constexpr (D) sw.r[2 * j + r][lane] = sum;
-              else dh2[j >> 1][j & 1][r] += sum;
+              else dh2[j >> 1][j & 1][r] = fmaf(sum, unit_inv(sm.c3t[8 * (j >> 1) + 2 * t + (j & 1)]), dh2[j >> 1][j & 1][r]);
             } else {  // slot (6, 0) of lane 0 and, from lane 1, slot (6, 1)
               const T o = __shfl_sync(0xffffffffu, sum, (lane & ~3) + 1);
               if constexpr (D) {
                 sw.r[24 + r][lane] = t == 0 ? sum : T(0);
                 sw.r[26 + r][lane] = t == 0 ? o : T(0);
               } else {
-                dh2[kT2 - 1][0][r] += t == 0 ? sum : T(0);
-                dh2[kT2 - 1][1][r] += t == 0 ? o : T(0);
+                dh2[kT2 - 1][0][r] = fmaf(t == 0 ? sum : T(0), unit_inv(sm.c3t[8 * (kT2 - 1) + 2 * t]), dh2[kT2 - 1][0][r]);
+                dh2[kT2 - 1][1][r] = fmaf(t == 0 ? o : T(0), unit_inv(sm.c3t[8 * (kT2 - 1) + 2 * t + 1]), dh2[kT2 - 1][1][r]);
               }
             }
           }
@@ -815,7 +811,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
 #pragma unroll
               for (int e = 0; e < 2; ++e)
 #pragma unroll
-                for (int r = 0; r < 2; ++r) dh2[p][e][r] += value(acc, 2 * r + e, sc3);
+                for (int r = 0; r < 2; ++r) dh2[p][e][r] += dig::join_f(acc, 2 * r + e);
             }
           }
         }
@@ -830,9 +826,10 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
             dh1[p][r] = T(0);
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
+              const T c3 = sm.c3t[8 * p + 2 * t + e];
               T g2;
-              if constexpr (D) g2 = sw.r[4 * p + 2 * e + r][lane] + value(acc, 2 * r + e, sc3);
-              else g2 = dh2[p][e][r];
+              if constexpr (D) g2 = sw.r[4 * p + 2 * e + r][lane] + value(acc, 2 * r + e, c3);
+              else g2 = dh2[p][e][r] * c3;
               const T dz = times_sech2(g2, h2_of<T>(A, h2, p, e, r) - h1[p][r]);
               if constexpr (D) sw.r[4 * p + 2 * e + r][lane] = dz;
               else dh2[p][e][r] = dz;
@@ -874,7 +871,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
         {
           T sc[2];
 #pragma unroll
-          for (int r = 0; r < 2; ++r) sc[r] = pow2t(ProdUnit<T>::v - ps.sw2 - sd2[r], T(0));
+          for (int r = 0; r < 2; ++r) sc[r] = pow2t(-sd2[r], T(0));
 #pragma unroll
           for (int n = 0; n < kT2T; ++n) {
             float acc[Fmt<T>::NO][4];
@@ -883,10 +880,10 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
             for (int e = 0; e < 2; ++e) {
               const int p = 2 * n + e;
               if (p >= kS1) break;
-              const T w1 = sm.w1[4 * p + t];
+              const T w1 = sm.w1[4 * p + t], c2 = sm.c2t[4 * p + t];
 #pragma unroll
               for (int r = 0; r < 2; ++r) {
-                const T g1 = dh1[p][r] + value(acc, 2 * r + e, sc[r]);
+                const T g1 = dh1[p][r] + value(acc, 2 * r + e, c2 * sc[r]);
                 ds[r] = fma(times_sech2(g1, h1[p][r]), w1, ds[r]);
               }
             }
@@ -961,32 +958,34 @@ __global__ void __launch_bounds__(32) k_dig_weights(const T* __restrict__ theta,
   const int lane = threadIdx.x, t = lane & 3, n = lane >> 2;  // B fragment: k rows 2t.., column n
   const int f = blockIdx.x, pair = blockIdx.y;
   const T* W = theta + (size_t)pair * kEmbParams;
-  const PairScale ps = scale[pair];
+  const PairScale& ps = scale[pair];
   const int tc = n >> 1, ec = n & 1;  // column n = 2 tc + ec
   typename DigWord<T>::U u[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {  // the lane's four k rows: 2t, 2t + 1, 2t + 8, 2t + 9
     const int hi = k >> 1, par = k & 1;
     T v = T(0);
-    int sw = ps.sw3;
+    int sw = 0;
     if (f < kF3) {
       const int p = (f - kF2) / kK2, s = (f - kF2) % kK2;
       const int kk = 4 * (4 * s + 2 * hi + par) + t, m = unit2(p, tc, ec);
-      sw = ps.sw2;
+      if (m >= 0) sw = ps.sw2[m];
       if (kk < kN1 && m >= 0) v = W[kEW2 + kk * kN2 + m];
     } else if (f < kF3T) {
       const int j = (f - kF3) / kK3, s = (f - kF3) % kK3;
       const int m = 2 * s + hi < kT2 ? unit2(2 * s + hi, t, par) : -1, mo = unit3m(j, tc);
+      if (mo >= 0) sw = ps.sw3[mo + kN2 * ec];
       if (m >= 0 && mo >= 0) v = W[kEW3 + m * kN3 + mo + kN2 * ec];
     } else if (f < kF2T) {
       const int p = (f - kF3T) / kK3T, s = (f - kF3T) % kK3T;
       const int j = 2 * s + hi;
       const int mi = j < kT3 ? unit3m(j, t) : -1, m = unit2(p, tc, ec);
+      if (m >= 0) sw = ps.swt3[m];
       if (mi >= 0 && m >= 0) v = W[kEW3 + m * kN3 + mi + kN2 * par];
     } else {
       const int r = (f - kF2T) / kK2T, s = (f - kF2T) % kK2T;
       const int m = 2 * s + hi < kT2 ? unit2(2 * s + hi, t, par) : -1, k1 = 4 * (2 * r + ec) + tc;
-      sw = ps.sw2;
+      if (k1 < kN1) sw = ps.swt2[k1];
       if (m >= 0 && k1 < kN1) v = W[kEW2 + k1 * kN2 + m];
     }
     u[k] = weight_digits(v, sw, T(0));
@@ -1005,27 +1004,36 @@ __global__ void __launch_bounds__(32) k_dig_weights(const T* __restrict__ theta,
   }
 }
 
-__device__ __forceinline__ long long bias_v(double b, int zs) { return __double2ll_rn(b * dig::pow2d(zs)); }
-__device__ __forceinline__ float bias_v(float b, int) { return b; }
+__device__ __forceinline__ void set_out(Out<double>& o, double b, int, int zs, int s) {
+  o.b = __double2ll_rn(b * dig::pow2d(zs));
+  o.zs = zs;
+  o.s = s;
+}
+__device__ __forceinline__ void set_out(Out<float>& o, float b, int sw, int, int) {
+  o.b = b;
+  o.c = pow2t(18 - sw, 0.f);
+}
 
 template <class T>
 __global__ void __launch_bounds__(128) k_dig_small(const T* __restrict__ theta, const PairScale* scale, PairSmall<T>* out) {
   const int pair = blockIdx.x, q = threadIdx.x;
   const T* W = theta + (size_t)pair * kEmbParams;
-  const PairScale ps = scale[pair];
+  const PairScale& ps = scale[pair];
   PairSmall<T>& o = out[pair];
   if (q < 4 * kS1) {
     o.w1[q] = q < kN1 ? W[kEW1 + q] : T(0);
     o.b1[q] = q < kN1 ? W[kEb1 + q] : T(0);
+    o.c2t[q] = q < kN1 ? pow2t(ProdUnit<T>::v - ps.swt2[q], T(0)) : T(1);
   }
   const int t = (q & 7) >> 1, e = q & 1;
   if (q < 8 * kT2) {
-    const int m = unit2(q >> 3, t, e);
-    o.b2[q] = m >= 0 ? bias_v(W[kEb2 + m], ps.zs2) : 0;
+    const int m = unit2(q >> 3, t, e), k = max(m, 0);  // no unit: zero digits, the scale of unit 0
+    set_out(o.o2[q], m >= 0 ? W[kEb2 + m] : T(0), ps.sw2[k], ps.zs2[k], ps.s2[k]);
+    o.c3t[q] = m >= 0 ? pow2t(ProdUnit<T>::v - ps.swt3[m], T(0)) : T(1);
   }
   if (q < 8 * kT3) {
-    const int m = unit3m(q >> 3, t);
-    o.b3[q] = m >= 0 ? bias_v(W[kEb3 + m + kN2 * e], ps.zs3) : 0;
+    const int m = unit3m(q >> 3, t), k = m >= 0 ? m + kN2 * e : 0;
+    set_out(o.o3[q], m >= 0 ? W[kEb3 + k] : T(0), ps.sw3[k], ps.zs3[k], ps.s3[k]);
   }
 }
 
@@ -1036,33 +1044,43 @@ int ceil_log2(double v) {
   return f == 0.5 ? e - 1 : e;
 }
 
-// Scales of one layer (K x N weights W, biases b, |inputs| <= in, activation scale 2^sh); false when the
-// weights are outside the range the fixed-point layer covers (or not finite).
-bool layer_scale(const double* W, const double* b, int K, int N, double in, bool fp64, int bits, int sh, int* sw, int* zs,
-                 int* s) {
-  double top = 0.0, bound = 0.0;
+// 2^sw times weights of at most `top`: half of the digits' range (FP64), 2^26 (1 - 2^-8) of 2^26 (FP32).
+int digit_scale(double top, bool fp64, int lowest) {
+  const int e = top > 0.0 ? std::max(ceil_log2(fp64 ? top : top * (1.0 + 1.0 / 128)), lowest) : 0;
+  return (fp64 ? Fmt<double>::BD * Fmt<double>::ND - 2 : Fmt<float>::BD * Fmt<float>::ND - 1) - e;
+}
+
+// Scales of one layer (K x N weights W, biases b, |inputs| <= in, FP64 activations with sh fraction bits): sw, zs and s
+// of every column, swt of every row; false when the weights are outside the range the fixed-point layer covers
+// (or not finite).
+bool layer_scale(const double* W, const double* b, int K, int N, double in, bool fp64, int sh, int* sw, int* zs, int* s,
+                 int* swt) {
+  std::vector<double> row(K, 0.0);
   for (int n = 0; n < N; ++n) {
-    double sum = std::fabs(b[n]);
+    double top = 0.0, sum = std::fabs(b[n]);
     for (int k = 0; k < K; ++k) {
       const double v = std::fabs(W[(size_t)k * N + n]);
       if (!(v <= 65536.0)) return false;
       top = std::fmax(top, v);
+      row[k] = std::fmax(row[k], v);
       sum += in * v;
     }
     if (!(sum <= 1048576.0)) return false;
-    bound = std::fmax(bound, sum);
+    sw[n] = digit_scale(top, fp64, fp64 ? -12 : -100);
+    zs[n] = std::min(52, 60 - (sum > 1.0 ? ceil_log2(sum) : 0));
+    s[n] = 72 + zs[n] - sh - sw[n];
+    if (fp64 && s[n] > 31) {  // large weights: fewer fraction bits in z
+      zs[n] -= s[n] - 31;
+      s[n] = 31;
+    }
+    if (fp64 && (s[n] < 1 || zs[n] < 40)) return false;
   }
-  // FP32 uses the digits' whole range: |W| 2^sw <= 2^26 (1 - 2^-8)
-  const int e = top > 0.0 ? std::max(ceil_log2(fp64 ? top : top * (1.0 + 1.0 / 128)), -12) : 0;
-  *sw = bits - (fp64 ? 2 : 1) - e;
-  *zs = std::min(52, 60 - (bound > 1.0 ? ceil_log2(bound) : 0));
-  *s = 72 + *zs - sh - *sw;
-  if (fp64 && *s > 31) {  // a wide weight range: fewer fraction bits in z
-    *zs -= *s - 31;
-    *s = 31;
-  }
-  return !fp64 || (*s >= 1 && *zs >= 40);
+  for (int k = 0; k < K; ++k) swt[k] = digit_scale(row[k], fp64, -100);
+  return true;
 }
+
+// A pair's scales stand before its constants and fragments.
+size_t scale_bytes(int npairs) { return (sizeof(PairScale) * npairs + 255) / 256 * 256; }
 
 template <class T>
 dp_status upload(Model* m) {
@@ -1073,17 +1091,17 @@ dp_status upload(Model* m) {
   m->dig_ok = true;
   for (int p = 0; p < np; ++p) {
     const double* W = m->theta_host.data() + (size_t)p * kEmbParams;
-    const bool ok2 = layer_scale(W + kEW2, W + kEb2, kN1, kN2, 1.0, d, bits, bits - 2, &sc[p].sw2, &sc[p].zs2, &sc[p].s2);
-    const bool ok3 = layer_scale(W + kEW3, W + kEb3, kN2, kN3, 2.0, d, bits, bits - 3, &sc[p].sw3, &sc[p].zs3, &sc[p].s3);
-    m->dig_ok = m->dig_ok && ok2 && ok3;
+    PairScale& q = sc[p];
+    m->dig_ok = m->dig_ok && layer_scale(W + kEW2, W + kEb2, kN1, kN2, 1.0, d, bits - 2, q.sw2, q.zs2, q.s2, q.swt2) &&
+                layer_scale(W + kEW3, W + kEb3, kN2, kN3, 2.0, d, bits - 3, q.sw3, q.zs3, q.s3, q.swt3);
   }
   if (!m->dig_ok) return DP_OK;
   unsigned char* base = static_cast<unsigned char*>(m->dig_emb);
   PairScale* dsc = reinterpret_cast<PairScale*>(base);
   DP_CUDA_TRY(m, cudaMemcpy(dsc, sc.data(), sizeof(PairScale) * np, cudaMemcpyHostToDevice));
   const T* th = sizeof(T) == 8 ? reinterpret_cast<const T*>(m->w64) : reinterpret_cast<const T*>(m->w32);
-  PairSmall<T>* sm = reinterpret_cast<PairSmall<T>*>(base + 1024);
-  uint4* fr = reinterpret_cast<uint4*>(base + 1024 + sizeof(PairSmall<T>) * np);
+  PairSmall<T>* sm = reinterpret_cast<PairSmall<T>*>(base + scale_bytes(np));
+  uint4* fr = reinterpret_cast<uint4*>(base + scale_bytes(np) + sizeof(PairSmall<T>) * np);
   k_dig_weights<T><<<dim3(kFrags, np), 32>>>(th, dsc, fr);
   k_dig_small<T><<<np, 128>>>(th, dsc, sm);
   m->launches += 2;
@@ -1100,9 +1118,8 @@ DigArgs<T> make_args(Model* m, int N) {
   a.rc = (T)m->rc; a.rs = (T)m->rs; a.winv = (T)(1.0 / (m->rc - m->rs)); a.switch_kind = m->switch_kind;
   a.stat = sizeof(T) == 8 ? reinterpret_cast<const T*>(m->stat64) : reinterpret_cast<const T*>(m->stat32);
   unsigned char* base = static_cast<unsigned char*>(m->dig_emb);
-  a.scale = reinterpret_cast<const PairScale*>(base);
-  a.small = reinterpret_cast<const PairSmall<T>*>(base + 1024);
-  a.frag = reinterpret_cast<const uint4*>(base + 1024 + sizeof(PairSmall<T>) * np);
+  a.small = reinterpret_cast<const PairSmall<T>*>(base + scale_bytes(np));
+  a.frag = reinterpret_cast<const uint4*>(base + scale_bytes(np) + sizeof(PairSmall<T>) * np);
   a.tab = static_cast<const dig::TanhTab*>(m->dig_tanh);
   a.itype = m->itype; a.nl_j = m->nl_j; a.nl_d = m->nl_d; a.nl_count = m->nl_count;
   a.Tm = static_cast<T*>(m->Tm);
@@ -1181,8 +1198,8 @@ dp_status backward(Model* m, int N) {
 
 size_t dig_emb_bytes(int ntypes, bool fp64) {
   const size_t np = (size_t)ntypes * ntypes;
-  return fp64 ? 1024 + np * (sizeof(PairSmall<double>) + (size_t)kFrags * SetWords<double>::v * 16)
-              : 1024 + np * (sizeof(PairSmall<float>) + (size_t)kFrags * SetWords<float>::v * 16);
+  return scale_bytes((int)np) + np * (fp64 ? sizeof(PairSmall<double>) + (size_t)kFrags * SetWords<double>::v * 16
+                                           : sizeof(PairSmall<float>) + (size_t)kFrags * SetWords<float>::v * 16);
 }
 size_t dig_tanh_bytes() { return sizeof(dig::TanhTab); }
 

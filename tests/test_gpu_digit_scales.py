@@ -1,0 +1,56 @@
+"""FP64 / FP32 nets whose weights or activations spread widely, against the FP64 oracle (GPU only).
+
+The digit products hold every operand relative to a scale, so what a scale covers (a column of weights, a row of
+activations) decides how many bits the small values keep.  Bars as for evenly scaled nets, from the arithmetic.
+FP32: about 100 terms a sum at 6e-8 each, 6e-6 on energies, with a factor of ten for the forces' cancellation.
+FP64: 1.1e-16 a rounding, sums of up to 1,600 terms (a random walk of 40) on both sides: 2e-14 on energies,
+a factor of ten for the forces."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2410_22867_gb300 import synth
+
+from _parity import errors
+from test_gpu_digits import _cluster
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+BARS = {"fp64": (2e-14, 2e-13), "fp32": (6e-6, 6e-5)}
+
+
+def _pairs():
+    return [(ti, tj) for ti in range(2) for tj in range(2)]
+
+
+def _check(w, prec, n=66, seed=66):
+    import paper_2410_22867_gb300 as dp
+    x, t, box = _cluster(n, seed)
+    ref = oracle.Model(w.to_blob()).compute(x, t, box)
+    m = dp.DPModel(w, prec, max_atoms=n)
+    e = errors(m.compute(torch.tensor(x, device="cuda"), torch.tensor(t, device="cuda"), box), ref, t)
+    m.close()
+    assert e["ei_rel"] <= BARS[prec][0] and e["f_rel"] <= BARS[prec][1], e
+
+
+def _outlier(layer, value):
+    """One weight of W2 or W3 of every pair far above the others.  Its input (unit 3) is a constant, so that its
+    output is saturated and the other columns decide the result; columns 9 are far below the others."""
+    w = synth.xavier_weights(("O", "H"), 6.0, 0.5, (46, 92), 1001)
+    for ti, tj in _pairs():
+        b = {k: w.block(f"emb{ti}{tj}.{k}") for k in ("W1", "b1", "W2", "b2", "W3", "b3")}
+        b["W1"][0, 3], b["b1"][3] = 0.0, 1.0
+        b["W2"][:, 3], b["b2"][3] = 0.0, 1.0
+        b["W2"][:, 9] *= 1e-6
+        b["W3"][:, 9] *= 1e-6
+        b[layer][3, 7] = value
+    return w
+
+
+# 65,535 and 65,600: just inside and just outside what the fixed-point layers take
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("layer", ["W2", "W3"])
+@pytest.mark.parametrize("value", [100.0, 16384.0, 65535.0, 65600.0])
+def test_one_large_embedding_weight(prec, layer, value):
+    _check(_outlier(layer, value), prec)
