@@ -81,12 +81,11 @@ __device__ __forceinline__ void split2(unsigned long long u0, unsigned long long
   out[5] = bytes_to_half2(__byte_perm(l0, l1, 0x0501));
   out[6] = bytes_to_half2(__byte_perm(l0, l1, 0x0400));
 }
-// FP32: x as three fp16 numbers that carry their own weights: the nearest multiples of 2^-G and of 2^-(G+9) of what
-// is left (nine bits each, by adding and subtracting 1.5 x 2^23 times the step), and the rest.  Subnormal
-// fp16 is exact in the products.  Five additions a value, where integer digits took ten instructions.
-template <int G>
+// FP32: |x| <= 256 as three fp16 numbers that carry their own weights: the nearest integer, the nearest multiple of 2^-9 of
+// what is left (nine bits each, by adding and subtracting 1.5 x 2^23 times the step), and the rest, which is
+// below 2^-10 and kept within 2^-22.  Five additions a value, where integer digits took ten instructions.
 __device__ __forceinline__ void split2f(float x0, float x1, uint32_t* out) {
-  constexpr float m0 = 12582912.f / (float)(1 << G), m1 = m0 / 512.f;
+  constexpr float m0 = 12582912.f, m1 = m0 / 512.f;
   const float a0 = __fsub_rn(__fadd_rn(x0, m0), m0), a1 = __fsub_rn(__fadd_rn(x1, m0), m0);
   const float r0 = __fsub_rn(x0, a0), r1 = __fsub_rn(x1, a1);
   const float b0 = __fsub_rn(__fadd_rn(r0, m1), m1), b1 = __fsub_rn(__fadd_rn(r1, m1), m1);

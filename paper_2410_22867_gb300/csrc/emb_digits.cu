@@ -137,6 +137,20 @@ __device__ __forceinline__ void env_row(const DigArgs<T>& a, int ti, Env<T>& v) 
   for (int c = 0; c < 4; ++c) v.R[c] = (v.R[c] - a.stat[ti * 4 + c]) * a.stat[(a.ntypes + ti) * 4 + c];
 }
 
+// Exponent e with |v| <= 2^e (v finite), from the bits; zero and tiny values give the lower limit.
+__device__ __forceinline__ int exp_above(double v) {
+  const int e = (__double2hiint(v) >> 20) & 0x7ff;
+  return max(e - 1022, -800);
+}
+__device__ __forceinline__ int exp_above(float v) {
+  const int e = (__float_as_int(v) >> 23) & 0xff;
+  return max(e - 126, -80);
+}
+__device__ __forceinline__ double pow2t(int e, double) { return dig::pow2d(e); }
+__device__ __forceinline__ float pow2t(int e, float) { return __int_as_float((127 + min(max(e, -126), 127)) << 23); }
+// 1 / c of a power of two c
+__device__ __forceinline__ float unit_inv(float c) { return __int_as_float((254 << 23) - __float_as_int(c)); }
+
 // ------------------------------------------------------------------ activations of either type
 // FP64: fixed point with 54 fraction bits; FP32: floats.
 __device__ __forceinline__ long long act1(double x, double w, double b, const dig::TanhTab* tab) {
@@ -144,45 +158,42 @@ __device__ __forceinline__ long long act1(double x, double w, double b, const di
 }
 __device__ __forceinline__ float act1(float x, float w, float b, const dig::TanhTab*) { return tanhf(fmaf(x, w, b)); }
 
-// tanh of element e's output.
-__device__ __forceinline__ long long act(const float (*acc)[4], int e, const Out<double>& o, const dig::TanhTab* tab) {
+// tanh of element e's output; u: the unit of the row's digits (FP32).
+__device__ __forceinline__ long long act(const float (*acc)[4], int e, const Out<double>& o, double, const dig::TanhTab* tab) {
   const dig::Pair64 p = dig::join(acc, e);
   const int r = 32 - o.s;
   const long long z = (p.hi << o.s) + ((p.lo + ((1ll << r) >> 1)) >> r) + o.b;
   return dig::tanh_fixed(z, o.zs, tab);
 }
-__device__ __forceinline__ float act(const float (*acc)[4], int e, const Out<float>& o, const dig::TanhTab*) {
-  return tanhf(fmaf(dig::join_f(acc, e), o.c, o.b));
+__device__ __forceinline__ float act(const float (*acc)[4], int e, const Out<float>& o, float u, const dig::TanhTab*) {
+  return tanhf(fmaf(dig::join_f(acc, e), o.c * u, o.b));
 }
 
-// The biased digits of activations: h1 (|h1| <= 1) and h2 (|h2| <= 2).
-__device__ __forceinline__ unsigned long long dig_h1(long long h) { return dig::biased(h); }
-__device__ __forceinline__ unsigned long long dig_h2(long long h) { return dig::biased((h + 1) >> 1); }
-__device__ __forceinline__ float dig_h1(float h) { return h; }  // FP32 splits the value itself
-__device__ __forceinline__ float dig_h2(float h) { return h; }
+// The biased digits of activations: h1 (|h1| <= 1) and h2 (|h2| <= 2); FP32: the value times f, below 256.
+__device__ __forceinline__ unsigned long long dig_h1(long long h, double) { return dig::biased(h); }
+__device__ __forceinline__ unsigned long long dig_h2(long long h, double) { return dig::biased((h + 1) >> 1); }
+__device__ __forceinline__ float dig_h1(float h, float f) { return h * f; }
+__device__ __forceinline__ float dig_h2(float h, float f) { return h * f; }
 __device__ __forceinline__ unsigned long long dig_of(double v) { return dig::biased(__double2ll_rn(v)); }
 __device__ __forceinline__ float dig_of(float v) { return v; }
 
 template <class T> struct DigWord;
 template <> struct DigWord<double> { using U = unsigned long long; };
 template <> struct DigWord<float> { using U = float; };
-// G: fraction bits of the leading FP32 digit, 7 for activations (|h| <= 2), 0 for gradients scaled below 256
-template <int G>
 __device__ __forceinline__ void split2(unsigned long long u0, unsigned long long u1, uint32_t* out) { dig::split2(u0, u1, out); }
-template <int G>
-__device__ __forceinline__ void split2(float u0, float u1, uint32_t* out) { dig::split2f<G>(u0, u1, out); }
+__device__ __forceinline__ void split2(float u0, float u1, uint32_t* out) { dig::split2f(u0, u1, out); }
 
 // A fragment of one k step (all digits) from the lane's four slots of rows g (u[0]) and g + 8 (u[1]); only the
 // first two slots unless `full`.
-template <class T, int G>
+template <class T>
 __device__ __forceinline__ void get_a(uint4* a, const typename DigWord<T>::U (*u)[4], bool full) {
   constexpr int ND = Fmt<T>::ND;
   uint32_t x[ND], y[ND], z[ND], w[ND];
-  split2<G>(u[0][0], u[0][1], x);
-  split2<G>(u[1][0], u[1][1], y);
+  split2(u[0][0], u[0][1], x);
+  split2(u[1][0], u[1][1], y);
   if (full) {
-    split2<G>(u[0][2], u[0][3], z);
-    split2<G>(u[1][2], u[1][3], w);
+    split2(u[0][2], u[0][3], z);
+    split2(u[1][2], u[1][3], w);
   }
 #pragma unroll
   for (int i = 0; i < ND; ++i) a[i] = make_uint4(x[i], y[i], full ? z[i] : 0u, full ? w[i] : 0u);
@@ -226,7 +237,7 @@ __device__ __forceinline__ void product(float (*acc)[4], const uint4* A, const u
         u[0][q] = ((unsigned long long)w.y << 32) | w.x;
         u[1][q] = ((unsigned long long)w.w << 32) | w.z;
       }
-      get_a<T, 0>(a, u, !tail);
+      get_a<T>(a, u, !tail);
     } else if constexpr (ST == kDigits) {
 #pragma unroll
       for (int i = 0; i < ND; ++i) {
@@ -254,7 +265,7 @@ __device__ __forceinline__ void product(float (*acc)[4], const uint4* A, const u
   }
 }
 // A of k step s into its store.
-template <class T, int G, Store ST>
+template <class T, Store ST>
 __device__ __forceinline__ void put_a(uint4* A, int s, bool full, int lane, const typename DigWord<T>::U (*u)[4]) {
   constexpr int ND = Fmt<T>::ND;
   if constexpr (ST == kWords) {
@@ -265,18 +276,19 @@ __device__ __forceinline__ void put_a(uint4* A, int s, bool full, int lane, cons
                                                 (uint32_t)(u[1][q] >> 32));
   } else if constexpr (ST == kDigits) {
     uint4 a[ND];
-    get_a<T, G>(a, u, full);
+    get_a<T>(a, u, full);
 #pragma unroll
     for (int i = 0; i < ND; ++i) {
       if (full) A[(s * ND + i) * 32 + lane] = a[i];
       else reinterpret_cast<uint2*>(A + s * ND * 32)[i * 32 + lane] = make_uint2(a[i].x, a[i].y);
     }
   } else {
-    get_a<T, G>(A + s * ND, u, full);
+    get_a<T>(A + s * ND, u, full);
   }
 }
-// FP32: the activation of h2 slot (p, e), row r, back from the digits in registers (24 bits and more).
-__device__ __forceinline__ float from_digits(const uint4* A, int p, int e, int r) {
+// FP32: the activation of h2 slot (p, e), row r, back from the digits in registers (their unit is u): within 2^-30 of the
+// row's largest.
+__device__ __forceinline__ float from_digits(const uint4* A, int p, int e, int r, float u) {
   constexpr int ND = Fmt<float>::ND;
   float v = 0.f;
 #pragma unroll
@@ -286,15 +298,32 @@ __device__ __forceinline__ float from_digits(const uint4* A, int p, int e, int r
     const __half2 x = *reinterpret_cast<const __half2*>(&h);
     v += e ? __high2float(x) : __low2float(x);
   }
-  return v;
+  return v * u;
+}
+
+// FP32: the digits of a tile's rows (g: r = 0, g + 8: r = 1) are relative to the row's largest activation: f = 2^(8 - e),
+// u = 1 / f with |h| <= 2^e in the lane's slots and, by shuffles, those of the row's other three lanes.  With a fixed
+// range a net whose activations are small lost bits (|h| ~ 1e-4: G 2e-4 off; now 8e-8, FMAs 1e-7).
+template <int M>
+__device__ __forceinline__ void row_scale(const float (*h)[2], float* f, float* u) {
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    float top = fabsf(h[0][r]);
+#pragma unroll
+    for (int p = 1; p < M; ++p) top = fmaxf(top, fabsf(h[p][r]));
+    top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 1));
+    top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 2));
+    f[r] = pow2t(8 - exp_above(top), 0.f);
+    u[r] = unit_inv(f[r]);
+  }
 }
 
 // Layers 1 and 2 of a tile: h1 [slot][row], h2 [n-tile][e][row] (rows g, g + 8; FP64), and the digits of h2
-// in A (shared memory, FP64) or A (registers, FP32, which takes h2 back from them).
+// in A (shared memory, FP64) or A (registers, FP32, which takes h2 back from them) with their units uh (FP32).
 template <class T, Store ST>
 __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const uint4* __restrict__ fr,
                                          T x0, T x1, const dig::TanhTab* tab, uint4* A, int lane,
-                                         typename Fmt<T>::V (*h1)[2], typename Fmt<T>::V (*h2)[2][2]) {
+                                         typename Fmt<T>::V (*h1)[2], typename Fmt<T>::V (*h2)[2][2], T* uh) {
   constexpr int ND = Fmt<T>::ND;
   constexpr bool D = sizeof(T) == 8;
   using V = typename Fmt<T>::V;
@@ -306,6 +335,8 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const uint4* __
     h1[p][0] = act1(x0, w, b, tab);
     h1[p][1] = act1(x1, w, b, tab);
   }
+  T f[2] = {T(1), T(1)}, u1[2] = {T(1), T(1)};
+  if constexpr (!D) row_scale<kS1>(h1, f, u1);
   uint4 A1r[D ? 1 : kK2 * ND];
   uint4* A1 = D ? A : A1r;
 #pragma unroll
@@ -314,11 +345,12 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const uint4* __
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-      for (int r = 0; r < 2; ++r) u[r][q] = 4 * s + q < kS1 ? dig_h1(h1[4 * s + q < kS1 ? 4 * s + q : 0][r]) : dig_h1(V(0));
-    put_a<T, 7, ST>(A1, s, true, lane, u);
+      for (int r = 0; r < 2; ++r) u[r][q] = 4 * s + q < kS1 ? dig_h1(h1[4 * s + q < kS1 ? 4 * s + q : 0][r], f[r]) : dig_h1(V(0), f[r]);
+    put_a<T, ST>(A1, s, true, lane, u);
   }
   if (D) __syncwarp();
   U u[2][4];
+  V hf[D ? 1 : 2 * kT2][2];  // FP32: h2, until the row's largest is known
 #pragma unroll
   for (int p = 0; p < kT2; ++p) {
     float acc[Fmt<T>::NO][4];
@@ -328,15 +360,23 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const uint4* __
       const Out<T> o = sm.o2[8 * p + 2 * t + e];
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const V h = h1[p][r] + act(acc, 2 * r + e, o, tab);
+        const V h = h1[p][r] + act(acc, 2 * r + e, o, u1[r], tab);
         if constexpr (D) h2[p][e][r] = h;
-        else u[r][2 * (p & 1) + e] = dig_h2(h);
+        else hf[2 * p + e][r] = h;
       }
     }
-    if constexpr (!D)
-      if ((p & 1) || p == kT2 - 1) put_a<T, 7, ST>(A, p >> 1, p & 1, lane, u);
   }
-  if constexpr (D) {
+  if constexpr (!D) {
+    row_scale<2 * kT2>(hf, f, uh);
+#pragma unroll
+    for (int p = 0; p < kT2; ++p) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) u[r][2 * (p & 1) + e] = dig_h2(hf[2 * p + e][r], f[r]);
+      if ((p & 1) || p == kT2 - 1) put_a<T, ST>(A, p >> 1, p & 1, lane, u);
+    }
+  } else {
     __syncwarp();
 #pragma unroll
     for (int s = 0; s < kK3; ++s) {
@@ -345,17 +385,17 @@ __device__ __forceinline__ void layers12(const PairSmall<T>& sm, const uint4* __
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           const int p = 2 * s + (q >> 1);
-          u[r][q] = p < kT2 ? dig_h2(h2[p < kT2 ? p : 0][q & 1][r]) : dig_h2(V(0));
+          u[r][q] = p < kT2 ? dig_h2(h2[p < kT2 ? p : 0][q & 1][r], f[r]) : dig_h2(V(0), f[r]);
         }
-      put_a<T, 7, ST>(A, s, s + 1 < kK3, lane, u);
+      put_a<T, ST>(A, s, s + 1 < kK3, lane, u);
     }
     __syncwarp();
   }
 }
 template <class T>
-__device__ __forceinline__ typename Fmt<T>::V h2_of(const uint4* A, const typename Fmt<T>::V (*h2)[2][2], int p, int e, int r) {
+__device__ __forceinline__ typename Fmt<T>::V h2_of(const uint4* A, const typename Fmt<T>::V (*h2)[2][2], int p, int e, int r, const T* uh) {
   if constexpr (sizeof(T) == 8) return h2[p][e][r];
-  else return from_digits(A, p, e, r);
+  else return from_digits(A, p, e, r, uh[r]);
 }
 
 __device__ __forceinline__ double to_t(long long v) { return (double)v; }  // times 2^-54 later
@@ -431,7 +471,8 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
         V h1[kS1][2], h2[D ? kT2 : 1][2][2];
         uint4 Ar[D ? 1 : kK3 * Fmt<T>::ND];
         uint4* A = D ? sw.A : Ar;
-        layers12<T, ST>(sm, fr, sw.R[g][0], sw.R[g + 8][0], tab, A, lane, h1, h2);
+        T uh[2] = {T(1), T(1)};
+        layers12<T, ST>(sm, fr, sw.R[g][0], sw.R[g + 8][0], tab, A, lane, h1, h2, uh);
 #pragma unroll
         for (int grp = 0; grp < 4; ++grp) {
 #pragma unroll
@@ -444,14 +485,14 @@ __global__ void __launch_bounds__(32 * FwdWarps<T>::v, 1) k_dig_fwd(DigArgs<T> a
             for (int r = 0; r < 2; ++r) {
               V res;
               if (j < 12) {
-                res = h2_of<T>(A, h2, j < 12 ? j >> 1 : 0, j & 1, r);
+                res = h2_of<T>(A, h2, j < 12 ? j >> 1 : 0, j & 1, r, uh);
               } else {  // unit 24 (lane 0 of the quad, its own) and unit 49 (held by lane 0, used by lane 1)
-                const V o = __shfl_sync(0xffffffffu, h2_of<T>(A, h2, 6, 1, r), lane & ~3);
-                res = t == 0 ? h2_of<T>(A, h2, 6, 0, r) : o;
+                const V o = __shfl_sync(0xffffffffu, h2_of<T>(A, h2, 6, 1, r, uh), lane & ~3);
+                res = t == 0 ? h2_of<T>(A, h2, 6, 0, r, uh) : o;
               }
 #pragma unroll
               for (int e = 0; e < 2; ++e)
-                sw.G[g + 8 * r][8 * jj + 2 * t + e] = to_t(res + act(acc, 2 * r + e, sm.o3[8 * j + 2 * t + e], tab));
+                sw.G[g + 8 * r][8 * jj + 2 * t + e] = to_t(res + act(acc, 2 * r + e, sm.o3[8 * j + 2 * t + e], uh[r], tab));
             }
           }
           __syncwarp();
@@ -593,20 +634,6 @@ struct BwdWarp {
 // 2,331 water atoms 325 and 282 us.
 constexpr int kBwdWarps64 = 6, kBwdWarps32 = 12, kBwdWarps32Types = 16;
 
-// Exponent e with |v| <= 2^e (v finite), from the bits; zero and tiny values give the lower limit.
-__device__ __forceinline__ int exp_above(double v) {
-  const int e = (__double2hiint(v) >> 20) & 0x7ff;
-  return max(e - 1022, -800);
-}
-__device__ __forceinline__ int exp_above(float v) {
-  const int e = (__float_as_int(v) >> 23) & 0xff;
-  return max(e - 126, -80);
-}
-__device__ __forceinline__ double pow2t(int e, double) { return dig::pow2d(e); }
-__device__ __forceinline__ float pow2t(int e, float) { return __int_as_float((127 + min(max(e, -126), 127)) << 23); }
-// 1 / c of a power of two c
-__device__ __forceinline__ float unit_inv(float c) { return __int_as_float((254 << 23) - __float_as_int(c)); }
-
 // Product value of element e (FP64: orders joined in units of 2^40; FP32: weights are 2^(18 - sw) times their digits).
 __device__ __forceinline__ double value(const float (*acc)[4], int e, double scale) {
   const dig::Pair64 p = dig::join(acc, e);
@@ -725,7 +752,8 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
         V h1[kS1][2], h2[D ? kT2 : 1][2][2];
         uint4 Ar[D ? 1 : kK3 * ND];
         uint4* A = D ? sw.A : Ar;
-        layers12<T, ST>(sm, fr, sw.x[g], sw.x[g + 8], tab, A, lane, h1, h2);
+        T uh[2] = {T(1), T(1)};
+        layers12<T, ST>(sm, fr, sw.x[g], sw.x[g + 8], tab, A, lane, h1, h2, uh);
         T R[2][4], dR[2][4];
 #pragma unroll
         for (int r = 0; r < 2; ++r)
@@ -759,15 +787,15 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
           for (int r = 0; r < 2; ++r) {
             V res;
             if (j < 12) {
-              res = h2_of<T>(A, h2, j < 12 ? j >> 1 : 0, j & 1, r);
+              res = h2_of<T>(A, h2, j < 12 ? j >> 1 : 0, j & 1, r, uh);
             } else {
-              const V o = __shfl_sync(0xffffffffu, h2_of<T>(A, h2, 6, 1, r), lane & ~3);
-              res = t == 0 ? h2_of<T>(A, h2, 6, 0, r) : o;
+              const V o = __shfl_sync(0xffffffffu, h2_of<T>(A, h2, 6, 1, r, uh), lane & ~3);
+              res = t == 0 ? h2_of<T>(A, h2, 6, 0, r, uh) : o;
             }
             T sum = T(0);
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-              const V t3 = act(acc, 2 * r + e, sm.o3[8 * j + 2 * t + e], tab);
+              const V t3 = act(acc, 2 * r + e, sm.o3[8 * j + 2 * t + e], uh[r], tab);
               const T G = to_t(res + t3);
               T dg = T(0);
 #pragma unroll
@@ -793,10 +821,10 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
             }
           }
           if constexpr (D) {
-            if ((j & 1) || j == kT3 - 1) put_a<T, 0, ST>(sw.Z, j >> 1, j & 1, lane, u);
+            if ((j & 1) || j == kT3 - 1) put_a<T, ST>(sw.Z, j >> 1, j & 1, lane, u);
           } else if ((j & 1) || j == kT3 - 1) {  // this k step against every n-tile of W3^T
             uint4 za[ND];
-            get_a<T, 0>(za, u, j & 1);
+            get_a<T>(za, u, j & 1);
 #pragma unroll
             for (int p = 0; p < kT3T; ++p) {
               const uint4* set = fr + (size_t)(kF3T + p * kK3T + (j >> 1)) * SetWords<T>::v;
@@ -830,7 +858,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
               T g2;
               if constexpr (D) g2 = sw.r[4 * p + 2 * e + r][lane] + value(acc, 2 * r + e, c3);
               else g2 = dh2[p][e][r] * c3;
-              const T dz = times_sech2(g2, h2_of<T>(A, h2, p, e, r) - h1[p][r]);
+              const T dz = times_sech2(g2, h2_of<T>(A, h2, p, e, r, uh) - h1[p][r]);
               if constexpr (D) sw.r[4 * p + 2 * e + r][lane] = dz;
               else dh2[p][e][r] = dz;
               top[r] = fmax(top[r], fabs(dz));
@@ -862,7 +890,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
                 }
                 z[r][q] = dig_of(v * f[r]);
               }
-            put_a<T, 0, ST>(A, s, s + 1 < kK2T, lane, z);  // the digits of h2 are no longer needed
+            put_a<T, ST>(A, s, s + 1 < kK2T, lane, z);  // the digits of h2 are no longer needed
           }
         }
         __syncwarp();
@@ -992,8 +1020,8 @@ __global__ void __launch_bounds__(32) k_dig_weights(const T* __restrict__ theta,
   }
   uint32_t lo[2 * Q], hi[2 * Q];
   lo[2 * Q - 1] = hi[2 * Q - 1] = 0u;  // an odd number of digits
-  split2<0>(u[0], u[1], lo);
-  split2<0>(u[2], u[3], hi);
+  split2(u[0], u[1], lo);
+  split2(u[2], u[3], hi);
   uint4* dst = frag + ((size_t)pair * kFrags + f) * SetWords<T>::v;
   if constexpr (sizeof(T) == 8) {
 #pragma unroll

@@ -92,7 +92,7 @@ __device__ __forceinline__ float fix_digits(float v, int e) {  // below 256
   return v * __int_as_float((127 + min(8 - e, 127)) << 23);
 }
 __device__ __forceinline__ void split2(unsigned long long u0, unsigned long long u1, uint32_t* out) { dig::split2(u0, u1, out); }
-__device__ __forceinline__ void split2(float u0, float u1, uint32_t* out) { dig::split2f<0>(u0, u1, out); }
+__device__ __forceinline__ void split2(float u0, float u1, uint32_t* out) { dig::split2f(u0, u1, out); }
 
 __device__ __forceinline__ void load4(const double* p, double* v) {
   const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);

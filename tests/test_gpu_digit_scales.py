@@ -54,3 +54,21 @@ def _outlier(layer, value):
 @pytest.mark.parametrize("value", [100.0, 16384.0, 65535.0, 65600.0])
 def test_one_large_embedding_weight(prec, layer, value):
     _check(_outlier(layer, value), prec)
+
+
+def _small(w1, fit):
+    """Activations of about w1 times the input in every row: no embedding biases, small first-layer weights; the fitting
+    nets' first layer scaled to match."""
+    w = synth.xavier_weights(("O", "H"), 6.0, 0.5, (46, 92), 1001)
+    for ti, tj in _pairs():
+        w.block(f"emb{ti}{tj}.W1")[...] *= w1
+        for k in ("b1", "b2", "b3"):
+            w.block(f"emb{ti}{tj}.{k}")[...] = 0.0
+    for t in range(2):
+        w.block(f"fit{t}.W1")[...] *= fit
+    return w
+
+
+@pytest.mark.parametrize("w1,fit", [(0.1, 1e3), (1e-2, 1e5), (1e-4, 1e9)])
+def test_small_activations_fp32(w1, fit):
+    _check(_small(w1, fit), "fp32")
