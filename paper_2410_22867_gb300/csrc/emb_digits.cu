@@ -154,7 +154,7 @@ __device__ __forceinline__ float unit_inv(float c) { return __int_as_float((254 
 // ------------------------------------------------------------------ activations of either type
 // FP64: fixed point with 54 fraction bits; FP32: floats.
 __device__ __forceinline__ long long act1(double x, double w, double b, const dig::TanhTab* tab) {
-  return dig::tanh_fixed(__double2ll_rn(fma(x, w, b) * 4503599627370496.0), 52, tab);
+  return dig::tanh_fixed(__double2ll_rn(fma(x, w, b) * 72057594037927936.0), 56, tab);  // saturates beyond 128
 }
 __device__ __forceinline__ float act1(float x, float w, float b, const dig::TanhTab*) { return tanhf(fmaf(x, w, b)); }
 
@@ -1095,7 +1095,7 @@ bool layer_scale(const double* W, const double* b, int K, int N, double in, bool
     }
     if (!(sum <= 1048576.0)) return false;
     sw[n] = digit_scale(top, fp64, fp64 ? -12 : -100);
-    zs[n] = std::min(52, 60 - (sum > 1.0 ? ceil_log2(sum) : 0));
+    zs[n] = std::min(56, 60 - (sum > 1.0 ? ceil_log2(sum) : 0));
     s[n] = 72 + zs[n] - sh - sw[n];
     if (fp64 && s[n] > 31) {  // large weights: fewer fraction bits in z
       zs[n] -= s[n] - 31;
@@ -1105,6 +1105,34 @@ bool layer_scale(const double* W, const double* b, int K, int N, double in, bool
   }
   for (int k = 0; k < K; ++k) swt[k] = digit_scale(row[k], fp64, -100);
   return true;
+}
+
+// FP64 activations have 54 fraction bits whatever their size, tanh an absolute error of 2^-55: on nets whose activations
+// are small that is worse than FMAs and a relative tanh (rms of h1 0.5: G 7e-17 off against 1.7e-16; 0.27: 1.3 / 1.8e-16;
+// 0.11: 3.1 / 1.9e-16; 0.01: 2.8e-15 / 1.9e-16).  True if the rms over units of h1 and of h2, over the inputs at 14
+// distances up to r_c, is at least kActivations.
+constexpr double kActivations = 0.2;
+bool activations_large(const Model* m, const double* W, int ti) {
+  double s1 = 0.0, s2 = 0.0;
+  for (int k = 2; k < 16; ++k) {
+    const double r = m->rc * (k + 0.5) / 16.0, u = (r - m->rs) / (m->rc - m->rs);
+    const double sw = u <= 0.0 ? 1.0 : m->switch_kind == 1 ? 0.5 * std::cos(3.14159265358979323846 * u) + 0.5
+                                                            : u * u * u * (-6.0 * u * u + 15.0 * u - 10.0) + 1.0;
+    const double x = (sw / r - m->davg_host[4 * ti]) / m->dstd_host[4 * ti];
+    double h1[kN1];
+    for (int q = 0; q < kN1; ++q) {
+      h1[q] = std::tanh(x * W[kEW1 + q] + W[kEb1 + q]);
+      s1 += h1[q] * h1[q];
+    }
+    for (int n = 0; n < kN2; ++n) {
+      double z = W[kEb2 + n];
+      for (int q = 0; q < kN1; ++q) z += h1[q] * W[kEW2 + q * kN2 + n];
+      const double h2 = h1[n % kN1] + std::tanh(z);
+      s2 += h2 * h2;
+    }
+  }
+  const double least = kActivations * kActivations * 14.0;
+  return s1 >= least * kN1 && s2 >= least * kN2;
 }
 
 // A pair's scales stand before its constants and fragments.
@@ -1121,7 +1149,8 @@ dp_status upload(Model* m) {
     const double* W = m->theta_host.data() + (size_t)p * kEmbParams;
     PairScale& q = sc[p];
     m->dig_ok = m->dig_ok && layer_scale(W + kEW2, W + kEb2, kN1, kN2, 1.0, d, bits - 2, q.sw2, q.zs2, q.s2, q.swt2) &&
-                layer_scale(W + kEW3, W + kEb3, kN2, kN3, 2.0, d, bits - 3, q.sw3, q.zs3, q.s3, q.swt3);
+                layer_scale(W + kEW3, W + kEb3, kN2, kN3, 2.0, d, bits - 3, q.sw3, q.zs3, q.s3, q.swt3) &&
+                (!d || m->ntypes > 3 || activations_large(m, W, p / m->ntypes));  // four types: the plain FP64 kernels do not fit
   }
   if (!m->dig_ok) return DP_OK;
   unsigned char* base = static_cast<unsigned char*>(m->dig_emb);

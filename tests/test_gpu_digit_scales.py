@@ -72,3 +72,9 @@ def _small(w1, fit):
 @pytest.mark.parametrize("w1,fit", [(0.1, 1e3), (1e-2, 1e5), (1e-4, 1e9)])
 def test_small_activations_fp32(w1, fit):
     _check(_small(w1, fit), "fp32")
+
+
+# 3 (rms of h1 0.25): the fixed-point layers; the others: the plain kernels
+@pytest.mark.parametrize("w1,fit", [(3.0, 10.0), (0.1, 1e3), (1e-2, 1e5), (1e-4, 1e9)])
+def test_small_activations_fp64(w1, fit):
+    _check(_small(w1, fit), "fp64")
