@@ -5,8 +5,8 @@
 // m16n8k16 B fragments (built once per weight upload, 15.7 MB a type in FP64, resident in L2).  A is read
 // in FP64 / FP32 and cut into digits on the way: lane (g, t) of a warp loads four consecutive k of rows
 // g and g + 8, which are its A fragment when k = 16 s + 4 t + {0, 1, 2, 3} stands at the fragment's columns
-// 2t, 2t + 1, 2t + 8, 2t + 9.  Rows carry a power of two of their own (largest element of the row, or
-// the bound of an activation), matrices one.
+// 2t, 2t + 1, 2t + 8, 2t + 9.  Rows of A carry a power of two of their own (largest element of the row, or
+// the bound of an activation), and so do the columns of B.
 //
 // Eight warps a CTA share a tile of 16 (8 / WK) rows: WK warps split K (their sums meet in shared
 // memory), so that a box of a few hundred atoms, where 16-row tiles times column blocks do not fill
@@ -34,6 +34,10 @@ __host__ __device__ __forceinline__ int mat_off(int q) {
   constexpr int big = (kKD / 16) * (kF / 8), small = (kF / 16) * (kF / 8);
   return q == 0 ? 0 : big + (q - 1) * small;
 }
+// Scales of a type's matrices, one an output column: the dropped digit products count against the largest weight of a
+// column (one for the whole matrix let a weight of 16,384 beside 0.03 put FP32 energies 7e-4 off).
+constexpr int kScales = 5 * kF + kKD;
+__host__ __device__ __forceinline__ int scale_off(int q) { return q * kF; }
 constexpr int kTypeFrags = 2 * (kKD / 16) * (kF / 8) + 4 * (kF / 16) * (kF / 8);
 
 // n-tiles of a warp.  FP32: three, so that two CTAs of 128 registers a thread fit an SM; six in one CTA reuse the
@@ -53,7 +57,7 @@ struct GemmArgs {
   const int* type_off;
   const int* type_count;
   const uint4* frag;       // [type][kTypeFrags][Q][32]
-  const int* wscale;       // [type][kMats]: |W| 2^sw within the digits' range
+  const int* wscale;       // [type][kScales]: a column's |w| 2^sw within the digits' range
   const T* A;              // [rows][K]
   const unsigned* rowmax;  // [rows] top bits of each row's largest |a|, or null: |a| < 2^a_exp
   int a_exp;
@@ -74,7 +78,7 @@ __device__ __forceinline__ unsigned top_bits(float v) { return (unsigned)__float
 // Exponent e with |v| < 2^e for all v with these top bits; not finite: a large one.
 __device__ __forceinline__ int exp_of(unsigned b, double) { return max((int)(b >> 20) - 1022, -800); }
 __device__ __forceinline__ int exp_of(unsigned b, float) {  // with the margin the full digit range needs
-  return max((int)((b + 0x10000u) >> 23) - 126, -80);
+  return max((int)((b + 0x10000u) >> 23) - 126, -110);
 }
 template <class T> struct RowBits { static constexpr int v = sizeof(T) == 8 ? 54 : 26; };
 
@@ -122,12 +126,15 @@ template <> struct Sum<float> {
   __device__ __forceinline__ void add(const float (*acc)[4], int e) { s += dig::join_f(acc, e); }
   __device__ __forceinline__ float value() const { return s; }
 };
-constexpr int kBadScale = -100000;  // a matrix with an infinity or a NaN: every product is NaN
+constexpr int kBadScale = -100000;  // a column with an infinity or a NaN: its products are NaN
 __device__ __forceinline__ double out_scale(int e, int sw, double) {  // 2^(40 - (54 - e) - sw)
-  return e > 1024 || sw == kBadScale ? __longlong_as_double(0x7ff8000000000000ll) : dig::pow2d(40 - 54 + e - sw);
+  return e > 1024 || sw == kBadScale ? __longlong_as_double(0x7ff8000000000000ll)
+                                     : dig::pow2d(min(max(40 - 54 + e - sw, -1022), 1023));
 }
-__device__ __forceinline__ float out_scale(int e, int sw, float) {    // 2^(36 - (26 - e) - sw)
-  return e > 128 || sw == kBadScale ? __int_as_float(0x7fc00000) : __int_as_float((127 + min(max(36 - 26 + e - sw, -126), 127)) << 23);
+__device__ __forceinline__ float out_scale(int e, int sw, float) {    // 2^(36 - (26 - e) - sw), down to the subnormals
+  if (e > 128 || sw == kBadScale) return __int_as_float(0x7fc00000);
+  const int x = 36 - 26 + e - sw;
+  return __int_as_float(x >= -126 ? (127 + min(x, 127)) << 23 : x >= -149 ? 1 << (x + 149) : 0);
 }
 
 // The fragments run through shared memory in stages of KS k steps by cp.async, ST stages deep: one pipeline for
@@ -162,7 +169,7 @@ __global__ void __launch_bounds__(32 * kWarps, sizeof(T) == 8 ? 1 : 2) k_dig_gem
   const Mat mt = mat_of(g.mat);
   const int ntile0 = blockIdx.y * NT, ntiles = mt.N / 8, ksteps = mt.K / 16;
   const uint4* fr = g.frag + ((size_t)ty * kTypeFrags + mat_off(g.mat)) * Q * 32;
-  const int sw = g.wscale[ty * kMats + g.mat];
+  const int* ws = g.wscale + ty * kScales + scale_off(g.mat);
   int ea[2];
   const T* ap[2];
   bool ok[2];
@@ -280,11 +287,11 @@ __global__ void __launch_bounds__(32 * kWarps, sizeof(T) == 8 ? 1 : 2) k_dig_gem
     } else {
       v = sum[n][e].value();
     }
-    v *= out_scale(ea[r], sw, T(0));
     const int col = 8 * (ntile0 + n) + 2 * tq + (e & 1);
     const bool in = ok[r] && ntile0 + n < ntiles;
     T out = T(0);
     if (in) {
+      v *= out_scale(ea[r], ws[col], T(0));
       const size_t o = (base + r0 + gr + 8 * r) * mt.N + col;
       if (g.mode == EPI_TANH) {
         out = gtanh(v + bias[col]);
@@ -365,25 +372,28 @@ __global__ void k_dig_head(int N, const int* __restrict__ itype, T* H3, const T*
 }
 
 // ------------------------------------------------------------------ weights
-// Scale exponent of every matrix (one block each): the largest |w|.
+// Element (k, n) of matrix q: W[k][n], or W[n][k] for a transpose.
 template <class T>
-__global__ void __launch_bounds__(1024) k_dig_fit_scale(const T* __restrict__ fit, int* wscale) {
-  __shared__ unsigned s[32];
-  const int ty = blockIdx.x / 3, q = blockIdx.x % 3;  // W1, W2, W3; the transposes share their scale
-  const T* W = fit + (size_t)ty * kFitParams + (q == 0 ? kFW1 : q == 1 ? kFW2 : kFW3);
-  const int n = (q == 0 ? kKD : kF) * kF;
+__device__ __forceinline__ T weight(const T* W, int q, const Mat& mt, int k, int n) {
+  return q < 3 ? W[(size_t)k * mt.N + n] : W[(size_t)n * mt.K + k];
+}
+__device__ __forceinline__ long mat_base(int q) { return q == 0 || q == 5 ? kFW1 : q == 1 || q == 4 ? kFW2 : kFW3; }
+
+// Scale exponent of every output column, one warp each: its largest |w|.
+template <class T>
+__global__ void __launch_bounds__(256) k_dig_fit_scale(const T* __restrict__ fit, int* wscale) {
+  const int c = blockIdx.x * 8 + (threadIdx.x >> 5), ty = blockIdx.y, lane = threadIdx.x & 31;
+  if (c >= kScales) return;
+  const int q = min(c / kF, kMats - 1), n = c - scale_off(q);
+  const Mat mt = mat_of(q);
+  const T* W = fit + (size_t)ty * kFitParams + mat_base(q);
   unsigned m = 0;
-  for (int k = threadIdx.x; k < n; k += 1024) m = max(m, top_bits(W[k]));
+  for (int k = lane; k < mt.K; k += 32) m = max(m, top_bits(weight(W, q, mt, k, n)));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 1; k < 32; ++k) m = max(m, s[k]);
-    const int e = max(exp_of(m, T(0)), sizeof(T) == 8 ? -60 : -30);
-    const int sw = e > (sizeof(T) == 8 ? 1024 : 128) ? kBadScale : RowBits<T>::v - e;
-    wscale[ty * kMats + q] = sw;
-    wscale[ty * kMats + 5 - q] = sw;
+  if (lane == 0) {
+    const int e = max(exp_of(m, T(0)), sizeof(T) == 8 ? -200 : -100);
+    wscale[ty * kScales + c] = e > (sizeof(T) == 8 ? 1024 : 128) ? kBadScale : RowBits<T>::v - e;
   }
 }
 
@@ -399,13 +409,11 @@ __global__ void __launch_bounds__(256) k_dig_fit_weights(const T* __restrict__ f
   const Mat mt = mat_of(q);
   const int ks = mt.K / 16, idx = f - mat_off(q), nt = idx / ks, s = idx % ks;
   const int col = 8 * nt + (lane >> 2), k0 = 16 * s + 4 * (lane & 3);
-  const T* W = fit + (size_t)ty * kFitParams +
-               (q == 0 || q == 5 ? kFW1 : q == 1 || q == 4 ? kFW2 : kFW3);
-  const int e = RowBits<T>::v - wscale[ty * kMats + q];
+  const T* W = fit + (size_t)ty * kFitParams + mat_base(q);
+  const int e = RowBits<T>::v - wscale[ty * kScales + scale_off(q) + col];
   decltype(fix_digits(T(0), 0)) u[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k)  // q < 3: W[k][n]; transposes: W[n][k] of a matrix with K columns
-    u[k] = fix_digits(q < 3 ? W[(size_t)(k0 + k) * mt.N + col] : W[(size_t)col * mt.K + k0 + k], e);
+  for (int k = 0; k < 4; ++k) u[k] = fix_digits(weight(W, q, mt, k0 + k, col), e);
   uint32_t lo[2 * Q], hi[2 * Q];
   lo[2 * Q - 1] = hi[2 * Q - 1] = 0u;
   split2(u[0], u[1], lo);
@@ -414,6 +422,9 @@ __global__ void __launch_bounds__(256) k_dig_fit_weights(const T* __restrict__ f
 #pragma unroll
   for (int p = 0; p < Q; ++p) dst[p * 32] = make_uint4(lo[2 * p], hi[2 * p], lo[2 * p + 1], hi[2 * p + 1]);
 }
+
+// A model's scales stand before its fragments.
+size_t scale_bytes(int ntypes) { return (sizeof(int) * kScales * ntypes + 255) / 256 * 256; }
 
 template <class T>
 const T* theta_of(const Model* m) {
@@ -424,8 +435,8 @@ template <class T>
 dp_status upload(Model* m) {
   const T* fit = theta_of<T>(m) + (size_t)m->ntypes * m->ntypes * kEmbParams;
   int* ws = static_cast<int*>(m->dig_fit);
-  uint4* fr = reinterpret_cast<uint4*>(static_cast<unsigned char*>(m->dig_fit) + 1024);
-  k_dig_fit_scale<T><<<3 * m->ntypes, 1024>>>(fit, ws);
+  uint4* fr = reinterpret_cast<uint4*>(static_cast<unsigned char*>(m->dig_fit) + scale_bytes(m->ntypes));
+  k_dig_fit_scale<T><<<dim3(cdiv(kScales, 8), m->ntypes), 256>>>(fit, ws);
   k_dig_fit_weights<T><<<dim3(cdiv(kTypeFrags, 8), m->ntypes), 256>>>(fit, ws, fr);
   m->launches += 2;
   DP_LAUNCH_CHECK(m);
@@ -459,7 +470,7 @@ dp_status run(Model* m, int N) {
   GemmArgs<T> g{};
   g.ntypes = m->ntypes; g.type_off = m->type_off; g.type_count = m->type_count;
   g.wscale = static_cast<const int*>(m->dig_fit);
-  g.frag = reinterpret_cast<const uint4*>(static_cast<unsigned char*>(m->dig_fit) + 1024);
+  g.frag = reinterpret_cast<const uint4*>(static_cast<unsigned char*>(m->dig_fit) + scale_bytes(m->ntypes));
   g.stride = kFitParams;
   // rows times column blocks against the SMs decide how far K is split inside a CTA: the least splitting
   // (most reuse of the fragments) that still gives four CTAs an SM
@@ -506,7 +517,7 @@ dp_status run(Model* m, int N) {
 }  // namespace
 
 size_t dig_fit_bytes(int ntypes, bool fp64) {
-  return 1024 + (size_t)ntypes * kTypeFrags * 512 * (fp64 ? dig::Frag<double>::Q : dig::Frag<float>::Q);
+  return scale_bytes(ntypes) + (size_t)ntypes * kTypeFrags * 512 * (fp64 ? dig::Frag<double>::Q : dig::Frag<float>::Q);
 }
 dp_status dig_fit_upload(Model* m) { return m->prec == DP_FP64 ? upload<double>(m) : upload<float>(m); }
 dp_status launch_dig_fitting(Model* m, int N) { return m->prec == DP_FP64 ? run<double>(m, N) : run<float>(m, N); }

@@ -78,3 +78,63 @@ def test_small_activations_fp32(w1, fit):
 @pytest.mark.parametrize("w1,fit", [(3.0, 10.0), (0.1, 1e3), (1e-2, 1e5), (1e-4, 1e9)])
 def test_small_activations_fp64(w1, fit):
     _check(_small(w1, fit), "fp64")
+
+
+def _fit_outlier(layer, value):
+    """One large weight in W1, W2 or W3 of both fitting nets whose input is never near zero (D_00 = |T_0|^2; units 3
+    made constant), so that its output is saturated; columns 9 far below the others."""
+    w = synth.xavier_weights(("O", "H"), 6.0, 0.5, (46, 92), 1001, fit_gain=10.0)
+    for t in range(2):
+        b = {k: w.block(f"fit{t}.{k}") for k in ("W1", "b1", "W2", "b2", "W3")}
+        b["W1"][:, 3], b["b1"][3] = 0.0, 1.0
+        b["W2"][:, 3], b["b2"][3] = 0.0, 1.0
+        for k in ("W1", "W2", "W3"):
+            b[k][:, 9] *= 1e-6
+        b[layer][0 if layer == "W1" else 3, 7] = value
+    return w
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("layer", ["W2", "W3"])
+@pytest.mark.parametrize("value", [1e5, 1e8])
+@pytest.mark.parametrize("n", [66, 3])
+def test_one_large_fitting_weight(prec, layer, value, n):
+    _check(_fit_outlier(layer, value), prec, n, n)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_one_large_descriptor_element(prec):
+    """D_00 about 1, the rest of its rows 1e-2 and 1e-4: embedding output 0 is near 1, the others near 1e-2."""
+    w = _small(1e-2, 100.0)
+    for ti, tj in _pairs():
+        w.block(f"emb{ti}{tj}.b3")[0] = 5.0
+    _check(w, prec)
+
+
+def test_captured_steps_follow_the_kernels():
+    """MD steps captured with one set of kernels are captured again when new parameters need the other one."""
+    import paper_2410_22867_gb300 as dp
+    s = synth.water_box(64, 3)
+    inside = synth.water_weights(1001)
+    outside = synth.water_weights(1001)
+    for ti, tj in _pairs():
+        b = {k: outside.block(f"emb{ti}{tj}.{k}") for k in ("W1", "b1", "W2")}
+        b["W1"][0, 3], b["b1"][3] = 0.0, 1.0
+        b["W2"][3, 7] = 1e5
+    v0 = synth.maxwell_boltzmann(s.masses()[s.types], 300.0, 5)
+    types = torch.tensor(s.types, device="cuda")
+
+    def run(m):
+        x, v = torch.tensor(s.coords, device="cuda"), torch.tensor(v0, device="cuda")
+        k = m.verlet(m.md_state(x, v, types, s.box, s.masses(), rebuild_every=2), 0.5, 4)
+        return k["forces"].clone(), k["potential"].clone()
+
+    m = dp.DPModel(inside, "fp64", max_atoms=s.natoms)
+    for w in (inside, outside, inside):
+        m.set_params(w.theta)
+        f, e = run(m)
+        fresh = dp.DPModel(w, "fp64", max_atoms=s.natoms)
+        f1, e1 = run(fresh)
+        assert float((f - f1).norm() / f1.norm()) <= 1e-11  # order of the atomic sums, 4 steps
+        assert abs(float(e - e1)) <= 1e-12 * abs(float(e1))
+        fresh.close()
