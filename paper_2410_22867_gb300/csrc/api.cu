@@ -441,7 +441,7 @@ dp_status upload_weights(Model* m) {
 
 // Everything made from w64 / w32: padded-slot terms and the operand copies.
 dp_status derive_weights(Model* m) {
-  const bool dig = m->dig_ok;
+  const bool dig = m->dig_ok, dig_fit = m->dig_fit_ok;
   DP_TRY(launch_pad_rows(m));
   if (m->prec == DP_MIX_BF16 || m->prec == DP_MIX_FP16) {
     DP_TRY(launch_tc_setup(m));
@@ -449,7 +449,7 @@ dp_status derive_weights(Model* m) {
   } else {
     DP_TRY(dig_upload(m));
     DP_TRY(dig_fit_upload(m));
-    if (m->dig_ok != dig) drop_graphs(m);  // captured steps hold the other embedding kernels
+    if (m->dig_ok != dig || m->dig_fit_ok != dig_fit) drop_graphs(m);  // captured steps hold the other kernels
   }
   return DP_OK;
 }

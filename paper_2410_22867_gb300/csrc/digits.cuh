@@ -21,6 +21,12 @@
 namespace dpg {
 namespace dig {
 
+// Largest ratio of a column's largest weight to the rms of its other nonzero weights that the digit products take.
+// All of a column is cut relative to its largest weight, and that one's input may be zero (a large weight saturates
+// its unit, whose gradient vanishes), so the others must keep their bits beside it: at 10 their cuts are 2^-52.5 (FP64)
+// of them, the error of the FMAs.  Normal weights reach 5.  Nets with more spread take the plain kernels (simt.cu).
+constexpr float kSpread = 10.f;
+
 template <class T> struct Fmt;
 template <> struct Fmt<double> {
   static constexpr int BD = 8, ND = 7, NO = 8;  // bits a digit, digits, product orders kept

@@ -1078,9 +1078,22 @@ int digit_scale(double top, bool fp64, int lowest) {
   return (fp64 ? Fmt<double>::BD * Fmt<double>::ND - 2 : Fmt<float>::BD * Fmt<float>::ND - 1) - e;
 }
 
+// No weight of a column (n of them, `stride` apart) above kSpread times the rms of its other nonzero ones.
+bool even_column(const double* w, int n, int stride) {
+  double top = 0.0, sum = 0.0;
+  int num = 0;
+  for (int k = 0; k < n; ++k) {
+    const double v = std::fabs(w[(size_t)k * stride]);
+    top = std::fmax(top, v);
+    sum += v * v;
+    num += v != 0.0;
+  }
+  return num <= 1 || top * top * (num - 1) <= dig::kSpread * dig::kSpread * (sum - top * top);
+}
+
 // Scales of one layer (K x N weights W, biases b, |inputs| <= in, FP64 activations with sh fraction bits): sw, zs and s
 // of every column, swt of every row; false when the weights are outside the range the fixed-point layer covers
-// (or not finite).
+// (or not finite), or spread too far.
 bool layer_scale(const double* W, const double* b, int K, int N, double in, bool fp64, int sh, int* sw, int* zs, int* s,
                  int* swt) {
   std::vector<double> row(K, 0.0);
@@ -1093,7 +1106,7 @@ bool layer_scale(const double* W, const double* b, int K, int N, double in, bool
       row[k] = std::fmax(row[k], v);
       sum += in * v;
     }
-    if (!(sum <= 1048576.0)) return false;
+    if (!(sum <= 1048576.0) || !even_column(W + n, K, N)) return false;
     sw[n] = digit_scale(top, fp64, fp64 ? -12 : -100);
     zs[n] = std::min(56, 60 - (sum > 1.0 ? ceil_log2(sum) : 0));
     s[n] = 72 + zs[n] - sh - sw[n];
@@ -1103,7 +1116,10 @@ bool layer_scale(const double* W, const double* b, int K, int N, double in, bool
     }
     if (fp64 && (s[n] < 1 || zs[n] < 40)) return false;
   }
-  for (int k = 0; k < K; ++k) swt[k] = digit_scale(row[k], fp64, -100);
+  for (int k = 0; k < K; ++k) {
+    if (!even_column(W + (size_t)k * N, N, 1)) return false;
+    swt[k] = digit_scale(row[k], fp64, -100);
+  }
   return true;
 }
 

@@ -126,13 +126,11 @@ template <> struct Sum<float> {
   __device__ __forceinline__ void add(const float (*acc)[4], int e) { s += dig::join_f(acc, e); }
   __device__ __forceinline__ float value() const { return s; }
 };
-constexpr int kBadScale = -100000;  // a column with an infinity or a NaN: its products are NaN
 __device__ __forceinline__ double out_scale(int e, int sw, double) {  // 2^(40 - (54 - e) - sw)
-  return e > 1024 || sw == kBadScale ? __longlong_as_double(0x7ff8000000000000ll)
-                                     : dig::pow2d(min(max(40 - 54 + e - sw, -1022), 1023));
+  return e > 1024 ? __longlong_as_double(0x7ff8000000000000ll) : dig::pow2d(min(max(40 - 54 + e - sw, -1022), 1023));
 }
 __device__ __forceinline__ float out_scale(int e, int sw, float) {    // 2^(36 - (26 - e) - sw), down to the subnormals
-  if (e > 128 || sw == kBadScale) return __int_as_float(0x7fc00000);
+  if (e > 128) return __int_as_float(0x7fc00000);
   const int x = 36 - 26 + e - sw;
   return __int_as_float(x >= -126 ? (127 + min(x, 127)) << 23 : x >= -149 ? 1 << (x + 149) : 0);
 }
@@ -379,9 +377,13 @@ __device__ __forceinline__ T weight(const T* W, int q, const Mat& mt, int k, int
 }
 __device__ __forceinline__ long mat_base(int q) { return q == 0 || q == 5 ? kFW1 : q == 1 || q == 4 ? kFW2 : kFW3; }
 
-// Scale exponent of every output column, one warp each: its largest |w|.
+__device__ __forceinline__ double from_top(unsigned b, double) { return __hiloint2double((int)b, 0); }
+__device__ __forceinline__ float from_top(unsigned b, float) { return __int_as_float((int)b); }
+
+// Scale exponent of every output column, one warp each: its largest |w|.  wide: set if a column has a weight above
+// kSpread times the rms of its other nonzero ones, or one that is not finite.
 template <class T>
-__global__ void __launch_bounds__(256) k_dig_fit_scale(const T* __restrict__ fit, int* wscale) {
+__global__ void __launch_bounds__(256) k_dig_fit_scale(const T* __restrict__ fit, int* wscale, int* wide) {
   const int c = blockIdx.x * 8 + (threadIdx.x >> 5), ty = blockIdx.y, lane = threadIdx.x & 31;
   if (c >= kScales) return;
   const int q = min(c / kF, kMats - 1), n = c - scale_off(q);
@@ -391,9 +393,29 @@ __global__ void __launch_bounds__(256) k_dig_fit_scale(const T* __restrict__ fit
   for (int k = lane; k < mt.K; k += 32) m = max(m, top_bits(weight(W, q, mt, k, n)));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  // squares of the weights relative to the largest (within 2^-20 in FP64, whose low word `top_bits` leaves out)
+  const T inv = T(1) / from_top(m, T(0));
+  float sum = 0.f;
+  int num = 0, tops = 0;
+  for (int k = lane; k < mt.K; k += 32) {
+    const T v = weight(W, q, mt, k, n);
+    const bool t = top_bits(v) == m;
+    const float x = t ? 0.f : (float)(v * inv);
+    sum = fmaf(x, x, sum);
+    num += v != T(0);
+    tops += t;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    num += __shfl_xor_sync(0xffffffffu, num, o);
+    tops += __shfl_xor_sync(0xffffffffu, tops, o);
+  }
   if (lane == 0) {
     const int e = max(exp_of(m, T(0)), sizeof(T) == 8 ? -200 : -100);
-    wscale[ty * kScales + c] = e > (sizeof(T) == 8 ? 1024 : 128) ? kBadScale : RowBits<T>::v - e;
+    wscale[ty * kScales + c] = RowBits<T>::v - e;
+    const bool even = m == 0 || num <= 1 || (float)(num - 1) <= dig::kSpread * dig::kSpread * (sum + (float)(tops - 1));
+    if (!even || e > (sizeof(T) == 8 ? 1024 : 128)) *wide = 1;
   }
 }
 
@@ -423,8 +445,8 @@ __global__ void __launch_bounds__(256) k_dig_fit_weights(const T* __restrict__ f
   for (int p = 0; p < Q; ++p) dst[p * 32] = make_uint4(lo[2 * p], hi[2 * p], lo[2 * p + 1], hi[2 * p + 1]);
 }
 
-// A model's scales stand before its fragments.
-size_t scale_bytes(int ntypes) { return (sizeof(int) * kScales * ntypes + 255) / 256 * 256; }
+// A model's scales and the flag of a wide column stand before its fragments.
+size_t scale_bytes(int ntypes) { return (sizeof(int) * ((size_t)kScales * ntypes + 1) + 255) / 256 * 256; }
 
 template <class T>
 const T* theta_of(const Model* m) {
@@ -436,9 +458,17 @@ dp_status upload(Model* m) {
   const T* fit = theta_of<T>(m) + (size_t)m->ntypes * m->ntypes * kEmbParams;
   int* ws = static_cast<int*>(m->dig_fit);
   uint4* fr = reinterpret_cast<uint4*>(static_cast<unsigned char*>(m->dig_fit) + scale_bytes(m->ntypes));
-  k_dig_fit_scale<T><<<dim3(cdiv(kScales, 8), m->ntypes), 256>>>(fit, ws);
-  k_dig_fit_weights<T><<<dim3(cdiv(kTypeFrags, 8), m->ntypes), 256>>>(fit, ws, fr);
-  m->launches += 2;
+  int* wide = ws + (size_t)kScales * m->ntypes;
+  DP_CUDA_TRY(m, cudaMemset(wide, 0, sizeof(int)));
+  k_dig_fit_scale<T><<<dim3(cdiv(kScales, 8), m->ntypes), 256>>>(fit, ws, wide);
+  int h = 0;
+  DP_CUDA_TRY(m, cudaMemcpy(&h, wide, sizeof(int), cudaMemcpyDeviceToHost));
+  m->dig_fit_ok = h == 0;
+  m->launches += 1;
+  if (m->dig_fit_ok) {
+    k_dig_fit_weights<T><<<dim3(cdiv(kTypeFrags, 8), m->ntypes), 256>>>(fit, ws, fr);
+    m->launches += 1;
+  }
   DP_LAUNCH_CHECK(m);
   return DP_OK;
 }

@@ -1,6 +1,6 @@
 // SIMT (CUDA-core) kernels of the FP64 and FP32 paths: environment matrix, tabulated embedding,
-// descriptor and the embedding backward that produces forces and virials; with the embedding net
-// itself only for weights outside the range of emb_digits.cu's fixed-point layers.
+// descriptor and the embedding backward that produces forces and virials; with the embedding and fitting nets
+// themselves only for weights outside the range of emb_digits.cu's and fit_digits.cu's digit products.
 //
 // Model (Section II-A, Fig. 1(b)): for each neighbour j of atom i,
 //   s = sw(r)/r, R_hat = ((s, s dx/r, s dy/r, s dz/r) - davg[ti]) / dstd[ti],
@@ -453,6 +453,160 @@ __global__ void __launch_bounds__(128) k_pad_rows(int nt, const double* __restri
   }
 }
 
+// ------------------------------------------------------------------ fitting net
+// For weights that spread too far for fit_digits.cu (digits.cuh kSpread); one GEMM and type a launch.
+enum EpiMode { EPI_TANH = 0, EPI_RES_TANH = 1, EPI_BWD = 2, EPI_NONE = 3 };
+
+template <class T>
+struct GemmArgs {
+  const int* type_off;   // device: first row of each type
+  const int* type_count; // device: rows of each type
+  int type;
+  int K, Ncol;
+  const T* A;            // [rows][K]
+  const T* B;            // [K][Ncol], or with TB its transpose [Ncol][K]
+  T* C;                  // [rows][Ncol]
+  const T* bias;         // [Ncol] (EPI_TANH, EPI_RES_TANH)
+  const T* res;          // [rows][Ncol] or [Ncol] (res_vec)
+  int res_vec;
+  const T* aux_in;       // [rows][Ncol]: EPI_BWD factor source
+  T* aux_out;            // [rows][Ncol]: EPI_RES_TANH tanh output / EPI_BWD pre-factor gradient
+  int mode;
+};
+
+constexpr int GBM = 64, GBN = 80, GBK = 16;
+
+template <class T, bool TB>
+__global__ void __launch_bounds__(256) k_fit_gemm(GemmArgs<T> g) {
+  __shared__ T As[GBK][GBM + 1];
+  __shared__ T Bs[GBK][GBN + 1];
+  const int rows = g.type_count[g.type];
+  const int r0 = blockIdx.x * GBM;
+  if (r0 >= rows) return;
+  const int row_base = g.type_off[g.type];
+  const int c0 = blockIdx.y * GBN;
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  T acc[4][5];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 5; ++q) acc[p][q] = T(0);
+  const T* A = g.A + (size_t)row_base * g.K;
+  for (int k0 = 0; k0 < g.K; k0 += GBK) {
+    for (int e = threadIdx.x; e < GBM * GBK; e += 256) {
+      int rr = e / GBK, kk = e % GBK;
+      int row = r0 + rr;
+      As[kk][rr] = (row < rows && k0 + kk < g.K) ? A[(size_t)row * g.K + k0 + kk] : T(0);
+    }
+    for (int e = threadIdx.x; e < GBK * GBN; e += 256) {
+      int kk = TB ? e % GBK : e / GBN, cc = TB ? e / GBK : e % GBN;
+      Bs[kk][cc] = (k0 + kk < g.K) ? (TB ? g.B[(size_t)(c0 + cc) * g.K + k0 + kk] : g.B[(size_t)(k0 + kk) * g.Ncol + c0 + cc])
+                                   : T(0);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < GBK; ++kk) {
+      T av[4], bv[5];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) av[p] = As[kk][ty * 4 + p];
+#pragma unroll
+      for (int q = 0; q < 5; ++q) bv[q] = Bs[kk][tx + 16 * q];
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 5; ++q) acc[p][q] += av[p] * bv[q];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    int row = r0 + ty * 4 + p;
+    if (row >= rows) continue;
+    size_t grow = (size_t)(row_base + row);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      int col = c0 + tx + 16 * q;
+      size_t o = grow * g.Ncol + col;
+      T v = acc[p][q];
+      if (g.mode == EPI_TANH) {
+        g.C[o] = dtanh<T>(v + g.bias[col]);
+      } else if (g.mode == EPI_RES_TANH) {
+        T t = dtanh<T>(v + g.bias[col]);
+        g.aux_out[o] = t;
+        g.C[o] = g.res[o] + t;
+      } else if (g.mode == EPI_BWD) {
+        T h = v + (g.res_vec ? g.res[col] : g.res[o]);
+        T f = g.aux_in[o];
+        if (g.aux_out) g.aux_out[o] = h;
+        g.C[o] = h * (T(1) - f * f);
+      } else {
+        g.C[o] = v;
+      }
+    }
+  }
+}
+
+// E_i = H3 . w4 + b4 + e_bias[t];  dZ3 = w4 * (1 - T3^2) written over H3.
+template <class T>
+__global__ void k_fit_head(const int* type_off, const int* type_count, int type, T* H3, const T* T3,
+                           const T* w4, const T* b4, const T* ebias, double* e_atom) {
+  const int lane = threadIdx.x & 31;
+  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (row >= type_count[type]) return;
+  const size_t r = (size_t)(type_off[type] + row);
+  T e = T(0);
+  for (int n = lane; n < kF; n += 32) {
+    T h = H3[r * kF + n], t = T3[r * kF + n], w = w4[n];
+    e += h * w;
+    H3[r * kF + n] = w * (T(1) - t * t);
+  }
+  e = warp_sum<T>(e);
+  if (lane == 0) e_atom[r] = (double)e + (double)b4[0] + (double)ebias[type];
+}
+
+template <class T>
+dp_status run_fitting(Model* m, int N) {
+  const T* w = (sizeof(T) == 8) ? reinterpret_cast<const T*>(m->w64) : reinterpret_cast<const T*>(m->w32);
+  T* act[5];
+  for (int q = 0; q < 5; ++q) act[q] = static_cast<T*>(m->act[q]);
+  const size_t emb_total = (size_t)m->ntypes * m->ntypes * kEmbParams;
+  const size_t ebias_off = emb_total + (size_t)m->ntypes * kFitParams;
+  const int gx = cdiv(N, GBM);
+  for (int t = 0; t < m->ntypes; ++t) {
+    const T* P = w + emb_total + (size_t)t * kFitParams;
+    GemmArgs<T> g{};
+    g.type_off = m->type_off; g.type_count = m->type_count; g.type = t;
+    // F1: H1 = tanh(D W1 + b1)
+    g.K = kKD; g.Ncol = kF; g.A = static_cast<const T*>(m->Dm); g.B = P + kFW1; g.C = act[0];
+    g.bias = P + kFb1; g.mode = EPI_TANH;
+    k_fit_gemm<T, false><<<dim3(gx, kF / GBN), 256, 0, m->stream>>>(g);
+    // F2: T2 = tanh(H1 W2 + b2), H2 = H1 + T2
+    g.K = kF; g.A = act[0]; g.B = P + kFW2; g.C = act[2]; g.bias = P + kFb2; g.res = act[0]; g.res_vec = 0;
+    g.aux_out = act[1]; g.mode = EPI_RES_TANH;
+    k_fit_gemm<T, false><<<dim3(gx, kF / GBN), 256, 0, m->stream>>>(g);
+    // F3: T3 = tanh(H2 W3 + b3), H3 = H2 + T3
+    g.A = act[2]; g.B = P + kFW3; g.C = act[4]; g.bias = P + kFb3; g.res = act[2]; g.aux_out = act[3];
+    k_fit_gemm<T, false><<<dim3(gx, kF / GBN), 256, 0, m->stream>>>(g);
+    // head: E_i, dZ3 = w4 (1 - T3^2) over H3
+    k_fit_head<T><<<cdiv(N, 8), 256, 0, m->stream>>>(m->type_off, m->type_count, t, act[4], act[3], P + kFw4,
+                                                     P + kFb4, w + ebias_off, m->e_atom);
+    // B3: dH2 = w4 + dZ3 W3^T ; dZ2 = dH2 (1 - T2^2)  (dH2 -> act[3], dZ2 -> act[2])
+    g.A = act[4]; g.B = P + kFW3; g.C = act[2]; g.res = P + kFw4; g.res_vec = 1;
+    g.aux_in = act[1]; g.aux_out = act[3]; g.mode = EPI_BWD;
+    k_fit_gemm<T, true><<<dim3(gx, kF / GBN), 256, 0, m->stream>>>(g);
+    // B2: dH1 = dH2 + dZ2 W2^T ; dZ1 = dH1 (1 - H1^2)  (dZ1 -> act[1])
+    g.A = act[2]; g.B = P + kFW2; g.C = act[1]; g.res = act[3]; g.res_vec = 0; g.aux_in = act[0];
+    g.aux_out = nullptr;
+    k_fit_gemm<T, true><<<dim3(gx, kF / GBN), 256, 0, m->stream>>>(g);
+    // B1: dD = dZ1 W1^T
+    g.K = kF; g.Ncol = kKD; g.A = act[1]; g.B = P + kFW1; g.C = static_cast<T*>(m->dD); g.mode = EPI_NONE;
+    k_fit_gemm<T, true><<<dim3(gx, kKD / GBN), 256, 0, m->stream>>>(g);
+    m->launches += 7;
+  }
+  DP_LAUNCH_CHECK(m);
+  return DP_OK;
+}
+
 template <class T>
 EmbArgs<T> make_emb_args(Model* m, int N) {
   EmbArgs<T> a{};
@@ -528,7 +682,8 @@ dp_status launch_descriptor(Model* m, int N) {
 }
 dp_status launch_fitting(Model* m, int N) {
   if (is_mixed(m)) return launch_mix_fitting(m, N);
-  return launch_dig_fitting(m, N);
+  if (m->dig_fit_ok) return launch_dig_fitting(m, N);
+  return m->prec == DP_FP64 ? run_fitting<double>(m, N) : run_fitting<float>(m, N);
 }
 dp_status launch_embed_backward(Model* m, int N, bool fold) {
   if (is_mixed(m)) return launch_mix_embed_backward(m, N, fold);

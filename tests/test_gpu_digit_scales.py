@@ -48,10 +48,24 @@ def _outlier(layer, value):
     return w
 
 
-# 65,535 and 65,600: just inside and just outside what the fixed-point layers take
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
 @pytest.mark.parametrize("layer", ["W2", "W3"])
-@pytest.mark.parametrize("value", [100.0, 16384.0, 65535.0, 65600.0])
+@pytest.mark.parametrize("value", [100.0, 16384.0])
+def test_one_large_embedding_weight_of_a_live_unit(prec, layer, value):
+    """As above, but unit 3 varies (its activations stay above 0.6): its gradient is a sum in which the large weight
+    meets the zero gradient of the output that it saturates."""
+    w = _outlier(layer, value)
+    for ti, tj in _pairs():
+        b = {k: w.block(f"emb{ti}{tj}.{k}") for k in ("W1", "b1", "W2", "b2")}
+        b["W1"][0, 3], b["b1"][3] = -0.4, 1.5
+        b["W2"][:, 3], b["b2"][3] = b["W2"][:, 4] * 0.3, 2.0
+    _check(w, prec)
+
+
+# 0.3: the digit products; from 100 on the plain kernels (the spread of the column, beyond 65,536 the size too)
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("layer", ["W2", "W3"])
+@pytest.mark.parametrize("value", [0.3, 100.0, 16384.0, 65535.0, 65600.0])
 def test_one_large_embedding_weight(prec, layer, value):
     _check(_outlier(layer, value), prec)
 
@@ -95,7 +109,7 @@ def _fit_outlier(layer, value):
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
-@pytest.mark.parametrize("layer", ["W2", "W3"])
+@pytest.mark.parametrize("layer", ["W1", "W2", "W3"])
 @pytest.mark.parametrize("value", [1e5, 1e8])
 @pytest.mark.parametrize("n", [66, 3])
 def test_one_large_fitting_weight(prec, layer, value, n):
@@ -109,6 +123,18 @@ def test_one_large_descriptor_element(prec):
     for ti, tj in _pairs():
         w.block(f"emb{ti}{tj}.b3")[0] = 5.0
     _check(w, prec)
+
+
+def test_infinite_fp32_weight():
+    """A parameter beyond FP32 makes a column infinite: its unit is saturated as in the oracle's FP64."""
+    import paper_2410_22867_gb300 as dp
+    x, t, box = _cluster(16, 16)
+    w = synth.xavier_weights(("O", "H"), 6.0, 0.5, (46, 92), 1001)
+    w.block("fit0.W2")[5, 5] = 1e300
+    ref = oracle.Model(w.to_blob()).compute(x, t, box)["atom_energy"]
+    m = dp.DPModel(w, "fp32", max_atoms=16)
+    e = m.compute(torch.tensor(x, device="cuda"), torch.tensor(t, device="cuda"), box)["atom_energy"].cpu().numpy()
+    assert np.abs(e - ref).max() <= BARS["fp32"][0] * np.abs(ref).mean()
 
 
 def test_captured_steps_follow_the_kernels():
@@ -130,7 +156,10 @@ def test_captured_steps_follow_the_kernels():
         return k["forces"].clone(), k["potential"].clone()
 
     m = dp.DPModel(inside, "fp64", max_atoms=s.natoms)
-    for w in (inside, outside, inside):
+    wide = synth.water_weights(1001)
+    for k in range(2):
+        wide.block(f"fit{k}.W2")[3, 7] = 100.0
+    for w in (inside, outside, wide, inside):
         m.set_params(w.theta)
         f, e = run(m)
         fresh = dp.DPModel(w, "fp64", max_atoms=s.natoms)
