@@ -576,7 +576,7 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
     A_(dig_emb, dig_emb_bytes(nt, prec == DP_FP64));
     A_(dig_dT, es * N * (4 * kN3 + 4));
     A_(dig_fit, dig_fit_bytes(nt, prec == DP_FP64));
-    A_(dig_max, 4 * 4 * N);
+    A_(dig_max, 4 * 6 * N);
     if (prec == DP_FP64) A_(dig_tanh, dig_tanh_bytes());
   }
   m->pg_cap = std::min(max_atoms, kPgAtoms);

@@ -179,7 +179,7 @@ struct Model {
   void* dig_tanh = nullptr;
   void* dig_dT = nullptr;     // [N][100][4], then [N][4] maxima
   void* dig_fit = nullptr;    // fitting weights as digit fragments (fit_digits.cu)
-  void* dig_max = nullptr;    // [4][N] top bits of the largest element of a row: D, dz3, dz2, dz1
+  void* dig_max = nullptr;    // [6][N] top bits of the largest element of a row: D, dz3, dz2, dz1, h1, h2
   bool dig_ok = false;        // the embedding weights are within the range of the fixed-point layers
   bool dig_fit_ok = false;    // likewise the fitting weights
   // mixed-precision path

@@ -5,8 +5,8 @@
 // m16n8k16 B fragments (built once per weight upload, 15.7 MB a type in FP64, resident in L2).  A is read
 // in FP64 / FP32 and cut into digits on the way: lane (g, t) of a warp loads four consecutive k of rows
 // g and g + 8, which are its A fragment when k = 16 s + 4 t + {0, 1, 2, 3} stands at the fragment's columns
-// 2t, 2t + 1, 2t + 8, 2t + 9.  Rows of A carry a power of two of their own (largest element of the row, or
-// the bound of an activation), and so do the columns of B.
+// 2t, 2t + 1, 2t + 8, 2t + 9.  Rows of A and columns of B carry a power of two of their own, from their largest element
+// (the activations too: with their bounds, 1 and 2, nets of small activations lost bits).
 //
 // Eight warps a CTA share a tile of 16 (8 / WK) rows: WK warps split K (their sums meet in shared
 // memory), so that a box of a few hundred atoms, where 16-row tiles times column blocks do not fill
@@ -59,9 +59,7 @@ struct GemmArgs {
   const uint4* frag;       // [type][kTypeFrags][Q][32]
   const int* wscale;       // [type][kScales]: a column's |w| 2^sw within the digits' range
   const T* A;              // [rows][K]
-  const unsigned* rowmax;  // [rows] top bits of each row's largest |a|, or null: |a| < 2^a_exp
-  int a_exp;
-  const T* w4;             // B3: the bound of dz3 is max |w4| of the type (in w4max), residual w4
+  const unsigned* rowmax;  // [rows] top bits of each row's largest |a|
   T* C;                    // [rows][N]
   const T* bias;           // theta: bias of type 0 (types bias_stride apart)
   long stride;             // parameters of a fitting block
@@ -177,7 +175,7 @@ __global__ void __launch_bounds__(32 * kWarps, sizeof(T) == 8 ? 1 : 2) k_dig_gem
     ok[r] = row < rows;
     const size_t gi = base + (ok[r] ? row : 0);
     ap[r] = g.A + gi * mt.K + 4 * tq;
-    ea[r] = g.rowmax ? exp_of(g.rowmax[gi], T(0)) : g.a_exp;
+    ea[r] = exp_of(g.rowmax[gi], T(0));
   }
   Sum<T> sum[NT][4];
   {
@@ -494,7 +492,7 @@ dp_status run(Model* m, int N) {
   for (int q = 0; q < 5; ++q) act[q] = static_cast<T*>(m->act[q]);
   unsigned* mx = static_cast<unsigned*>(m->dig_max);
   const size_t R = (size_t)m->max_atoms;
-  DP_CUDA_TRY(m, cudaMemsetAsync(mx + 2 * R, 0, 4 * 2 * R, m->stream));
+  DP_CUDA_TRY(m, cudaMemsetAsync(mx + 2 * R, 0, 4 * 4 * R, m->stream));
   k_dig_rowmax<T><<<cdiv(N, 8), 256, 0, m->stream>>>(N, static_cast<const T*>(m->Dm), mx);
   m->launches += 1;
   GemmArgs<T> g{};
@@ -518,13 +516,15 @@ dp_status run(Model* m, int N) {
   } while (0)
   // F1: H1 = tanh(D W1 + b1)
   g.mat = 0; g.A = static_cast<const T*>(m->Dm); g.rowmax = mx; g.C = act[0]; g.bias = fit + kFb1; g.mode = EPI_TANH;
+  g.outmax = mx + 4 * R;
   DP_GO(g);
-  // F2: T2 = tanh(H1 W2 + b2), H2 = H1 + T2   (|H1| <= 1 < 2^1, |H2| <= 2 < 2^2)
-  g.mat = 1; g.A = act[0]; g.rowmax = nullptr; g.a_exp = 1; g.C = act[2]; g.bias = fit + kFb2; g.res = act[0];
-  g.aux_out = act[1]; g.mode = EPI_RES_TANH;
+  // F2: T2 = tanh(H1 W2 + b2), H2 = H1 + T2
+  g.mat = 1; g.A = act[0]; g.rowmax = mx + 4 * R; g.C = act[2]; g.bias = fit + kFb2; g.res = act[0];
+  g.aux_out = act[1]; g.mode = EPI_RES_TANH; g.outmax = mx + 5 * R;
   DP_GO(g);
   // F3: T3 = tanh(H2 W3 + b3), H3 = H2 + T3
-  g.mat = 2; g.A = act[2]; g.a_exp = 2; g.C = act[4]; g.bias = fit + kFb3; g.res = act[2]; g.aux_out = act[3];
+  g.mat = 2; g.A = act[2]; g.rowmax = mx + 5 * R; g.C = act[4]; g.bias = fit + kFb3; g.res = act[2]; g.aux_out = act[3];
+  g.outmax = nullptr;
   DP_GO(g);
   k_dig_head<T><<<cdiv(N, 8), 256, 0, m->stream>>>(N, m->itype, act[4], act[3], fit, ebias, m->e_atom, mx + R);
   m->launches += 1;

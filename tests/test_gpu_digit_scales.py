@@ -167,3 +167,19 @@ def test_captured_steps_follow_the_kernels():
         assert float((f - f1).norm() / f1.norm()) <= 1e-11  # order of the atomic sums, 4 steps
         assert abs(float(e - e1)) <= 1e-12 * abs(float(e1))
         fresh.close()
+
+
+def _small_fit(gain):
+    """Fitting activations of about `gain`: no fitting biases, first-layer weights scaled down."""
+    w = synth.xavier_weights(("O", "H"), 6.0, 0.5, (46, 92), 1001)
+    for t in range(2):
+        w.block(f"fit{t}.W1")[...] *= gain
+        for k in ("b1", "b2", "b3", "b4"):
+            w.block(f"fit{t}.{k}")[...] = 0.0
+    return w
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("gain", [1e-2, 1e-4, 1e-6])
+def test_small_fitting_activations(prec, gain):
+    _check(_small_fit(gain), prec)
