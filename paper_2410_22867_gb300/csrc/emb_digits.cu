@@ -659,23 +659,29 @@ __device__ __forceinline__ double widen(float v) {
   const uint32_t x = e == 255u ? 0x7ffu : e + 896u;
   return __hiloint2double((int)((b & 0x80000000u) | (e == 0u ? 0u : (x << 20) | (m >> 3))), (int)(e == 0u ? 0u : m << 29));
 }
-// Sum over a tile's rows of g (plain) or -g d, in FP64; FP32 rows with exact products and a compensated sum
-// (two floats, 48 bits), widened once a tile: the FP64 form was 18% of the FP64 pipe and a chain of 16 DFMAs.
-__device__ __forceinline__ double tile_sum(const double* g, const double* d, bool plain, int rows) {
+// Sum over a tile's rows first, first + 2, ... of g (plain) or -g d, in FP64.  FP32 rows: exact products, and sums of three
+// floats (70 bits and more, so no less than FP64's 53) that are widened once a tile; the FP64 form was 18% of the FP64
+// pipe and a chain of 16 DFMAs.
+__device__ __forceinline__ double tile_sum(const double* g, const double* d, bool plain, int first, int rows) {
   double s = 0.0;
-  for (int k = 0; k < rows; ++k) s = fma(g[k], plain ? 1.0 : -d[k], s);
+  for (int k = first; k < rows; k += 2) s = fma(g[k], plain ? 1.0 : -d[k], s);
   return s;
 }
-__device__ __forceinline__ double tile_sum(const float* g, const float* d, bool plain, int rows) {
-  float s = 0.f, c = 0.f;
-  for (int k = 0; k < rows; ++k) {
+__device__ __forceinline__ float two_sum(float& s, float x) {  // s += x; returns what was rounded off
+  const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+  const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+  s = t;
+  return r;
+}
+__device__ __forceinline__ double tile_sum(const float* g, const float* d, bool plain, int first, int rows) {
+  float s = 0.f, c = 0.f, l = 0.f;
+  for (int k = first; k < rows; k += 2) {
     const float x = g[k], y = plain ? 1.f : -d[k];
     const float p = __fmul_rn(x, y), e = __fmaf_rn(x, y, -p);
-    const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
-    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b)), e));
-    s = t;
+    const float r = two_sum(s, p), q = two_sum(c, e);
+    l = __fadd_rn(l, __fadd_rn(two_sum(c, r), q));
   }
-  return (double)s + (double)c;
+  return (double)s + ((double)c + (double)l);
 }
 
 // Embedding backward with recompute, prod_force and the per-atom virial.  Everything downstream of
@@ -707,7 +713,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
     for (int c = 0; c < 4; ++c) bmax[c] = a.dTmax[(size_t)i * 4 + c];
     int q0 = 0;
     bool any = false;
-    double mine = 0.0;  // lanes 0..2: centre force, 3..11: virial
+    double mine = 0.0;  // lanes 0..2: centre force, 3..11: virial, over even rows; 12..23: odd rows
     for (int tj = 0; tj < a.ntypes; ++tj) {
       const int cnt = a.nl_count[(size_t)i * a.ntypes + tj];
       const int nt = (cnt + 15) >> 4;
@@ -956,14 +962,15 @@ __global__ void __launch_bounds__(32 * W, 1) k_dig_bwd(DigArgs<T> a) {
           }
         }
         __syncwarp();
-        if (lane < 12) {  // lane c: sum of g_c; lane 3 + 3 p + q: -sum of g_p d_q
-          const int rows = min(16, cnt - base);
-          const int c = lane < 3 ? lane : (lane - 3) / 3, q = lane < 3 ? 0 : (lane - 3) % 3;
-          mine += tile_sum(sw.g3[c], sw.env[q], lane < 3, rows);
+        if (lane < 24) {  // k = c: sum of g_c; k = 3 + 3 p + q: -sum of g_p d_q
+          const int k = lane < 12 ? lane : lane - 12;
+          const int c = k < 3 ? k : (k - 3) / 3, q = k < 3 ? 0 : (k - 3) % 3;
+          mine += tile_sum(sw.g3[c], sw.env[q], k < 3, lane >= 12, min(16, cnt - base));
         }
       }
     }
     if (any) {
+      mine += __shfl_down_sync(0xffffffffu, mine, 12);
       if (lane < 3) atomicAdd(&a.force[3 * (size_t)i + lane], mine);
       else if (lane < 12) atomicAdd(&a.vir_atom[(size_t)i * 9 + lane - 3], mine);
     }

@@ -183,3 +183,17 @@ def _small_fit(gain):
 @pytest.mark.parametrize("gain", [1e-2, 1e-4, 1e-6])
 def test_small_fitting_activations(prec, gain):
     _check(_small_fit(gain), prec)
+
+
+@pytest.mark.parametrize("n", [64, 256])
+def test_fp32_force_sums_are_fp64(n):
+    """The net force of an FP32 model: every pair force enters with both signs, and sums in FP64 of 24-bit values (29 bits
+    to spare) are exact but for the pairs 2^-29 below the largest.  Bar: a fiftieth of what one rounding of the
+    largest force at every addition (two a neighbour, about 95 neighbours) would leave as a random walk."""
+    import paper_2410_22867_gb300 as dp
+    from _parity import env_stats
+    s = synth.water_box(n, 1)
+    m = dp.DPModel(synth.normalised_weights("water", env_stats()), "fp32", max_atoms=s.natoms)
+    f = m.compute(torch.tensor(s.coords, device="cuda"), torch.tensor(s.types, device="cuda"), s.box)["forces"].cpu().numpy()
+    net = np.abs(f.astype(np.longdouble).sum(0)).max()
+    assert float(net) <= 0.02 * 2.0 ** -53 * np.sqrt(2 * 95 * s.natoms) * np.abs(f).max()
