@@ -105,6 +105,7 @@ struct Model {
   float* tab32 = nullptr;
   float* tab_nodes32 = nullptr;  // FP32 node data for the shared-memory table kernels (tab_mix.cu)
   void* tab_mem = nullptr;
+  size_t tab_bytes = 0;
   // 16-bit operand copies for the tensor-core kernels (per type), laid out by those kernels
   void* tc_weights = nullptr;
   void* emb_img = nullptr;    // mixed precision: per embedding pair, the forward's MMA operand

@@ -95,27 +95,30 @@ __global__ void k_tab_coef(int npairs, int n, double h, const double* __restrict
 
 dp_status launch_tabulate(Model* m, double x0, double x1, int n) {
   DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));
-  if (m->tab_mem) {
+  m->tab_n = 0;
+  const int npairs = m->ntypes * m->ntypes;
+  const size_t nodes = (size_t)npairs * (n + 1) * kN3 * 3;        // doubles
+  const size_t coef = (size_t)npairs * n * kN3 * 8;               // entries
+  const size_t bytes = n == 0 ? 0 : nodes * 8 + coef * 8 + coef * 4 + nodes * 4;
+  // a table of the same size (new parameters) is rebuilt where it is: captured MD steps hold its address
+  if (m->tab_mem && m->tab_bytes != bytes) {
     DP_CUDA_TRY(m, cudaFree(m->tab_mem));
     m->tab_mem = nullptr;
     m->tab64 = nullptr;
     m->tab32 = nullptr;
     m->tab_nodes32 = nullptr;
   }
-  m->tab_n = 0;
   if (n == 0) return DP_OK;
-  const int npairs = m->ntypes * m->ntypes;
-  const size_t nodes = (size_t)npairs * (n + 1) * kN3 * 3;        // doubles
-  const size_t coef = (size_t)npairs * n * kN3 * 8;               // entries
-  const size_t bytes = nodes * 8 + coef * 8 + coef * 4 + nodes * 4;
-  void* mem = nullptr;
-  cudaError_t e = cudaMalloc(&mem, bytes);
-  if (e != cudaSuccess) {
-    m->last_error = std::string("table allocation: ") + cudaGetErrorString(e);
-    return DP_ERR_OOM;
+  if (!m->tab_mem) {
+    cudaError_t e = cudaMalloc(&m->tab_mem, bytes);
+    if (e != cudaSuccess) {
+      m->tab_mem = nullptr;
+      m->last_error = std::string("table allocation: ") + cudaGetErrorString(e);
+      return DP_ERR_OOM;
+    }
+    m->tab_bytes = bytes;
   }
-  m->tab_mem = mem;
-  double* v = static_cast<double*>(mem);
+  double* v = static_cast<double*>(m->tab_mem);
   m->tab64 = v + nodes;
   m->tab32 = reinterpret_cast<float*>(m->tab64 + coef);
   m->tab_nodes32 = m->tab32 + coef;
