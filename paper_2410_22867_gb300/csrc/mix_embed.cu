@@ -1233,7 +1233,8 @@ __global__ void k_scan_fix(int N, int nblk, int* rowoff, const int* blk) {
 // Zeroes what an evaluation accumulates: forces (both arrays), per-replica virials, and the partial T
 // of the (atom, type) segments that the forward does not store whole: those without rows and those
 // split between two CTAs (chunks of `per` rows as in k_mix_embed_fwd with `grid` CTAs).  Clearing all
-// of Tseg wrote 1.6 KB an atom and type (38 us a step at 131,072 atoms).  One warp per atom.
+// of Tseg wrote 1.6 KB an atom and type (38 us a step at 131,072 atoms).  One warp per atom.  Tseg null: the
+// shared-memory table kernels store every segment whole.
 __global__ void __launch_bounds__(256) k_mix_zero(int N, int ntypes, int grid, int nrep, const int* __restrict__ rowoff,
                                                   float4* Tseg, double* force, float4* force32, double* vir_rep) {
   const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -1241,6 +1242,7 @@ __global__ void __launch_bounds__(256) k_mix_zero(int N, int ntypes, int grid, i
   if (i >= N) return;
   if (lane < 3) force[(size_t)i * 3 + lane] = 0.0;
   if (lane == 3) force32[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!Tseg) return;
   int total = 0;
   for (int tj = 0; tj < ntypes; ++tj) total += rowoff[(size_t)tj * (N + 1) + N];
   const int per = max(kRows, (total + grid - 1) / grid);
@@ -1510,7 +1512,8 @@ dp_status launch_mix_descriptor(Model* m, int N) {
   const void* fn = reinterpret_cast<const void*>(fk);
   DP_CUDA_TRY(m, ensure_smem(fn, kFwdSmem));
   const int grid = tuned_grid(m, 0, num_sms() * blocks_per_sm(fn, kRows, kFwdSmem, kTmemCols));
-  k_mix_zero<<<cdiv(N, 8), 256, 0, m->stream>>>(N, m->ntypes, grid, m->nrep, m->rowoff, reinterpret_cast<float4*>(m->Tseg),
+  k_mix_zero<<<cdiv(N, 8), 256, 0, m->stream>>>(N, m->ntypes, grid, m->nrep, m->rowoff,
+                                                tab_smem_path(m, N) ? nullptr : reinterpret_cast<float4*>(m->Tseg),
                                                 m->force, reinterpret_cast<float4*>(m->force32), m->vir_rep);
   if (tab_smem_path(m, N)) {
     const dp_status st = launch_tab_forward(m, N);

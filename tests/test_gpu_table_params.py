@@ -1,5 +1,5 @@
-"""New parameters for a tabulated model whose MD steps are captured: the table is rebuilt where it is, so that the
-captured steps read the new one (GPU only).  Bars: the order of atomic force sums over 4 steps, as in
+"""Tabulated models: new parameters while MD steps are captured (the table is rebuilt where it is, so that the captured
+steps read the new one), and the autotuner (GPU only).  Bars: the order of atomic force sums over 4 steps, as in
 test_gpu_params_device.py."""
 import pytest
 
@@ -41,3 +41,19 @@ def test_captured_steps_use_the_new_table(prec, bar):
     fresh.tabulate(64)
     f1 = run(fresh)
     assert float((f - f1).norm() / f1.norm()) <= bar
+
+
+def test_autotune_leaves_kernels_of_one_shape():
+    """The shared-memory table kernels have one launch shape: nothing is tuned for them; below their range it is."""
+    import paper_2410_22867_gb300 as dp
+    for cells, large in ((6, True), (3, False)):
+        s = synth.copper_fcc(cells, 1)
+        m = dp.DPModel(synth.copper_weights(1001), "mix_fp16", max_atoms=s.natoms)
+        m.tabulate(256)
+        x, t = torch.tensor(s.coords, device="cuda"), torch.tensor(s.types, device="cuda")
+        f0 = m.compute(x, t, s.box)["forces"]
+        g = m.autotune(1)
+        assert g[2] > 0 and g[3] > 0 and (g[0] > 0) != large and (g[1] > 0) != large, g
+        f1 = m.compute(x, t, s.box)["forces"]
+        assert float((f0 - f1).norm() / f0.norm()) <= 1e-3  # as test_gpu_params_device.py's mixed bar
+        m.close()
