@@ -431,12 +431,17 @@ extern "C" {
 
 const char* dp_version(void) { return "dpgb300 0.1"; }
 
-// Device copies of the parameters from m->theta_host (and davg / dstd): theta in FP64 and
-// FP32, normalisation statistics, and the tensor-core operand copies: 16-bit ones for the mixed
-// precisions, digit fragments for FP64 / FP32.  Synchronous.
+// Leading parameters that m->theta_host keeps: all of them for the mixed precisions' 16-bit copies, the embedding nets'
+// (for the scales of their digits) otherwise.
+static size_t host_params(const Model* m) {
+  return is_mixed(m) ? (size_t)m->ntheta : (size_t)m->ntypes * m->ntypes * kEmbParams;
+}
+
+// Device copies of the parameters: theta in FP64 and FP32, padded-slot terms and the tensor-core operand copies:
+// 16-bit ones for the mixed precisions, digit fragments for FP64 / FP32.  Synchronous.
 dp_status derive_weights(Model* m);
-dp_status upload_weights(Model* m) {
-  const std::vector<double>& theta = m->theta_host;
+dp_status upload_weights(Model* m, const std::vector<double>& theta) {
+  m->theta_host.assign(theta.begin(), theta.begin() + host_params(m));
   std::vector<float> t32(theta.begin(), theta.end());
   DP_CUDA_TRY(m, cudaMemcpy(m->w64, theta.data(), 8 * theta.size(), cudaMemcpyHostToDevice));
   DP_CUDA_TRY(m, cudaMemcpy(m->w32, t32.data(), 4 * t32.size(), cudaMemcpyHostToDevice));
@@ -531,7 +536,6 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
   m->S = m->sel_off[ntypes];
   m->VS = m->vcap_off[ntypes];
   m->ntheta = (long long)P.theta.size();
-  m->theta_host = P.theta;
   m->davg_host = P.davg; m->dstd_host = P.dstd;
   if ((prec == DP_MIX_BF16 || prec == DP_MIX_FP16) && !tc_available(m))
     return fail(DP_ERR_UNSUPPORTED, "mixed precision needs the tensor-core kernels (sm_103a GPU)");
@@ -609,7 +613,7 @@ dp_status dp_create(dp_model** out, int ntypes, const char* const* type_map, dou
   }
   {
     dp_status s1 = upload_stats(m);
-    if (s1 == DP_OK) s1 = upload_weights(m);
+    if (s1 == DP_OK) s1 = upload_weights(m, P.theta);
     if (s1 != DP_OK) return fail(s1, m->last_error);
   }
   if (cudaMemset(m->err, 0, 16) != cudaSuccess) return fail(DP_ERR_CUDA, "memset failed");
@@ -689,8 +693,7 @@ dp_status dp_set_params(dp_model* h, const double* theta, long long ntheta) {
   for (long long q = 0; q < ntheta; ++q)
     if (!std::isfinite(theta[q])) { m->last_error = "non-finite parameter"; return DP_ERR_WEIGHTS; }
   DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));
-  m->theta_host.assign(theta, theta + ntheta);
-  DP_TRY(upload_weights(m));
+  DP_TRY(upload_weights(m, std::vector<double>(theta, theta + ntheta)));
   DP_CUDA_TRY(m, cudaDeviceSynchronize());
   if (m->tab_n > 0) DP_TRY(launch_tabulate(m, m->tab_x0, m->tab_x0 + m->tab_n * m->tab_h, m->tab_n));
   return DP_OK;
@@ -702,9 +705,7 @@ dp_status dp_set_params_device(dp_model* h, const void* theta, int is_fp32, long
   if (!theta) { m->last_error = "null theta"; return DP_ERR_ARG; }
   if (ntheta != m->ntheta) { m->last_error = "ntheta does not match the model"; return DP_ERR_ARG; }
   DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));
-  // The host keeps the parameters that host code reads: all of them for the mixed precisions' 16-bit copies,
-  // the embedding nets' (for the scales of their digits) otherwise.
-  const size_t keep = is_mixed(m) ? (size_t)ntheta : (size_t)m->ntypes * m->ntypes * kEmbParams;
+  const size_t keep = host_params(m);
   std::vector<double> host(keep);
   std::vector<float> host32(is_fp32 ? keep : 0);
   DP_TRY(launch_check_finite(m, theta, is_fp32 != 0, ntheta, m->err + 1));
@@ -715,7 +716,7 @@ dp_status dp_set_params_device(dp_model* h, const void* theta, int is_fp32, long
   DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));
   if (bad) { m->last_error = "non-finite parameter"; return DP_ERR_WEIGHTS; }
   if (is_fp32) std::copy(host32.begin(), host32.end(), host.begin());
-  std::copy(host.begin(), host.end(), m->theta_host.begin());
+  m->theta_host = std::move(host);
   DP_TRY(launch_copy_params(m, theta, is_fp32 != 0, ntheta));
   DP_CUDA_TRY(m, cudaStreamSynchronize(m->stream));  // derive_weights also uses the legacy default stream
   DP_TRY(derive_weights(m));

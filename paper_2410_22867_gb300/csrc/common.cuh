@@ -82,7 +82,7 @@ struct Model {
   cudaStream_t capture_stream = nullptr;  // owned; graphs are captured here, replayed on `stream`
   std::string last_error;
   long long ntheta = 0;
-  std::vector<double> theta_host;
+  std::vector<double> theta_host;  // the parameters that host code reads (host_params)
   std::vector<double> davg_host, dstd_host;
 
   // weights (device)
