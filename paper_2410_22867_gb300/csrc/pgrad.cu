@@ -885,11 +885,13 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
     DP_CUDA_TRY(m, cudaMemcpyAsync(m->pg_roff, roffs.data(), sizeof(int) * roffs.size(), cudaMemcpyHostToDevice,
                                    m->stream));
 
-  // workspace
+  // workspace: T and its adjoint, then one area that the fitting net (steps 2 to 5) and the neighbour rows
+  // (steps 1 and 6) use in turn
   T* ws = static_cast<T*>(m->pg_ws);
   const size_t C = (size_t)cap;
   T* TT = ws;
-  T* Y = TT + C * 800;
+  T* TB = TT + C * 800;
+  T* Y = TB + C * 800;
   T* Yb = Y + 2 * C * kKD;
   T* F1 = Yb + 2 * C * kKD;
   T* F2 = F1 + 2 * C * kF;
@@ -897,9 +899,8 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
   T* H = F3 + 2 * C * kF;
   T* U = H + 2 * C * kF;
   T* G = U + 2 * C * kF;
-  T* TB = G + 2 * C * kF;
   const size_t RW = (size_t)m->pg_rows;
-  T* geo = TB + C * 800;
+  T* geo = Y;
   T* H1 = geo + RW * kPgGeo;
   T* H2 = H1 + 2 * RW * kN1;
   T* TZ = H2 + 2 * RW * kN2;
@@ -1008,9 +1009,9 @@ dp_status run_param_grad(Model* m, int N, double* grad) {
 }  // namespace
 
 size_t param_grad_workspace_bytes(int cap, int rows, bool fp64) {
-  const size_t per_atom = 800 + 2 * 2 * (size_t)kKD + 6 * 2 * (size_t)kF + 800;
+  const size_t fit = 2 * 2 * (size_t)kKD + 6 * 2 * (size_t)kF;  // per atom
   const size_t per_row = kPgGeo + 2 * (size_t)(kN1 + kN2 + kN2 + kN3 + kN2 + kN2 + kN1) + 1;
-  return ((size_t)cap * per_atom + (size_t)rows * per_row) * (fp64 ? 8 : 4);
+  return ((size_t)cap * 1600 + std::max((size_t)cap * fit, (size_t)rows * per_row)) * (fp64 ? 8 : 4);
 }
 
 dp_status launch_param_grad(Model* m, int N, const double* F0, double E0, double cE, double cF, double* grad,
