@@ -26,14 +26,14 @@ __global__ void k_unpermute(int N, const int* __restrict__ perm, const double* _
 
 // Per-replica energy and virial: sums of the per-atom values (caller order), or for the
 // virial the per-replica accumulator vir_rep when the backward produced one.  Deterministic:
-// block (c, r) sums chunk c (kRedChunk atoms) of replica r over a fixed strided partition and a fixed
+// block (c, r) sums chunk c (`chunk` atoms) of replica r over a fixed strided partition and a fixed
 // tree of warp shuffles; with one chunk per replica it writes the result, otherwise its partial,
 // which k_rep_final adds in a fixed order.  NQ = 1 (no per-atom virial) or 10 quantities: FP64 adds are
 // slow here, and the mixed precisions paid for ten columns of zeros (9.8 us a call, now 2.9).
 constexpr int kRedThreads = 256;
 constexpr int kRedChunk = 2048;
 template <int NQ>
-__global__ void __launch_bounds__(kRedThreads) k_rep_reduce(int nrep, int nchunk, const int* __restrict__ rep_off,
+__global__ void __launch_bounds__(kRedThreads) k_rep_reduce(int nrep, int chunk, int nchunk, const int* __restrict__ rep_off,
                                                            const double* __restrict__ e_user,
                                                            const double* __restrict__ vir_user,
                                                            const double* __restrict__ vir_rep, double* energy,
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kRedThreads) k_rep_reduce(int nrep, int nchunk
   const int r = blockIdx.y, c = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (r >= nrep) return;
   const int rb = rep_off[r], re = rep_off[r + 1];
-  const int beg = min(re, rb + c * kRedChunk), end = min(re, beg + kRedChunk);
+  const int beg = min(re, rb + c * chunk), end = min(re, beg + chunk);
   double acc[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
@@ -205,9 +205,10 @@ dp_status launch_copy_params(Model* m, const void* theta, bool fp32, long long n
   return DP_OK;
 }
 
-// Chunk slots of the reduction workspace: every replica may need ceil(max_atoms / kRedChunk).
+// Chunk slots of the reduction workspace: one box in chunks of kRedChunk atoms, any replicas in chunks four times as
+// large (a replica may hold nearly all atoms).
 size_t rep_reduce_slots(int max_atoms, int max_reps) {
-  return (size_t)max_reps * ((size_t)max_atoms / kRedChunk + 1);
+  return (size_t)max_reps * ((size_t)max_atoms / (4 * kRedChunk) + 1) + (size_t)max_atoms / kRedChunk;
 }
 
 namespace {
@@ -215,13 +216,11 @@ namespace {
 // Per-replica sums of per-atom values (energy, and the per-atom virial unless vir_rep holds it).
 dp_status launch_rep_reduce(Model* m, const double* e_user, const double* vir_user, const double* vir_rep,
                             double* energy, double* virial, const int* err) {
-  const int nchunk = std::max(1, (m->max_rep_atoms + kRedChunk - 1) / kRedChunk);
-  if (nchunk > 1 && (size_t)m->nrep * nchunk > m->red_cap) {
-    m->last_error = "reduction workspace too small";
-    return DP_ERR_CAPACITY;
-  }
+  int chunk = kRedChunk;
+  while ((size_t)m->nrep * cdiv(m->max_rep_atoms, chunk) > m->red_cap) chunk *= 2;  // ends at 4 kRedChunk
+  const int nchunk = std::max(1, cdiv(m->max_rep_atoms, chunk));
   const auto fn = vir_user ? k_rep_reduce<10> : k_rep_reduce<1>;
-  fn<<<dim3(nchunk, m->nrep), kRedThreads, 0, m->stream>>>(m->nrep, nchunk, m->rep_off_dev, e_user, vir_user, vir_rep,
+  fn<<<dim3(nchunk, m->nrep), kRedThreads, 0, m->stream>>>(m->nrep, chunk, nchunk, m->rep_off_dev, e_user, vir_user, vir_rep,
                                                            energy, virial, m->red_part, err);
   m->launches += 1;
   if (nchunk > 1) {
