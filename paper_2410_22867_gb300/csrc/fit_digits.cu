@@ -124,14 +124,27 @@ template <> struct Sum<float> {
   __device__ __forceinline__ void add(const float (*acc)[4], int e) { s += dig::join_f(acc, e); }
   __device__ __forceinline__ float value() const { return s; }
 };
-__device__ __forceinline__ double out_scale(int e, int sw, double) {  // 2^(40 - (54 - e) - sw)
-  return e > 1024 ? __longlong_as_double(0x7ff8000000000000ll) : dig::pow2d(min(max(40 - 54 + e - sw, -1022), 1023));
-}
-__device__ __forceinline__ float out_scale(int e, int sw, float) {    // 2^(36 - (26 - e) - sw), down to the subnormals
-  if (e > 128) return __int_as_float(0x7fc00000);
-  const int x = 36 - 26 + e - sw;
-  return __int_as_float(x >= -126 ? (127 + min(x, 127)) << 23 : x >= -149 ? 1 << (x + 149) : 0);
-}
+// The unit of a product is that of its row (|a| < 2^e) times that of its column (|w| 2^sw within the digits' range):
+// 2^(40 - (54 - e) - sw) in FP64 (exponents added: the FP64 pipe is scarce), 2^(36 - (26 - e) - sw) in FP32 (two normal
+// numbers multiplied).  A row that is not finite: NaN.
+template <class T> struct Units;
+template <> struct Units<double> {
+  using V = int;
+  static constexpr int kBad = 1 << 20;
+  __device__ static __forceinline__ V row(int e) { return e > 1024 ? kBad : e - 34; }
+  __device__ static __forceinline__ V col(int sw) { return 20 - sw; }
+  __device__ static __forceinline__ double both(V r, V c) {
+    return r == kBad ? __longlong_as_double(0x7ff8000000000000ll) : dig::pow2d(min(max(r + c, -1022), 1023));
+  }
+};
+template <> struct Units<float> {
+  using V = float;
+  __device__ static __forceinline__ V row(int e) {
+    return e > 128 ? __int_as_float(0x7fc00000) : __int_as_float((127 + e - 8) << 23);
+  }
+  __device__ static __forceinline__ V col(int sw) { return __int_as_float((127 + 18 - sw) << 23); }
+  __device__ static __forceinline__ float both(V r, V c) { return r * c; }
+};
 
 // The fragments run through shared memory in stages of KS k steps by cp.async, ST stages deep: one pipeline for
 // the warps that share a part of K (they multiply the same fragments).  Loads straight
@@ -269,6 +282,14 @@ __global__ void __launch_bounds__(32 * kWarps, sizeof(T) == 8 ? 1 : 2) k_dig_gem
     __syncthreads();
   }
   if (r0 >= rows) return;
+  using U = Units<T>;
+  const typename U::V ru[2] = {U::row(ea[0]), U::row(ea[1])};
+  typename U::V cu[NT][2];
+#pragma unroll
+  for (int n = 0; n < NT; ++n)
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+      cu[n][c] = ntile0 + n < ntiles ? U::col(ws[8 * (ntile0 + n) + 2 * tq + c]) : typename U::V(0);
   const T* bias = g.bias + (long)ty * g.stride;
   const T* resv = g.res + (g.res_vec ? (long)ty * g.stride : 0);
 #pragma unroll
@@ -287,7 +308,7 @@ __global__ void __launch_bounds__(32 * kWarps, sizeof(T) == 8 ? 1 : 2) k_dig_gem
     const bool in = ok[r] && ntile0 + n < ntiles;
     T out = T(0);
     if (in) {
-      v *= out_scale(ea[r], ws[col], T(0));
+      v *= U::both(ru[r], cu[n][e & 1]);
       const size_t o = (base + r0 + gr + 8 * r) * mt.N + col;
       if (g.mode == EPI_TANH) {
         out = gtanh(v + bias[col]);
