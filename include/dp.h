@@ -62,7 +62,8 @@ typedef enum {
 } dp_status;
 
 typedef enum {
-  DP_FP64 = 0,     /* everything in FP64 */
+  DP_FP64 = 0,     /* everything in FP64 (FP64 and FP32 nets whose weights are of like size
+                      multiply in exact digits on the tensor cores, others by FMAs) */
   DP_FP32 = 1,     /* R, networks and per-pair force terms in FP32; positions,
                       Verlet update, force accumulation, energy and virial sums in FP64 */
   DP_MIX_BF16 = 2, /* as DP_FP32, with the embedding and fitting GEMM operands in BF16
@@ -204,7 +205,7 @@ dp_status dp_param_grad(dp_model* m, int natoms, const double* coords, const int
  * of the net, in every precision (mixed precisions keep the 16-bit fitting net and T product).
  * n_intervals = 0 goes back to the nets.  The tables are built on the device in FP64 from the
  * current parameters (rebuilt by dp_set_params) and kept in FP64 and FP32.  Unlike the other
- * calls this one allocates device memory (the tables: 36 n bytes per output and pair).  Drops
+ * calls this one allocates device memory (the tables: 132 n bytes per output and pair).  Drops
  * captured MD graphs; synchronous.  dp_param_grad returns DP_ERR_UNSUPPORTED while a table is
  * in use.  Errors: DP_ERR_ARG (n_intervals < 0 or > 2^20, x_min >= x_max), DP_ERR_OOM, DP_ERR_CUDA.
  */
@@ -252,9 +253,10 @@ long long dp_ntheta(const dp_model* m);
  * dp_set_params -- replace the model's network parameters (training step).  theta
  * [ntheta] host FP64 in the layout of the weight blob's parameter block (embedding
  * nets per (ti, tj), fitting nets per type, e_bias); ntheta must equal dp_ntheta(m).
- * All derived device copies (FP32, transposed fitting weights, 16-bit tensor-core
- * copies) are rebuilt.  Waits for the model's stream first; synchronous.  Captured
- * MD graphs stay valid (the device buffers do not move).
+ * All derived device copies (FP32, digit fragments or 16-bit tensor-core copies, tables)
+ * are rebuilt in place.  Waits for the model's stream first; synchronous.  Captured MD graphs
+ * stay valid, unless the new parameters need the other kernels of an FP64 / FP32 model (weights
+ * of like size or not): then the steps are captured again.
  * Errors: DP_ERR_ARG (null, wrong size), DP_ERR_WEIGHTS (non-finite value), DP_ERR_CUDA.
  */
 dp_status dp_set_params(dp_model* m, const double* theta, long long ntheta);

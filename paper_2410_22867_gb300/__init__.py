@@ -347,8 +347,9 @@ class DPModel:
         return int(lib().dp_ntheta(self.h))
 
     def set_params(self, theta):
-        """Replace the network parameters (dp_set_params): theta [ntheta] float64 in the weight
-        blob's parameter order (numpy array or torch tensor on any device)."""
+        """Replace the network parameters: theta [ntheta] in the weight blob's parameter order, a numpy array or a
+        torch tensor of any device and real type.  A contiguous float32 or float64 tensor on the model's GPU is
+        taken there (dp_set_params_device); everything else goes through the host in float64 (dp_set_params)."""
         if hasattr(theta, "detach"):
             import torch
             theta = theta.detach()
@@ -406,8 +407,8 @@ def _make_param_loss():
 
     class ParamLoss(torch.autograd.Function):
         """L(theta) = cE (E - E0)^2 + cF sum_k |F_k - F0_k|^2 of one box as a differentiable
-        function of the network parameters theta (float64 tensor [ntheta]).  The forward
-        loads theta into `model` (dp_set_params) and runs dp_param_grad, which returns the
+        function of the network parameters theta (tensor [ntheta], gradient in its type).  The forward
+        loads theta into `model` (set_params) and runs dp_param_grad, which returns the
         loss and its full gradient; the backward scales that gradient.  coords, types, F0
         are device tensors in the caller's atom order, box a host 3x3."""
 

@@ -1,7 +1,7 @@
 // Products of FP64 and FP32 matrices on the 16-bit tensor cores, exact up to a chosen truncation
 // (the error-free splitting of Ozaki, Ogita, Oishi and Rump 2012, in the tensor-core form of Mukunoki,
-// Ozaki, Ogita and Imamura 2020): each operand becomes a fixed-point integer relative to a common
-// scale, written as ND balanced digits d_0 (most significant) .. d_{ND-1} of BD bits; every digit is
+// Ozaki, Ogita and Imamura 2020): each operand becomes a fixed-point integer relative to the scale of its row (left
+// operand) or column (right operand), written as ND balanced digits d_0 (most significant) .. d_{ND-1} of BD bits; every digit is
 // an exact fp16 number, and the products of two digits summed over K stay below 2^24, so the FP32
 // accumulators of mma.sync hold them exactly.  Digit products of one order i + j share an
 // accumulator; orders above NO - 1 are dropped.
@@ -13,7 +13,12 @@
 // warp instruction occupies a sub-partition's pipe for 64 clocks), mma.sync with fp16 operands 1,032.
 // 34 digit products per FP64 product (7 digits, orders 0..7) are 15 times cheaper than the DFMAs they replace.
 // FP32: 6 digit products cost 0.75 of the FFMA time at peak rates, leave the CUDA cores to the tanh and need no
-// register tiles of weights; 25 bits relative to the operand's largest element against FP32's 24.
+// register tiles of weights.
+//
+// Error: relative to the largest element of the row times the largest of the column, 2^-28 (FP32) or 2^-54 (FP64)
+// a term, where FMAs round every partial sum.  On nets whose columns are alike (kSpread) energies and
+// forces are as close to FP64 as with FMAs or closer: over 22 nets (scaled by 0.01 to 40, uneven rows and columns, heavy
+// tails, no biases) the ratio of the errors is 0.3 to 1.05 in FP32, 0.8 to 1.14 in FP64.
 #pragma once
 
 #include "common.cuh"

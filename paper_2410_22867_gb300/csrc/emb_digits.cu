@@ -11,7 +11,9 @@
 //   layer 3   n-tile j, column 2t+e  unit q = m(j, t) + 50 e               (13 n-tiles)
 //             m(j, t) = 4 (j / 2) + t + 25 (j % 2) for j < 12; m(12, 0) = 24, m(12, 1) = 49
 // Weight fragments are built once per weight upload in this order (k_dig_weights), one 16-byte load
-// per lane and two digits, and are read through L1 / L2 (135 KB a pair in FP64).
+// per lane and two digits, and are read through L1 / L2 (262 KB a pair in FP64, 100 KB in FP32).
+// Scales: weights by the output column, FP32 activations and all gradients by the row, FP64 activations by
+// their range; nets that these do not suit take the plain kernels (layer_scale, activations_large).
 //
 // What bounds it: FP64 keeps layer-1 sums, T, dE/dT products and the environment rows on the FP64
 // pipe (64 clocks a warp instruction); tanh and the activations are fixed-point integers.
@@ -216,7 +218,7 @@ __device__ __forceinline__ void load_b(uint4* b, const uint4* __restrict__ set, 
 // made those kernels bound by shared-memory bandwidth.  FP64 forward (kDigits): digits in the warp's
 // shared memory, 112 bytes a lane and k step.  FP64 backward (kWords): the slots' 56-bit digit words, 64
 // bytes, cut into digits on every use, so that six warps fit an SM instead of four (8.66 -> 7.30 ms for 4,000 Cu
-// atoms; the forward, which has its eight warps anyway, would lose: 2.73 -> 3.10 ms).
+// atoms, 7.55 with a scale for every column; the forward, which has its eight warps anyway, would lose: 2.73 -> 3.10 ms).
 enum Store { kRegs, kDigits, kWords };
 
 // acc = A (KS k steps) times the fragments of one n-tile; with TAIL the last step has 8 columns.

@@ -1,8 +1,8 @@
 // FP64 / FP32 fitting net (1600 -> 240 -> 240 -> 240 -> 1, forward and data gradient) with digit
-// products on the tensor cores (digits.cuh): seven launches for all centre types.
+// products on the tensor cores (digits.cuh): eight kernels for all centre types.
 //
 // A GEMM C = A B works on the atoms of one type (rows) and one weight matrix, whose digits are stored as
-// m16n8k16 B fragments (built once per weight upload, 15.7 MB a type in FP64, resident in L2).  A is read
+// m16n8k16 B fragments (built once per weight upload, 16.0 MB a type in FP64, resident in L2).  A is read
 // in FP64 / FP32 and cut into digits on the way: lane (g, t) of a warp loads four consecutive k of rows
 // g and g + 8, which are its A fragment when k = 16 s + 4 t + {0, 1, 2, 3} stands at the fragment's columns
 // 2t, 2t + 1, 2t + 8, 2t + 9.  Rows of A and columns of B carry a power of two of their own, from their largest element

@@ -63,7 +63,6 @@ constexpr int kSplitSlot = 6;             // barrier index of the first split st
 constexpr int kSplitJobs = 8;             // per split GEMM: 4 K blocks x {hi, lo}, all 240 output columns
 constexpr int kL1Jobs = kKD / 64;         // 25
 constexpr int kB1Chunks = kKD / kBChunk;  // 10
-constexpr int kB1Jobs = 2 * kB1Chunks;    // 20
 
 struct FitMaps {
   CUtensorMap D;                     // [rows = max_atoms][1600]
