@@ -214,15 +214,15 @@ TANH_PER_NEIGHBOUR = 175
 # and its SHA-1 at the capture: when the file has changed since, the figure no longer describes
 # the kernel and `traffic` is reported as null.
 TRAFFIC_PER_ROW = {
-    ("embedding_backward", "mix_fp16"): {"bytes_per_unit": (171.784448e6 + 4.521984e6) / 5726060, "unit": "row",
+    ("embedding_backward", "mix_fp16"): {"bytes_per_unit": (171.547136e6 + 3.744768e6) / 5726060, "unit": "row",
                                          "source": "paper_2410_22867_gb300/csrc/mix_embed.cu",
-                                         "sha1": "6f6ae8c2452f3221d1e7684b71aefd4ddf1483f5"},
-    ("embedding_forward", "mix_fp16"): {"bytes_per_unit": (95.683328e6 + 21.243904e6) / 5726060, "unit": "row",
+                                         "sha1": "d56b31cc32ba327024a1ee9d6c9f317e2b88540d"},
+    ("embedding_forward", "mix_fp16"): {"bytes_per_unit": (95.686912e6 + 21.238528e6) / 5726060, "unit": "row",
                                         "source": "paper_2410_22867_gb300/csrc/mix_embed.cu",
-                                        "sha1": "6f6ae8c2452f3221d1e7684b71aefd4ddf1483f5"},
-    ("fitting", "mix_fp16"): {"bytes_per_unit": (106.631680e6 + 75.120640e6) / 32000, "unit": "atom",
+                                        "sha1": "d56b31cc32ba327024a1ee9d6c9f317e2b88540d"},
+    ("fitting", "mix_fp16"): {"bytes_per_unit": (106.717952e6 + 75.449600e6) / 32000, "unit": "atom",
                               "source": "paper_2410_22867_gb300/csrc/mix_fit.cu",
-                              "sha1": "a9afad59b8d8cbab7736d97dcdeeb23fd961956c"},
+                              "sha1": "055dc06088903dde54ba7679fc6f4fbfd02b0d19"},
 }
 
 
