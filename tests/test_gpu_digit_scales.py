@@ -197,3 +197,36 @@ def test_fp32_force_sums_are_fp64(n):
     f = m.compute(torch.tensor(s.coords, device="cuda"), torch.tensor(s.types, device="cuda"), s.box)["forces"].cpu().numpy()
     net = np.abs(f.astype(np.longdouble).sum(0)).max()
     assert float(net) <= 0.02 * 2.0 ** -53 * np.sqrt(2 * 95 * s.natoms) * np.abs(f).max()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("nmol", [21, 22, 64, 65])
+def test_plain_kernels_in_a_box(prec, nmol):
+    """Both nets by FMAs, at the edges of the fitting GEMM's 64-row blocks (one, two and three of hydrogens)."""
+    import paper_2410_22867_gb300 as dp
+    s = synth.water_box(nmol, nmol)
+    w = synth.xavier_weights(("O", "H"), 6.0, 0.5, (46, 92), 1001, fit_gain=10.0)
+    for ti, tj in _pairs():
+        w.block(f"emb{ti}{tj}.W3")[3, 7] = 3.0
+    for t in range(2):
+        w.block(f"fit{t}.W2")[3, 7] = 2.0
+    ref = oracle.Model(w.to_blob()).compute(s.coords, s.types, s.box)
+    m = dp.DPModel(w, prec, max_atoms=s.natoms)
+    e = errors(m.compute(torch.tensor(s.coords, device="cuda"), torch.tensor(s.types, device="cuda"), s.box), ref, s.types)
+    m.close()
+    assert e["ei_rel"] <= BARS[prec][0] and e["f_rel"] <= BARS[prec][1], e
+
+
+# 40 times larger embedding weights carry 40 times the error of the sums; at 1e6 (plain kernels) tanh is a step whose rare
+# unsaturated places carry 1e6 times it
+@pytest.mark.parametrize("prec,scale,f_bar", [("fp32", 40.0, 40 * BARS["fp32"][1]), ("fp64", 1e6, 1e6 * BARS["fp64"][1])])
+def test_forces_of_large_embedding_weights(prec, scale, f_bar):
+    import paper_2410_22867_gb300 as dp
+    from test_gpu_digits import _weights
+    x, t, box = _cluster(66, 66)
+    w = _weights(scale)
+    ref = oracle.Model(w.to_blob()).compute(x, t, box)
+    m = dp.DPModel(w, prec, max_atoms=66)
+    e = errors(m.compute(torch.tensor(x, device="cuda"), torch.tensor(t, device="cuda"), box), ref, t)
+    m.close()
+    assert e["ei_rel"] <= 40 * BARS["fp32"][0] and e["f_rel"] <= f_bar, e
