@@ -1102,9 +1102,9 @@ bool even_column(const double* w, int n, int stride) {
 
 // Scales of one layer (K x N weights W, biases b, |inputs| <= in, FP64 activations with sh fraction bits): sw, zs and s
 // of every column, swt of every row; false when the weights are outside the range the fixed-point layer covers
-// (or not finite), or spread too far.
-bool layer_scale(const double* W, const double* b, int K, int N, double in, bool fp64, int sh, int* sw, int* zs, int* s,
-                 int* swt) {
+// (or not finite), or with `even` spread too far.
+bool layer_scale(const double* W, const double* b, int K, int N, double in, bool fp64, bool even, int sh, int* sw, int* zs,
+                 int* s, int* swt) {
   std::vector<double> row(K, 0.0);
   for (int n = 0; n < N; ++n) {
     double top = 0.0, sum = std::fabs(b[n]);
@@ -1115,7 +1115,7 @@ bool layer_scale(const double* W, const double* b, int K, int N, double in, bool
       row[k] = std::fmax(row[k], v);
       sum += in * v;
     }
-    if (!(sum <= 1048576.0) || !even_column(W + n, K, N)) return false;
+    if (!(sum <= 1048576.0) || (even && !even_column(W + n, K, N))) return false;
     sw[n] = digit_scale(top, fp64, fp64 ? -12 : -100);
     zs[n] = std::min(56, 60 - (sum > 1.0 ? ceil_log2(sum) : 0));
     s[n] = 72 + zs[n] - sh - sw[n];
@@ -1126,7 +1126,7 @@ bool layer_scale(const double* W, const double* b, int K, int N, double in, bool
     if (fp64 && (s[n] < 1 || zs[n] < 40)) return false;
   }
   for (int k = 0; k < K; ++k) {
-    if (!even_column(W + (size_t)k * N, N, 1)) return false;
+    if (even && !even_column(W + (size_t)k * N, N, 1)) return false;
     swt[k] = digit_scale(row[k], fp64, -100);
   }
   return true;
@@ -1169,13 +1169,16 @@ dp_status upload(Model* m) {
   constexpr int bits = Fmt<T>::BD * Fmt<T>::ND;
   constexpr bool d = sizeof(T) == 8;
   std::vector<PairScale> sc(np);
+  // The plain FP64 kernels keep all pairs of a centre type in shared memory, which holds three: four types multiply in
+  // digits whatever their spread.
+  const bool even = !d || m->ntypes <= 3;
   m->dig_ok = true;
   for (int p = 0; p < np; ++p) {
     const double* W = m->theta_host.data() + (size_t)p * kEmbParams;
     PairScale& q = sc[p];
-    m->dig_ok = m->dig_ok && layer_scale(W + kEW2, W + kEb2, kN1, kN2, 1.0, d, bits - 2, q.sw2, q.zs2, q.s2, q.swt2) &&
-                layer_scale(W + kEW3, W + kEb3, kN2, kN3, 2.0, d, bits - 3, q.sw3, q.zs3, q.s3, q.swt3) &&
-                (!d || m->ntypes > 3 || activations_large(m, W, p / m->ntypes));  // four types: the plain FP64 kernels do not fit
+    m->dig_ok = m->dig_ok && layer_scale(W + kEW2, W + kEb2, kN1, kN2, 1.0, d, even, bits - 2, q.sw2, q.zs2, q.s2, q.swt2) &&
+                layer_scale(W + kEW3, W + kEb3, kN2, kN3, 2.0, d, even, bits - 3, q.sw3, q.zs3, q.s3, q.swt3) &&
+                (!d || !even || activations_large(m, W, p / m->ntypes));
   }
   if (!m->dig_ok) return DP_OK;
   unsigned char* base = static_cast<unsigned char*>(m->dig_emb);

@@ -230,3 +230,26 @@ def test_forces_of_large_embedding_weights(prec, scale, f_bar):
     e = errors(m.compute(torch.tensor(x, device="cuda"), torch.tensor(t, device="cuda"), box), ref, t)
     m.close()
     assert e["ei_rel"] <= 40 * BARS["fp32"][0] and e["f_rel"] <= f_bar, e
+
+
+@pytest.mark.parametrize("kind", ["even", "outlier", "small"])
+def test_four_types_fp64(kind):
+    """FP64 models of four atom types have no plain embedding kernels: digits take them whatever their spread (bars of the
+    other FP64 tests)."""
+    import paper_2410_22867_gb300 as dp
+    x, t, box = _cluster(40, 40)
+    t = (np.arange(40) % 4).astype(np.int32)
+    w = synth.xavier_weights(("A", "B", "C", "D"), 6.0, 0.5, (20, 20, 20, 20), 1001)
+    for ti in range(4):
+        for tj in range(4):
+            if kind == "outlier":
+                w.block(f"emb{ti}{tj}.W3")[3, 7] = 100.0
+            if kind == "small":
+                w.block(f"emb{ti}{tj}.W1")[...] *= 1e-2
+                for k in ("b1", "b2", "b3"):
+                    w.block(f"emb{ti}{tj}.{k}")[...] = 0.0
+    ref = oracle.Model(w.to_blob()).compute(x, t, box)
+    m = dp.DPModel(w, "fp64", max_atoms=40)
+    e = errors(m.compute(torch.tensor(x, device="cuda"), torch.tensor(t, device="cuda"), box), ref, t)
+    m.close()
+    assert e["ei_rel"] <= 1e-10 and e["f_rel"] <= 1e-9, e

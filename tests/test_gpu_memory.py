@@ -3,6 +3,8 @@ one area, since they are never in use together.  2,048 water atoms in FP32, from
 33 KB an atom of lists and evaluation buffers (65 MiB), the weights and their copies (30 MiB), the gradient's two
 T arrays (12.5 MiB) and the larger of its areas, 32,768 rows of 709 values (89 MiB): 197 MiB, and 10% for the
 granularity of the allocations."""
+import gc
+
 import pytest
 
 from paper_2410_22867_gb300 import synth
@@ -13,6 +15,7 @@ pytestmark = pytest.mark.gpu
 
 def test_gradient_areas_are_shared():
     import paper_2410_22867_gb300 as dp
+    gc.collect()  # models of other tests
     dp.DPModel(synth.water_weights(), "fp32", max_atoms=64).close()  # what is allocated once per process
     torch.cuda.synchronize()
     before = torch.cuda.mem_get_info()[0]
@@ -32,6 +35,7 @@ def test_reduction_slots_of_many_replicas():
     w = synth.xavier_weights(("O", "H"), 3.0, 0.5, (8, 16), 1001)
 
     def taken(reps):
+        gc.collect()
         torch.cuda.synchronize()
         before = torch.cuda.mem_get_info()[0]
         m = dp.DPModel(w, "fp32", max_atoms=131072, max_replicas=reps, skin=0.5)
