@@ -260,6 +260,7 @@ inline cudaError_t ensure_smem(const void* fn, size_t smem, bool one_cta = false
                                one_cta ? (int)std::min<size_t>(100, (smem + 2048) * 100 / (228 * 1024) + 1)
                                        : (int)cudaSharedmemCarveoutMaxShared);
   if (err == cudaSuccess) done.push_back({fn, smem});
+  else cudaGetLastError();  // returned to the caller: another model's next launch check must not find it
   return err;
 }
 

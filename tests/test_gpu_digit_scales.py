@@ -233,15 +233,16 @@ def test_forces_of_large_embedding_weights(prec, scale, f_bar):
 
 
 @pytest.mark.parametrize("kind", ["even", "outlier", "small"])
-def test_four_types_fp64(kind):
-    """FP64 models of four atom types have no plain embedding kernels: digits take them whatever their spread (bars of the
-    other FP64 tests)."""
+@pytest.mark.parametrize("nt", [3, 4])
+def test_many_types_fp64(kind, nt):
+    """FP64 models of three atom types are the largest that the plain embedding kernels hold; with four, digits take them
+    whatever their spread (bars of the other FP64 tests)."""
     import paper_2410_22867_gb300 as dp
     x, t, box = _cluster(40, 40)
-    t = (np.arange(40) % 4).astype(np.int32)
-    w = synth.xavier_weights(("A", "B", "C", "D"), 6.0, 0.5, (20, 20, 20, 20), 1001)
-    for ti in range(4):
-        for tj in range(4):
+    t = (np.arange(40) % nt).astype(np.int32)
+    w = synth.xavier_weights(tuple("ABCD"[:nt]), 6.0, 0.5, (20,) * nt, 1001)
+    for ti in range(nt):
+        for tj in range(nt):
             if kind == "outlier":
                 w.block(f"emb{ti}{tj}.W3")[3, 7] = 100.0
             if kind == "small":
@@ -253,3 +254,19 @@ def test_four_types_fp64(kind):
     e = errors(m.compute(torch.tensor(x, device="cuda"), torch.tensor(t, device="cuda"), box), ref, t)
     m.close()
     assert e["ei_rel"] <= 1e-10 and e["f_rel"] <= 1e-9, e
+
+
+def test_a_refused_launch_leaves_other_models_alone():
+    """FP64 tables of four types do not fit shared memory: that model's call is refused, another model's calls run."""
+    import paper_2410_22867_gb300 as dp
+    x, t, box = _cluster(16, 16)
+    x, box0 = torch.tensor(x, device="cuda"), box
+    four = dp.DPModel(synth.xavier_weights(tuple("ABCD"), 6.0, 0.5, (20,) * 4, 1001), "fp64", max_atoms=16)
+    four.tabulate(16)
+    other = dp.DPModel(synth.xavier_weights(("O", "H"), 6.0, 0.5, (46, 92), 1001), "fp64", max_atoms=16)
+    tt = torch.tensor(t, device="cuda")
+    with pytest.raises(dp.DPError):
+        four.compute(x, tt, box0)
+    e = other.compute(x, tt, box0)["energy"]
+    assert torch.isfinite(e).all()
+    dp.DPModel(synth.water_weights(), "fp32", max_atoms=16).close()
